@@ -466,20 +466,10 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(bv[0]), "=f"(bv[1]), "=f"(bv[2]), "=f"(bv[3]) : "r"(ba));
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(bv[4]), "=f"(bv[5]), "=f"(bv[6]), "=f"(bv[7]) : "r"(ba + 16));
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
+            for (int e = 0; e < 8; ++e)
               if (add_bias) y[e] = __fadd_rn(y[e], bv[e]);
-              if (p.f.relu == 1) y[e] = fmaxf(y[e], 0.f);
-              else if (p.f.relu) y[e] = apply_activation(y[e], p.f.relu);
-            }
-            float uu[8];
-            float edge = ofast ? 0.f : 1.f;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) uu[e] = quant_magic(y[e], orcp, edge);
-            uint32_t w0 = pack4_low_bytes(uu[0], uu[1], uu[2], uu[3]), w1 = pack4_low_bytes(uu[4], uu[5], uu[6], uu[7]);
-            if (edge >= 0.5f) {   // some estimate sits on a rounding boundary (or the step has no usable reciprocal)
-              w0 = quant4(make_float4(y[0], y[1], y[2], y[3]), ostep, orcp, false);
-              w1 = quant4(make_float4(y[4], y[5], y[6], y[7]), ostep, orcp, false);
-            }
+            uint32_t w0, w1;
+            q8_codes8(y, p.f.relu, ostep, orcp, ofast, w0, w1);
             packed[2 * (sub + u)] = w0;
             packed[2 * (sub + u) + 1] = w1;
             continue;

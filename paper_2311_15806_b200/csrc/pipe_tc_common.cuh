@@ -154,24 +154,113 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, int (&v)[8]) {
                : "memory");
 }
 
-// The code clamp(rne(v / s)) of the fused inner-layer epilogue without a conversion instruction: the estimate
-// t = v * rn(1 / s), clamped to +-127 (a t beyond 127 has a true quotient above 126.9999, whose code is 127),
-// is added to 1.5 * 2^23, where the spacing of binary32 is one, so the addition itself rounds to the nearest
-// integer, ties to even, and leaves the code in the low byte of the sum.  `edge` collects the largest
-// |t - code| + |t| * 2^-21: at 0.5 or more an estimate lies so close to a rounding boundary that the IEEE
-// quotient, which defines the code, may round the other way, and the caller divides.
-__device__ __forceinline__ float quant_magic(float v, float r, float& edge) {
-  const float t = fminf(fmaxf(__fmul_rn(v, r), -127.f), 127.f);
+// The codes clamp(rne(sigma(v) / s)) of the fused inner-layer epilogue, eight at a time, without a conversion
+// instruction, a division or a full-precision exp / erf on the common path.  An estimate t of sigma(v) / s, clamped to
+// +-127 (a t beyond 127 has a true quotient above 126.9, whose code is 127), is added to 1.5 * 2^23, where the spacing
+// of binary32 is one, so the addition itself rounds to the nearest integer, ties to even, and leaves the code in the
+// low byte of the sum.  `edge` collects the largest |t - code| + (bound on the error of t): at 0.5 or more an estimate
+// lies so close to a rounding boundary that what DEFINES the code -- apply_activation in binary32, then the IEEE
+// quotient -- may round the other way, and codes4_exact evaluates the definition.  The codes are therefore the same
+// bits as with the definition everywhere.
+// Why: the drain is bound by its instructions.  With expf / erff and a division per output the SiLU and GeLU drains
+// took longer than the MMAs they should hide behind.  Measured before -> after (K = 4, M = 2, T = 4096): 4096 -> 11008
+// with SiLU 596 -> 342 us (fp32 output: 302), 768 -> 3072 with GeLU 175 -> 84 us (fp32 output: 57), and with ReLU, which
+// gains from the fallback being out of line, 86 -> 69 us.
+__device__ __forceinline__ float code_magic(float t, float err, float& edge) {
   const float u = __fadd_rn(t, 12582912.f);
   const float d = __fsub_rn(t, __fsub_rn(u, 12582912.f));
-  edge = fmaxf(edge, __fmaf_rn(fabsf(t), 4.76837158203125e-07f, fabsf(d)));
+  edge = fmaxf(edge, __fadd_rn(fabsf(d), err));
   return u;
+}
+__device__ __forceinline__ float ex2_approx(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+// sigma(v) for kinds 2 to 4 of apply_activation, estimated, and `slack`: a bound on the distance from apply_activation's
+// binary32 value as a fraction of |estimate| (SiLU, sigmoid) or of |v| (GeLU).
+//   SiLU v q and sigmoid q, q = 1 / (1 + 2^(-v log2 e)), on the approximate exponential and reciprocal: the rounded
+//     argument of the exponential contributes |v| 1.5 * 2^-24, the exponential 2^-22, the reciprocal, the other
+//     roundings and the reference's own less than 2^-21 together.  (Beyond v = -86 the exponential overflows and the
+//     estimate is 0 where sigma is below 1e-35: no usable step, all above 1e-30, makes that a code other than 0.)
+//   GeLU max(v, 0) - |v| h(|v|), h = (1 - erf(|v| / sqrt 2)) / 2 by formula 7.1.26 of Abramowitz and Stegun (absolute
+//     error 1.5e-7 in erf) with halved coefficients.
+// Over every binary32 v in +-80 the largest distance measured is 0.50 (SiLU), 0.39 (GeLU), 0.50 (sigmoid) of the bound.
+template <int KIND>
+__device__ __forceinline__ float smooth_estimate(float v, float& slack) {
+  if constexpr (KIND == 3) {
+    const float av = fabsf(v);
+    const float t = rcp_approx(__fmaf_rn(0.23164189f, av, 1.f));            // 0.3275911 / sqrt 2
+    const float e = ex2_approx(__fmul_rn(__fmul_rn(v, v), -0.72134752f));   // exp(-v^2 / 2)
+    float h = __fmaf_rn(t, 0.5307027145f, -0.7265760135f);
+    h = __fmaf_rn(t, h, 0.7107068705f);
+    h = __fmaf_rn(t, h, -0.142248368f);
+    h = __fmaf_rn(t, h, 0.127414796f);
+    h = __fmul_rn(__fmul_rn(t, h), e);
+    slack = 9.5367431640625e-07f;                                           // 2^-20
+    return __fmaf_rn(-av, h, fmaxf(v, 0.f));
+  } else {
+    const float q = rcp_approx(__fadd_rn(1.f, ex2_approx(__fmul_rn(v, -1.44269504f))));
+    slack = __fmaf_rn(fabsf(v), 1.1920928955078125e-07f, 1.430511474609375e-06f);   // |v| 2^-23 + 1.5 * 2^-20
+    return KIND == 2 ? __fmul_rn(v, q) : q;
+  }
+}
+
+// Four codes by the definition (out of line: the drain's loop is sensitive to its instruction footprint).
+static __device__ __noinline__ uint32_t codes4_exact(float a, float b, float c, float d, int kind, float s) {
+  return quant_lane_exact(apply_activation(a, kind), s) | (quant_lane_exact(apply_activation(b, kind), s) << 8) |
+         (quant_lane_exact(apply_activation(c, kind), s) << 16) | (quant_lane_exact(apply_activation(d, kind), s) << 24);
 }
 
 __device__ __forceinline__ uint32_t pack4_low_bytes(float a, float b, float c, float d) {
   const uint32_t ab = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x0040);
   const uint32_t cd = __byte_perm(__float_as_uint(c), __float_as_uint(d), 0x0040);
   return __byte_perm(ab, cd, 0x5410);
+}
+
+template <int KIND>
+__device__ __forceinline__ void smooth_codes8(const float (&y)[8], float r, float (&uu)[8], float& edge) {
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    float slack;
+    const float a = smooth_estimate<KIND>(y[e], slack);
+    const float t = fminf(fmaxf(__fmul_rn(a, r), -127.f), 127.f);
+    // + 2^-21 |t|: the product with rn(1 / s) in place of the IEEE quotient (for GeLU |t| <= |v| r up to the slack)
+    const float err = KIND == 3 ? __fmul_rn(fabsf(y[e]), __fmul_rn(r, slack + 4.76837158203125e-07f))
+                                : __fmul_rn(fabsf(t), __fadd_rn(slack, 4.76837158203125e-07f));
+    uu[e] = code_magic(t, err, edge);
+  }
+}
+
+// kind: the activation; s: the output step; r = rn(1 / s), usable when `fast`.
+__device__ __forceinline__ void q8_codes8(const float (&y)[8], int kind, float s, float r, bool fast, uint32_t& w0, uint32_t& w1) {
+  float uu[8];
+  float edge = fast ? 0.f : 1.f;
+  if (kind < 2) {
+    const float lo = kind == 1 ? 0.f : -127.f;   // ReLU: max(v, 0) r = max(v r, 0)
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const float t = fminf(fmaxf(__fmul_rn(y[e], r), lo), 127.f);
+      uu[e] = code_magic(t, __fmul_rn(fabsf(t), 4.76837158203125e-07f), edge);
+    }
+  } else if (kind == 2) {
+    smooth_codes8<2>(y, r, uu, edge);
+  } else if (kind == 3) {
+    smooth_codes8<3>(y, r, uu, edge);
+  } else {
+    smooth_codes8<4>(y, r, uu, edge);
+  }
+  w0 = pack4_low_bytes(uu[0], uu[1], uu[2], uu[3]);
+  w1 = pack4_low_bytes(uu[4], uu[5], uu[6], uu[7]);
+  if (edge >= 0.5f) {   // an estimate too close to a rounding boundary to decide (or the step has no usable reciprocal)
+    w0 = codes4_exact(y[0], y[1], y[2], y[3], kind, s);
+    w1 = codes4_exact(y[4], y[5], y[6], y[7], kind, s);
+  }
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -279,3 +279,24 @@ def test_requantized_convolution_matches_oracle(oracle, N, Hh, Ww, Cc, O, kh, kw
         torch.cuda.synchronize()
         assert B.pipe_poll_status() == B.PIPE_OK
         np.testing.assert_array_equal(y2.cpu().numpy().view(np.uint32), f2.y.view(np.uint32))
+
+
+@pytest.mark.parametrize("kernel", [B.KERNEL_TCGEN05, B.KERNEL_TCGEN05_PAIR])
+@pytest.mark.parametrize("act", [B.ACT_IDENTITY, B.ACT_RELU, B.ACT_SILU, B.ACT_GELU, B.ACT_SIGMOID])
+def test_estimated_codes_equal_the_definition(kernel, act):
+    """The tensor-core epilogues decide a code from an estimate of sigma(y) / step and evaluate the definition (binary32
+    sigma, IEEE division) only next to a rounding boundary; the CUDA-core kernel always evaluates it: the same bits.
+    A million outputs per step put some quotients within 2^-20 of a boundary; steps from one that leaves a handful of
+    codes over one that clamps most outputs to one whose reciprocal is not usable."""
+    H.ensure_built()
+    rng = np.random.default_rng(40 + act)
+    O, I, T = 512, 128, 2000
+    W = _w(rng, O, I) * 30.0                       # outputs of a few units, where the smooth functions bend
+    bias = rng.standard_normal(O).astype(np.float32)
+    layer = H.gpu_expand(H.desc_of(O, I, 4, 2, 8, 32), W)
+    xq, sx = H.gpu_quantize(rng.standard_normal((T, I)).astype(np.float32))
+    for step in (0.5, 0.031, 0.0171, 1e-4, 1e-31):
+        want, _ = H.gpu_ensemble_q8(layer, [xq], [sx], [step], bias, relu=act, kernel=B.KERNEL_REFERENCE, want_partials=False)
+        got, _ = H.gpu_ensemble_q8(layer, [xq], [sx], [step], bias, relu=act, kernel=kernel, want_partials=False)
+        assert B.pipe_poll_status() == B.PIPE_OK
+        np.testing.assert_array_equal(got[0], want[0])
