@@ -210,6 +210,12 @@ struct ForwardArgs {
   int64_t ldyq;
 };
 
+inline bool has_zero_point(const ForwardArgs& a) {
+  for (int m = 0; m < a.num_branches; ++m)
+    if (a.branch[m].zp) return true;
+  return false;
+}
+
 // Tensor map of a row-major byte matrix [rows, inner_bytes] with row pitch pitch_bytes (a multiple of 16) and
 // a box of box_inner x box_rows bytes; swizzle128 selects the 128-byte swizzle.  False when the driver entry
 // point is missing or the encoding fails.

@@ -91,11 +91,22 @@ static pipe_status run_forward(const LayerInfo& L, const void* d_blob, int M, co
 static pipe_status dispatch_forward(const ForwardArgs& a, const LayerInfo& L, int M, int64_t T, const int32_t* const* zp,
                                     cudaStream_t stream) {
   const int choice = kernel_choice();
-  if (zp) {   // asymmetric codes: the CUDA-core kernel folds the zero point in (the others decline)
+  if (zp) {
+    // asymmetric codes: the SM-pair kernel and, up to 15 tokens, the weight-streaming kernel form the row sums beside the
+    // products (row of ones); the CUDA-core kernel takes every other shape.  Measured against the CUDA-core kernel from
+    // 128 x 128 to 3072 x 3072 and 1 to 2048 tokens: equal (host-bound) at 128 x 128, faster everywhere else.
     if (static_cast<int64_t>(255) * L.qmax * L.I >= (static_cast<int64_t>(1) << 31)) return PIPE_ERR_ACC_OVERFLOW;
     for (int m = 0; m < M; ++m)
       if (reinterpret_cast<uintptr_t>(zp[m]) & 3) return PIPE_ERR_ALIGNMENT;
-    return (choice == 0 || choice == 1) ? forward_reference(a, stream) : PIPE_ERR_UNSUPPORTED;
+    if (choice == 1) return forward_reference(a, stream);
+    if (choice != 0) return PIPE_ERR_UNSUPPORTED;
+    // (the tensor-core accumulators hold 2^(8-b) times the sums)
+    pipe_status st = PIPE_ERR_UNSUPPORTED;
+    if (((static_cast<int64_t>(255) * L.qmax * L.I) << (8 - L.bits)) < (static_cast<int64_t>(1) << 31)) {
+      if (T <= 16) st = forward_stream(a, stream);
+      if (st == PIPE_ERR_UNSUPPORTED) st = forward_tcgen05_pair(a, stream);
+    }
+    return st == PIPE_ERR_UNSUPPORTED ? forward_reference(a, stream) : st;
   }
   if (choice == 1) return forward_reference(a, stream);
   if (choice == 2) return forward_tcgen05(a, stream);

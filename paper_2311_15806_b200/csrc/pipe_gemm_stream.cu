@@ -159,7 +159,10 @@ __device__ __forceinline__ int rows_before(const int32_t* cum, int c, int O, int
 // branches -- an absent chunk takes part with zero weights -- so that the slabs' load-and-MMA chains are one block the
 // compiler may interleave (cfg4a T = 1, five slabs per warp: 17.6 -> 16.8 us; cfg4b T = 1, two: 21.2 -> 19.4 us; with the
 // slots of the general kernel, five, a launch with two slabs per warp would do 2.5 times its work that way).
-template <int BITS, int NT, int NP, bool SUMMED, int FULL>
+// ZP: asymmetric activations, sum_i (c - z) q = sum_i c q - z sum_i q.  The last token column of the MMAs (7, or 15 with
+// two token tiles) is fed ones instead of a token, so its accumulators are the row sums of the codes; the epilogue reads
+// them from the neighbouring lane that holds that column.
+template <int BITS, int NT, int NP, bool SUMMED, int FULL, bool ZP>
 __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __grid_constant__ Params p) {
   constexpr int SPW = FULL ? FULL : ((NP * NT <= 2) ? 5 : (NP * NT == 4 ? 2 : 1));   // slabs per consumer warp and pass
   constexpr int CHK = 128 / BITS;               // codes per 16-byte chunk
@@ -451,6 +454,7 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
               const int r = gid + 8 * t;
               const int c16 = (within >> 4) + v;
               xv[v][t] = lds128(sgen, kbs * kXTile + r * 128 + ((c16 ^ (r & 7)) << 4));
+              if (ZP && t == NT - 1 && gid == 7) xv[v][t] = make_uint4(0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u);
             }
 #pragma unroll
           for (int s = 0; s < SPW; ++s) {
@@ -532,6 +536,8 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
         bool first_chain = true;
         int next_order = 1;   // orders below this one have had their predictor boundaries handled
         const float bv = biastab[li * 8 + gid];
+        int zp = 0;
+        if constexpr (ZP) zp = br.zp ? __ldg(br.zp) : 0;
         auto close_chain = [&]() {
 #pragma unroll
           for (int t = 0; t < NT; ++t)
@@ -567,11 +573,14 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
             if constexpr (SUMMED) close_up_to(ko);
             const float cs = cstab[(li * p.nkmax + ko) * 8 + gid];
             const int row = slabmeta[li * p.nkmax + ko] + gid, roff = p.f.order[br.k_begin + ko].row_off;
+            // (row gid's sums: column 8 NT - 1, i.e. the second column of lane 4 gid + 3's last token tile)
+            int zr = 0;
+            if constexpr (ZP) zr = zp * (__shfl_sync(0xffffffffu, a4[NT - 1][2 * half + 1], lane | 3) >> p.shift);
 #pragma unroll
             for (int t = 0; t < NT; ++t)
 #pragma unroll
               for (int e = 0; e < 2; ++e) {
-                const int a = a4[t][2 * half + e] >> p.shift;   // exact: the sum carries a factor 2^shift
+                const int a = (a4[t][2 * half + e] >> p.shift) - zr;   // exact: the sum carries a factor 2^shift
                 y[t][e] = __fmaf_rn(__int2float_rn(a), cs, y[t][e]);
                 const int tok = 8 * t + 2 * tig + e;
                 if (p.f.partials && tok < p.f.T) p.f.partials[static_cast<int64_t>(tok) * p.f.total_rows + roff + row] = a;
@@ -667,7 +676,9 @@ static bool kernel_info(void (*kern)(const Params), int dyn_wanted_or_0, int* sm
 
 static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, uint32_t split_mask = 0) {
   using namespace st;
-  if (a.T > 16 || a.g % 8 != 0 || a.O % 8 != 0) return PIPE_ERR_UNSUPPORTED;
+  const bool zp = has_zero_point(a);   // (its row sums take the place of a token)
+  if (a.T > (zp ? 15 : 16) || a.g % 8 != 0 || a.O % 8 != 0) return PIPE_ERR_UNSUPPORTED;
+  if (zp && a.q8_out) return PIPE_ERR_UNSUPPORTED;
   if (a.ldxq % 16 != 0) return PIPE_ERR_UNSUPPORTED;   // tensor-map row pitch
   for (int m = 0; m < a.num_branches; ++m)
     if (reinterpret_cast<uintptr_t>(a.branch[m].xq) & 15) return PIPE_ERR_UNSUPPORTED;
@@ -678,7 +689,7 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, uint
   p.f = a;
   p.prefetch = a.blob_settled ? 1 : 0;
   p.split_mask = split_mask;
-  const int nt = a.T <= 8 ? 1 : 2;
+  const int nt = a.T <= (zp ? 7 : 8) ? 1 : 2;
   const int np = max_cluster <= 2 ? 1 : (max_cluster <= 4 ? 2 : 4);
   const int spw = (np * nt <= 2) ? 5 : (np * nt == 4 ? 2 : 1);
   p.kblocks = ceil_div(a.I, 128);
@@ -692,28 +703,30 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, uint
   p.pass_slabs = kGroupWarps * spw;
   // (the kernel instantiation depends only on bits, tokens and orders, all known here)
   void (*kern)(const Params) = nullptr;
-#define PIPE_ST_PICK(B, S)                                                                     \
-  if (nt == 1) kern = np == 1 ? stream_forward_kernel<B, 1, 1, S, 0> : (np == 2 ? stream_forward_kernel<B, 1, 2, S, 0> : stream_forward_kernel<B, 1, 4, S, 0>); \
-  else kern = np == 1 ? stream_forward_kernel<B, 2, 1, S, 0> : (np == 2 ? stream_forward_kernel<B, 2, 2, S, 0> : stream_forward_kernel<B, 2, 4, S, 0>);
-  if (split_mask == 0) {
-    if (a.bits == 8) { PIPE_ST_PICK(8, false) } else if (a.bits == 4) { PIPE_ST_PICK(4, false) } else { PIPE_ST_PICK(2, false) }
+#define PIPE_ST_PICK(B, S, Z)                                                                  \
+  if (nt == 1) kern = np == 1 ? stream_forward_kernel<B, 1, 1, S, 0, Z> : (np == 2 ? stream_forward_kernel<B, 1, 2, S, 0, Z> : stream_forward_kernel<B, 1, 4, S, 0, Z>); \
+  else kern = np == 1 ? stream_forward_kernel<B, 2, 1, S, 0, Z> : (np == 2 ? stream_forward_kernel<B, 2, 2, S, 0, Z> : stream_forward_kernel<B, 2, 4, S, 0, Z>);
+  if (zp) {
+    if (a.bits == 8) { PIPE_ST_PICK(8, false, true) } else if (a.bits == 4) { PIPE_ST_PICK(4, false, true) } else { PIPE_ST_PICK(2, false, true) }
+  } else if (split_mask == 0) {
+    if (a.bits == 8) { PIPE_ST_PICK(8, false, false) } else if (a.bits == 4) { PIPE_ST_PICK(4, false, false) } else { PIPE_ST_PICK(2, false, false) }
   } else {   // a summed ensemble on a shared input: the epilogue that closes the predictors' chains
-    if (a.bits == 8) { PIPE_ST_PICK(8, true) } else if (a.bits == 4) { PIPE_ST_PICK(4, true) } else { PIPE_ST_PICK(2, true) }
+    if (a.bits == 8) { PIPE_ST_PICK(8, true, false) } else if (a.bits == 4) { PIPE_ST_PICK(4, true, false) } else { PIPE_ST_PICK(2, true, false) }
   }
 #undef PIPE_ST_PICK
   // the same kernel without per-slab branches, by slab slots per warp (one order pair; up to 8 tokens: 2 to 5 slots,
   // 9 to 16 tokens: 2 or 3 -- more would spill)
   auto full_kernel = [&](int slots) -> void (*)(const Params) {
-    if (split_mask != 0 || np != 1) return nullptr;
+    if (split_mask != 0 || np != 1 || zp) return nullptr;
 #define PIPE_ST_FULL(B)                                                                                       \
   if (nt == 1) {                                                                                              \
-    if (slots == 2) return stream_forward_kernel<B, 1, 1, false, 2>;                                          \
-    if (slots == 3) return stream_forward_kernel<B, 1, 1, false, 3>;                                          \
-    if (slots == 4) return stream_forward_kernel<B, 1, 1, false, 4>;                                          \
-    if (slots == 5) return stream_forward_kernel<B, 1, 1, false, 5>;                                          \
+    if (slots == 2) return stream_forward_kernel<B, 1, 1, false, 2, false>;                                          \
+    if (slots == 3) return stream_forward_kernel<B, 1, 1, false, 3, false>;                                          \
+    if (slots == 4) return stream_forward_kernel<B, 1, 1, false, 4, false>;                                          \
+    if (slots == 5) return stream_forward_kernel<B, 1, 1, false, 5, false>;                                          \
   } else {                                                                                                    \
-    if (slots == 2) return stream_forward_kernel<B, 2, 1, false, 2>;                                          \
-    if (slots == 3) return stream_forward_kernel<B, 2, 1, false, 3>;                                          \
+    if (slots == 2) return stream_forward_kernel<B, 2, 1, false, 2, false>;                                          \
+    if (slots == 3) return stream_forward_kernel<B, 2, 1, false, 3, false>;                                          \
   }
     if (a.bits == 8) { PIPE_ST_FULL(8) } else if (a.bits == 4) { PIPE_ST_FULL(4) } else { PIPE_ST_FULL(2) }
 #undef PIPE_ST_FULL
@@ -778,7 +791,7 @@ pipe_status forward_stream(const ForwardArgs& a, cudaStream_t stream) {
   const bool sum_mode = a.num_branches > 1 && a.branch[1].accumulate;
   if (!sum_mode) return launch_stream(a, stream);
   // predictors that share input and step: one launch on the cluster of all orders, the chains added in registers
-  if (!a.q8_out) {
+  if (!a.q8_out && !has_zero_point(a)) {
     bool shared = true;
     for (int m = 1; m < a.num_branches; ++m)
       shared = shared && a.branch[m].xq == a.branch[0].xq && a.branch[m].sx == a.branch[0].sx &&

@@ -33,6 +33,13 @@ constexpr int kSub = 2;              // reduction blocks per ring stage: every b
                                      // commit is paid once per stage, and each costs its thread on the order of a
                                      // hundred cycles, so a stage carries two blocks (eight MMAs)
 constexpr int kMaxN = 256;           // stacked weight rows per tile
+// Asymmetric activations (ZP): sum_i (c - z) q = sum_i c q - z sum_i q, and the row sums of the weight codes come out of
+// the MMAs themselves: the last row of every activation tile holds ones, so a tile carries 127 tokens per CTA and lane
+// 127 of its accumulators the sums (of the widened codes: 2^(8-b) times, like everything in the accumulator).  One row
+// in 128 is cheaper than summing the codes in the unpack warps, whose inner loop paces the long layers, and the
+// expanded layer needs no further section.  (768 -> 3072, int4, K = 4, M = 2, T = 709: 392 us on the CUDA-core kernel,
+// which alone took a zero point before, 27 us here; T = 2048: 1025 against 45 us.)
+constexpr int kTileTokensZp = kTileM - 1;
 constexpr int kMaxClusterOrders = 8;
 constexpr int kUnpackWarps = 6;   // 16 warps per CTA: 128 registers per thread (see the one-SM kernel)
 constexpr int kEpiWarps = 8;
@@ -448,6 +455,9 @@ struct EpiCtx {
   int part, nparts;  // share of the 16-channel groups this warp drains (two warps per lane quarter)
   float* stg;        // 32 rows x 16 floats, swizzled
   uint32_t zero_s;   // shared address of eight zero floats
+  const int* zp_s;   // ZP: zero point of every branch
+  int* zrow;         // ZP: [2][kMaxN] zero point times row sum of every stacked row, by accumulator buffer
+  uint32_t zbar0;    // ZP: 2 barriers, the buffer's products are complete
 };
 
 // Epilogue role (8 warps, one TMEM lane quarter each; a lane owns one token row of a token tile).
@@ -468,7 +478,7 @@ struct EpiCtx {
 // outputs are summed after the layer (Sec. 3.2): every predictor's chain starts from zero, the bias closes the first
 // one, and the chains are added in ascending predictor order in this thread -- the same additions, in the same
 // order, as one launch per predictor summing into y, without the read-modify-write of y.
-template <int NKMAX, bool PARTIALS, bool Q8, bool SUMMED, bool SHORT_K>
+template <int NKMAX, bool PARTIALS, bool Q8, bool SUMMED, bool SHORT_K, bool ZP>
 __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) {
   constexpr int CH = (NKMAX <= 2) ? 2 : 1;   // chunks per batch of accumulator loads
   // STRAIGHT: the chain of a chunk without branches (see below).  It trades some arithmetic on pruned (chunk, order)
@@ -540,7 +550,7 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
     // convolution the warp holds half of an 8 x 8 pixel patch (4 image rows of 8 pixels).
     const int ttile = 2 * t.tt + x.rank;
     bool tile_ok = ttile < p.ntok_tiles;
-    int64_t tok_base = static_cast<int64_t>(ttile) * kTileM + q * 32;
+    int64_t tok_base = static_cast<int64_t>(ttile) * (ZP ? kTileTokensZp : kTileM) + q * 32;
     int eh = 4, ew = 8;
     if (p.f.conv_on) {
       const int patch = 2 * ttile + (q >> 1);
@@ -555,21 +565,22 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
     // a patch on the right or lower edge of the output may hang over it
     auto inside = [&](int r) -> bool { return (r >> 3) < eh && (r & 7) < ew; };
     const int64_t tok_own = token_of(lane);
-    const bool own_ok = tile_ok && (p.f.conv_on ? inside(lane) : tok_own < p.f.T);
+    const bool own_ok = tile_ok && (p.f.conv_on ? inside(lane) : tok_own < p.f.T) && !(ZP && q == 3 && lane == 31);
     float* srow[4];        // the four rows this lane stores, at channel c0 + 4 * sj
     uint32_t srow_ok = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int64_t tok = token_of(sr0 + 8 * i);
       srow[i] = Q8 ? nullptr : br.y + tok * p.f.ldy + c0 + 4 * sj;
-      if (tile_ok && (p.f.conv_on ? inside(sr0 + 8 * i) : tok < p.f.T)) srow_ok |= 1u << i;
+      if (tile_ok && (p.f.conv_on ? inside(sr0 + 8 * i) : tok < p.f.T) && !(ZP && q == 3 && sr0 + 8 * i == 31)) srow_ok |= 1u << i;
     }
     const bool vec_ok = y_vec && ((reinterpret_cast<uintptr_t>(br.y) & 15) == 0);
     // Tensor stores (one per full 16-channel group, issued by one lane, straight from the staging block) where the
     // host found the output eligible: they leave the warp with neither the second pass over the staging block nor
     // the store instructions, and rows beyond T -- for a convolution, pixels beyond the image -- are clipped by
     // the copy engine.  A sum into y keeps the path through registers, which alone adds in binary32 round-to-nearest.
-    const bool tma_out = !Q8 && ((p.y_tma >> t.m) & 1u) && !br.accumulate && tile_ok;
+    // (ZP: the last quarter holds 31 tokens; its row of sums must not be stored over the next tile's first token)
+    const bool tma_out = !Q8 && ((p.y_tma >> t.m) & 1u) && !br.accumulate && tile_ok && !(ZP && q == 3);
     int ty1 = static_cast<int>(tok_base), ty2 = 0, ty3 = 0;   // coordinates behind the channel: token, or (x, y, image)
     if (p.f.conv_on) {
       const int patch = 2 * ttile + (q >> 1);
@@ -601,6 +612,27 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
     // over were computed after every epilogue warp of the pair had finished that tile.
     if (rec_issuer && tcount >= 1 && tile + x.npairs < x.num_tiles) fetch_record(tcount + 1, tile + x.npairs);
     const uint32_t tbase = x.tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * kAccCols;
+    if constexpr (ZP) {
+      // The two warps of the last lane quarter read the row of sums, half of the columns each.  (A buffer's products are
+      // rewritten two tiles later, when every warp has released the accumulators of this one.)
+      int* zr = x.zrow + buf * kMaxN;
+      if (q == 3) {
+        const int zp = x.zp_s[t.m];
+#pragma unroll 1
+        for (int c = x.part * 8; c < kMaxN; c += 8 * x.nparts) {
+          int v[8];
+          tmem_ld8(tbase + c, v);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (lane == 31) {
+            *reinterpret_cast<int4*>(zr + c) = make_int4(zp * v[0], zp * v[1], zp * v[2], zp * v[3]);
+            *reinterpret_cast<int4*>(zr + c + 4) = make_int4(zp * v[4], zp * v[5], zp * v[6], zp * v[7]);
+          }
+        }
+        if (lane == 31) mbar_arrive(x.zbar0 + 8u * buf);
+      }
+      __syncwarp();
+      if (!mbar_wait(x.zbar0 + 8u * buf, aph, x.abort_flag, p.f.status)) break;
+    }
     for (int grp = x.part; grp < ngrp && tile_ok; grp += x.nparts) {
       // bias of this lane's channel quad: needed in the store phase only, so its latency is hidden
       const bool quad_ok = 2 * grp + (sj >> 1) < nch;
@@ -681,6 +713,13 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
             const uint32_t ca = (STRAIGHT && cols[u][ko] < 0) ? x.zero_s : cscale_s + static_cast<uint32_t>(cols[u][ko] * 4);
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(cs[0]), "=f"(cs[1]), "=f"(cs[2]), "=f"(cs[3]) : "r"(ca));
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(cs[4]), "=f"(cs[5]), "=f"(cs[6]), "=f"(cs[7]) : "r"(ca + 16));
+            if constexpr (ZP) {
+              const int* zr = x.zrow + buf * kMaxN + (cols[u][ko] >= 0 ? cols[u][ko] : 0);
+              const int4 z0 = *reinterpret_cast<const int4*>(zr), z1 = *reinterpret_cast<const int4*>(zr + 4);
+              const int zz[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
+#pragma unroll
+              for (int e = 0; e < 8; ++e) acc[u][ko][e] -= zz[e];
+            }
             if constexpr (PARTIALS) {
 #pragma unroll
               for (int e = 0; e < 8; ++e) {
@@ -818,7 +857,7 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
   __syncwarp();
 }
 
-template <bool Q8, bool SUMMED, bool SHORT_K>
+template <bool Q8, bool SUMMED, bool SHORT_K, bool ZP = false>
 __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_constant__ Params p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t bars[2 * kMaxRing + 4];  // full[3] done[3] tmem_full[2] tmem_empty[2]
@@ -832,6 +871,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
   __shared__ __align__(16) float cfold_s[kRecBufs][kMaxN];            // s_k * lambda_x of the stacked rows of those tiles
   __shared__ uint64_t pre_bars[kRecBufs];
   __shared__ __align__(16) float zero8_s[8];
+  __shared__ __align__(16) int zrow_s[ZP ? 2 * kMaxN : 4];
+  __shared__ int zp_s[ZP ? PIPE_MAX_ORDERS : 1];
+  __shared__ uint64_t z_bars[2];
   __shared__ float sx_s[2 * PIPE_MAX_ORDERS];                        // lambda_x of every branch, then the fused epilogue's output steps
   __shared__ __align__(1024) float epi_stage[kEpiWarps][32 * 16];   // per epilogue warp: 32 token rows x 16 channels (the
                                                                     // source of tensor stores with the 64-byte swizzle)
@@ -869,6 +911,19 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
       else if (Q8) v = __ldg(p.f.branch[m].out_scale);
     }
     sx_s[i] = v;
+    if constexpr (ZP) {
+      if (i < PIPE_MAX_ORDERS) zp_s[i] = (m < p.f.num_branches && p.f.branch[m].zp) ? __ldg(p.f.branch[m].zp) : 0;
+    }
+  }
+  if constexpr (ZP) {
+    // the row of ones behind the 127 token rows of every activation tile of the ring (sixteen equal bytes per piece,
+    // whatever the swizzle does with the pieces); the copies never write it
+    for (int i = threadIdx.x; i < p.depth * kSub * (kKStep / 4); i += kThreads) {
+      const int w = i % (kKStep / 4), tile = i / (kKStep / 4);
+      uint8_t* row = g.stage_gen + (tile / kSub) * kStageBytes + (tile % kSub) * kABytes + kTileTokensZp * kKStep;
+      reinterpret_cast<uint32_t*>(row)[w] = 0x01010101u;
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (threadIdx.x == 0) {
     abort_flag_s = 0;
@@ -895,6 +950,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
     for (int b = 0; b < 2; ++b) {
       mbar_init(g.tfull0 + 8u * b, 1);
       mbar_init(g.tempty0 + 8u * b, 2 * kEpiWarps);
+      if (ZP) mbar_init(smem_u32(&z_bars[b]), 2);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -954,7 +1010,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
         const uint32_t dst = g.stage0 + rp.slot * kStageBytes + sub * kABytes + (p.f.conv_on ? half * (kABytes / 2) : 0);
         // reduction block kb = (filter tap, 128-channel chunk); the tap shifts the patch window
         const int c0 = p.f.conv_on ? chunk * kKStep : kb * kKStep;
-        const int c1 = p.f.conv_on ? p.f.csw * pw0 + tw - p.f.cpw : ttile * kTileM;
+        const int c1 = p.f.conv_on ? p.f.csw * pw0 + tw - p.f.cpw : ttile * (ZP ? kTileTokensZp : kTileM);
         const int c2 = p.f.csh * ph0 + th - p.f.cph;
         if (p.f.conv_on) {   // block kb + kSub, for the next stage
           chunk += kSub;
@@ -970,7 +1026,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
         // ahead of the MMAs, so the barrier's phase of the slot's use before may still be collecting its arrivals,
         // and an early arrival would be counted into that phase)
         if (!mbar_wait(g.done0 + 8u * rp.slot, rp.phase ^ 1, g.abort_flag, p.f.status)) break;
-        if (g.rank == 0 && lane == 0) mbar_expect_tx(g.full0 + 8u * rp.slot, 2 * nsub * kABytes);
+        if (g.rank == 0 && lane == 0) mbar_expect_tx(g.full0 + 8u * rp.slot, 2 * nsub * (ZP ? kTileTokensZp * kKStep : kABytes));
         if (sub >= nsub) continue;
         if (!p.f.conv_on) tma_pair_load_2d(dst, &p.tmap_a[m], c0, c1, bar);   // rows beyond T read zeros
         else tma_pair_load_4d(dst, &p.tmap_a[m], c0, c1, c2, pn, bar);
@@ -1062,14 +1118,17 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
     e.nparts = kEpiWarps / 4;
     e.stg = epi_stage[ew];
     e.zero_s = smem_u32(zero8_s);
+    e.zp_s = zp_s;
+    e.zrow = zrow_s;
+    e.zbar0 = smem_u32(z_bars);
     if (p.f.partials) {   // verification output: every integer accumulator is also written out
-      if (p.nkmax <= 2) epilogue_role<2, true, Q8, SUMMED, SHORT_K>(p, e);
-      else if (p.nkmax <= 4) epilogue_role<4, true, Q8, SUMMED, SHORT_K>(p, e);
-      else epilogue_role<8, true, Q8, SUMMED, SHORT_K>(p, e);
+      if (p.nkmax <= 2) epilogue_role<2, true, Q8, SUMMED, SHORT_K, ZP>(p, e);
+      else if (p.nkmax <= 4) epilogue_role<4, true, Q8, SUMMED, SHORT_K, ZP>(p, e);
+      else epilogue_role<8, true, Q8, SUMMED, SHORT_K, ZP>(p, e);
     } else {
-      if (p.nkmax <= 2) epilogue_role<2, false, Q8, SUMMED, SHORT_K>(p, e);
-      else if (p.nkmax <= 4) epilogue_role<4, false, Q8, SUMMED, SHORT_K>(p, e);
-      else epilogue_role<8, false, Q8, SUMMED, SHORT_K>(p, e);
+      if (p.nkmax <= 2) epilogue_role<2, false, Q8, SUMMED, SHORT_K, ZP>(p, e);
+      else if (p.nkmax <= 4) epilogue_role<4, false, Q8, SUMMED, SHORT_K, ZP>(p, e);
+      else epilogue_role<8, false, Q8, SUMMED, SHORT_K, ZP>(p, e);
     }
   }
 
@@ -1110,12 +1169,14 @@ static const DeviceSetup& device_setup() {
     int smem_max = 0, sms = 0;
     if (cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return;
-    cudaFuncAttributes f0, f1, f2;
+    cudaFuncAttributes f0, f1, f2, f3;
     if (cudaFuncGetAttributes(&f0, tc2_forward_kernel<false, false, false>) != cudaSuccess) return;
     if (cudaFuncGetAttributes(&f1, tc2_forward_kernel<true, false, false>) != cudaSuccess) return;
     if (cudaFuncGetAttributes(&f2, tc2_forward_kernel<false, true, false>) != cudaSuccess) return;
+    if (cudaFuncGetAttributes(&f3, tc2_forward_kernel<false, false, false, true>) != cudaSuccess) return;
     size_t fixed_b = f0.sharedSizeBytes > f1.sharedSizeBytes ? f0.sharedSizeBytes : f1.sharedSizeBytes;
     fixed_b = fixed_b > f2.sharedSizeBytes ? fixed_b : f2.sharedSizeBytes;
+    fixed_b = fixed_b > f3.sharedSizeBytes ? fixed_b : f3.sharedSizeBytes;
     const int fixed = static_cast<int>(fixed_b);
     d.depth = (smem_max - fixed - 1024) / kStageBytes;   // static shared memory, alignment slack
     if (d.depth > kMaxRing) d.depth = kMaxRing;
@@ -1128,6 +1189,7 @@ static const DeviceSetup& device_setup() {
     if (cudaFuncSetAttribute(tc2_forward_kernel<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
     if (cudaFuncSetAttribute(tc2_forward_kernel<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
     if (cudaFuncSetAttribute(tc2_forward_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
+    if (cudaFuncSetAttribute(tc2_forward_kernel<false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1184,7 +1246,10 @@ static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_
   const int row_bytes = direct ? round_up(a.I, kKStep) : a.kernel_row_bytes;   // bytes of a row over all reduction blocks
   if (direct) p.f.bits = 8;   // the kernel then treats the layer as one of int8 codes
   p.nkmax = max_cluster;
-  p.ntok_tiles = static_cast<int>(ceil_div<int64_t>(a.T, kTileM));
+  const bool zp = has_zero_point(a);   // asymmetric activations: 127 tokens per tile, see kTileTokensZp
+  const int tile_tokens = zp ? kTileTokensZp : kTileM;
+  if (zp && (a.conv_on || a.q8_out)) return PIPE_ERR_UNSUPPORTED;
+  p.ntok_tiles = static_cast<int>(ceil_div<int64_t>(a.T, tile_tokens));
   p.conv_pw = p.conv_pp = p.conv_np = p.conv_chunks = 1;
   if (a.conv_on) {
     p.conv_pw = ceil_div(a.cWo, 8);
@@ -1195,7 +1260,7 @@ static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_
   }
   // (a single token tile: the second CTA of a pair then stages zeros and stores nothing, but still unpacks its half of
   // every block, which is what such a launch spends its time on)
-  if (p.ntok_tiles == 1 && kernel_choice() == 0) {
+  if (p.ntok_tiles == 1 && kernel_choice() == 0 && !zp) {
     // ... unless the whole layer is a handful of blocks: then nothing is there to share and the one-SM kernel's shorter
     // set-up wins (a forced choice of this kernel still takes the launch)
     int64_t rows = 0;
@@ -1239,7 +1304,7 @@ static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_
   } else
   for (int m = 0; m < a.num_branches; ++m) {
     if (!make_map_2d(&p.tmap_a[m], a.branch[m].xq, static_cast<uint64_t>(a.I), static_cast<uint64_t>(a.T),
-                     static_cast<uint64_t>(a.ldxq), kKStep, kTileM, CU_TENSOR_MAP_SWIZZLE_128B))
+                     static_cast<uint64_t>(a.ldxq), kKStep, tile_tokens, CU_TENSOR_MAP_SWIZZLE_128B))
       return PIPE_ERR_CUDA;
   }
   // fp32 outputs that tensor stores can write: 16-byte aligned rows of at least one box
@@ -1270,7 +1335,8 @@ static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_
   cfg.numAttrs = 2;
   // (a reduction axis of at most 8 blocks: the drain paces the layer, see STRAIGHT in the epilogue)
   const bool short_k = p.kblocks <= 8;
-  const cudaError_t e = a.q8_out    ? (short_k ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<true, false, true>, p)
+  const cudaError_t e = zp          ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<false, false, false, true>, p)
+                        : a.q8_out  ? (short_k ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<true, false, true>, p)
                                                : cudaLaunchKernelEx(&cfg, tc2_forward_kernel<true, false, false>, p))
                         : split_mask ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<false, true, false>, p)
                         : short_k    ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<false, false, true>, p)
@@ -1287,7 +1353,7 @@ pipe_status forward_tcgen05_pair(const ForwardArgs& a, cudaStream_t stream) {
   // Predictors that share one input (the first layer of an ensemble, Sec. 3.2): ONE launch on the cluster of all
   // orders -- the activations are staged once, the MMAs run at the width of the whole cluster, and the epilogue
   // closes each predictor's chain and adds them in ascending order in registers.
-  if (a.sum_blk && a.sum_rec && !a.q8_out) {
+  if (a.sum_blk && a.sum_rec && !a.q8_out && !has_zero_point(a)) {
     bool shared = true;
     for (int m = 1; m < a.num_branches; ++m)
       shared = shared && a.branch[m].xq == a.branch[0].xq && a.branch[m].sx == a.branch[0].sx &&

@@ -138,7 +138,7 @@ def test_zero_point_forward_matches_the_oracle(oracle, O, I, T, bits, K, g, n_ke
         want_part[:, lo:hi] = f.partials[:, lo:hi]
         k0 += split[m]
     np.testing.assert_array_equal(part.cpu().numpy(), want_part)
-    # the tensor-core kernels decline the zero point instead of ignoring it
+    # a forced tensor-core kernel declines the zero point instead of ignoring it
     B.pipe_diag_select_kernel(B.KERNEL_TCGEN05)
     try:
         with pytest.raises(B.PipeError) as ei:
@@ -186,6 +186,47 @@ def test_unstructured_mask_matches_the_oracle(oracle, O, I, bits, K, g, keep_ele
     f = oracle.forward(e, xo, so)
     np.testing.assert_array_equal(part, f.partials)
     np.testing.assert_array_equal(y.view(np.uint32), f.y.view(np.uint32))
+
+
+# around the 7 / 15 tokens beside which the streaming kernel fits its column of ones and the 127 of a pair CTA's tile
+ZP_ROUTE_CASES = [
+    # O,   I,   bits, K, g, n_keep, M, int8_copy
+    (200, 144, 4, 4, 8, 9, 2, False),
+    (264, 1008, 8, 2, 8, 17, 1, False),
+    (320, 272, 2, 8, 16, 7, 4, False),
+    (136, 400, 3, 3, 8, 6, 1, True),
+]
+
+
+@pytest.mark.parametrize("T", [1, 7, 8, 15, 16, 126, 127, 128, 254, 255, 381])
+@pytest.mark.parametrize("O,I,bits,K,g,n_keep,M,int8_copy", ZP_ROUTE_CASES)
+def test_zero_point_on_the_tensor_cores_equals_the_cuda_core_kernel(O, I, bits, K, g, n_keep, M, int8_copy, T):
+    """The row sums formed beside the products give the bits of the CUDA-core kernel, which sums the codes themselves (and
+    is compared with the oracle above): outputs, partial sums, summed predictors, absent and extreme zero points."""
+    H.ensure_built()
+    rng = np.random.default_rng(3 * O + T)
+    W = _w(rng, O, I, heavy=(bits == 2))
+    bias = torch.from_numpy(rng.standard_normal(O).astype(np.float32)).cuda()
+    layer = H.gpu_expand(H.desc_of(O, I, bits, K, g, n_keep, M, int8_copy=int8_copy), W)
+    xq = [torch.from_numpy(rng.integers(-128, 128, (T, I)).astype(np.int8)).cuda() for _ in range(M)]
+    sx = [torch.tensor([0.01 * (1 + m)], device="cuda") for m in range(M)]
+    zp = [torch.tensor([z], dtype=torch.int32, device="cuda") for z in (-128, 127, 3)[:M]] + [None] * (M - 3)
+    R = layer.layout.total_rows
+    for sums in (False, True):
+        def run(choice):
+            ys = [torch.full((T, O), float("nan"), device="cuda") for _ in range(M)]
+            part = torch.zeros((T, R), dtype=torch.int32, device="cuda")
+            B.pipe_diag_select_kernel(choice)
+            try:
+                B.pipe_ensemble_forward_zp(layer.desc, layer.blob, xq, sx, zp, ys, bias, sums, part)
+            finally:
+                B.pipe_diag_select_kernel(B.KERNEL_AUTO)
+            torch.cuda.synchronize()
+            return [y.view(torch.int32) for y in (ys[:1] if sums else ys)] + [part]
+        want, got = run(B.KERNEL_REFERENCE), run(B.KERNEL_AUTO)
+        assert B.pipe_poll_status() == B.PIPE_OK
+        for a, b in zip(want, got):
+            assert torch.equal(a, b)
 
 
 @pytest.mark.parametrize("kernel", [B.KERNEL_REFERENCE, B.KERNEL_TCGEN05, B.KERNEL_TCGEN05_PAIR, B.KERNEL_STREAM, B.KERNEL_DECODE_TC, B.KERNEL_AUTO])
