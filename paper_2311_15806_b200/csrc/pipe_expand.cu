@@ -1,10 +1,12 @@
 // pipe_expand_weights: residual expansion of a weight matrix (Sec. 3.1, Eq. 2-3 and the masked
 // form), with the per-channel symmetric quantizer of Eq. 1.
 //
-// Per order: [group select, orders >= 2] -> one fused pass over the kept rows that (order 1: finds the
-// row maximum,) divides, rounds, packs both code layouts, updates the residual with one FMA per
-// element and leaves the next order's row absmax behind.  All kernels are
-// HBM-bound streaming passes: 128-bit loads, warp-shuffle reductions, one block per row.
+// Most layers: one pass over W that quantizes every row K times in registers, one block that decides which order keeps
+// which group, one copy of the kept rows' codes to their orders (expand_chain_kernel and behind it).
+// Masks over single weights, the L2 score and row lengths that path does not take, per order: [group select, orders >= 2]
+// -> one fused pass over the kept rows that (order 1: finds the row maximum,) divides, rounds, packs both code layouts,
+// updates the residual with one FMA per element and leaves the next order's row absmax behind: streaming passes,
+// 128-bit loads, warp-shuffle reductions, one block per row.
 #include <cstring>
 #include <mutex>
 
@@ -527,10 +529,9 @@ constexpr int kTableThreads = 256;
 // greedy rule "close the block when the next group would take it beyond the limit" needs, for a block that starts at
 // group b, the first group whose running sum from b exceeds the limit (or that would be the block's max_groups + 1-th):
 // the sums are non-decreasing, so the lanes test 32 candidates at a time and the first hit is the cut.
-__global__ void __launch_bounds__(kTableThreads) block_table_kernel(const __grid_constant__ BlockTableArgs a) {
+__device__ __forceinline__ void cut_table(const BlockTableArgs& a, const int m) {
   __shared__ int pre_s[kTableChunk];            // inclusive running sum of the chunk's rows
   __shared__ int part_s[kTableThreads];
-  const int m = blockIdx.x;
   int32_t* out = a.out[m];
   if (!out) return;
   int cur_rows = 0, cur_groups = 0, n = 0;      // (warp 0: the same in every lane)
@@ -604,6 +605,8 @@ __global__ void __launch_bounds__(kTableThreads) block_table_kernel(const __grid
     out[0] = n <= a.cap[m] ? n : 0;
   }
 }
+
+__global__ void __launch_bounds__(kTableThreads) block_table_kernel(const __grid_constant__ BlockTableArgs a) { cut_table(a, blockIdx.x); }
 
 // Block records (layout in pipe.h): one thread block per (block of a table, table).
 struct BlockRecordArgs {
@@ -681,8 +684,481 @@ __global__ void block_record_kernel(const __grid_constant__ BlockRecordArgs a) {
   }
 }
 
-__global__ void write_header_kernel(uint32_t* hdr, pipe_layer_desc d) {
-  if (threadIdx.x == 0) {
+// ------------------------------------------------------------------------------------------------
+// The expansion with ONE pass over the weights.
+//
+// How often a row has been quantized decides its residual: the residual entering a row's (j+1)-th quantization, its
+// "level" j, does not depend on WHICH orders kept the row.  So a row's scales and codes of all K levels come from one
+// pass with the row in registers (expand_chain_kernel); which order uses which level is known as soon as the group
+// maxima of every level are (select_orders_kernel, one block, walks the orders); and a third kernel copies the kept
+// rows' packed codes from level storage to their orders (place_orders_kernel).
+// Against one pass per order this neither writes nor re-reads the fp32 residual (8 bytes an element and order) and
+// pays with codes of levels that no order uses (b / 8 bytes each, and their arithmetic): 4096 x 11008 and back, int4,
+// K = 4, gamma = 0.5: 600 -> 280 us; 8192 x 8192 ternary, K = 8, gamma = 0.25 (8 levels computed, 2.75 used on
+// average): 464 -> 247 us.  The level storage takes the place of the residual in the workspace.
+// Layers this does not take (chain_fits) run one pass per order: the unstructured mask and the L2 score need the
+// residual itself, rows beyond 16384 do not fit a block's registers, and rows that are not whole 16-code chunks.
+struct ChainOut {
+  uint8_t* codes;
+  uint8_t* kcodes;
+  uint8_t* wcodes;
+  float* scales;
+};
+struct ChainArgs {
+  const float* W;
+  int64_t ldw;
+  ChainOut out[PIPE_MAX_ORDERS];   // levels below `direct` go straight to the order of that number
+  int direct;                      // 1, or K when every order keeps every row
+  uint8_t* temp;                   // packed codes (streaming field order, row-major) of the levels from `direct` on
+  int temp_pitch;
+  float* lvl_scale;                // [K][O]
+  uint32_t* lvl_max;               // [K][G] largest magnitude bits of the group's rows entering a level
+  int O, I, I_pad, g, G, K, qmax;
+  int canon_row_bytes;
+  int* status;
+};
+
+// Both packed layouts of 16 codes given as the four bytes of four words.
+template <int BITS>
+__device__ __forceinline__ void pack_bytes(const uint32_t (&wv)[4], uint32_t (&kern)[4]) {
+  if (BITS == 8) {
+#pragma unroll
+    for (int w = 0; w < 4; ++w) kern[w] = wv[w];
+  } else if (BITS == 4) {
+#pragma unroll
+    for (int w = 0; w < 2; ++w) kern[w] = (wv[2 * w] & 0x0F0F0F0Fu) | ((wv[2 * w + 1] << 4) & 0xF0F0F0F0u);
+  } else {
+    kern[0] = (wv[0] & 0x03030303u) | ((wv[1] & 0x03030303u) << 2) | ((wv[2] & 0x03030303u) << 4) | ((wv[3] & 0x03030303u) << 6);
+  }
+}
+// A word of the canonical layout from the same codes' word of the streaming layout (see include/pipe.h).
+template <int BITS>
+__device__ __forceinline__ uint32_t canon_of_kern(uint32_t k) {
+  if (BITS == 8) return k;
+  uint32_t c = 0;
+  if (BITS == 4) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t t = (k >> (4 * h)) & 0x0F0F0F0Fu;
+      const uint32_t u = (t | (t >> 4)) & 0x00FF00FFu;
+      c |= ((u | (u >> 8)) & 0xFFFFu) << (16 * h);
+    }
+  } else {
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const uint32_t t = (k >> (2 * h)) & 0x03030303u;
+      const uint32_t u = (t | (t >> 6)) & 0x000F000Fu;
+      c |= ((u | (u >> 12)) & 0xFFu) << (8 * h);
+    }
+  }
+  return c;
+}
+// The int8 codes (four per word) of field h of a streaming-layout word, sign extended byte by byte.
+template <int BITS>
+__device__ __forceinline__ uint32_t bytes_of_kern(uint32_t k, int h) {
+  if (BITS == 8) return k;
+  if (BITS == 4) {
+    const uint32_t t = (k >> (4 * h)) & 0x0F0F0F0Fu;
+    return t | ((t & 0x08080808u) * 0x1Eu);
+  }
+  const uint32_t t = (k >> (2 * h)) & 0x03030303u;
+  return t | ((t & 0x02020202u) * 0x7Eu);
+}
+
+// Four elements through all levels up to j by the definition (out of line: a few chunks in a thousand): residual after
+// level j and its codes as the bytes of a word.  lvl_s: the scales of the levels below j.
+__device__ __forceinline__ float code_by_division(float x, float s, float fq) {
+  float c = 0.f;
+  if (s != 0.f) c = fminf(fmaxf(rintf(__fdiv_rn(x, s)), -fq), fq);
+  return c;
+}
+static __device__ __noinline__ void replay_quad(const float4* src, const float* lvl_s, int j, float s, float fq, float4* resid, uint32_t* codes) {
+  const float4 v = src ? __ldg(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+  float x[4] = {v.x, v.y, v.z, v.w};
+  uint32_t b = 0;
+#pragma unroll 1
+  for (int l = 0; l <= j; ++l) {
+    const float sl = l < j ? lvl_s[l] : s;
+    b = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float q = code_by_division(x[e], sl, fq);
+      x[e] = __fmaf_rn(-sl, q, x[e]);
+      b |= (static_cast<uint32_t>(static_cast<int>(q)) & 0xffu) << (8 * e);
+    }
+  }
+  *resid = make_float4(x[0], x[1], x[2], x[3]);
+  *codes = b;
+}
+
+constexpr int kChainMaxI = 16384;
+
+// One block per row, PER chunks of 16 consecutive elements per thread.  Bound by its instructions, so per element
+// and level there are four beside the packing: r * (1 / s) + 1.5 * 2^23 (the fused addition rounds to nearest even and
+// leaves the code in the low byte), the code as a float, the residual, its maximum.  What DEFINES the code is the IEEE
+// quotient; it and the estimate can differ only next to a rounding boundary, where |residual| is within
+// s * |t| * 2^-22 of s / 2: so the maximum that the next level needs anyway tells whether a chunk has to be divided
+// (the reciprocal is off by 2^-23, the quotient's own rounding by 2^-24, relative; |t| <= qmax because |x| <= amax,
+// which is also why no clamp is needed while s has a usable reciprocal).
+// (11 instructions per element and level in all, against 16 with an estimate, its distance and the update one after the
+// other and one chunk per thread; the issue slots are 77 % busy, DRAM 45 %: 11008 x 4096 in 78 us, the ternary
+// 8192 x 8192 with its eight levels in 190.)
+template <int BITS, int PER, int MAXT, int MINB>   // PER: 16-code chunks per thread
+__global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_constant__ ChainArgs p) {
+  __shared__ uint32_t part[2][32];
+  __shared__ float lvl_s[PIPE_MAX_ORDERS];
+  const int o = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  const float fq = static_cast<float>(p.qmax);
+  constexpr float kMagic = 12582912.f;
+  constexpr int kWords = BITS / 2;            // packed words of 16 codes
+  constexpr int kStepBytes = 128 * BITS / 8;
+  // |residual| / s from which a chunk is divided: 1/2 - (qmax 2^-22 + 2^-23)
+  const float near_half = 0.5f - (fq * 2.384185791015625e-07f + 1.1920928955078125e-07f);
+  float r[PER][16];
+  uint32_t mk = 0;
+#pragma unroll
+  for (int c = 0; c < PER; ++c) {
+    const int e0 = (tid + c * blockDim.x) * 16;
+    if (e0 < p.I) {
+      const float4* src = reinterpret_cast<const float4*>(p.W + static_cast<int64_t>(o) * p.ldw + e0);
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        const float4 v = __ldg(src + w);
+        r[c][4 * w] = v.x; r[c][4 * w + 1] = v.y; r[c][4 * w + 2] = v.z; r[c][4 * w + 3] = v.w;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 16; ++e) r[c][e] = 0.f;
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < PER; ++c)
+#pragma unroll
+    for (int e = 0; e < 16; ++e) mk = max(mk, abs_key(r[c][e]));
+  uint8_t* temp_row = p.temp + static_cast<int64_t>(o) * p.temp_pitch;   // this row in the level being written
+  const int64_t temp_step = static_cast<int64_t>(p.O) * p.temp_pitch;
+#pragma unroll 1
+  for (int j = 0; j < p.K; ++j) {
+    // largest magnitude entering this level (one barrier per level: the partial maxima alternate between two rows)
+    mk = __reduce_max_sync(0xffffffffu, mk);
+    if (lane == 0) part[j & 1][warp] = mk;
+    __syncthreads();
+    mk = __reduce_max_sync(0xffffffffu, lane < nwarps ? part[j & 1][lane] : 0u);
+    const float s = __fdiv_rn(__uint_as_float(mk), fq);
+    const bool direct = j < p.direct;
+    if (tid == 0) {
+      lvl_s[j] = s;   // (read at later levels, behind their barriers)
+      if (j == 0 && mk >= 0x7f800000u) raise_status(p.status, PIPE_ERR_NONFINITE);
+      (direct ? p.out[j].scales : p.lvl_scale + static_cast<int64_t>(j) * p.O)[o] = s;
+      if (j > 0 && p.direct == 1) atomicMax(p.lvl_max + static_cast<int64_t>(j) * p.G + o / p.g, mk);
+    }
+    const bool fast = quant_step_is_fast(s);
+    float rcp = 0.f;
+    if (fast) asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rcp) : "f"(s));
+    const float limit = fast ? s * near_half : -1.f;
+    mk = 0;
+#pragma unroll
+    for (int c = 0; c < PER; ++c) {
+      uint32_t wv[4], kern[4];
+      float m = 0.f;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        float u[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          float& x = r[c][4 * w + e];
+          u[e] = __fmaf_rn(x, rcp, kMagic);
+          x = __fmaf_rn(-s, __fsub_rn(u[e], kMagic), x);   // exact new residual, rounded once
+          m = fmaxf(m, fabsf(x));
+        }
+        wv[w] = __byte_perm(__byte_perm(__float_as_uint(u[0]), __float_as_uint(u[1]), 0x0040),
+                            __byte_perm(__float_as_uint(u[2]), __float_as_uint(u[3]), 0x0040), 0x5410);
+      }
+      const int chunk = tid + c * blockDim.x, e0 = chunk * 16;
+      if (m >= limit) {
+        // (the old residual is overwritten: the chunk goes through all levels again, divided)
+        m = 0.f;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          float4 v;
+          replay_quad(e0 < p.I ? reinterpret_cast<const float4*>(p.W + static_cast<int64_t>(o) * p.ldw + e0) + w : nullptr, lvl_s, j, s, fq, &v, &wv[w]);
+          r[c][4 * w] = v.x; r[c][4 * w + 1] = v.y; r[c][4 * w + 2] = v.z; r[c][4 * w + 3] = v.w;
+          m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+        }
+      }
+      mk = max(mk, __float_as_uint(m));
+      pack_bytes<BITS>(wv, kern);
+      auto store = [](uint8_t* dst, const uint32_t (&w)[4]) {
+        if constexpr (kWords == 4) *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+        else if constexpr (kWords == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
+        else *reinterpret_cast<uint32_t*>(dst) = w[0];
+      };
+      if (!direct) {
+        if (e0 < p.I) store(temp_row + chunk * (2 * BITS), kern);
+      } else {
+        const ChainOut& out = p.out[j];
+        if (e0 < p.I_pad) {
+          store(out.kcodes + (static_cast<int64_t>(e0 >> 7) * p.O + o) * kStepBytes + (e0 & 127) * BITS / 8, kern);
+          if (out.wcodes)
+            *reinterpret_cast<uint4*>(out.wcodes + (static_cast<int64_t>(e0 >> 7) * p.O + o) * 128 + ((((e0 & 127) >> 4) ^ (o & 7)) << 4)) =
+                make_uint4(wv[0], wv[1], wv[2], wv[3]);
+        }
+        if (e0 < p.I) {
+          uint32_t canon[4];
+#pragma unroll
+          for (int w = 0; w < 4; ++w) canon[w] = w < kWords ? canon_of_kern<BITS>(kern[w]) : 0u;
+          store(out.codes + static_cast<int64_t>(o) * p.canon_row_bytes + chunk * (2 * BITS), canon);
+        }
+      }
+    }
+    if (!direct) temp_row += temp_step;
+  }
+}
+
+// Which order keeps which group at which level, all orders in one block: per order the n_keep groups of largest score
+// (the maximum at the group's present level; ties to the lower index, as everywhere; non-negative floats order like
+// their bits).  The n_keep-th largest score is found by cutting the interval that holds it into up to 256 bins and
+// counting, usually twice (bisecting the bits instead, one block-wide count per bit, took 9 us per order where this
+// takes under 3), then the kept groups are compacted in index order.
+constexpr int kSelThreads = 1024;
+constexpr int kSelPer = 8;
+constexpr int kSelMaxGroups = kSelThreads * kSelPer;
+struct SelectArgs {
+  const uint32_t* lvl_max;   // [K][G]
+  int32_t* lvl_of;           // [K][n_keep]: level of every kept slot of an order (order 1 is dense: level 0)
+  int32_t* cum[PIPE_MAX_ORDERS];
+  int32_t* kept[PIPE_MAX_ORDERS];
+  int G, K, n_keep;
+};
+
+__global__ void __launch_bounds__(kSelThreads) select_orders_kernel(const __grid_constant__ SelectArgs p) {
+  __shared__ uint32_t part[2][32], part_lo[32];
+  __shared__ int hist[256];
+  __shared__ int found_bin, found_need, found_exact;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nch = (p.G + kSelThreads - 1) / kSelThreads;
+  if (tid < 256) hist[tid] = 0;
+  // key: score at the group's present level, plus one (0: no group); next: at the level behind it, asked for ahead of use
+  uint32_t lvl[kSelPer], key[kSelPer], next[kSelPer];
+  auto score = [&](int c, uint32_t l) -> uint32_t {
+    const int j = c * kSelThreads + tid;
+    return c < nch && j < p.G && l < static_cast<uint32_t>(p.K) ? __ldg(p.lvl_max + static_cast<int64_t>(l) * p.G + j) + 1u : 0u;
+  };
+#pragma unroll
+  for (int c = 0; c < kSelPer; ++c) {
+    lvl[c] = 1;
+    key[c] = score(c, 1);
+  }
+  for (int k = 1; k < p.K; ++k) {
+    uint32_t lo = 0xffffffffu, hi = 0;
+#pragma unroll
+    for (int c = 0; c < kSelPer; ++c) {
+      next[c] = score(c, lvl[c] + 1);
+      if (c < nch && key[c] != 0) {
+        lo = min(lo, key[c]);
+        hi = max(hi, key[c]);
+      }
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) {
+      part_lo[warp] = lo;
+      part[0][warp] = hi;
+    }
+    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, part_lo[lane]);
+    hi = __reduce_max_sync(0xffffffffu, part[0][lane]);
+    // of the keys in [lo, hi] the `need` largest are kept, those above hi are kept already
+    int need = p.n_keep;
+    uint32_t thr = lo;
+    int ties = p.G;            // how many of the keys equal to the threshold are kept, lowest index first
+    while (true) {
+      if (lo == hi) {
+        thr = lo;
+        ties = need;
+        break;
+      }
+      const int width = 32 - __clz(hi - lo);
+      const int sh = width > 8 ? width - 8 : 0;
+#pragma unroll
+      for (int c = 0; c < kSelPer; ++c)
+        if (c < nch && key[c] >= lo && key[c] <= hi) atomicAdd(&hist[(key[c] - lo) >> sh], 1);
+      __syncthreads();
+      if (warp == 0) {
+        // lane L holds the bins 8 L .. 8 L + 7 (and clears them for the next use); suffix sums over the lanes
+        int h[8], tot = 0;
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+          h[b] = hist[8 * lane + b];
+          hist[8 * lane + b] = 0;
+          tot += h[b];
+        }
+        int suf = tot;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const int v = __shfl_down_sync(0xffffffffu, suf, d);
+          if (lane + d < 32) suf += v;
+        }
+        int above = suf - tot;   // keys in the lanes' bins behind this one's
+        if (above < need && suf >= need) {
+#pragma unroll
+          for (int b = 7; b >= 0; --b) {
+            if (above < need && above + h[b] >= need) {
+              found_bin = 8 * lane + b;
+              found_need = need - above;
+              found_exact = above + h[b] == need;
+            }
+            above += h[b];
+          }
+        }
+      }
+      __syncthreads();
+      lo += static_cast<uint32_t>(found_bin) << sh;
+      if (found_exact) {
+        thr = lo;
+        break;
+      }
+      need = found_need;
+      hi = min(hi, lo + ((1u << sh) - 1u));
+    }
+    int gt_run = 0, eq_run = 0;
+#pragma unroll
+    for (int c = 0; c < kSelPer; ++c) {
+      if (c >= nch) continue;
+      const int j = c * kSelThreads + tid;
+      const unsigned gt = __ballot_sync(0xffffffffu, key[c] > thr), eq = __ballot_sync(0xffffffffu, key[c] == thr);
+      // (the rows of `part` alternate; the row for c = 0 is the one the interval's maximum did not use)
+      if (lane == 0) part[(c + 1) & 1][warp] = (__popc(gt) << 16) | __popc(eq);
+      __syncthreads();
+      const int mine = static_cast<int>(part[(c + 1) & 1][lane]);
+      const int before = __reduce_add_sync(0xffffffffu, lane < warp ? mine : 0), all = __reduce_add_sync(0xffffffffu, mine);
+      const unsigned below = (1u << lane) - 1u;
+      const int gb = gt_run + (before >> 16) + __popc(gt & below), eb = eq_run + (before & 0xffff) + __popc(eq & below);
+      const bool keep = ((gt >> lane) & 1u) || (((eq >> lane) & 1u) && eb < ties);
+      const int pos = gb + min(eb, ties);
+      if (j < p.G) {
+        p.cum[k][j] = pos;
+        if (keep) {
+          p.kept[k][pos] = j;
+          p.lvl_of[static_cast<int64_t>(k) * p.n_keep + pos] = static_cast<int>(lvl[c]);
+          ++lvl[c];
+          key[c] = next[c];
+        }
+      }
+      gt_run += all >> 16;
+      eq_run += all & 0xffff;
+    }
+    if (tid == 0) p.cum[k][p.G] = p.n_keep;
+    __syncthreads();   // `part` and the found bin are free for the next order
+  }
+}
+
+// The kept rows' codes from level storage to their orders (both layouts, and the int8 copy where the layer keeps one),
+// one block per (order, kept group); the first blocks cut the channel-block and decode-unit tables meanwhile, whose
+// serial walk would otherwise stand alone at the end of the expansion (18 us on 4096 -> 11008).
+// UW: words a thread moves at a time, 4 where rows are whole 16-byte pieces, else the words of 16 codes.
+struct PlaceArgs {
+  ChainOut out[PIPE_MAX_ORDERS];
+  const int32_t* kept[PIPE_MAX_ORDERS];
+  const int32_t* lvl_of;
+  const float* lvl_scale;
+  const uint8_t* temp;
+  int temp_pitch;
+  int O, g, n_keep, rows;          // rows: kept rows of a sparse order
+  int canon_row_bytes, kblocks, tables;
+  BlockTableArgs tab;
+};
+
+template <int BITS, int UW>
+__global__ void __launch_bounds__(kTableThreads) place_orders_kernel(const __grid_constant__ PlaceArgs p) {
+  if (blockIdx.x < static_cast<unsigned>(p.tables)) {
+    cut_table(p.tab, blockIdx.x);
+    return;
+  }
+  const int b = blockIdx.x - p.tables;
+  const int k = 1 + b / p.n_keep, slot = b % p.n_keep;
+  const int j = p.kept[k][slot], lvl = p.lvl_of[static_cast<int64_t>(k) * p.n_keep + slot];
+  const ChainOut& out = p.out[k];
+  const int n0 = slot * p.g, o0 = j * p.g;
+  const uint8_t* src = p.temp + (static_cast<int64_t>(lvl - 1) * p.O + o0) * p.temp_pitch;
+  for (int u = threadIdx.x; u < p.g; u += kTableThreads) out.scales[n0 + u] = p.lvl_scale[static_cast<int64_t>(lvl) * p.O + o0 + u];
+  constexpr int kStepBytes = 128 * BITS / 8;
+  constexpr int UB = 4 * UW;                    // bytes of a piece
+  constexpr int kPieces = kStepBytes / UB;      // pieces of a row in one reduction block
+  const int per = p.g * kPieces;                // pieces of the group in one reduction block
+  const int tid = threadIdx.x;
+  const int kpar = per <= kTableThreads ? kTableThreads / per : 1;
+  const int kb0 = per <= kTableThreads ? tid / per : 0;
+  if (kb0 >= kpar) return;
+  for (int q = per <= kTableThreads ? tid % per : tid; q < per; q += kTableThreads) {
+    const int u = q / kPieces, piece = q % kPieces, n = n0 + u;
+    const uint8_t* row = src + static_cast<int64_t>(u) * p.temp_pitch + piece * UB;
+    uint8_t* crow = out.codes + static_cast<int64_t>(n) * p.canon_row_bytes + piece * UB;
+    uint8_t* krow = out.kcodes + static_cast<int64_t>(n) * kStepBytes + piece * UB;
+    const int64_t kstep = static_cast<int64_t>(p.rows) * kStepBytes;
+#pragma unroll 4
+    for (int kb = kb0; kb < p.kblocks; kb += kpar) {
+      const int byte0 = kb * kStepBytes + piece * UB;
+      const bool in_row = byte0 < p.canon_row_bytes;
+      uint32_t w[UW];
+#pragma unroll
+      for (int i = 0; i < UW; ++i) w[i] = 0u;
+      if (in_row) {
+        if constexpr (UW == 4) {
+          const uint4 v = __ldg(reinterpret_cast<const uint4*>(row + kb * kStepBytes));
+          w[0] = v.x, w[1] = v.y, w[2] = v.z, w[3] = v.w;
+        } else if constexpr (UW == 2) {
+          const uint2 v = __ldg(reinterpret_cast<const uint2*>(row + kb * kStepBytes));
+          w[0] = v.x, w[1] = v.y;
+        } else {
+          w[0] = __ldg(reinterpret_cast<const uint32_t*>(row + kb * kStepBytes));
+        }
+      }
+      uint32_t c[UW];
+#pragma unroll
+      for (int i = 0; i < UW; ++i) c[i] = canon_of_kern<BITS>(w[i]);
+      uint8_t* kd = krow + kb * kstep;
+      uint8_t* cd = crow + kb * kStepBytes;
+      if constexpr (UW == 4) {
+        *reinterpret_cast<uint4*>(kd) = make_uint4(w[0], w[1], w[2], w[3]);
+        if (in_row) *reinterpret_cast<uint4*>(cd) = make_uint4(c[0], c[1], c[2], c[3]);
+      } else if constexpr (UW == 2) {
+        *reinterpret_cast<uint2*>(kd) = make_uint2(w[0], w[1]);
+        if (in_row) *reinterpret_cast<uint2*>(cd) = make_uint2(c[0], c[1]);
+      } else {
+        *reinterpret_cast<uint32_t*>(kd) = w[0];
+        if (in_row) *reinterpret_cast<uint32_t*>(cd) = c[0];
+      }
+      if (out.wcodes) {
+        // 16 codes are one 16-byte piece of the operand layout, at its place in the swizzled row
+        constexpr int kPer16 = BITS / 2;          // words of 16 codes
+        uint8_t* wrow = out.wcodes + (static_cast<int64_t>(kb) * p.rows + n) * 128;
+#pragma unroll
+        for (int i = 0; i < UW / kPer16; ++i) {
+          uint32_t v[4];
+#pragma unroll
+          for (int h = 0; h < 4; ++h) v[h] = bytes_of_kern<BITS>(w[i * kPer16 + h * BITS / 8], h % (8 / BITS));
+          const int p16 = piece * (UW / kPer16) + i;
+          *reinterpret_cast<uint4*>(wrow + ((p16 ^ (n & 7)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]);
+        }
+      }
+    }
+  }
+}
+
+// Header, the trivial kept lists (order 1; every order where all groups are kept) and zeroed level maxima.
+struct ChainInitArgs {
+  uint32_t* hdr;
+  pipe_layer_desc desc;
+  int32_t* cum[PIPE_MAX_ORDERS];
+  int32_t* kept[PIPE_MAX_ORDERS];
+  int lists, G;
+  uint32_t* lvl_max;
+  int64_t n_max;
+};
+
+__device__ __forceinline__ void write_header(uint32_t* hdr, const pipe_layer_desc& d) {
+  {
     hdr[0] = kBlobMagic;
     hdr[1] = 1;  // format version
     int32_t* o = reinterpret_cast<int32_t*>(hdr + 2);
@@ -690,6 +1166,43 @@ __global__ void write_header_kernel(uint32_t* hdr, pipe_layer_desc d) {
     o[4] = d.group_size; o[5] = d.keep_groups; o[6] = d.num_branches;
     for (int m = 0; m < PIPE_MAX_ORDERS; ++m) o[7 + m] = d.branch_orders[m];
   }
+}
+__global__ void write_header_kernel(uint32_t* hdr, pipe_layer_desc d) {
+  if (threadIdx.x == 0) write_header(hdr, d);
+}
+
+__global__ void __launch_bounds__(256) chain_init_kernel(const __grid_constant__ ChainInitArgs p) {
+  const int64_t i0 = blockIdx.x * 256ll + threadIdx.x, step = gridDim.x * 256ll;
+  if (i0 == 0) write_header(p.hdr, p.desc);
+  for (int64_t i = i0; i < p.n_max; i += step) p.lvl_max[i] = 0u;
+  for (int k = 0; k < p.lists; ++k)
+    for (int64_t j = i0; j <= p.G; j += step) {
+      p.cum[k][j] = static_cast<int32_t>(j);
+      if (j < p.G) p.kept[k][j] = static_cast<int32_t>(j);
+    }
+}
+
+// The chain's level storage inside the expansion workspace; false: the layer runs one pass per order.
+struct ChainPlan {
+  uint64_t temp, lvl_scale, lvl_max, lvl_of;   // byte offsets
+  int temp_pitch;
+};
+static bool chain_fits(const LayerInfo& L, const float* W, int64_t ldw, ChainPlan* c) {
+  if (L.keep_elems > 0 || L.score_mode != PIPE_SCORE_MAXABS) return false;
+  if (L.I % 16 != 0 || round_up(L.I, kKernelKAlign) > kChainMaxI || L.G > kSelMaxGroups) return false;
+  if ((reinterpret_cast<uintptr_t>(W) & 15) || ldw % 4 != 0) return false;
+  const int levels = L.n_keep == L.G ? 0 : L.K - 1;   // levels that need storage
+  c->temp_pitch = round_up(L.lay.canon_row_bytes, 16);
+  uint64_t off = 0;
+  c->temp = off;
+  off += round_up<uint64_t>(static_cast<uint64_t>(levels) * L.O * c->temp_pitch, 256);
+  c->lvl_scale = off;
+  if (levels) off += round_up<uint64_t>(static_cast<uint64_t>(L.K) * L.O * 4, 256);
+  c->lvl_max = off;
+  if (levels) off += round_up<uint64_t>(static_cast<uint64_t>(L.K) * L.G * 4, 256);
+  c->lvl_of = off;
+  if (levels) off += round_up<uint64_t>(static_cast<uint64_t>(L.K) * L.n_keep * 4, 256);
+  return off <= L.lay.expand_ws_bytes;   // (more than 32 bits of codes per element beyond order 1 does not fit)
 }
 
 }  // namespace pipe
@@ -737,120 +1250,200 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
   }
   uint8_t* blob = static_cast<uint8_t*>(d_blob);
 
-  write_header_kernel<<<1, 32, 0, s>>>(reinterpret_cast<uint32_t*>(blob), *desc);
-  count_launch(1);
-  for (int k = 0; k < L.K; ++k) {
-    int32_t* kept = reinterpret_cast<int32_t*>(blob + L.lay.kept_off[k]);
-    int32_t* cum = reinterpret_cast<int32_t*>(blob + L.lay.cum_off[k]);
-    const bool dense = (k == 0) || (L.n_keep == L.G);
-    if (!dense && L.G <= kFusedGroups && L.score_mode == PIPE_SCORE_MAXABS) {
-      group_select_kernel<<<1, kFusedGroups, 0, s>>>(a, L.G, L.g, L.n_keep, cum, kept);
-      count_launch(1);
-    } else {
-      if (!dense && L.score_mode == PIPE_SCORE_L2) {
-        // (a sparse order is never the first, so the current residual is in the workspace)
-        row_sumsq_kernel<<<ceil_div(L.O, 8), 256, 0, s>>>(resid, I4, L.O, L.I, rowsq);
-        group_score_l2_kernel<<<ceil_div(L.G, 256), 256, 0, s>>>(rowsq, L.G, L.g, score64);
-        group_rank_kernel<double><<<ceil_div(L.G, 8), 256, 0, s>>>(score64, L.G, L.n_keep, keep);
-        count_launch(3);
-      } else if (!dense) {
-        group_score_kernel<<<ceil_div(L.G, 256), 256, 0, s>>>(a, L.G, L.g, score);
-        group_rank_kernel<float><<<ceil_div(L.G, 8), 256, 0, s>>>(score, L.G, L.n_keep, keep);
-        count_launch(2);
-      }
-      group_compact_kernel<<<1, 1024, 0, s>>>(dense ? nullptr : keep, L.G, cum, kept);
-      count_launch(1);
+  // channel-block tables (entries 0 .. M) and decode-unit tables (entries M + 1 .. 2 M + 1: the same cut with the
+  // layout's row limits), one thread block per table
+  BlockTableArgs t;
+  std::memset(&t, 0, sizeof(t));
+  t.G = L.G;
+  t.g = L.g;
+  bool any = false, any_blk = false;
+  for (int m = 0; m <= L.M; ++m) {
+    const int k0 = (m < L.M) ? L.branch_begin[m] : 0, k1 = (m < L.M) ? L.branch_begin[m + 1] : L.K;
+    if (L.lay.blk_off[m] != 0) {
+      t.nk[m] = k1 - k0;
+      for (int q = 0; q < k1 - k0; ++q) t.cum[m][q] = reinterpret_cast<const int32_t*>(blob + L.lay.cum_off[k0 + q]);
+      t.out[m] = reinterpret_cast<int32_t*>(blob + L.lay.blk_off[m]);
+      t.cap[m] = L.lay.blk_cap[m];
+      // even blocks: the fewest blocks that could hold the cluster's rows, their mean size plus one group of slack
+      int64_t R = 0;
+      for (int k = k0; k < k1; ++k) R += L.lay.rows[k];
+      t.limit[m] = block_row_limit(R, L.O, k1 - k0, L.g);
+      any = any_blk = true;
     }
-    QuantizeRowsArgs q;
-    q.src = (k == 0) ? d_W : resid;
-    q.ld_src = (k == 0) ? ldw : I4;
-    q.dst = (k + 1 < L.K) ? resid : nullptr;
-    q.ld_dst = I4;
-    q.a = a;
-    q.first = (k == 0) ? 1 : 0;
-    q.status = status;
-    q.kept = kept;
-    q.codes = blob + L.lay.codes_off[k];
-    q.kcodes = blob + L.lay.kcodes_off[k];
-    q.wcodes = L.lay.wcodes_off[k] ? blob + L.lay.wcodes_off[k] : nullptr;
-    q.scales = reinterpret_cast<float*>(blob + L.lay.scales_off[k]);
-    q.I = L.I; q.g = L.g; q.qmax = L.qmax;
-    q.canon_row_bytes = L.lay.canon_row_bytes;
-    q.kernel_row_bytes = L.lay.kernel_row_bytes;
-    q.rows = L.lay.rows[k];
-    q.mask_thr = nullptr;
-    q.mask_cut = nullptr;
-    if (L.keep_elems > 0 && k > 0) {
-      row_topn_kernel<<<L.O, 256, 0, s>>>(resid, I4, L.I, L.keep_elems, mask_thr, mask_cut);
-      count_launch(1);
-      q.mask_thr = mask_thr;
-      q.mask_cut = mask_cut;
+    if (L.lay.dec_off[m] != 0) {
+      const int e = L.M + 1 + m;
+      t.nk[e] = k1 - k0;
+      for (int q = 0; q < k1 - k0; ++q) t.cum[e][q] = reinterpret_cast<const int32_t*>(blob + L.lay.cum_off[k0 + q]);
+      t.out[e] = reinterpret_cast<int32_t*>(blob + L.lay.dec_off[m]);
+      t.cap[e] = L.G;
+      t.limit[e] = L.lay.dec_limit[m];
+      any = true;
     }
-    const int rows = L.lay.rows[k];
-    if (L.bits == 8) quantize_rows_kernel<8><<<rows, kRowThreads, 0, s>>>(q);
-    else if (L.bits == 4) quantize_rows_kernel<4><<<rows, kRowThreads, 0, s>>>(q);
-    else quantize_rows_kernel<2><<<rows, kRowThreads, 0, s>>>(q);
-    count_launch(1);
   }
-  {
-    // channel-block tables (entries 0 .. M) and decode-unit tables (entries M + 1 .. 2 M + 1: the same cut with the
-    // layout's row limits) in one launch, one thread block per table
-    BlockTableArgs t;
-    std::memset(&t, 0, sizeof(t));
-    t.G = L.G;
-    t.g = L.g;
-    bool any = false, any_blk = false;
-    for (int m = 0; m <= L.M; ++m) {
-      const int k0 = (m < L.M) ? L.branch_begin[m] : 0, k1 = (m < L.M) ? L.branch_begin[m + 1] : L.K;
-      if (L.lay.blk_off[m] != 0) {
-        t.nk[m] = k1 - k0;
-        for (int q = 0; q < k1 - k0; ++q) t.cum[m][q] = reinterpret_cast<const int32_t*>(blob + L.lay.cum_off[k0 + q]);
-        t.out[m] = reinterpret_cast<int32_t*>(blob + L.lay.blk_off[m]);
-        t.cap[m] = L.lay.blk_cap[m];
-        // even blocks: the fewest blocks that could hold the cluster's rows, their mean size plus one group of slack
-        int64_t R = 0;
-        for (int k = k0; k < k1; ++k) R += L.lay.rows[k];
-        t.limit[m] = block_row_limit(R, L.O, k1 - k0, L.g);
-        any = any_blk = true;
-      }
-      if (L.lay.dec_off[m] != 0) {
-        const int e = L.M + 1 + m;
-        t.nk[e] = k1 - k0;
-        for (int q = 0; q < k1 - k0; ++q) t.cum[e][q] = reinterpret_cast<const int32_t*>(blob + L.lay.cum_off[k0 + q]);
-        t.out[e] = reinterpret_cast<int32_t*>(blob + L.lay.dec_off[m]);
-        t.cap[e] = L.G;
-        t.limit[e] = L.lay.dec_limit[m];
-        any = true;
-      }
+  const int tables = any ? 2 * (L.M + 1) : 0;
+
+  ChainPlan plan;
+  if (chain_fits(L, d_W, ldw, &plan)) {
+    const bool dense = L.K == 1 || L.n_keep == L.G;
+    ChainInitArgs ini;
+    std::memset(&ini, 0, sizeof(ini));
+    ChainArgs ch;
+    std::memset(&ch, 0, sizeof(ch));
+    SelectArgs sel;
+    std::memset(&sel, 0, sizeof(sel));
+    PlaceArgs pl;
+    std::memset(&pl, 0, sizeof(pl));
+    for (int k = 0; k < L.K; ++k) {
+      ini.cum[k] = sel.cum[k] = reinterpret_cast<int32_t*>(blob + L.lay.cum_off[k]);
+      ini.kept[k] = sel.kept[k] = reinterpret_cast<int32_t*>(blob + L.lay.kept_off[k]);
+      pl.kept[k] = sel.kept[k];
+      ChainOut& out = ch.out[k];
+      out.codes = blob + L.lay.codes_off[k];
+      out.kcodes = blob + L.lay.kcodes_off[k];
+      out.wcodes = L.lay.wcodes_off[k] ? blob + L.lay.wcodes_off[k] : nullptr;
+      out.scales = reinterpret_cast<float*>(blob + L.lay.scales_off[k]);
+      pl.out[k] = out;
     }
-    if (any) {
-      block_table_kernel<<<2 * (L.M + 1), kTableThreads, 0, s>>>(t);
+    ini.hdr = reinterpret_cast<uint32_t*>(blob);
+    ini.desc = *desc;
+    ini.lists = dense ? L.K : 1;
+    ini.G = L.G;
+    ini.lvl_max = reinterpret_cast<uint32_t*>(ws + plan.lvl_max);
+    ini.n_max = dense ? 0 : static_cast<int64_t>(L.K) * L.G;
+    const int64_t init_n = ini.n_max > L.G + 1 ? ini.n_max : L.G + 1;
+    const int64_t init_grid = ceil_div<int64_t>(init_n, 256);
+    chain_init_kernel<<<static_cast<int>(init_grid < 64 ? init_grid : 64), 256, 0, s>>>(ini);
+    ch.W = d_W;
+    ch.ldw = ldw;
+    ch.direct = dense ? L.K : 1;
+    ch.temp = ws + plan.temp;
+    ch.temp_pitch = plan.temp_pitch;
+    ch.lvl_scale = reinterpret_cast<float*>(ws + plan.lvl_scale);
+    ch.lvl_max = ini.lvl_max;
+    ch.O = L.O; ch.I = L.I; ch.I_pad = round_up(L.I, kKernelKAlign); ch.g = L.g; ch.G = L.G; ch.K = L.K; ch.qmax = L.qmax;
+    ch.canon_row_bytes = L.lay.canon_row_bytes;
+    ch.status = status;
+    // Two chunks per thread at 64 registers.  Between 8192 and 12288 elements three, at 80: one or two blocks of up to
+    // 384 threads are too few to hide each other's barriers there (4096 x 11008: 151 -> 143 us for the whole expansion;
+    // 11008 x 4096: 128 against 137; one chunk per thread 145 and 198, four 130 and 147).
+    const bool long_rows = ch.I_pad > 8192 && ch.I_pad <= 12288;
+    const int threads = round_up(ceil_div(ch.I_pad / 16, long_rows ? 3 : 2), 32);
+#define PIPE_CHAIN(B)                                                                       \
+  if (long_rows) expand_chain_kernel<B, 3, 256, 3><<<L.O, threads, 0, s>>>(ch);             \
+  else expand_chain_kernel<B, 2, 512, 2><<<L.O, threads, 0, s>>>(ch);
+    if (L.bits == 8) { PIPE_CHAIN(8) } else if (L.bits == 4) { PIPE_CHAIN(4) } else { PIPE_CHAIN(2) }
+#undef PIPE_CHAIN
+    count_launch(2);
+    if (!dense) {
+      sel.lvl_max = ini.lvl_max;
+      sel.lvl_of = reinterpret_cast<int32_t*>(ws + plan.lvl_of);
+      sel.G = L.G; sel.K = L.K; sel.n_keep = L.n_keep;
+      select_orders_kernel<<<1, kSelThreads, 0, s>>>(sel);
+      pl.lvl_of = sel.lvl_of;
+      pl.lvl_scale = ch.lvl_scale;
+      pl.temp = ch.temp;
+      pl.temp_pitch = plan.temp_pitch;
+      pl.O = L.O; pl.g = L.g; pl.n_keep = L.n_keep; pl.rows = L.n_keep * L.g;
+      pl.canon_row_bytes = L.lay.canon_row_bytes;
+      pl.kblocks = ceil_div(L.I, kKernelKAlign);
+      pl.tables = tables;
+      pl.tab = t;
+      const int grid = tables + (L.K - 1) * L.n_keep;
+      const bool whole = L.lay.canon_row_bytes % 16 == 0;
+      if (L.bits == 8) place_orders_kernel<8, 4><<<grid, kTableThreads, 0, s>>>(pl);
+      else if (L.bits == 4 && whole) place_orders_kernel<4, 4><<<grid, kTableThreads, 0, s>>>(pl);
+      else if (L.bits == 4) place_orders_kernel<4, 2><<<grid, kTableThreads, 0, s>>>(pl);
+      else if (whole) place_orders_kernel<2, 4><<<grid, kTableThreads, 0, s>>>(pl);
+      else place_orders_kernel<2, 1><<<grid, kTableThreads, 0, s>>>(pl);
+      count_launch(2);
+    } else if (tables) {
+      block_table_kernel<<<tables, kTableThreads, 0, s>>>(t);
       count_launch(1);
     }
-    if (any_blk) {
-      // the records of the blocks just cut
-      BlockRecordArgs r;
-      std::memset(&r, 0, sizeof(r));
-      r.g = L.g;
-      r.status = status;
-      int max_cap = 0;
-      for (int m = 0; m <= L.M; ++m) {
-        if (L.lay.rec_off[m] == 0) continue;
-        const int k0 = (m < L.M) ? L.branch_begin[m] : 0, k1 = (m < L.M) ? L.branch_begin[m + 1] : L.K;
-        r.nk[m] = k1 - k0;
-        for (int q = 0; q < k1 - k0; ++q) {
-          r.cum[m][q] = reinterpret_cast<const int32_t*>(blob + L.lay.cum_off[k0 + q]);
-          r.scales[m][q] = reinterpret_cast<const float*>(blob + L.lay.scales_off[k0 + q]);
+  } else {
+    write_header_kernel<<<1, 32, 0, s>>>(reinterpret_cast<uint32_t*>(blob), *desc);
+    count_launch(1);
+    for (int k = 0; k < L.K; ++k) {
+      int32_t* kept = reinterpret_cast<int32_t*>(blob + L.lay.kept_off[k]);
+      int32_t* cum = reinterpret_cast<int32_t*>(blob + L.lay.cum_off[k]);
+      const bool dense = (k == 0) || (L.n_keep == L.G);
+      if (!dense && L.G <= kFusedGroups && L.score_mode == PIPE_SCORE_MAXABS) {
+        group_select_kernel<<<1, kFusedGroups, 0, s>>>(a, L.G, L.g, L.n_keep, cum, kept);
+        count_launch(1);
+      } else {
+        if (!dense && L.score_mode == PIPE_SCORE_L2) {
+          // (a sparse order is never the first, so the current residual is in the workspace)
+          row_sumsq_kernel<<<ceil_div(L.O, 8), 256, 0, s>>>(resid, I4, L.O, L.I, rowsq);
+          group_score_l2_kernel<<<ceil_div(L.G, 256), 256, 0, s>>>(rowsq, L.G, L.g, score64);
+          group_rank_kernel<double><<<ceil_div(L.G, 8), 256, 0, s>>>(score64, L.G, L.n_keep, keep);
+          count_launch(3);
+        } else if (!dense) {
+          group_score_kernel<<<ceil_div(L.G, 256), 256, 0, s>>>(a, L.G, L.g, score);
+          group_rank_kernel<float><<<ceil_div(L.G, 8), 256, 0, s>>>(score, L.G, L.n_keep, keep);
+          count_launch(2);
         }
-        r.tbl[m] = reinterpret_cast<const int32_t*>(blob + L.lay.blk_off[m]);
-        r.out[m] = blob + L.lay.rec_off[m];
-        r.cap[m] = L.lay.rec_cap[m];
-        max_cap = max_cap > r.cap[m] ? max_cap : r.cap[m];
-      }
-      if (max_cap > 0) {
-        block_record_kernel<<<dim3(max_cap, L.M + 1), 256, 0, s>>>(r);
+        group_compact_kernel<<<1, 1024, 0, s>>>(dense ? nullptr : keep, L.G, cum, kept);
         count_launch(1);
       }
+      QuantizeRowsArgs q;
+      q.src = (k == 0) ? d_W : resid;
+      q.ld_src = (k == 0) ? ldw : I4;
+      q.dst = (k + 1 < L.K) ? resid : nullptr;
+      q.ld_dst = I4;
+      q.a = a;
+      q.first = (k == 0) ? 1 : 0;
+      q.status = status;
+      q.kept = kept;
+      q.codes = blob + L.lay.codes_off[k];
+      q.kcodes = blob + L.lay.kcodes_off[k];
+      q.wcodes = L.lay.wcodes_off[k] ? blob + L.lay.wcodes_off[k] : nullptr;
+      q.scales = reinterpret_cast<float*>(blob + L.lay.scales_off[k]);
+      q.I = L.I; q.g = L.g; q.qmax = L.qmax;
+      q.canon_row_bytes = L.lay.canon_row_bytes;
+      q.kernel_row_bytes = L.lay.kernel_row_bytes;
+      q.rows = L.lay.rows[k];
+      q.mask_thr = nullptr;
+      q.mask_cut = nullptr;
+      if (L.keep_elems > 0 && k > 0) {
+        row_topn_kernel<<<L.O, 256, 0, s>>>(resid, I4, L.I, L.keep_elems, mask_thr, mask_cut);
+        count_launch(1);
+        q.mask_thr = mask_thr;
+        q.mask_cut = mask_cut;
+      }
+      const int rows = L.lay.rows[k];
+      if (L.bits == 8) quantize_rows_kernel<8><<<rows, kRowThreads, 0, s>>>(q);
+      else if (L.bits == 4) quantize_rows_kernel<4><<<rows, kRowThreads, 0, s>>>(q);
+      else quantize_rows_kernel<2><<<rows, kRowThreads, 0, s>>>(q);
+      count_launch(1);
+    }
+    if (tables) {
+      block_table_kernel<<<tables, kTableThreads, 0, s>>>(t);
+      count_launch(1);
+    }
+  }
+  if (any_blk) {
+    // the records of the blocks just cut
+    BlockRecordArgs r;
+    std::memset(&r, 0, sizeof(r));
+    r.g = L.g;
+    r.status = status;
+    int max_cap = 0;
+    for (int m = 0; m <= L.M; ++m) {
+      if (L.lay.rec_off[m] == 0) continue;
+      const int k0 = (m < L.M) ? L.branch_begin[m] : 0, k1 = (m < L.M) ? L.branch_begin[m + 1] : L.K;
+      r.nk[m] = k1 - k0;
+      for (int q = 0; q < k1 - k0; ++q) {
+        r.cum[m][q] = reinterpret_cast<const int32_t*>(blob + L.lay.cum_off[k0 + q]);
+        r.scales[m][q] = reinterpret_cast<const float*>(blob + L.lay.scales_off[k0 + q]);
+      }
+      r.tbl[m] = reinterpret_cast<const int32_t*>(blob + L.lay.blk_off[m]);
+      r.out[m] = blob + L.lay.rec_off[m];
+      r.cap[m] = L.lay.rec_cap[m];
+      max_cap = max_cap > r.cap[m] ? max_cap : r.cap[m];
+    }
+    if (max_cap > 0) {
+      block_record_kernel<<<dim3(max_cap, L.M + 1), 256, 0, s>>>(r);
+      count_launch(1);
     }
   }
   mark_expansion(s);   // a forward call that follows on this stream must not read the blob ahead of its dependency wait

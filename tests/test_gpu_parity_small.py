@@ -50,6 +50,44 @@ def test_expand_weights_bit_exact(oracle, O, I, bits, K, g, n_keep):
     H.assert_expansion_matches(layer, e, oracle)
 
 
+# Both expansions and the lines between them: rows from one 16-code chunk to the most a block's registers hold and one
+# chunk more, group counts around the selection block's 1024 and its 8192, orders whose level storage just fits or does
+# not fit the workspace, every order dense, rows that are no whole 16-byte pieces, the int8 copy.
+EXPAND_ROUTE_CASES = [
+    # O,    I,     bits, K, g, n_keep, int8_copy
+    (64, 16, 4, 3, 8, 3, True),
+    (40, 144, 8, 4, 8, 2, True),
+    (40, 2304, 8, 5, 8, 2, False),
+    (48, 528, 2, 8, 16, 1, True),
+    (48, 560, 4, 4, 16, 2, True),
+    (64, 256, 2, 16, 8, 3, False),
+    (64, 2064, 3, 5, 8, 8, True),
+    (128, 784, 6, 3, 8, 5, True),
+    (16, 16384, 4, 3, 8, 1, False),
+    (16, 16400, 4, 3, 8, 1, False),
+    (1023, 16, 4, 3, 1, 500, False),
+    (8200, 32, 2, 4, 8, 1000, False),
+    (8192, 16, 4, 3, 1, 4097, False),
+    (8193, 16, 4, 3, 1, 77, False),
+]
+
+
+@pytest.mark.parametrize("ties", [False, True])
+@pytest.mark.parametrize("O,I,bits,K,g,n_keep,int8_copy", EXPAND_ROUTE_CASES)
+def test_expand_weights_on_every_route(oracle, O, I, bits, K, g, n_keep, int8_copy, ties):
+    rng = np.random.default_rng(O + I)
+    W = _w(rng, O, I, heavy=True)
+    if ties:                                  # many groups of equal score: the lower index wins
+        W = np.ascontiguousarray(W[rng.integers(0, max(1, O // (4 * g)), O // g).repeat(g) * g + np.tile(np.arange(g), O // g)])
+        W[-g:] = 0.0
+    if bits in (3, 6):
+        e = oracle.expand_ex(W, bits, K, g, n_keep)
+    else:
+        e = oracle.expand(W, bits, K, g, n_keep)
+    layer = H.gpu_expand(H.desc_of(O, I, bits, K, g, n_keep, int8_copy=int8_copy), W)
+    H.assert_expansion_matches(layer, e, oracle)
+
+
 @pytest.mark.parametrize("bits", [8, 4, 2])
 def test_expand_weights_at_rounding_boundaries(oracle, bits):
     """Rows whose entries sit on, and a few ulps beside, the boundaries (k + 1/2) * s of their own scale: the
