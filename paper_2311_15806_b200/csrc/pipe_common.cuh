@@ -95,26 +95,11 @@ inline int block_count_bound(int64_t R, int O, int G, int nk, int g) {
 // Raise a device-side error: first error wins.
 __device__ inline void raise_status(int* status, int code) { atomicCAS(status, 0, code); }
 
-// clamp(rne(v / s)) as an int8 lane.  The IEEE quotient is what defines the code (Eq. 1 with true
-// division), but a division costs an order of magnitude more than a multiplication, so the quotient is
-// first estimated as t = v * r with r = rn(1 / s): t is within a relative 2^-22.9 of the real quotient,
-// as is the IEEE quotient itself (2^-24), so both round to the same integer unless the estimate lies
-// within |t| * 2^-21 of a rounding boundary (an odd multiple of one half) -- only then, a few times in a
-// hundred thousand, is the division carried out.  Beyond +-130 both clamp.
-__device__ __forceinline__ uint32_t quant_lane(float v, float s, float r) {
-  const float t = __fmul_rn(v, r);
-  float q = rintf(t);
-  const float at = fabsf(t);
-  if (at > 130.f) {
-    q = copysignf(127.f, t);
-  } else if (0.5f - fabsf(__fsub_rn(t, q)) <= at * 4.76837158203125e-07f) {
-    q = rintf(__fdiv_rn(v, s));
-  }
-  q = fminf(fmaxf(q, -127.f), 127.f);
-  return static_cast<uint32_t>(static_cast<int>(q)) & 0xffu;
-}
-
-// The same code with the division always carried out; a zero step gives the code 0 (Eq. 1 on an all-zero tensor).
+// clamp(rne(v / s)) as an int8 lane.  The IEEE quotient is what defines the code (Eq. 1 with true division), but a
+// division costs an order of magnitude more than a multiplication, so the quantizers estimate it as t = v * r with
+// r = rn(1 / s): t is within a relative 2^-22.9 of the real quotient, as is the IEEE quotient itself (2^-24), so both round
+// to the same integer unless the estimate lies within |t| * 2^-21 of a rounding boundary (an odd multiple of one half) --
+// only then, a few times in a hundred thousand, is the division carried out, by this.  A zero step gives the code 0.
 __device__ __forceinline__ uint32_t quant_lane_exact(float v, float s) {
   float q = 0.f;
   if (s != 0.f) q = fminf(fmaxf(rintf(__fdiv_rn(v, s)), -127.f), 127.f);
@@ -124,10 +109,19 @@ __device__ __forceinline__ uint32_t quant_lane_exact(float v, float s) {
 // The estimate needs a reciprocal that neither overflows nor is subnormal.
 __device__ __forceinline__ bool quant_step_is_fast(float s) { return s >= 1e-30f && s <= 1e30f; }
 
-// Four codes as the bytes of one word, lowest address first.
-__device__ __forceinline__ uint32_t quant4(const float4& f, float s, float r, bool fast) {
-  if (fast) return quant_lane(f.x, s, r) | (quant_lane(f.y, s, r) << 8) | (quant_lane(f.z, s, r) << 16) | (quant_lane(f.w, s, r) << 24);
-  return quant_lane_exact(f.x, s) | (quant_lane_exact(f.y, s) << 8) | (quant_lane_exact(f.z, s) << 16) | (quant_lane_exact(f.w, s) << 24);
+// Rounding without a conversion instruction: t + 1.5 * 2^23, where the spacing of binary32 is one, is t rounded to the
+// nearest integer, ties to even, and holds it in the low byte.  edge: the largest |t - code| + err so far; at 0.5 or more
+// an estimate t that is off by up to err may round the other way.
+__device__ __forceinline__ float code_magic(float t, float err, float& edge) {
+  const float u = __fadd_rn(t, 12582912.f);
+  const float d = __fsub_rn(t, __fsub_rn(u, 12582912.f));
+  edge = fmaxf(edge, __fadd_rn(fabsf(d), err));
+  return u;
+}
+__device__ __forceinline__ uint32_t pack4_low_bytes(float a, float b, float c, float d) {
+  const uint32_t ab = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x0040);
+  const uint32_t cd = __byte_perm(__float_as_uint(c), __float_as_uint(d), 0x0040);
+  return __byte_perm(ab, cd, 0x5410);
 }
 
 // sigma of Eq. 9 for an inner layer (Sec. 3.2 names ReLU, SiLU, GeLU and sigmoid), in binary32: kind 0 identity,

@@ -166,12 +166,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, int (&v)[8]) {
 // took longer than the MMAs they should hide behind.  Measured before -> after (K = 4, M = 2, T = 4096): 4096 -> 11008
 // with SiLU 596 -> 342 us (fp32 output: 302), 768 -> 3072 with GeLU 175 -> 84 us (fp32 output: 57), and with ReLU, which
 // gains from the fallback being out of line, 86 -> 69 us.
-__device__ __forceinline__ float code_magic(float t, float err, float& edge) {
-  const float u = __fadd_rn(t, 12582912.f);
-  const float d = __fsub_rn(t, __fsub_rn(u, 12582912.f));
-  edge = fmaxf(edge, __fadd_rn(fabsf(d), err));
-  return u;
-}
 __device__ __forceinline__ float ex2_approx(float x) {
   float r;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -215,12 +209,6 @@ __device__ __forceinline__ float smooth_estimate(float v, float& slack) {
 static __device__ __noinline__ uint32_t codes4_exact(float a, float b, float c, float d, int kind, float s) {
   return quant_lane_exact(apply_activation(a, kind), s) | (quant_lane_exact(apply_activation(b, kind), s) << 8) |
          (quant_lane_exact(apply_activation(c, kind), s) << 16) | (quant_lane_exact(apply_activation(d, kind), s) << 24);
-}
-
-__device__ __forceinline__ uint32_t pack4_low_bytes(float a, float b, float c, float d) {
-  const uint32_t ab = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x0040);
-  const uint32_t cd = __byte_perm(__float_as_uint(c), __float_as_uint(d), 0x0040);
-  return __byte_perm(ab, cd, 0x5410);
 }
 
 template <int KIND>

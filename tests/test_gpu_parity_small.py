@@ -167,6 +167,37 @@ def test_quantize_act_bit_exact(oracle, T, I):
     np.testing.assert_array_equal(xq.cpu().numpy(), xq_o)
 
 
+# One launch of one cluster from 256 to 32768 quads (one or four per thread), two passes beyond (the last case has a part
+# that the range pass does not keep in L2); rows that are no whole quads or have a pitch go chunk by chunk.
+QUANT_ROUTE_CASES = [(1, 4), (1, 1020), (1, 1024), (8, 4096), (8, 4100), (32, 4096), (33, 4096), (64, 4096), (65, 4096), (300, 4097),
+                     (2000, 1000), (5300, 4096)]
+
+
+@pytest.mark.parametrize("pitch", [0, 4, 5])
+@pytest.mark.parametrize("T,I", QUANT_ROUTE_CASES)
+def test_quantize_act_on_every_route(oracle, T, I, pitch):
+    rng = np.random.default_rng(T + I + pitch)
+    x = (rng.standard_normal((T, I)) * 2.5).astype(np.float32)
+    x[T // 2, I - 1] = -17.0                  # the maximum sits at an end
+    xd = torch.zeros((T, I + pitch), device="cuda")
+    xd[:, :I] = torch.from_numpy(x).cuda()
+    ws = B.alloc_bytes(256)
+    ws.fill_(0xFF)                            # the workspace's contents do not matter
+    sx = torch.zeros(1, device="cuda")
+    zp = torch.full((1,), 99, dtype=torch.int32, device="cuda")
+    xq = torch.full((T, I + pitch), 55, dtype=torch.int8, device="cuda")
+    B.pipe_quantize_act(xd[:, :I], xq[:, :I], sx, ws)
+    want, want_s = oracle.quantize_act(x)
+    assert sx.cpu().numpy().view(np.uint32)[0] == np.float32(want_s).view(np.uint32)
+    np.testing.assert_array_equal(xq[:, :I].cpu().numpy(), want)
+    for bits, asym in ((8, True), (4, False), (6, True)):
+        B.pipe_quantize_act_ex(xd[:, :I], xq[:, :I], sx, zp, ws, bits, asym)
+        want, want_s, want_z = oracle.quantize_act_ex(x, bits, asym)
+        assert sx.cpu().numpy().view(np.uint32)[0] == np.float32(want_s).view(np.uint32) and int(zp.item()) == want_z
+        np.testing.assert_array_equal(xq[:, :I].cpu().numpy(), want)
+    assert bool((xq[:, I:] == 55).all()) and B.pipe_poll_status() == B.PIPE_OK
+
+
 def test_quantize_act_at_rounding_boundaries(oracle):
     """Values placed on, and one or two ulps beside, the rounding boundaries (k + 1/2) * lambda_x: the code is
     defined by the IEEE quotient, so a kernel that estimates the quotient must fall back to the true
