@@ -59,6 +59,7 @@ using namespace tcc;
 struct Params {
   CUtensorMap tmap_a[PIPE_MAX_ORDERS];  // one per branch input
   CUtensorMap tmap_y[PIPE_MAX_ORDERS];  // one per branch output (fp32), valid where y_tma has the branch's bit
+  CUtensorMap tmap_w;                   // int8 codes: the streaming sections from kbase on as rows of 128 bytes, box of 8 rows
   uint32_t y_tma;                       // branches whose fp32 output the epilogue may write with tensor stores
   ForwardArgs f;
   int ntt, kblocks;       // ntt: pairs of token tiles; kblocks: reduction blocks of 128 lanes
@@ -253,17 +254,17 @@ struct Rings {
 // when six warps each had 8 KiB outstanding), reads them into registers, and only then overwrites the slot with the
 // widened rows; nothing else is staged.  A lane's item i is the 16-byte chunk 32 i + lane of those packed rows
 // (RPI = 32 / CPR rows per item).
-// int8 codes need no widening and fill the slot exactly; they are loaded through registers.
+// int8 codes need no widening: they arrive by tensor copies of eight rows whose 128-byte swizzle is the operand layout
+// (through registers, which this replaced, a block took 2 us: 4096 x 4096, K = 2, T = 100: 66 -> 20 us, T = 4096:
+// 348 -> 96 us).
 template <int BITS>
 __device__ __forceinline__ void unpack_role(const Params& p, const Rings& g, int uw, int lane, uint32_t pkbar) {
   constexpr int CPR = BITS;                // 16-byte chunks per packed row per block: 8, 4, 2
   constexpr int RPI = 32 / CPR;            // rows per item: 4, 8, 16
   constexpr int ITEMS = (kMaxN / 2) / RPI; // items of a full half tile: 32, 16, 8
-  constexpr int PASS = ITEMS > 16 ? 16 : ITEMS;   // items held in registers at a time
   constexpr int OUT_PER_CHUNK = 8 / BITS;  // 16-byte vectors written per chunk read
   constexpr int PK = kKStep * BITS / 8;    // packed bytes of a row of a block
   constexpr int kPackedOff = kBtBytes - (kMaxN / 2) * PK;   // sub-byte codes: where the packed rows land in the slot
-  const uint4* kb16 = reinterpret_cast<const uint4*>(p.kbase);
   const int my_tiles = (g.num_tiles - g.pair + g.npairs - 1) / g.npairs;
   if (my_tiles <= 0) return;
   const int slots_per_tile = kSub * p.ksteps;
@@ -281,6 +282,7 @@ __device__ __forceinline__ void unpack_role(const Params& p, const Rings& g, int
   // block (16-byte units relative to kbase), bytes, and byte offset inside the packed rows of the half tile
   uint32_t run_off = 0, run_stp = 0, run_bytes = 0, run_dst = 0;
   int n_items = 0, mine = 0;               // items / rows of this CTA's half tile that exist
+  int w_row = 0, w_step = 0;               // int8 codes: row of this lane's eight rows in tmap_w at block 0, and per block
   int kbs = uw, ti = 0;                    // block position inside the tile, tile index
   while (kbs >= slots_per_tile) {
     kbs -= slots_per_tile;
@@ -318,6 +320,16 @@ __device__ __forceinline__ void unpack_role(const Params& p, const Rings& g, int
           run_dst = static_cast<uint32_t>(a - h0) * PK;
         }
       }
+      if (BITS == 8 && !p.direct) {
+        // lane i < 16 brings the rows h0 + 8 i .. + 7 of the stacked tile, which lie in one order (groups are multiples of 8)
+        const int r = h0 + 8 * lane;
+#pragma unroll
+        for (int q = 0; q < kMaxClusterOrders; ++q)
+          if (q < t.nk && r >= t.rowbase[q] && r < t.rowbase[q + 1]) {
+            w_row = static_cast<int>(p.koff[t.k0 + q] >> 3) + t.start[q] + (r - t.rowbase[q]);
+            w_step = p.f.order[t.k0 + q].rows;
+          }
+      }
     }
     const uint32_t gs = static_cast<uint32_t>(ti) * p.ksteps + static_cast<uint32_t>(kbs / kSub);   // stage number
     const uint32_t slot = gs % p.depth, use = gs / p.depth;
@@ -325,44 +337,7 @@ __device__ __forceinline__ void unpack_role(const Params& p, const Rings& g, int
     const bool real = kbs < p.kblocks && mine > 0;     // false: the empty position behind an odd block count
     const uint32_t bt_off = slot * kStageBytes + kStageBOff + sub * kBtBytes;
     uint8_t* bt = g.stage_gen + bt_off;
-    bool through_registers = false;
-    if constexpr (BITS == 8) through_registers = !p.direct;
-    if (through_registers) {
-      if constexpr (BITS == 8) {
-#pragma unroll
-      for (int pass = 0; pass < ITEMS / PASS; ++pass) {
-        uint4 w[PASS];
-        if (real) {
-#pragma unroll
-          for (int i = 0; i < PASS; ++i) {
-            const int item = i + PASS * pass;
-            // the run that holds the item's first row
-            const int byte0 = item * RPI * PK;
-            uint32_t src = 0;
-#pragma unroll
-            for (int q = 0; q < kMaxClusterOrders; ++q) {
-              const uint32_t ro = __shfl_sync(0xffffffffu, run_off + static_cast<uint32_t>(kbs) * run_stp, q);
-              const uint32_t rd = __shfl_sync(0xffffffffu, run_dst, q), rbts = __shfl_sync(0xffffffffu, run_bytes, q);
-              if (static_cast<uint32_t>(byte0) >= rd && static_cast<uint32_t>(byte0) < rd + rbts) src = ro + ((byte0 - rd) >> 4);
-            }
-            if (item < n_items) w[i] = __ldg(kb16 + src + lane);
-          }
-        }
-        // the stage is free once the MMAs of its previous use have completed (first pass of the block only)
-        if (pass == 0 && !mbar_wait(g.done0 + 8u * slot, (use & 1) ^ 1, g.abort_flag, p.f.status)) return;
-        if (real) {
-#pragma unroll
-          for (int i = 0; i < PASS; ++i) {
-            const int item = i + PASS * pass;
-            if (item >= n_items) continue;
-            const int row0 = item * RPI;   // rows row0 + lr; the item's parity moves the row inside its 8-row atom
-            uint8_t* row = bt + (row0 >> 3) * 1024 + (row0 & 7) * 128 + out_lane;
-            *reinterpret_cast<uint4*>(row + ((lc ^ ((row0 + lr) & 7)) << 4)) = w[i];
-          }
-        }
-      }
-      }
-    } else {
+    {
       // (int8 rows in the operand layout -- the layer's int8 copy -- are complete when their copies have landed)
       // everything the copies need is prepared before the wait for the slot: what follows the wait is on the
       // critical path of the ring (the barrier of the packed rows belongs to this warp alone, so its byte count can
@@ -373,10 +348,13 @@ __device__ __forceinline__ void unpack_role(const Params& p, const Rings& g, int
       if (real && lane == 0) mbar_expect_tx(bar, static_cast<uint32_t>(mine) * PK);
       if (!mbar_wait(g.done0 + 8u * slot, (use & 1) ^ 1, g.abort_flag, p.f.status)) return;
       if (real) {
+        if (BITS == 8 && !p.direct && 8 * lane < mine)
+          tma_load_2d(g.stage0 + bt_off + lane * 1024, &p.tmap_w, 0, w_row + kbs * w_step, bar);
         if (run_bytes != 0) {
-          asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
-                       "r"(run_bytes), "r"(bar)
-                       : "memory");
+          if (BITS != 8 || p.direct)
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+                         "r"(run_bytes), "r"(bar)
+                         : "memory");
           // ... and this warp's next block into L2, a use of the ring (some 5000 cycles) ahead: where the weights come from
           // HBM -- few token tiles -- the copy then finds them there (11008 -> 4096, T = 100: 48.1 -> 44.9 us, 4096 ->
           // 11008, T = 1024: 96.7 -> 91.3; two uses ahead 47.8, three 45.5), and it costs nothing measurable elsewhere
@@ -1302,6 +1280,16 @@ static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_
     p.koff[k] = static_cast<uint32_t>(d >> 4);
   }
   p.depth = ds.depth;
+  if (p.f.bits == 8 && !direct) {
+    uint64_t rows = 0;
+    for (int k = k_lo; k < k_hi; ++k) {
+      const uint64_t end = (static_cast<uint64_t>(p.koff[k]) >> 3) + static_cast<uint64_t>(a.order[k].rows) * ceil_div(a.I, kKStep);
+      rows = end > rows ? end : rows;
+      if ((p.koff[k] & 7) != 0 || rows > INT32_MAX) return PIPE_ERR_UNSUPPORTED;
+    }
+    if (!make_map_2d(&p.tmap_w, p.kbase, kKStep, rows, kKStep, kKStep, 8, CU_TENSOR_MAP_SWIZZLE_128B)) return PIPE_ERR_CUDA;
+  }
+
   if (a.conv_on) {
     for (int m = 0; m < a.num_branches; ++m)
       if (!make_map_nhwc(&p.tmap_a[m], a.branch[m].xq, a.cN, a.cH, a.cW, a.cC, a.csh, a.csw)) return PIPE_ERR_CUDA;
