@@ -220,7 +220,8 @@ bool make_tensor_map_2d_u8(CUtensorMap* map, const void* base, uint64_t inner_by
 pipe_status forward_reference(const ForwardArgs& a, cudaStream_t stream);
 pipe_status forward_tcgen05(const ForwardArgs& a, cudaStream_t stream);
 pipe_status forward_tcgen05_pair(const ForwardArgs& a, cudaStream_t stream);   // two-SM form (clusters of two CTAs)
-pipe_status forward_stream(const ForwardArgs& a, cudaStream_t stream);
+// (slices: more than 16 tokens too, in slices of 16, where the launch is small enough for the rule in launch_stream)
+pipe_status forward_stream(const ForwardArgs& a, cudaStream_t stream, bool slices);
 pipe_status forward_decode_tc(const ForwardArgs& a, cudaStream_t stream);      // T <= 16 on tcgen05 (decode-unit tables)
 
 }  // namespace pipe

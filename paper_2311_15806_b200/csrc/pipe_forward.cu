@@ -92,7 +92,7 @@ static pipe_status dispatch_forward(const ForwardArgs& a, const LayerInfo& L, in
                                     cudaStream_t stream) {
   const int choice = kernel_choice();
   if (zp) {
-    // asymmetric codes: the SM-pair kernel and, up to 15 tokens, the weight-streaming kernel form the row sums beside the
+    // asymmetric codes: the SM-pair kernel and, in slices of 15 tokens, the weight-streaming kernel form the row sums beside the
     // products (row of ones); the CUDA-core kernel takes every other shape.  Measured against the CUDA-core kernel from
     // 128 x 128 to 3072 x 3072 and 1 to 2048 tokens: equal (host-bound) at 128 x 128, faster everywhere else.
     if (static_cast<int64_t>(255) * L.qmax * L.I >= (static_cast<int64_t>(1) << 31)) return PIPE_ERR_ACC_OVERFLOW;
@@ -103,23 +103,23 @@ static pipe_status dispatch_forward(const ForwardArgs& a, const LayerInfo& L, in
     // (the tensor-core accumulators hold 2^(8-b) times the sums)
     pipe_status st = PIPE_ERR_UNSUPPORTED;
     if (((static_cast<int64_t>(255) * L.qmax * L.I) << (8 - L.bits)) < (static_cast<int64_t>(1) << 31)) {
-      if (T <= 16) st = forward_stream(a, stream);
+      st = forward_stream(a, stream, true);
       if (st == PIPE_ERR_UNSUPPORTED) st = forward_tcgen05_pair(a, stream);
     }
     return st == PIPE_ERR_UNSUPPORTED ? forward_reference(a, stream) : st;
   }
   if (choice == 1) return forward_reference(a, stream);
   if (choice == 2) return forward_tcgen05(a, stream);
-  if (choice == 3) return forward_stream(a, stream);
+  if (choice == 3) return forward_stream(a, stream, false);
   if (choice == 4) return forward_tcgen05_pair(a, stream);
   if (choice == 5) return forward_decode_tc(a, stream);
-  // T <= 16: weight streaming; from two token tiles on the SM-pair kernel; the one-SM kernel for what lies between
-  // and for layers without channel-block tables; the CUDA-core kernel for every other shape
+  // T <= 16, and small layers in slices of 16 tokens: weight streaming; then the SM-pair kernel; the one-SM kernel for
+  // layers without channel-block tables and what the pair kernel leaves it; the CUDA-core kernel for every other shape
   pipe_status st = PIPE_ERR_UNSUPPORTED;
   // (the small-token tcgen05 kernel, choice 5, is measured slower than the weight-streaming kernel -- widening the
   // codes through shared memory for the tensor core triples the shared-memory traffic per weight byte -- and is
   // therefore not on the automatic path)
-  if (T <= 16) st = forward_stream(a, stream);
+  st = forward_stream(a, stream, true);
   if (T <= 16 && st == PIPE_ERR_UNSUPPORTED) st = forward_decode_tc(a, stream);
   if (st == PIPE_ERR_UNSUPPORTED) st = forward_tcgen05_pair(a, stream);
   if (st == PIPE_ERR_UNSUPPORTED) st = forward_tcgen05(a, stream);

@@ -1,4 +1,5 @@
-// Small-token kernel of the expanded layer (Appendix B, Eq. 9; Sec. 3.2 for the branches), T <= 16.
+// Small-token kernel of the expanded layer (Appendix B, Eq. 9; Sec. 3.2 for the branches): up to 16 tokens, and small
+// layers on more tokens in slices of 16 (gridDim.y; see the rule in launch_stream).
 //
 // With a handful of tokens the layer is bound by streaming the packed weight codes from HBM once,
 // so the kernel is built around the byte stream.  A "slab" is 8 consecutive output channels of
@@ -55,6 +56,7 @@ struct Params {
   int prefetch;           // the expanded layer is not being written by the launch before: weights may be fetched ahead of the dependency wait
   uint32_t split_mask;    // summed ensemble on one shared input, run as ONE cluster of all orders: bit k marks the order (k > 0)
                           // that opens the next predictor, whose chain the epilogue starts from zero
+  int slice_tokens;       // tokens of a slice: the CTAs of slice z compute the tokens [z, z + 1) * slice_tokens
   int ctas_per_branch;    // every branch has its own CTAs, so no CTA's range crosses a branch boundary
 };
 
@@ -190,6 +192,8 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
   const int depth = p.depth;
 
   // this CTA's slabs: [s0, s0 + cnt), all of one branch
+  const int tok0 = static_cast<int>(blockIdx.y) * p.slice_tokens;
+  const int tok_end = min(static_cast<int>(p.f.T), tok0 + p.slice_tokens);
   const int my_branch = static_cast<int>(blockIdx.x) / p.ctas_per_branch, cib = static_cast<int>(blockIdx.x) % p.ctas_per_branch;
   const int base = p.slabs_per_branch / p.ctas_per_branch, rem = p.slabs_per_branch % p.ctas_per_branch;
   const int s0 = my_branch * p.slabs_per_branch + cib * base + min(cib, rem);
@@ -320,7 +324,7 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
             if (kb < p.kblocks) {
               if (idx == 0) {
                 // activations: token rows beyond T and reduction bytes beyond I come back as zeros
-                if (what != 1) tma_load_2d(sbase + kbs * kXTile, &p.tmap_x[P.branch], kb * 128, 0, bar);
+                if (what != 1) tma_load_2d(sbase + kbs * kXTile, &p.tmap_x[P.branch], kb * 128, tok0, bar);
               } else if (what != 2 && P.seg_rows[idx - 1] > 0) {
                 const int ko = idx - 1;
                 const OrderView& ov = p.f.order[br.k_begin + ko];
@@ -582,8 +586,8 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
               for (int e = 0; e < 2; ++e) {
                 const int a = (a4[t][2 * half + e] >> p.shift) - zr;   // exact: the sum carries a factor 2^shift
                 y[t][e] = __fmaf_rn(__int2float_rn(a), cs, y[t][e]);
-                const int tok = 8 * t + 2 * tig + e;
-                if (p.f.partials && tok < p.f.T) p.f.partials[static_cast<int64_t>(tok) * p.f.total_rows + roff + row] = a;
+                const int tok = tok0 + 8 * t + 2 * tig + e;
+                if (p.f.partials && tok < tok_end) p.f.partials[static_cast<int64_t>(tok) * p.f.total_rows + roff + row] = a;
               }
           }
         }
@@ -598,8 +602,8 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
         for (int t = 0; t < NT; ++t)
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
-            const int tok = 8 * t + 2 * tig + e;
-            if (tok >= p.f.T) continue;
+            const int tok = tok0 + 8 * t + 2 * tig + e;
+            if (tok >= tok_end) continue;
             float v = y[t][e];
             if (bias) v = __fadd_rn(v, bv);
             if (p.f.q8_out) {
@@ -674,10 +678,12 @@ static bool kernel_info(void (*kern)(const Params), int dyn_wanted_or_0, int* sm
 
 }  // namespace st
 
-static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, uint32_t split_mask = 0) {
+static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool slices, uint32_t split_mask = 0) {
   using namespace st;
   const bool zp = has_zero_point(a);   // (its row sums take the place of a token)
-  if (a.T > (zp ? 15 : 16) || a.g % 8 != 0 || a.O % 8 != 0) return PIPE_ERR_UNSUPPORTED;
+  const int slice_tokens = zp ? 15 : 16;
+  const int nslices = static_cast<int>(ceil_div<int64_t>(a.T < 4096 ? a.T : 4096, slice_tokens));
+  if ((a.T > slice_tokens && !slices) || nslices * a.num_branches > kPlanSMs || a.g % 8 != 0 || a.O % 8 != 0) return PIPE_ERR_UNSUPPORTED;
   if (zp && a.q8_out) return PIPE_ERR_UNSUPPORTED;
   if (a.ldxq % 16 != 0) return PIPE_ERR_UNSUPPORTED;   // tensor-map row pitch
   for (int m = 0; m < a.num_branches; ++m)
@@ -689,6 +695,7 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, uint
   p.f = a;
   p.prefetch = a.blob_settled ? 1 : 0;
   p.split_mask = split_mask;
+  p.slice_tokens = slice_tokens;
   const int nt = a.T <= (zp ? 7 : 8) ? 1 : 2;
   const int np = max_cluster <= 2 ? 1 : (max_cluster <= 4 ? 2 : 4);
   const int spw = (np * nt <= 2) ? 5 : (np * nt == 4 ? 2 : 1);
@@ -734,11 +741,18 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, uint
   };
   int smem_max = 0, sms = 0, fixed = 0;
   if (!kernel_info(kern, 0, &smem_max, &sms, &fixed)) return PIPE_ERR_CUDA;
-  p.ctas_per_branch = sms / a.num_branches;
+  p.ctas_per_branch = sms / (a.num_branches * nslices);
   if (p.ctas_per_branch < 1) return PIPE_ERR_UNSUPPORTED;
   if (p.ctas_per_branch > p.slabs_per_branch) p.ctas_per_branch = p.slabs_per_branch;
   const int grid = p.ctas_per_branch * a.num_branches;
   p.own_max = ceil_div(p.slabs_per_branch, p.ctas_per_branch);
+  // More than 16 tokens: every slice of 16 streams the weights again (from L2), for which the launch needs neither the
+  // tile set-up nor the long pipeline of the SM-pair kernel.  That pays while a CTA's slabs fit one pass and its share of a
+  // reduction block stays small.  Measured, slices against pair kernel: 256 x 256 int8, T = 64: 5.3 / 7.5 us; 512 x 4096
+  // int4 K = 3, T = 256: 11.7 / 18.5; 3072 x 768 M = 2, T = 48: 7.4 / 12.5; 11008 -> 4096 M = 2, T = 32: 32.8 / 43.4 (14 KiB);
+  // beyond one pass 1024 x 1024 M = 2, T = 200: 12.5 / 11.9, 3072 x 768, T = 100: 15.7 / 11.9; beyond 20 KiB 4096 x 4096
+  // int8 K = 2, T = 64: 28.8 / 20.2 (28 KiB), T = 48: 19.1 / 20.1 (22 KiB).
+  if (nslices > 1 && (p.own_max > p.pass_slabs || p.own_max * 8 * max_cluster * p.pk > (20 << 10))) return PIPE_ERR_UNSUPPORTED;
   // one pass whose slab slots are (nearly) all taken: the kernel without per-slab branches, with just the slots it needs
   {
     const int slots = ceil_div(p.own_max, kGroupWarps);
@@ -775,7 +789,7 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, uint
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.gridDim = dim3(grid, nslices, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = dyn;
   cfg.stream = stream;
@@ -786,10 +800,10 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, uint
   return launch_status();
 }
 
-pipe_status forward_stream(const ForwardArgs& a, cudaStream_t stream) {
+pipe_status forward_stream(const ForwardArgs& a, cudaStream_t stream, bool slices) {
   if (a.T == 0) return PIPE_OK;
   const bool sum_mode = a.num_branches > 1 && a.branch[1].accumulate;
-  if (!sum_mode) return launch_stream(a, stream);
+  if (!sum_mode) return launch_stream(a, stream, slices);
   // predictors that share input and step: one launch on the cluster of all orders, the chains added in registers
   if (!a.q8_out && !has_zero_point(a)) {
     bool shared = true;
@@ -805,7 +819,7 @@ pipe_status forward_stream(const ForwardArgs& a, cudaStream_t stream) {
       one.branch[0].accumulate = 0;
       uint32_t split = 0;
       for (int m = 1; m < a.num_branches; ++m) split |= 1u << a.branch[m].k_begin;
-      const pipe_status st = launch_stream(one, stream, split);
+      const pipe_status st = launch_stream(one, stream, slices, split);
       if (st != PIPE_ERR_UNSUPPORTED) return st;
     }
   }
@@ -813,7 +827,7 @@ pipe_status forward_stream(const ForwardArgs& a, cudaStream_t stream) {
     ForwardArgs one = a;
     one.num_branches = 1;
     one.branch[0] = a.branch[m];
-    pipe_status st = launch_stream(one, stream);
+    pipe_status st = launch_stream(one, stream, slices);
     if (st != PIPE_OK) return st;
   }
   return PIPE_OK;

@@ -1243,9 +1243,9 @@ static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_
   }
   // (a single token tile: the second CTA of a pair then stages zeros and stores nothing, but still unpacks its half of
   // every block, which is what such a launch spends its time on)
-  if (p.ntok_tiles == 1 && kernel_choice() == 0 && !zp) {
-    // ... unless the whole layer is a handful of blocks: then nothing is there to share and the one-SM kernel's shorter
-    // set-up wins (a forced choice of this kernel still takes the launch)
+  if (p.ntok_tiles == 1 && kernel_choice() == 0 && !zp && a.bits == 2 && !direct) {
+    // ... unless the layer is a handful of blocks of 2-bit codes, where the one-SM kernel is ahead (512 x 768, K = 4:
+    // 10.0 against 11.4 us; with 4 and 8 bits the pair is: 512 x 4096 18.4 against 24.8, 256 x 2304 10.8 against 40)
     int64_t rows = 0;
     for (int m = 0; m < a.num_branches; ++m)
       for (int k = a.branch[m].k_begin; k < a.branch[m].k_end; ++k) rows += a.order[k].rows;

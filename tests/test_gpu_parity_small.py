@@ -745,3 +745,38 @@ def test_two_layer_convolutional_ensemble_chain(oracle):
         rows1.append(_lower_im2col(q.reshape(N, Hh, Ww, C1), 3, 3, 1, 1, 1)[0])
     want, _ = oracle.ensemble(e2, np.stack(rows1), steps, split, bias=b2, sum_branches=True)
     np.testing.assert_array_equal(y.cpu().numpy().view(np.uint32), want.view(np.uint32))
+
+
+# T around the slices of 16 (15 beside a zero point) in which small layers on more than 16 tokens stream their weights,
+# and around the last T that the rule gives them
+@pytest.mark.parametrize("T", [17, 31, 32, 33, 100, 161])
+@pytest.mark.parametrize("O,I,bits,K,g,n_keep,M", [(128, 144, 4, 4, 8, 9, 2), (264, 400, 8, 2, 8, 33, 1), (320, 272, 2, 8, 16, 7, 4),
+                                                   (1024, 128, 4, 2, 8, 64, 1)])
+def test_small_layers_in_token_slices(O, I, bits, K, g, n_keep, M, T):
+    rng = np.random.default_rng(O + T)
+    layer = H.gpu_expand(H.desc_of(O, I, bits, K, g, n_keep, M), _w(rng, O, I, heavy=(bits == 2)))
+    bias = torch.from_numpy(rng.standard_normal(O).astype(np.float32)).cuda()
+    xq = [torch.from_numpy(rng.integers(-127, 128, (T, I)).astype(np.int8)).cuda() for _ in range(M)]
+    sx = [torch.tensor([0.01 * (1 + m)], device="cuda") for m in range(M)]
+    step = [torch.tensor([0.3], device="cuda")] * M
+
+    def run(choice):
+        B.pipe_diag_select_kernel(choice)
+        try:
+            ys = [torch.full((T, O), float("nan"), device="cuda") for _ in range(M)]
+            one = [torch.full((T, O), float("nan"), device="cuda") for _ in range(3)]
+            yq = [torch.full((T, O), 99, dtype=torch.int8, device="cuda") for _ in range(M)]
+            part = torch.zeros((T, layer.layout.total_rows), dtype=torch.int32, device="cuda")
+            B.pipe_ensemble_forward(layer.desc, layer.blob, xq, sx, ys, bias, False, part)
+            B.pipe_ensemble_forward(layer.desc, layer.blob, xq, sx, one[:1], bias, True)
+            B.pipe_ensemble_forward(layer.desc, layer.blob, xq[:1] * M, sx[:1] * M, one[1:2], bias, True)
+            B.pipe_expanded_linear(layer.desc, layer.blob, xq[0], sx[0], one[2], bias)
+            B.pipe_ensemble_forward_q8(layer.desc, layer.blob, xq, sx, step, yq, bias, B.ACT_RELU)
+        finally:
+            B.pipe_diag_select_kernel(B.KERNEL_AUTO)
+        torch.cuda.synchronize()
+        return [y.view(torch.int32) for y in ys + one] + yq + [part]
+
+    for a, b in zip(run(B.KERNEL_REFERENCE), run(B.KERNEL_AUTO)):
+        assert torch.equal(a, b)
+    assert B.pipe_poll_status() == B.PIPE_OK
