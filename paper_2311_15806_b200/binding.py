@@ -123,6 +123,13 @@ def lib() -> C.CDLL:
     return _lib
 
 
+try:
+    _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+except AttributeError:   # a torch build without CUDA, or one that no longer has these
+    _current_device = lambda: None                                           # noqa: E731
+    _raw_stream = lambda _: int(torch.cuda.current_stream().cuda_stream)     # noqa: E731
+
+
 def _check(status: int, where: str) -> None:
     if status != PIPE_OK:
         raise PipeError(status, where)
@@ -130,7 +137,8 @@ def _check(status: int, where: str) -> None:
 
 def _stream_ptr(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the raw handle of torch.cuda.current_stream() without building the Stream object (2 us of a 10 us call)
+        return _raw_stream(_current_device())
     return int(stream.cuda_stream)
 
 
