@@ -164,8 +164,16 @@ __device__ __forceinline__ int rows_before(const int32_t* cum, int c, int O, int
 // ZP: asymmetric activations, sum_i (c - z) q = sum_i c q - z sum_i q.  The last token column of the MMAs (7, or 15 with
 // two token tiles) is fed ones instead of a token, so its accumulators are the row sums of the codes; the epilogue reads
 // them from the neighbouring lane that holds that column.
-template <int BITS, int NT, int NP, bool SUMMED, int FULL, bool ZP>
+//
+// MODE 0: every branch writes its own output.  1: a summed ensemble whose predictors share one input, as one cluster of all
+// orders.  2: the same for TWO predictors of at most two orders each on inputs of their own: order pair q of a slab belongs
+// to predictor q and meets predictor q's activation tile, of which a stage then holds two.  (More pairs than two do not
+// leave a warp the registers for its slabs; such ensembles run one launch per predictor, each adding into y.  11008 -> 4096,
+// K = 4, two predictors: T = 1 37 us in two launches, 24.3 in one, T = 13 40 and 26.9.)
+template <int BITS, int NT, int NP, int MODE, int FULL, bool ZP>
 __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __grid_constant__ Params p) {
+  constexpr bool SUMMED = MODE != 0;
+  constexpr int NX = MODE == 2 ? 2 : 1;         // activation tiles of a reduction block
   constexpr int SPW = FULL ? FULL : ((NP * NT <= 2) ? 5 : (NP * NT == 4 ? 2 : 1));   // slabs per consumer warp and pass
   constexpr int CHK = 128 / BITS;               // codes per 16-byte chunk
   constexpr int KBPS = (BITS == 2) ? 2 : 1;     // reduction blocks per stage
@@ -267,7 +275,7 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
   __syncthreads();
   if (threadIdx.x < npass) {
     Pass& P = passes[threadIdx.x];
-    int off = KBPS * kXTile;
+    int off = NX * KBPS * kXTile;
     int wb = 0;
     for (int ko = 0; ko < kMaxOrd; ++ko) {
       P.seg_off[ko] = off;
@@ -307,26 +315,26 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
           int nkb = 0;
 #pragma unroll
           for (int kbs = 0; kbs < KBPS; ++kbs) nkb += (ks * KBPS + kbs < p.kblocks) ? 1 : 0;
-          mbar_expect_tx(bar, static_cast<uint32_t>(nkb * (kXTile + P.wbytes)));
+          mbar_expect_tx(bar, static_cast<uint32_t>(nkb * (NX * kXTile + P.wbytes)));
         }
       }
       __syncwarp();
       if (*abort_flag) break;
       // jobs of a stage: per reduction block, the activation tile and then one run of rows per order
       // (what: 0 all of them, 1 the weights only, 2 the activation tiles only)
-      const int njobs = KBPS * (1 + nk);
+      const int njobs = KBPS * (NX + nk);
       auto issue_jobs = [&](int what) {
-        for (int j0 = 0; j0 < KBPS * (1 + p.nkmax); j0 += kJobLanes) {   // same trip count in every lane; lanes without a job idle
+        for (int j0 = 0; j0 < KBPS * (NX + p.nkmax); j0 += kJobLanes) {   // same trip count in every lane; lanes without a job idle
           const int j = j0 + job0;
           if (valid && j < njobs) {
-            const int kbs = j / (1 + nk), idx = j - kbs * (1 + nk);
+            const int kbs = j / (NX + nk), idx = j - kbs * (NX + nk);
             const int kb = ks * KBPS + kbs;
             if (kb < p.kblocks) {
-              if (idx == 0) {
+              if (idx < NX) {
                 // activations: token rows beyond T and reduction bytes beyond I come back as zeros
-                if (what != 1) tma_load_2d(sbase + kbs * kXTile, &p.tmap_x[P.branch], kb * 128, tok0, bar);
-              } else if (what != 2 && P.seg_rows[idx - 1] > 0) {
-                const int ko = idx - 1;
+                if (what != 1) tma_load_2d(sbase + (idx * KBPS + kbs) * kXTile, &p.tmap_x[P.branch + idx], kb * 128, tok0, bar);
+              } else if (what != 2 && P.seg_rows[idx - NX] > 0) {
+                const int ko = idx - NX;
                 const OrderView& ov = p.f.order[br.k_begin + ko];
                 const uint8_t* src = ov.kcodes + (static_cast<size_t>(kb) * ov.rows + P.seg_row0[ko]) * p.pk;
                 bulk_load(sbase + P.seg_off[ko] + kbs * P.seg_rows[ko] * p.pk, src, static_cast<uint32_t>(P.seg_rows[ko] * p.pk), bar);
@@ -357,6 +365,7 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
   } else {
     // ================================================================== consumer warps
     if (p.prefetch) asm volatile("griddepcontrol.wait;" ::: "memory");   // (the steps and the bias are the caller's data)
+    const int ksecond = MODE == 2 ? __ffs(p.split_mask) - 1 : 0;   // MODE 2: first order of the second predictor
     // scale products s_k * lambda_x and bias of every own slab (needed at the end of a pass only;
     // the loads overlap the first copies)
     for (int e = threadIdx.x; e < cnt * p.nkmax * 8; e += 32 * kConsWarps) {
@@ -365,7 +374,7 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
       const BranchArgs& br = p.f.branch[branch];
       const int row0 = slabmeta[li * p.nkmax + ko];
       float v = 0.f;
-      if (row0 >= 0) v = __fmul_rn(__ldg(p.f.order[br.k_begin + ko].scales + row0 + r), __ldg(br.sx));
+      if (row0 >= 0) v = __fmul_rn(__ldg(p.f.order[br.k_begin + ko].scales + row0 + r), __ldg((MODE == 2 && ko >= ksecond) ? p.f.branch[1].sx : br.sx));
       cstab[e] = v;
     }
     for (int e = threadIdx.x; e < cnt * 8; e += 32 * kConsWarps) {
@@ -394,28 +403,31 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
       if (lane < SPW) {
         int* ct = mychunks + lane * centries;
         const int sl = wg + kGroupWarps * lane;
-        int n = 0;
+        int n = 0, present = 0;
         if (sl < nsl) {
           for (int ko = 0; ko < nk; ++ko) {
             const int row0 = slabmeta[(P.lb + sl) * p.nkmax + ko];
             if (row0 < 0) continue;
+            if (MODE == 2 && ko >= ksecond && n < 2) n = 2;
             ct[2 + 3 * n] = P.seg_off[ko] + (row0 - P.seg_row0[ko]) * p.pk;
             ct[3 + 3 * n] = P.seg_rows[ko] * p.pk;
+            present |= 1 << n;
             ++n;
           }
         }
-        ct[0] = n;
+        ct[0] = MODE == 2 ? present : n;
       }
       __syncwarp();
-      int nchunks[SPW];
+      int nchunks[SPW];   // kept orders of the slab; MODE 2: bit ci set where position ci is taken
+      auto have = [&](int s, int ci) { return MODE == 2 ? ((nchunks[s] >> ci) & 1) != 0 : ci < nchunks[s]; };
       uint32_t woff[SPW][2 * NP], wstr[SPW][2 * NP];
 #pragma unroll
       for (int s = 0; s < SPW; ++s) {
         nchunks[s] = mychunks[s * centries];
 #pragma unroll
         for (int ci = 0; ci < 2 * NP; ++ci) {
-          woff[s][ci] = ci < nchunks[s] ? mychunks[s * centries + 2 + 3 * ci] : 0;
-          wstr[s][ci] = ci < nchunks[s] ? mychunks[s * centries + 3 + 3 * ci] : 0;
+          woff[s][ci] = have(s, ci) ? mychunks[s * centries + 2 + 3 * ci] : 0;
+          wstr[s][ci] = have(s, ci) ? mychunks[s * centries + 3 + 3 * ci] : 0;
         }
       }
       int acc[SPW][NP][NT][4];
@@ -450,15 +462,15 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
           // integers, and zero times anything is zero).
           const bool live = ks * KBPS + kbs < p.kblocks;
           const uint32_t wbyte = static_cast<uint32_t>(gid * p.pk + ((within * BITS) >> 3));
-          uint4 xv[XCH][NT];
+          uint4 xv[NX][XCH][NT];
 #pragma unroll
-          for (int v = 0; v < XCH; ++v)
+          for (int v = 0; v < NX * XCH; ++v)
 #pragma unroll
             for (int t = 0; t < NT; ++t) {
               const int r = gid + 8 * t;
-              const int c16 = (within >> 4) + v;
-              xv[v][t] = lds128(sgen, kbs * kXTile + r * 128 + ((c16 ^ (r & 7)) << 4));
-              if (ZP && t == NT - 1 && gid == 7) xv[v][t] = make_uint4(0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u);
+              const int c16 = (within >> 4) + v % XCH;
+              xv[v / XCH][v % XCH][t] = lds128(sgen, (v / XCH * KBPS + kbs) * kXTile + r * 128 + ((c16 ^ (r & 7)) << 4));
+              if (ZP && t == NT - 1 && gid == 7) xv[v / XCH][v % XCH][t] = make_uint4(0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u);
             }
 #pragma unroll
           for (int s = 0; s < SPW; ++s) {
@@ -470,13 +482,13 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
                 // replaced by zero weights)
                 wa = lds128(sgen, woff[s][2 * q] + kbs * wstr[s][2 * q] + wbyte);
                 wb = lds128(sgen, woff[s][2 * q + 1] + kbs * wstr[s][2 * q + 1] + wbyte);
-                const bool ha = live && 2 * q < nchunks[s], hb = live && 2 * q + 1 < nchunks[s];
+                const bool ha = live && have(s, 2 * q), hb = live && have(s, 2 * q + 1);
                 wa = ha ? wa : make_uint4(0, 0, 0, 0);
                 wb = hb ? wb : make_uint4(0, 0, 0, 0);
               } else {
-                if (2 * q >= nchunks[s]) continue;
+                if (!have(s, 2 * q)) continue;
                 if (live) wa = lds128(sgen, woff[s][2 * q] + kbs * wstr[s][2 * q] + wbyte);
-                if (live && 2 * q + 1 < nchunks[s]) wb = lds128(sgen, woff[s][2 * q + 1] + kbs * wstr[s][2 * q + 1] + wbyte);
+                if (live && have(s, 2 * q + 1)) wb = lds128(sgen, woff[s][2 * q + 1] + kbs * wstr[s][2 * q + 1] + wbyte);
               }
 #pragma unroll
               for (int mm = 0; mm < 2 * XCH; ++mm) {
@@ -485,7 +497,8 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
                 frag<BITS>(wb, mm, b0, b1);
 #pragma unroll
                 for (int t = 0; t < NT; ++t) {
-                  const uint32_t xw[4] = {xv[mm >> 1][t].x, xv[mm >> 1][t].y, xv[mm >> 1][t].z, xv[mm >> 1][t].w};
+                  const uint4& xr = xv[MODE == 2 ? q : 0][mm >> 1][t];
+                  const uint32_t xw[4] = {xr.x, xr.y, xr.z, xr.w};
                   // tile rows 0-7: first order of the pair, rows 8-15: second order
                   mma_s8(acc[s][q][t], a0, b0, a1, b1, xw[2 * (mm & 1)], xw[2 * (mm & 1) + 1]);
                 }
@@ -504,7 +517,7 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
         if (sl >= nsl) continue;
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
-          if (2 * q >= nchunks[s]) continue;
+          if (!have(s, 2 * q)) continue;
 #pragma unroll
           for (int t = 0; t < NT; ++t)
 #pragma unroll
@@ -521,9 +534,14 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
         // kept orders of the slab, ascending (at most 2 * NP)
         int kos[2 * NP];
         int nch = 0;
+        if constexpr (MODE == 2) {
+#pragma unroll
+          for (int ci = 0; ci < 2 * NP; ++ci) kos[ci] = -1;
+        }
 #pragma unroll
         for (int ko = 0; ko < kMaxOrd; ++ko)
           if (ko < nk && slabmeta[li * p.nkmax + ko] >= 0) {
+            if (MODE == 2 && ko >= ksecond && nch < 2) nch = 2;
 #pragma unroll
             for (int ci = 0; ci < 2 * NP; ++ci)
               if (ci == nch) kos[ci] = ko;
@@ -559,7 +577,7 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
         };
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
-          if (2 * q >= nch) continue;
+          if (MODE == 2 ? kos[2 * q] < 0 : 2 * q >= nch) continue;
           int a4[NT][4];
 #pragma unroll
           for (int t = 0; t < NT; ++t)
@@ -572,7 +590,7 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
             const int ci = 2 * q + half;
-            if (ci >= nch) continue;
+            if (MODE == 2 ? kos[ci] < 0 : ci >= nch) continue;
             const int ko = kos[ci];
             if constexpr (SUMMED) close_up_to(ko);
             const float cs = cstab[(li * p.nkmax + ko) * 8 + gid];
@@ -636,11 +654,12 @@ struct KernelInfo {
   const void* fn = nullptr;
   int fixed = 0, dyn_set = 0;
 };
+constexpr int kMaxKernels = 128;   // instantiations of the kernel (90)
 struct DeviceCache {
   std::mutex mu;
   bool ready = false;
   int smem_max = 0, sms = 0, n = 0;
-  KernelInfo k[64];
+  KernelInfo k[kMaxKernels];
 };
 
 static bool kernel_info(void (*kern)(const Params), int dyn_wanted_or_0, int* smem_max, int* sms, int* fixed) {
@@ -659,7 +678,7 @@ static bool kernel_info(void (*kern)(const Params), int dyn_wanted_or_0, int* sm
   for (int i = 0; i < c.n; ++i)
     if (c.k[i].fn == reinterpret_cast<const void*>(kern)) ki = &c.k[i];
   if (!ki) {
-    if (c.n >= 64) return false;
+    if (c.n >= kMaxKernels) return false;
     cudaFuncAttributes fattr;
     if (cudaFuncGetAttributes(&fattr, kern) != cudaSuccess) return false;
     ki = &c.k[c.n++];
@@ -678,7 +697,7 @@ static bool kernel_info(void (*kern)(const Params), int dyn_wanted_or_0, int* sm
 
 }  // namespace st
 
-static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool slices, uint32_t split_mask = 0) {
+static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool slices, uint32_t split_mask = 0, bool distinct = false) {
   using namespace st;
   const bool zp = has_zero_point(a);   // (its row sums take the place of a token)
   const int slice_tokens = zp ? 15 : 16;
@@ -686,7 +705,7 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
   if ((a.T > slice_tokens && !slices) || nslices * a.num_branches > kPlanSMs || a.g % 8 != 0 || a.O % 8 != 0) return PIPE_ERR_UNSUPPORTED;
   if (zp && a.q8_out) return PIPE_ERR_UNSUPPORTED;
   if (a.ldxq % 16 != 0) return PIPE_ERR_UNSUPPORTED;   // tensor-map row pitch
-  for (int m = 0; m < a.num_branches; ++m)
+  for (int m = 0; m < (distinct ? 2 : a.num_branches); ++m)
     if (reinterpret_cast<uintptr_t>(a.branch[m].xq) & 15) return PIPE_ERR_UNSUPPORTED;
   int max_cluster = 0;
   for (int m = 0; m < a.num_branches; ++m) max_cluster = max(max_cluster, a.branch[m].k_end - a.branch[m].k_begin);
@@ -697,7 +716,7 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
   p.split_mask = split_mask;
   p.slice_tokens = slice_tokens;
   const int nt = a.T <= (zp ? 7 : 8) ? 1 : 2;
-  const int np = max_cluster <= 2 ? 1 : (max_cluster <= 4 ? 2 : 4);
+  const int np = distinct ? 2 : max_cluster <= 2 ? 1 : (max_cluster <= 4 ? 2 : 4);
   const int spw = (np * nt <= 2) ? 5 : (np * nt == 4 ? 2 : 1);
   p.kblocks = ceil_div(a.I, 128);
   p.pk = 128 * a.bits / 8;
@@ -714,26 +733,38 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
   if (nt == 1) kern = np == 1 ? stream_forward_kernel<B, 1, 1, S, 0, Z> : (np == 2 ? stream_forward_kernel<B, 1, 2, S, 0, Z> : stream_forward_kernel<B, 1, 4, S, 0, Z>); \
   else kern = np == 1 ? stream_forward_kernel<B, 2, 1, S, 0, Z> : (np == 2 ? stream_forward_kernel<B, 2, 2, S, 0, Z> : stream_forward_kernel<B, 2, 4, S, 0, Z>);
   if (zp) {
-    if (a.bits == 8) { PIPE_ST_PICK(8, false, true) } else if (a.bits == 4) { PIPE_ST_PICK(4, false, true) } else { PIPE_ST_PICK(2, false, true) }
+    if (a.bits == 8) { PIPE_ST_PICK(8, 0, true) } else if (a.bits == 4) { PIPE_ST_PICK(4, 0, true) } else { PIPE_ST_PICK(2, 0, true) }
   } else if (split_mask == 0) {
-    if (a.bits == 8) { PIPE_ST_PICK(8, false, false) } else if (a.bits == 4) { PIPE_ST_PICK(4, false, false) } else { PIPE_ST_PICK(2, false, false) }
+    if (a.bits == 8) { PIPE_ST_PICK(8, 0, false) } else if (a.bits == 4) { PIPE_ST_PICK(4, 0, false) } else { PIPE_ST_PICK(2, 0, false) }
+  } else if (distinct) {
+    if (a.bits == 8) kern = nt == 1 ? stream_forward_kernel<8, 1, 2, 2, 0, false> : stream_forward_kernel<8, 2, 2, 2, 0, false>;
+    else if (a.bits == 4) kern = nt == 1 ? stream_forward_kernel<4, 1, 2, 2, 0, false> : stream_forward_kernel<4, 2, 2, 2, 0, false>;
+    else kern = nt == 1 ? stream_forward_kernel<2, 1, 2, 2, 0, false> : stream_forward_kernel<2, 2, 2, 2, 0, false>;
   } else {   // a summed ensemble on a shared input: the epilogue that closes the predictors' chains
-    if (a.bits == 8) { PIPE_ST_PICK(8, true, false) } else if (a.bits == 4) { PIPE_ST_PICK(4, true, false) } else { PIPE_ST_PICK(2, true, false) }
+    if (a.bits == 8) { PIPE_ST_PICK(8, 1, false) } else if (a.bits == 4) { PIPE_ST_PICK(4, 1, false) } else { PIPE_ST_PICK(2, 1, false) }
   }
 #undef PIPE_ST_PICK
   // the same kernel without per-slab branches, by slab slots per warp (one order pair; up to 8 tokens: 2 to 5 slots,
   // 9 to 16 tokens: 2 or 3 -- more would spill)
   auto full_kernel = [&](int slots) -> void (*)(const Params) {
+    if (distinct) {   // one or two slots
+#define PIPE_ST_DIST(B)                                                                                                   \
+  if (slots == 1) return nt == 1 ? stream_forward_kernel<B, 1, 2, 2, 1, false> : stream_forward_kernel<B, 2, 2, 2, 1, false>; \
+  if (slots == 2) return nt == 1 ? stream_forward_kernel<B, 1, 2, 2, 2, false> : stream_forward_kernel<B, 2, 2, 2, 2, false>;
+      if (a.bits == 8) { PIPE_ST_DIST(8) } else if (a.bits == 4) { PIPE_ST_DIST(4) } else { PIPE_ST_DIST(2) }
+#undef PIPE_ST_DIST
+      return nullptr;
+    }
     if (split_mask != 0 || np != 1 || zp) return nullptr;
 #define PIPE_ST_FULL(B)                                                                                       \
   if (nt == 1) {                                                                                              \
-    if (slots == 2) return stream_forward_kernel<B, 1, 1, false, 2, false>;                                          \
-    if (slots == 3) return stream_forward_kernel<B, 1, 1, false, 3, false>;                                          \
-    if (slots == 4) return stream_forward_kernel<B, 1, 1, false, 4, false>;                                          \
-    if (slots == 5) return stream_forward_kernel<B, 1, 1, false, 5, false>;                                          \
+    if (slots == 2) return stream_forward_kernel<B, 1, 1, 0, 2, false>;                                          \
+    if (slots == 3) return stream_forward_kernel<B, 1, 1, 0, 3, false>;                                          \
+    if (slots == 4) return stream_forward_kernel<B, 1, 1, 0, 4, false>;                                          \
+    if (slots == 5) return stream_forward_kernel<B, 1, 1, 0, 5, false>;                                          \
   } else {                                                                                                    \
-    if (slots == 2) return stream_forward_kernel<B, 2, 1, false, 2, false>;                                          \
-    if (slots == 3) return stream_forward_kernel<B, 2, 1, false, 3, false>;                                          \
+    if (slots == 2) return stream_forward_kernel<B, 2, 1, 0, 2, false>;                                          \
+    if (slots == 3) return stream_forward_kernel<B, 2, 1, 0, 3, false>;                                          \
   }
     if (a.bits == 8) { PIPE_ST_FULL(8) } else if (a.bits == 4) { PIPE_ST_FULL(4) } else { PIPE_ST_FULL(2) }
 #undef PIPE_ST_FULL
@@ -752,11 +783,13 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
   // int4 K = 3, T = 256: 11.7 / 18.5; 3072 x 768 M = 2, T = 48: 7.4 / 12.5; 11008 -> 4096 M = 2, T = 32: 32.8 / 43.4 (14 KiB);
   // beyond one pass 1024 x 1024 M = 2, T = 200: 12.5 / 11.9, 3072 x 768, T = 100: 15.7 / 11.9; beyond 20 KiB 4096 x 4096
   // int8 K = 2, T = 64: 28.8 / 20.2 (28 KiB), T = 48: 19.1 / 20.1 (22 KiB).
-  if (nslices > 1 && (p.own_max > p.pass_slabs || p.own_max * 8 * max_cluster * p.pk > (20 << 10))) return PIPE_ERR_UNSUPPORTED;
+  // (Two predictors in one launch, MODE 2, against one launch each, both in slices: 3072 -> 768, T = 32: 11.6 / 18.3 us,
+  // 4 KiB; 11008 -> 4096: 46.5 / 41.1, 14 KiB.)
+  if (nslices > 1 && (p.own_max > p.pass_slabs || p.own_max * 8 * max_cluster * p.pk > ((distinct ? 8 : 20) << 10))) return PIPE_ERR_UNSUPPORTED;
   // one pass whose slab slots are (nearly) all taken: the kernel without per-slab branches, with just the slots it needs
   {
     const int slots = ceil_div(p.own_max, kGroupWarps);
-    void (*kern_full)(const Params) = (p.own_max > kGroupWarps) ? full_kernel(slots) : nullptr;
+    void (*kern_full)(const Params) = (p.own_max > kGroupWarps || distinct) ? full_kernel(slots) : nullptr;
     if (kern_full) {
       kern = kern_full;
       p.pass_slabs = kGroupWarps * slots;
@@ -767,7 +800,7 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
   if (ceil_div(p.own_max, p.pass_slabs) > kMaxPasses) return PIPE_ERR_UNSUPPORTED;
   // a stage holds one reduction block (two for 2-bit codes) of every order for the slabs of a pass, all kept
   const int pass_cap = p.pass_slabs < p.own_max ? p.pass_slabs : p.own_max;
-  p.stage_bytes = round_up(p.kbps * (kXTile + pass_cap * 8 * max_cluster * p.pk), 1024);
+  p.stage_bytes = round_up(p.kbps * ((distinct ? 2 : 1) * kXTile + pass_cap * 8 * max_cluster * p.pk), 1024);
   const int table_bytes = p.own_max * (max_cluster * 4 + max_cluster * 32 + 32) + kConsWarps * spw * (1 + 3 * max_cluster) * 4 +
                           p.pass_slabs * np * nt * 4 * 32 * 4;
   const int avail = smem_max - fixed - 1024 - round_up(table_bytes, 16);
@@ -779,7 +812,7 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
   p.depth -= p.depth % kProdWarps;   // every producer warp owns depth / kProdWarps slots
   if (p.depth < kProdWarps) return PIPE_ERR_UNSUPPORTED;
   const int dyn = 1024 + p.depth * p.stage_bytes + round_up(table_bytes, 16);
-  for (int m = 0; m < a.num_branches; ++m)
+  for (int m = 0; m < (distinct ? 2 : a.num_branches); ++m)
     if (!make_tensor_map_2d_u8(&p.tmap_x[m], a.branch[m].xq, static_cast<uint64_t>(a.I), static_cast<uint64_t>(a.T),
                                static_cast<uint64_t>(a.ldxq), 128, 16, true))
       return PIPE_ERR_CUDA;
@@ -811,7 +844,10 @@ pipe_status forward_stream(const ForwardArgs& a, cudaStream_t stream, bool slice
       shared = shared && a.branch[m].xq == a.branch[0].xq && a.branch[m].sx == a.branch[0].sx &&
                a.branch[m].k_begin == a.branch[m - 1].k_end && a.branch[m].y == a.branch[0].y;
     const int k0 = a.branch[0].k_begin, k1 = a.branch[a.num_branches - 1].k_end;
-    if (shared && k0 == 0) {
+    // (two predictors of at most two orders each on inputs of their own: one launch as well)
+    const bool distinct = !shared && a.num_branches == 2 && a.branch[1].k_begin == a.branch[0].k_end && a.branch[1].y == a.branch[0].y &&
+                          a.branch[0].k_end - k0 <= 2 && k1 - a.branch[1].k_begin <= 2;
+    if ((shared || distinct) && k0 == 0) {
       ForwardArgs one = a;
       one.num_branches = 1;
       one.branch[0] = a.branch[0];
@@ -819,7 +855,7 @@ pipe_status forward_stream(const ForwardArgs& a, cudaStream_t stream, bool slice
       one.branch[0].accumulate = 0;
       uint32_t split = 0;
       for (int m = 1; m < a.num_branches; ++m) split |= 1u << a.branch[m].k_begin;
-      const pipe_status st = launch_stream(one, stream, slices, split);
+      const pipe_status st = launch_stream(one, stream, slices, split, distinct);
       if (st != PIPE_ERR_UNSUPPORTED) return st;
     }
   }

@@ -780,3 +780,33 @@ def test_small_layers_in_token_slices(O, I, bits, K, g, n_keep, M, T):
     for a, b in zip(run(B.KERNEL_REFERENCE), run(B.KERNEL_AUTO)):
         assert torch.equal(a, b)
     assert B.pipe_poll_status() == B.PIPE_OK
+
+
+# two predictors on inputs of their own, summed, in one launch of the streaming kernel: one slab slot per warp, two, more
+# (several passes), clusters of one order, every code width; token counts around a tile, two tiles and the first slice
+@pytest.mark.parametrize("T", [1, 8, 9, 16, 17])
+@pytest.mark.parametrize("O,I,bits,K,g,n_keep", [(6144, 160, 4, 4, 8, 300), (12288, 144, 4, 3, 8, 600), (256, 400, 8, 2, 8, 20),
+                                                 (512, 400, 2, 4, 16, 9), (5000, 272, 8, 3, 8, 200)])
+def test_two_summed_predictors_stream_in_one_launch(O, I, bits, K, g, n_keep, T):
+    M = 2
+    rng = np.random.default_rng(O + T)
+    layer = H.gpu_expand(H.desc_of(O, I, bits, K, g, n_keep, M), _w(rng, O, I, heavy=(bits == 2)))
+    bias = torch.from_numpy(rng.standard_normal(O).astype(np.float32)).cuda()
+    xq = [torch.from_numpy(rng.integers(-127, 128, (T, I)).astype(np.int8)).cuda() for _ in range(M)]
+    sx = [torch.tensor([0.01 * (1 + m)], device="cuda") for m in range(M)]
+    out = []
+    for choice in (B.KERNEL_REFERENCE, B.KERNEL_AUTO):
+        y = torch.full((T, O), float("nan"), device="cuda")
+        part = torch.zeros((T, layer.layout.total_rows), dtype=torch.int32, device="cuda")
+        B.pipe_diag_select_kernel(choice)
+        try:
+            before = B.pipe_launch_count()
+            B.pipe_ensemble_forward(layer.desc, layer.blob, xq, sx, [y], bias, True, part)
+            launches = B.pipe_launch_count() - before
+        finally:
+            B.pipe_diag_select_kernel(B.KERNEL_AUTO)
+        torch.cuda.synchronize()
+        out.append((y.view(torch.int32), part))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    assert T > 16 or launches == 1
+    assert B.pipe_poll_status() == B.PIPE_OK
