@@ -51,7 +51,8 @@ constexpr int kStageBOff = kSub * kABytes;
 constexpr int kTmemCols = 512;
 constexpr int kAccCols = 256;
 constexpr int kMaxRing = 3;
-constexpr int kRecBufs = 3;    // copies of block records in shared memory (this tile, the next, the one before)
+constexpr int kRecBufs = 4;    // copies of block records in shared memory: a tile's, the next tile's, whose tables are made
+                               // while this tile drains, the one on its way, and one that slower warps may still be reading
 constexpr int kTileRing = 8;   // tiles whose stacked-row count the unpack warps keep for the MMA issuer (they are at
                                // most a ring of stages, i.e. three tiles, ahead of it)
 using namespace tcc;
@@ -422,6 +423,11 @@ __device__ __forceinline__ void unpack_role(const Params& p, const Rings& g, int
   }
 }
 
+__device__ __forceinline__ float4 load_row(const float* src, bool vec) {
+  if (vec) return *reinterpret_cast<const float4*>(src);
+  return make_float4(src[0], src[1], src[2], src[3]);
+}
+
 struct EpiCtx {
   uint32_t tmem_base, tfull0, tempty0;
   uint32_t recbar0;   // kRecBufs barriers: the block record of the tile has landed
@@ -437,6 +443,7 @@ struct EpiCtx {
   uint32_t tempty_lead0;   // the accumulator-released barriers of the pair's first CTA (cluster address)
   int part, nparts;  // share of the 16-channel groups this warp drains (two warps per lane quarter)
   float* stg;        // 32 rows x 16 floats, swizzled
+  float* bias_s;     // fused epilogue: [kRecBufs][PIPE_BLOCK_CHANNELS] bias of the tiles' channels (in the staging blocks' place)
   uint32_t zero_s;   // shared address of eight zero floats
   const int* zp_s;   // ZP: zero point of every branch
   int* zrow;         // ZP: [2][kMaxN] zero point times row sum of every stacked row, by accumulator buffer
@@ -461,7 +468,8 @@ struct EpiCtx {
 // outputs are summed after the layer (Sec. 3.2): every predictor's chain starts from zero, the bias closes the first
 // one, and the chains are added in ascending predictor order in this thread -- the same additions, in the same
 // order, as one launch per predictor summing into y, without the read-modify-write of y.
-template <int NKMAX, bool PARTIALS, bool Q8, bool SUMMED, bool SHORT_K, bool ZP>
+// ACC: the result is added to y (a summed ensemble's later predictors); with a zero point that is found out at run time.
+template <int NKMAX, bool PARTIALS, bool Q8, bool SUMMED, bool SHORT_K, bool ZP, bool ACC>
 __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) {
   constexpr int CH = (NKMAX <= 2) ? 2 : 1;   // chunks per batch of accumulator loads
   // STRAIGHT: the chain of a chunk without branches (see below).  It trades some arithmetic on pruned (chunk, order)
@@ -493,38 +501,57 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
                  "l"(src), "r"(kRecBytes), "r"(bar)
                  : "memory");
   };
-  if (rec_issuer) {
-    if (x.pair < x.num_tiles) fetch_record(0, x.pair);
-    if (x.pair + x.npairs < x.num_tiles) fetch_record(1, x.pair + x.npairs);
+  // Tables of the pair's tile number tc, by all epilogue threads of the CTA, a tile ahead of their use so that no warp
+  // waits for the slowest one between two tiles (made at the tile's start they cost 4500 cycles of the 20 000 a tile of
+  // 768 -> 3072 drains for; its fused GeLU layer 84 -> 77 us without): the products c = s_k * lambda_x of the stacked rows (once per CTA instead
+  // of once per token row) and, for the fused epilogue, the bias of the tile's channels.
+  auto make_tables = [&](uint32_t tc, int tile) -> bool {
+    const uint32_t i = tc % kRecBufs, ph = (tc / kRecBufs) & 1;
+    if (!mbar_wait(x.recbar0 + 8u * i, ph, x.abort_flag, p.f.status)) return false;
+    int m, cb, tt;
+    locate_tile(p, x.tile_base, tile, m, cb, tt);
+    const float sx = x.sx_s[m];
+    const uint32_t rec = x.rec0 + i * kRecBytes;
+    const int et = (x.warp - 2 - kUnpackWarps) * 32 + lane;   // this thread among the epilogue threads
+    if constexpr (Q8) {
+      int c0, c1;
+      asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(c0), "=r"(c1) : "r"(rec));
+      const bool bias = p.f.branch[m].add_bias && p.f.bias;
+      for (int c = et; c < c1 - c0; c += 32 * kEpiWarps) x.bias_s[i * PIPE_BLOCK_CHANNELS + c] = bias ? __ldg(p.f.bias + c0 + c) : 0.f;
+    }
+    for (int r = et; r < kMaxN; r += 32 * kEpiWarps) {
+      float sc;
+      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(sc) : "r"(rec + kRecScaleOff + 4u * r));
+      x.cfold[i * kMaxN + r] = __fmul_rn(sc, sx);
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(x.prebar0 + 8u * i);
+    return true;
+  };
+  bool tables_ok = true;
+  if (x.pair < x.num_tiles) {
+    if (rec_issuer) {
+      fetch_record(0, x.pair);
+      if (x.pair + x.npairs < x.num_tiles) fetch_record(1, x.pair + x.npairs);
+    }
+    __syncwarp();
+    tables_ok = make_tables(0, x.pair);
   }
-  for (int tile = x.pair; tile < x.num_tiles; tile += x.npairs, ++tcount) {
+  for (int tile = x.pair; tables_ok && tile < x.num_tiles; tile += x.npairs, ++tcount) {
     struct { int m, cb, tt, k0; } t;
     locate_tile(p, x.tile_base, tile, t.m, t.cb, t.tt);
     const BranchArgs& br = p.f.branch[t.m];
     t.k0 = br.k_begin;
+    const bool accumulate = ACC || (ZP && br.accumulate);
     const int buf = tcount & 1;
     const uint32_t aph = (tcount >> 1) & 1;
-    const float sx = x.sx_s[t.m];
     const uint32_t rec_s = x.rec0 + (tcount % kRecBufs) * kRecBytes;
-    if (!mbar_wait(x.recbar0 + 8u * (tcount % kRecBufs), (tcount / kRecBufs) & 1, x.abort_flag, p.f.status)) break;
+    if (!mbar_wait(x.prebar0 + 8u * (tcount % kRecBufs), (tcount / kRecBufs) & 1, x.abort_flag, p.f.status)) break;
     int c0, c1;
     asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(c0), "=r"(c1) : "r"(rec_s));
     const int nch = (c1 - c0) >> 3;       // at most PIPE_BLOCK_CHANNELS / 8
     const uint32_t colmap_s = rec_s + kRecColmapOff;
-    // The products c = s_k * lambda_x of the tile's stacked rows, once per CTA instead of once per token row.
-    float* cf = x.cfold + (tcount % kRecBufs) * kMaxN;
-    {
-      const int et = (x.warp - 2 - kUnpackWarps) * 32 + lane;   // this thread among the epilogue threads
-      for (int r = et; r < kMaxN; r += 32 * kEpiWarps) {
-        float sc;
-        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(sc) : "r"(rec_s + kRecScaleOff + 4u * r));
-        cf[r] = __fmul_rn(sc, sx);
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(x.prebar0 + 8u * (tcount % kRecBufs));
-      if (!mbar_wait(x.prebar0 + 8u * (tcount % kRecBufs), (tcount / kRecBufs) & 1, x.abort_flag, p.f.status)) break;
-    }
-    const uint32_t cscale_s = smem_u32(cf);
+    const uint32_t cscale_s = smem_u32(x.cfold + (tcount % kRecBufs) * kMaxN);
     // The accumulators hold 2^(8-b) times the sums; float(2^(8-b) a) = 2^(8-b) float(a) exactly, so the shift is
     // taken as a multiplication by 2^-(8-b) after the conversion (exact for every int32, and on the pipe with the
     // most issue slots); only the verification output needs the shifted integers themselves.
@@ -563,7 +590,7 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
     // the store instructions, and rows beyond T -- for a convolution, pixels beyond the image -- are clipped by
     // the copy engine.  A sum into y keeps the path through registers, which alone adds in binary32 round-to-nearest.
     // (ZP: the last quarter holds 31 tokens; its row of sums must not be stored over the next tile's first token)
-    const bool tma_out = !Q8 && ((p.y_tma >> t.m) & 1u) && !br.accumulate && tile_ok && !(ZP && q == 3);
+    const bool tma_out = !Q8 && ((p.y_tma >> t.m) & 1u) && !accumulate && tile_ok && !(ZP && q == 3);
     int ty1 = static_cast<int>(tok_base), ty2 = 0, ty3 = 0;   // coordinates behind the channel: token, or (x, y, image)
     if (p.f.conv_on) {
       const int patch = 2 * ttile + (q >> 1);
@@ -583,7 +610,6 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
       // the block starts at a multiple of 8 channels; 16-byte stores need the row piece aligned as well
       const uintptr_t bits = reinterpret_cast<uintptr_t>(br.yq) | static_cast<uintptr_t>(p.f.ldyq) | static_cast<uintptr_t>(c0);
       qalign = (bits & 15) == 0 ? 16 : ((bits & 3) == 0 ? 4 : 1);
-      for (int c = lane; c < c1 - c0; c += 32) x.stg[c] = (br.add_bias && p.f.bias) ? __ldg(p.f.bias + c0 + c) : 0.f;
     }
     const bool add_bias = !SUMMED && br.add_bias && p.f.bias;   // (a summed ensemble adds it inside the chain)
     const float* bias_q = add_bias ? p.f.bias + c0 + 4 * sj : nullptr;
@@ -591,9 +617,13 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
     __syncwarp();
     if (!mbar_wait(x.tfull0 + 8u * buf, aph, x.abort_flag, p.f.status)) break;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // The record of the NEXT tile goes into the copy the tile before the last one used: the accumulators just handed
-    // over were computed after every epilogue warp of the pair had finished that tile.
-    if (rec_issuer && tcount >= 1 && tile + x.npairs < x.num_tiles) fetch_record(tcount + 1, tile + x.npairs);
+    // The record of the tile after the next goes into the copy the tile before the last one used, the next tile's tables
+    // overwrite those of the tile before that: the accumulators just handed over were computed after every epilogue warp
+    // of the pair had finished both.
+    if (rec_issuer && tile + 2 * x.npairs < x.num_tiles) fetch_record(tcount + 2, tile + 2 * x.npairs);
+    __syncwarp();
+    if (tile + x.npairs < x.num_tiles) tables_ok = make_tables(tcount + 1, tile + x.npairs);
+    if (!tables_ok) break;
     const uint32_t tbase = x.tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * kAccCols;
     if constexpr (ZP) {
       // The two warps of the last lane quarter read the row of sums, half of the columns each.  (A buffer's products are
@@ -623,6 +653,15 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
       if (!Q8 && add_bias && quad_ok && !(tma_out && 2 * grp + 1 < nch)) {
         const float* bp = bias_q + 16 * grp;
         bq = make_float4(__ldg(bp), __ldg(bp + 1), __ldg(bp + 2), __ldg(bp + 3));
+      }
+      // (a sum into y: the rows this lane will add to are under way while the chain runs)
+      float4 o[4];
+      if (ACC && quad_ok) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if ((srow_ok >> i) & 1u) o[i] = load_row(srow[i] + 16 * grp, vec_ok);
+        }
       }
       // ---- this lane's row: 16 channels into the staging block (as 16 codes into registers for the fused epilogue)
       const bool use_tma = tma_out && 2 * grp + 1 < nch;
@@ -732,7 +771,7 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
           if constexpr (Q8) {
             // bias last, sigma, then Q of the next layer (Sec. 3.2): eight codes of this lane's own row
             float bv[8];
-            const uint32_t ba = smem_u32(x.stg) + static_cast<uint32_t>(chunk * 32);
+            const uint32_t ba = smem_u32(x.bias_s + (tcount % kRecBufs) * PIPE_BLOCK_CHANNELS) + static_cast<uint32_t>(chunk * 32);
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(bv[0]), "=f"(bv[1]), "=f"(bv[2]), "=f"(bv[3]) : "r"(ba));
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(bv[4]), "=f"(bv[5]), "=f"(bv[6]), "=f"(bv[7]) : "r"(ba + 16));
 #pragma unroll
@@ -808,7 +847,10 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
         continue;
       }
       __syncwarp();
-      // ---- 8 rows x 64 bytes per store instruction; the bias joins here, after the whole chain
+      // ---- 8 rows x 64 bytes per store instruction; the bias joins here, after the whole chain.  A sum into y read
+      // its rows here once, one after the other between the stores, each waiting for L2: 2900 cycles per group, more than
+      // half of a short launch (both launches of a summed 3 x 3 convolution 512 -> 512 on 32 x 14 x 14: 93 -> 67 us; of
+      // 3072 -> 768, T = 4096: 60 -> 52).
       if (quad_ok) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -816,17 +858,13 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
           float4 v;
           asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(stg_r + static_cast<uint32_t>(i * 8 * 64)));
           if (add_bias) v = make_float4(__fadd_rn(v.x, bq.x), __fadd_rn(v.y, bq.y), __fadd_rn(v.z, bq.z), __fadd_rn(v.w, bq.w));
-          float* dst = srow[i] + 16 * grp;
-          if (vec_ok) {
-            if (br.accumulate) {
-              const float4 o = *reinterpret_cast<const float4*>(dst);
-              v = make_float4(__fadd_rn(o.x, v.x), __fadd_rn(o.y, v.y), __fadd_rn(o.z, v.z), __fadd_rn(o.w, v.w));
-            }
-            *reinterpret_cast<float4*>(dst) = v;
-          } else {
-            if (br.accumulate) v = make_float4(__fadd_rn(dst[0], v.x), __fadd_rn(dst[1], v.y), __fadd_rn(dst[2], v.z), __fadd_rn(dst[3], v.w));
-            dst[0] = v.x, dst[1] = v.y, dst[2] = v.z, dst[3] = v.w;
+          if (accumulate) {
+            if (!ACC) o[i] = load_row(srow[i] + 16 * grp, vec_ok);
+            v = make_float4(__fadd_rn(o[i].x, v.x), __fadd_rn(o[i].y, v.y), __fadd_rn(o[i].z, v.z), __fadd_rn(o[i].w, v.w));
           }
+          float* dst = srow[i] + 16 * grp;
+          if (vec_ok) *reinterpret_cast<float4*>(dst) = v;
+          else dst[0] = v.x, dst[1] = v.y, dst[2] = v.z, dst[3] = v.w;
         }
       }
       __syncwarp();
@@ -840,7 +878,7 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
   __syncwarp();
 }
 
-template <bool Q8, bool SUMMED, bool SHORT_K, bool ZP = false>
+template <bool Q8, bool SUMMED, bool SHORT_K, bool ZP = false, bool ACC = false>
 __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_constant__ Params p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t bars[2 * kMaxRing + 4];  // full[3] done[3] tmem_full[2] tmem_empty[2]
@@ -858,6 +896,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
   __shared__ int zp_s[ZP ? PIPE_MAX_ORDERS : 1];
   __shared__ uint64_t z_bars[2];
   __shared__ float sx_s[2 * PIPE_MAX_ORDERS];                        // lambda_x of every branch, then the fused epilogue's output steps
+  static_assert(kRecBufs * PIPE_BLOCK_CHANNELS <= kEpiWarps * 32 * 16, "the fused epilogue's bias tables");
   __shared__ __align__(1024) float epi_stage[kEpiWarps][32 * 16];   // per epilogue warp: 32 token rows x 16 channels (the
                                                                     // source of tensor stores with the 64-byte swizzle)
 
@@ -1100,18 +1139,19 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
     e.part = ew >> 2;
     e.nparts = kEpiWarps / 4;
     e.stg = epi_stage[ew];
+    e.bias_s = &epi_stage[0][0];
     e.zero_s = smem_u32(zero8_s);
     e.zp_s = zp_s;
     e.zrow = zrow_s;
     e.zbar0 = smem_u32(z_bars);
     if (p.f.partials) {   // verification output: every integer accumulator is also written out
-      if (p.nkmax <= 2) epilogue_role<2, true, Q8, SUMMED, SHORT_K, ZP>(p, e);
-      else if (p.nkmax <= 4) epilogue_role<4, true, Q8, SUMMED, SHORT_K, ZP>(p, e);
-      else epilogue_role<8, true, Q8, SUMMED, SHORT_K, ZP>(p, e);
+      if (p.nkmax <= 2) epilogue_role<2, true, Q8, SUMMED, SHORT_K, ZP, ACC>(p, e);
+      else if (p.nkmax <= 4) epilogue_role<4, true, Q8, SUMMED, SHORT_K, ZP, ACC>(p, e);
+      else epilogue_role<8, true, Q8, SUMMED, SHORT_K, ZP, ACC>(p, e);
     } else {
-      if (p.nkmax <= 2) epilogue_role<2, false, Q8, SUMMED, SHORT_K, ZP>(p, e);
-      else if (p.nkmax <= 4) epilogue_role<4, false, Q8, SUMMED, SHORT_K, ZP>(p, e);
-      else epilogue_role<8, false, Q8, SUMMED, SHORT_K, ZP>(p, e);
+      if (p.nkmax <= 2) epilogue_role<2, false, Q8, SUMMED, SHORT_K, ZP, ACC>(p, e);
+      else if (p.nkmax <= 4) epilogue_role<4, false, Q8, SUMMED, SHORT_K, ZP, ACC>(p, e);
+      else epilogue_role<8, false, Q8, SUMMED, SHORT_K, ZP, ACC>(p, e);
     }
   }
 
@@ -1172,6 +1212,8 @@ static const DeviceSetup& device_setup() {
     if (cudaFuncSetAttribute(tc2_forward_kernel<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
     if (cudaFuncSetAttribute(tc2_forward_kernel<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
     if (cudaFuncSetAttribute(tc2_forward_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
+    if (cudaFuncSetAttribute(tc2_forward_kernel<false, false, true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
+    if (cudaFuncSetAttribute(tc2_forward_kernel<false, false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
     if (cudaFuncSetAttribute(tc2_forward_kernel<false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -1330,6 +1372,9 @@ static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_
   const cudaError_t e = zp          ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<false, false, false, true>, p)
                         : a.q8_out  ? (short_k ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<true, false, true>, p)
                                                : cudaLaunchKernelEx(&cfg, tc2_forward_kernel<true, false, false>, p))
+                        : a.branch[0].accumulate
+                            ? (short_k ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<false, false, true, false, true>, p)
+                                       : cudaLaunchKernelEx(&cfg, tc2_forward_kernel<false, false, false, false, true>, p))
                         : split_mask ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<false, true, false>, p)
                         : short_k    ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<false, false, true>, p)
                                      : cudaLaunchKernelEx(&cfg, tc2_forward_kernel<false, false, false>, p);
