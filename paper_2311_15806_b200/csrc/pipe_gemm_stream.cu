@@ -52,6 +52,7 @@ struct Params {
   int kbps;               // reduction blocks per stage (2 for 2-bit codes, else 1)
   int nstages;            // stages per pass
   int nkmax;              // most orders any branch has
+  int chunk_ints;         // words of one slab's entry in the chunk table: chunk_entry_ints
   int own_max;            // most slabs any CTA owns
   int prefetch;           // the expanded layer is not being written by the launch before: weights may be fetched ahead of the dependency wait
   uint32_t split_mask;    // summed ensemble on one shared input, run as ONE cluster of all orders: bit k marks the order (k > 0)
@@ -59,6 +60,14 @@ struct Params {
   int slice_tokens;       // tokens of a slice: the CTAs of slice z compute the tokens [z, z + 1) * slice_tokens
   int ctas_per_branch;    // every branch has its own CTAs, so no CTA's range crosses a branch boundary
 };
+
+// A slab's entry in the chunk table: one word, then three per position.  Positions are the kept orders, ascending -- but
+// with two predictors on inputs of their own (MODE 2) the second one starts at position 2 however few the first one has.
+constexpr int kChunkWords = 3;
+inline int chunk_entry_ints(int nkmax, bool two_inputs) {
+  const int positions = two_inputs && nkmax < 4 ? 4 : nkmax;
+  return 1 + kChunkWords * positions;
+}
 
 struct Pass {
   int branch, lb, le;                 // local slab range [lb, le) of the CTA's own slabs
@@ -192,8 +201,8 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
   int* slabmeta = reinterpret_cast<int*>(tables);                                   // [own][nkmax] first row or -1
   float* cstab = reinterpret_cast<float*>(slabmeta + p.own_max * p.nkmax);          // [own][nkmax][8] s_k * lambda_x
   float* biastab = cstab + p.own_max * p.nkmax * 8;                                 // [own][8]
-  int* chunktab = reinterpret_cast<int*>(biastab + p.own_max * 8);                  // [warp][SPW][1 + 3 * nkmax]
-  int* sums = chunktab + kConsWarps * SPW * (1 + 3 * p.nkmax);                          // [pass slab][NP][NT * 4][32 lanes]
+  int* chunktab = reinterpret_cast<int*>(biastab + p.own_max * 8);                  // [warp][SPW][chunk_ints]
+  int* sums = chunktab + kConsWarps * SPW * p.chunk_ints;                               // [pass slab][NP][NT * 4][32 lanes]
   const uint8_t* stage_gen = smem_raw + (stage0 - smem_u32(smem_raw));
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8u * kMaxDepth;
   const uint32_t sums_ready = empty0 + 8u * kMaxDepth, sums_free = sums_ready + 8u;
@@ -386,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
     }
     asm volatile("bar.sync 1, %0;" ::"r"(32 * kConsWarps) : "memory");   // every consumer warp arrives here unconditionally
 
-    const int centries = 1 + 3 * p.nkmax;
+    const int centries = p.chunk_ints;
     const int grp = warp / kGroupWarps, wg = warp % kGroupWarps;
     bool ok = true;
     for (int pi = 0; pi < npass && ok; ++pi) {
@@ -409,8 +418,8 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
             const int row0 = slabmeta[(P.lb + sl) * p.nkmax + ko];
             if (row0 < 0) continue;
             if (MODE == 2 && ko >= ksecond && n < 2) n = 2;
-            ct[2 + 3 * n] = P.seg_off[ko] + (row0 - P.seg_row0[ko]) * p.pk;
-            ct[3 + 3 * n] = P.seg_rows[ko] * p.pk;
+            ct[2 + kChunkWords * n] = P.seg_off[ko] + (row0 - P.seg_row0[ko]) * p.pk;
+            ct[3 + kChunkWords * n] = P.seg_rows[ko] * p.pk;
             present |= 1 << n;
             ++n;
           }
@@ -426,8 +435,8 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
         nchunks[s] = mychunks[s * centries];
 #pragma unroll
         for (int ci = 0; ci < 2 * NP; ++ci) {
-          woff[s][ci] = have(s, ci) ? mychunks[s * centries + 2 + 3 * ci] : 0;
-          wstr[s][ci] = have(s, ci) ? mychunks[s * centries + 3 + 3 * ci] : 0;
+          woff[s][ci] = have(s, ci) ? mychunks[s * centries + 2 + kChunkWords * ci] : 0;
+          wstr[s][ci] = have(s, ci) ? mychunks[s * centries + 3 + kChunkWords * ci] : 0;
         }
       }
       int acc[SPW][NP][NT][4];
@@ -724,6 +733,7 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
   p.kbps = a.bits == 2 ? 2 : 1;
   p.nstages = ceil_div(p.kblocks, p.kbps);
   p.nkmax = max_cluster;
+  p.chunk_ints = chunk_entry_ints(max_cluster, distinct);
   p.slabs_per_branch = a.O / 8;
   p.total_slabs = p.slabs_per_branch * a.num_branches;
   p.pass_slabs = kGroupWarps * spw;
@@ -801,7 +811,7 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
   // a stage holds one reduction block (two for 2-bit codes) of every order for the slabs of a pass, all kept
   const int pass_cap = p.pass_slabs < p.own_max ? p.pass_slabs : p.own_max;
   p.stage_bytes = round_up(p.kbps * ((distinct ? 2 : 1) * kXTile + pass_cap * 8 * max_cluster * p.pk), 1024);
-  const int table_bytes = p.own_max * (max_cluster * 4 + max_cluster * 32 + 32) + kConsWarps * spw * (1 + 3 * max_cluster) * 4 +
+  const int table_bytes = p.own_max * (max_cluster * 4 + max_cluster * 32 + 32) + kConsWarps * spw * p.chunk_ints * 4 +
                           p.pass_slabs * np * nt * 4 * 32 * 4;
   const int avail = smem_max - fixed - 1024 - round_up(table_bytes, 16);
   p.depth = avail / p.stage_bytes;

@@ -783,14 +783,14 @@ def test_small_layers_in_token_slices(O, I, bits, K, g, n_keep, M, T):
 
 
 # two predictors on inputs of their own, summed, in one launch of the streaming kernel: one slab slot per warp, two, more
-# (several passes), clusters of one order, every code width; token counts around a tile, two tiles and the first slice
+# (several passes), every code width; token counts around a tile, two tiles and the first slice
 @pytest.mark.parametrize("T", [1, 8, 9, 16, 17])
 @pytest.mark.parametrize("O,I,bits,K,g,n_keep", [(6144, 160, 4, 4, 8, 300), (12288, 144, 4, 3, 8, 600), (256, 400, 8, 2, 8, 20),
                                                  (512, 400, 2, 4, 16, 9), (5000, 272, 8, 3, 8, 200)])
-def test_two_summed_predictors_stream_in_one_launch(O, I, bits, K, g, n_keep, T):
+def test_two_summed_predictors_stream_in_one_launch(O, I, bits, K, g, n_keep, T, branch_orders=None):
     M = 2
     rng = np.random.default_rng(O + T)
-    layer = H.gpu_expand(H.desc_of(O, I, bits, K, g, n_keep, M), _w(rng, O, I, heavy=(bits == 2)))
+    layer = H.gpu_expand(H.desc_of(O, I, bits, K, g, n_keep, M, branch_orders), _w(rng, O, I, heavy=(bits == 2)))
     bias = torch.from_numpy(rng.standard_normal(O).astype(np.float32)).cuda()
     xq = [torch.from_numpy(rng.integers(-127, 128, (T, I)).astype(np.int8)).cuda() for _ in range(M)]
     sx = [torch.tensor([0.01 * (1 + m)], device="cuda") for m in range(M)]
@@ -810,3 +810,13 @@ def test_two_summed_predictors_stream_in_one_launch(O, I, bits, K, g, n_keep, T)
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
     assert T > 16 or launches == 1
     assert B.pipe_poll_status() == B.PIPE_OK
+
+
+# the same with predictors of fewer than two orders: the second one's chunks still begin behind two positions of the first.
+# Two slabs per CTA, four (every warp's slot taken), two slots per warp, several passes; nearly every group keeps all orders
+@pytest.mark.parametrize("T", [1, 3, 5, 9, 16])
+@pytest.mark.parametrize("bits", [8, 4, 2])
+@pytest.mark.parametrize("O", [2048, 4096, 6144, 12288])
+@pytest.mark.parametrize("branch_orders", [(1, 1), (1, 2), (2, 1)])
+def test_summed_predictors_of_one_order_stream_in_one_launch(O, bits, branch_orders, T):
+    test_two_summed_predictors_stream_in_one_launch(O, 272, bits, sum(branch_orders), 16, O // 16 - 9, T, list(branch_orders))

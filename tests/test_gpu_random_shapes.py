@@ -46,3 +46,20 @@ def test_random_shapes_on_few_tokens_match_oracle(oracle, O, I, T, bits, K, g, n
     ensemble on a shared input as one launch included."""
     TP.test_forward_matches_oracle(oracle, B.KERNEL_AUTO, O, I, T, bits, K, g, n_keep, M)
     assert B.pipe_poll_status() == B.PIPE_OK
+
+
+def _summed_cases(n, seed):
+    rng = np.random.default_rng(seed)
+    out = []
+    for _ in range(n):
+        bits, g = int(rng.choice([8, 4, 2])), int(rng.choice([8, 16]))
+        split = [int(rng.integers(1, 3)), int(rng.integers(1, 3))]
+        G = int(np.exp(rng.uniform(np.log(4), np.log(12288 // g))))
+        out.append((G * g, int(rng.integers(1, 40)) * 16, bits, sum(split), g, int(rng.integers(1, G + 1)), int(rng.integers(1, 17)), split))
+    return out
+
+
+@pytest.mark.parametrize("O,I,bits,K,g,n_keep,T,split", _summed_cases(32, 20231118))
+def test_random_summed_predictors_on_inputs_of_their_own(O, I, bits, K, g, n_keep, T, split):
+    """Two predictors of one or two orders each, every output width up to 12288: one launch, the CUDA-core kernel's bits."""
+    TP.test_two_summed_predictors_stream_in_one_launch(O, I, bits, K, g, n_keep, T, split)
