@@ -389,7 +389,8 @@ pipe_status pipe_ensemble_forward(const pipe_layer_desc* desc, const void* d_blo
  * sum_i c q - z_m * sum_i q; everything after it is unchanged.  h_zp_m: HOST array of M device pointers to one int32
  * each (NULL entries mean 0).  d_partials receives acc_k with the zero point taken out.  PIPE_ERR_ACC_OVERFLOW
  * cannot be excluded by the descriptor alone here: |c - z| reaches 255, so the layer must satisfy
- * 255 * qmax * I < 2^31 (checked).  Runs on the tensor-core kernels where the shape allows it (they form the row sums
+ * 255 * qmax * I < 2^31 (checked).  (That is with a zero point inside the code range; any other is taken as well, and acc_k
+ * is then exact while z_m * sum_i q and acc_k fit 32 bits.)  Runs on the tensor-core kernels where the shape allows it (they form the row sums
  * of the codes beside the products), on the CUDA-core kernel otherwise; the results are the same bits.
  */
 pipe_status pipe_ensemble_forward_zp(const pipe_layer_desc* desc, const void* d_blob, const int8_t* const* h_xq_m,

@@ -637,8 +637,10 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
           tmem_ld8(tbase + c, v);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           if (lane == 31) {
-            *reinterpret_cast<int4*>(zr + c) = make_int4(zp * v[0], zp * v[1], zp * v[2], zp * v[3]);
-            *reinterpret_cast<int4*>(zr + c + 4) = make_int4(zp * v[4], zp * v[5], zp * v[6], zp * v[7]);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = zp * (v[e] >> p.shift);
+            *reinterpret_cast<int4*>(zr + c) = make_int4(v[0], v[1], v[2], v[3]);
+            *reinterpret_cast<int4*>(zr + c + 4) = make_int4(v[4], v[5], v[6], v[7]);
           }
         }
         if (lane == 31) mbar_arrive(x.zbar0 + 8u * buf);
@@ -739,10 +741,13 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
               const int* zr = x.zrow + buf * kMaxN + (cols[u][ko] >= 0 ? cols[u][ko] : 0);
               const int4 z0 = *reinterpret_cast<const int4*>(zr), z1 = *reinterpret_cast<const int4*>(zr + 4);
               const int zz[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
+              // (both without the factor 2^shift: a zero point outside the code range would carry the difference beyond 32 bits)
 #pragma unroll
-              for (int e = 0; e < 8; ++e) acc[u][ko][e] -= zz[e];
-            }
-            if constexpr (PARTIALS) {
+              for (int e = 0; e < 8; ++e) {
+                acc[u][ko][e] = (acc[u][ko][e] >> p.shift) - zz[e];
+                y[e] = __fmaf_rn(__int2float_rn(acc[u][ko][e]), cs[e], y[e]);
+              }
+            } else if constexpr (PARTIALS) {
 #pragma unroll
               for (int e = 0; e < 8; ++e) {
                 const int a = acc[u][ko][e] >> p.shift;  // exact: the accumulator holds 2^shift times the sum

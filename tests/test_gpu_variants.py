@@ -229,6 +229,34 @@ def test_zero_point_on_the_tensor_cores_equals_the_cuda_core_kernel(O, I, bits, 
             assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("T", [9, 128, 300])
+@pytest.mark.parametrize("bits,I,z", [(2, 4096, 30000), (4, 1008, -200000), (3, 1008, 200000), (8, 400, 30000)])
+def test_zero_point_outside_the_code_range(bits, I, z, T):
+    """The tensor cores hold 2^(8-b) times the sums, which a large zero point would take beyond 32 bits although
+    z * sum q itself fits (|z| qmax I < 1.6e9 here): the zero point has to join after that factor is gone."""
+    H.ensure_built()
+    rng = np.random.default_rng(bits + T)
+    O = 3072                                                              # (T = 9 streams the weights, the others do not)
+    W = rng.uniform(0.01, 0.02, (O, I)).astype(np.float32)                # (codes of one sign: large row sums)
+    layer = H.gpu_expand(H.desc_of(O, I, bits, 2, 16, 99), W)
+    xq = torch.from_numpy(rng.integers(-128, 128, (T, I)).astype(np.int8)).cuda()
+    sx, zp = torch.tensor([0.01], device="cuda"), torch.tensor([z], dtype=torch.int32, device="cuda")
+    out = []
+    for choice in (B.KERNEL_REFERENCE, B.KERNEL_AUTO):
+        for want_part in (False, True):
+            y = torch.full((T, O), float("nan"), device="cuda")
+            part = torch.zeros((T, layer.layout.total_rows), dtype=torch.int32, device="cuda") if want_part else None
+            B.pipe_diag_select_kernel(choice)
+            try:
+                B.pipe_ensemble_forward_zp(layer.desc, layer.blob, [xq], [sx], [zp], [y], None, False, part)
+            finally:
+                B.pipe_diag_select_kernel(B.KERNEL_AUTO)
+            torch.cuda.synchronize()
+            out.append((y.view(torch.int32), part))
+    assert B.pipe_poll_status() == B.PIPE_OK
+    assert all(torch.equal(y, out[0][0]) for y, _ in out) and torch.equal(out[1][1], out[3][1])
+
+
 @pytest.mark.parametrize("kernel", [B.KERNEL_REFERENCE, B.KERNEL_TCGEN05, B.KERNEL_TCGEN05_PAIR, B.KERNEL_STREAM, B.KERNEL_DECODE_TC, B.KERNEL_AUTO])
 @pytest.mark.parametrize("act", [B.ACT_SILU, B.ACT_GELU, B.ACT_SIGMOID])
 def test_smooth_activations_in_the_fused_epilogue(oracle, kernel, act):
