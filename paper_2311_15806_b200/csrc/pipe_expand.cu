@@ -765,29 +765,51 @@ __device__ __forceinline__ uint32_t bytes_of_kern(uint32_t k, int h) {
   return t | ((t & 0x02020202u) * 0x7Eu);
 }
 
-// Four elements through all levels up to j by the definition (out of line: a few chunks in a thousand): residual after
-// level j and its codes as the bytes of a word.  lvl_s: the scales of the levels below j.
+// The estimate of one level (see expand_chain_kernel): the reciprocal of its step, and the residual magnitude from which a
+// code has to be divided for.  A step of zero quantizes nothing: with rcp = 0 every code is 0 and the residual stays.
+__device__ __forceinline__ void level_estimate(float s, float near_half, float& rcp, float& limit) {
+  const bool fast = quant_step_is_fast(s);
+  rcp = 0.f;
+  if (fast) asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rcp) : "f"(s));
+  limit = fast ? s * near_half : s == 0.f ? __uint_as_float(0x7f800000u) : -1.f;
+}
 __device__ __forceinline__ float code_by_division(float x, float s, float fq) {
   float c = 0.f;
   if (s != 0.f) c = fminf(fmaxf(rintf(__fdiv_rn(x, s)), -fq), fq);
   return c;
 }
-static __device__ __noinline__ void replay_quad(const float4* src, const float* lvl_s, int j, float s, float fq, float4* resid, uint32_t* codes) {
+// Four elements through all levels up to j (out of line: a few chunks in a thousand): residual after level j and its codes
+// as the bytes of a word.  lvl_s: the scales of the levels below j.  Divides only where the estimate cannot decide, like the
+// levels themselves: weights on a coarse grid (an integer model's) put many quotients on a boundary, at several levels.
+static __device__ __noinline__ void replay_quad(const float4* src, const float* lvl_s, int j, float s, float fq, float near_half, float4* resid, uint32_t* codes) {
   const float4 v = src ? __ldg(src) : make_float4(0.f, 0.f, 0.f, 0.f);
-  float x[4] = {v.x, v.y, v.z, v.w};
-  uint32_t b = 0;
+  float x[4] = {v.x, v.y, v.z, v.w}, q[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
   for (int l = 0; l <= j; ++l) {
     const float sl = l < j ? lvl_s[l] : s;
-    b = 0;
+    float rcp, limit, x1[4];
+    level_estimate(sl, near_half, rcp, limit);
+    float m = 0.f;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const float q = code_by_division(x[e], sl, fq);
-      x[e] = __fmaf_rn(-sl, q, x[e]);
-      b |= (static_cast<uint32_t>(static_cast<int>(q)) & 0xffu) << (8 * e);
+      q[e] = __fsub_rn(__fmaf_rn(x[e], rcp, 12582912.f), 12582912.f);
+      x1[e] = __fmaf_rn(-sl, q[e], x[e]);
+      m = fmaxf(m, fabsf(x1[e]));
     }
+    if (m >= limit) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        q[e] = code_by_division(x[e], sl, fq);
+        x1[e] = __fmaf_rn(-sl, q[e], x[e]);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) x[e] = x1[e];
   }
   *resid = make_float4(x[0], x[1], x[2], x[3]);
+  uint32_t b = 0;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) b |= (static_cast<uint32_t>(static_cast<int>(q[e])) & 0xffu) << (8 * e);
   *codes = b;
 }
 
@@ -852,10 +874,8 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
       (direct ? p.out[j].scales : p.lvl_scale + static_cast<int64_t>(j) * p.O)[o] = s;
       if (j > 0 && p.direct == 1) atomicMax(p.lvl_max + static_cast<int64_t>(j) * p.G + o / p.g, mk);
     }
-    const bool fast = quant_step_is_fast(s);
-    float rcp = 0.f;
-    if (fast) asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rcp) : "f"(s));
-    const float limit = fast ? s * near_half : -1.f;
+    float rcp, limit;
+    level_estimate(s, near_half, rcp, limit);
     mk = 0;
 #pragma unroll
     for (int c = 0; c < PER; ++c) {
@@ -876,12 +896,12 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
       }
       const int chunk = tid + c * blockDim.x, e0 = chunk * 16;
       if (m >= limit) {
-        // (the old residual is overwritten: the chunk goes through all levels again, divided)
+        // (the old residual is overwritten: the chunk goes through all levels again)
         m = 0.f;
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
           float4 v;
-          replay_quad(e0 < p.I ? reinterpret_cast<const float4*>(p.W + static_cast<int64_t>(o) * p.ldw + e0) + w : nullptr, lvl_s, j, s, fq, &v, &wv[w]);
+          replay_quad(e0 < p.I ? reinterpret_cast<const float4*>(p.W + static_cast<int64_t>(o) * p.ldw + e0) + w : nullptr, lvl_s, j, s, fq, near_half, &v, &wv[w]);
           r[c][4 * w] = v.x; r[c][4 * w + 1] = v.y; r[c][4 * w + 2] = v.z; r[c][4 * w + 3] = v.w;
           m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
         }
