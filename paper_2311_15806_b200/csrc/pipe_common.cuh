@@ -210,6 +210,22 @@ inline bool has_zero_point(const ForwardArgs& a) {
   return false;
 }
 
+// A summed ensemble as one launch per predictor, in order, so that y = ((y_1 + y_2) + ...) is formed in a fixed order.
+// launch(args, queue) with queue = false only says whether the kernel takes a predictor: all are asked before the first is
+// queued, for a kernel that declines a later one would have its launches repeated by the next kernel.
+template <class Launch>
+inline pipe_status launch_each_predictor(const ForwardArgs& a, Launch launch) {
+  for (int queue = 0; queue < 2; ++queue)
+    for (int m = 0; m < a.num_branches; ++m) {
+      ForwardArgs one = a;
+      one.num_branches = 1;
+      one.branch[0] = a.branch[m];
+      const pipe_status st = launch(one, queue != 0);
+      if (st != PIPE_OK) return st;
+    }
+  return PIPE_OK;
+}
+
 // Tensor map of a row-major byte matrix [rows, inner_bytes] with row pitch pitch_bytes (a multiple of 16) and
 // a box of box_inner x box_rows bytes; swizzle128 selects the 128-byte swizzle.  False when the driver entry
 // point is missing or the encoding fails.

@@ -463,7 +463,8 @@ static const DeviceSetup& device_setup() {
 
 }  // namespace dec
 
-static pipe_status launch_dec(const ForwardArgs& a, cudaStream_t stream) {
+// (queue = false: only say whether the kernel takes the call)
+static pipe_status launch_dec(const ForwardArgs& a, cudaStream_t stream, bool queue = true) {
   using namespace dec;
   if (a.T > kMaxTok || a.conv_on) return PIPE_ERR_UNSUPPORTED;
   if (a.bits == 8) return PIPE_ERR_UNSUPPORTED;   // int8 rows need no widening; the weight-streaming kernel takes them
@@ -505,6 +506,7 @@ static pipe_status launch_dec(const ForwardArgs& a, cudaStream_t stream) {
     if ((d & 15) || end >= 0xffffffffull) return PIPE_ERR_UNSUPPORTED;
     p.koff[k] = static_cast<uint32_t>(d >> 4);
   }
+  if (!queue) return PIPE_OK;
   for (int m = 0; m < a.num_branches; ++m)
     if (!make_map_2d(&p.tmap_x[m], a.branch[m].xq, static_cast<uint64_t>(a.I), static_cast<uint64_t>(a.T),
                      static_cast<uint64_t>(a.ldxq), kKStep, kMaxTok, CU_TENSOR_MAP_SWIZZLE_128B))
@@ -537,16 +539,8 @@ pipe_status forward_decode_tc(const ForwardArgs& a, cudaStream_t stream) {
   if (a.T == 0) return PIPE_OK;
   const bool sum_mode = a.num_branches > 1 && a.branch[1].accumulate;
   if (!sum_mode) return launch_dec(a, stream);
-  // Summed ensemble: one launch per branch, in order, so that y = ((y_1 + y_2) + ...) is formed in a fixed order
-  // (each branch then runs under the plan that was laid out for all of them, which only costs balance).
-  for (int m = 0; m < a.num_branches; ++m) {
-    ForwardArgs one = a;
-    one.num_branches = 1;
-    one.branch[0] = a.branch[m];
-    pipe_status st = launch_dec(one, stream);
-    if (st != PIPE_OK) return st;
-  }
-  return PIPE_OK;
+  // (each predictor of a summed ensemble runs under the plan that was laid out for all of them, which only costs balance)
+  return launch_each_predictor(a, [&](const ForwardArgs& one, bool queue) { return launch_dec(one, stream, queue); });
 }
 
 }  // namespace pipe

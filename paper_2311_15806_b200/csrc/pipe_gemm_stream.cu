@@ -706,7 +706,9 @@ static bool kernel_info(void (*kern)(const Params), int dyn_wanted_or_0, int* sm
 
 }  // namespace st
 
-static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool slices, uint32_t split_mask = 0, bool distinct = false) {
+// (queue = false: only say whether the kernel takes the call)
+static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool slices, uint32_t split_mask = 0, bool distinct = false,
+                                 bool queue = true) {
   using namespace st;
   const bool zp = has_zero_point(a);   // (its row sums take the place of a token)
   const int slice_tokens = zp ? 15 : 16;
@@ -821,6 +823,7 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
   if (p.depth > round_up(most_stages, kProdWarps)) p.depth = round_up(most_stages, kProdWarps);
   p.depth -= p.depth % kProdWarps;   // every producer warp owns depth / kProdWarps slots
   if (p.depth < kProdWarps) return PIPE_ERR_UNSUPPORTED;
+  if (!queue) return PIPE_OK;
   const int dyn = 1024 + p.depth * p.stage_bytes + round_up(table_bytes, 16);
   for (int m = 0; m < (distinct ? 2 : a.num_branches); ++m)
     if (!make_tensor_map_2d_u8(&p.tmap_x[m], a.branch[m].xq, static_cast<uint64_t>(a.I), static_cast<uint64_t>(a.T),
@@ -869,14 +872,7 @@ pipe_status forward_stream(const ForwardArgs& a, cudaStream_t stream, bool slice
       if (st != PIPE_ERR_UNSUPPORTED) return st;
     }
   }
-  for (int m = 0; m < a.num_branches; ++m) {
-    ForwardArgs one = a;
-    one.num_branches = 1;
-    one.branch[0] = a.branch[m];
-    pipe_status st = launch_stream(one, stream, slices);
-    if (st != PIPE_OK) return st;
-  }
-  return PIPE_OK;
+  return launch_each_predictor(a, [&](const ForwardArgs& one, bool queue) { return launch_stream(one, stream, slices, 0, false, queue); });
 }
 
 }  // namespace pipe

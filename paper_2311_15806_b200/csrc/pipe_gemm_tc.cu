@@ -795,7 +795,8 @@ static const DeviceSetup& device_setup() {
 
 }  // namespace tc
 
-static pipe_status launch_tc(const ForwardArgs& a, cudaStream_t stream) {
+// (queue = false: only say whether the kernel takes the call)
+static pipe_status launch_tc(const ForwardArgs& a, cudaStream_t stream, bool queue = true) {
   using namespace tc;
   const DeviceSetup& ds = device_setup();
   if (ds.status != PIPE_OK) return ds.status;
@@ -875,6 +876,7 @@ static pipe_status launch_tc(const ForwardArgs& a, cudaStream_t stream) {
   if (p.depth > kMaxRing) p.depth = kMaxRing;
   if (p.depth < 2) return PIPE_ERR_UNSUPPORTED;
   const int dyn_smem = p.depth * p.stage_bytes + 1024;
+  if (!queue) return PIPE_OK;
 
   if (a.conv_on) {
     for (int m = 0; m < a.num_branches; ++m)
@@ -897,16 +899,7 @@ pipe_status forward_tcgen05(const ForwardArgs& a, cudaStream_t stream) {
   if (a.T == 0) return PIPE_OK;
   const bool sum_mode = a.num_branches > 1 && a.branch[1].accumulate;
   if (!sum_mode) return launch_tc(a, stream);
-  // Summed ensemble: one launch per branch, in order, so that y = ((y_1 + y_2) + ...) is formed
-  // by the same thread in a fixed order.
-  for (int m = 0; m < a.num_branches; ++m) {
-    ForwardArgs one = a;
-    one.num_branches = 1;
-    one.branch[0] = a.branch[m];
-    pipe_status st = launch_tc(one, stream);
-    if (st != PIPE_OK) return st;
-  }
-  return PIPE_OK;
+  return launch_each_predictor(a, [&](const ForwardArgs& one, bool queue) { return launch_tc(one, stream, queue); });
 }
 
 }  // namespace pipe

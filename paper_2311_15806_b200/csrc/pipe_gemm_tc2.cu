@@ -1242,7 +1242,8 @@ static const DeviceSetup& device_setup() {
 
 }  // namespace tc2
 
-static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_t split_mask = 0) {
+// (queue = false: only say whether the kernel takes the call)
+static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_t split_mask = 0, bool queue = true) {
   using namespace tc2;
   const DeviceSetup& ds = device_setup();
   if (ds.status != PIPE_OK) return ds.status;
@@ -1334,8 +1335,9 @@ static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_
       rows = end > rows ? end : rows;
       if ((p.koff[k] & 7) != 0 || rows > INT32_MAX) return PIPE_ERR_UNSUPPORTED;
     }
-    if (!make_map_2d(&p.tmap_w, p.kbase, kKStep, rows, kKStep, kKStep, 8, CU_TENSOR_MAP_SWIZZLE_128B)) return PIPE_ERR_CUDA;
+    if (queue && !make_map_2d(&p.tmap_w, p.kbase, kKStep, rows, kKStep, kKStep, 8, CU_TENSOR_MAP_SWIZZLE_128B)) return PIPE_ERR_CUDA;
   }
+  if (!queue) return PIPE_OK;
 
   if (a.conv_on) {
     for (int m = 0; m < a.num_branches; ++m)
@@ -1415,16 +1417,7 @@ pipe_status forward_tcgen05_pair(const ForwardArgs& a, cudaStream_t stream) {
       if (st != PIPE_ERR_UNSUPPORTED) return st;
     }
   }
-  // Summed ensemble: one launch per branch, in order, so that y = ((y_1 + y_2) + ...) is formed
-  // by the same thread in a fixed order.
-  for (int m = 0; m < a.num_branches; ++m) {
-    ForwardArgs one = a;
-    one.num_branches = 1;
-    one.branch[0] = a.branch[m];
-    pipe_status st = launch_tc2(one, stream);
-    if (st != PIPE_OK) return st;
-  }
-  return PIPE_OK;
+  return launch_each_predictor(a, [&](const ForwardArgs& one, bool queue) { return launch_tc2(one, stream, 0, queue); });
 }
 
 }  // namespace pipe

@@ -873,3 +873,27 @@ def test_two_summed_predictors_stream_in_one_launch(O, I, bits, K, g, n_keep, T,
 @pytest.mark.parametrize("branch_orders", [(1, 1), (1, 2), (2, 1)])
 def test_summed_predictors_of_one_order_stream_in_one_launch(O, bits, branch_orders, T):
     test_two_summed_predictors_stream_in_one_launch(O, 272, bits, sum(branch_orders), 16, O // 16 - 9, T, list(branch_orders))
+
+
+@pytest.mark.parametrize("O,I,bits,g,n_keep,T", [(3072, 1024, 8, 8, 384, 64), (4096, 1024, 4, 8, 256, 48)])
+def test_a_declined_predictor_declines_the_ensemble(O, I, bits, g, n_keep, T):
+    """Predictors of one and three orders, summed: the rule for token slices takes the first one alone.  Both run on the
+    pair kernel then, and nothing has been queued before: two launches, the CUDA-core kernel's bits."""
+    rng = np.random.default_rng(T)
+    layer = H.gpu_expand(H.desc_of(O, I, bits, 4, g, n_keep, 2, [1, 3]), _w(rng, O, I))
+    xq = [torch.from_numpy(rng.integers(-127, 128, (T, I)).astype(np.int8)).cuda() for _ in range(2)]
+    sx = [torch.tensor([0.01 * (1 + m)], device="cuda") for m in range(2)]
+    ys = []
+    for choice in (B.KERNEL_REFERENCE, B.KERNEL_AUTO):
+        y = torch.full((T, O), float("nan"), device="cuda")
+        B.pipe_diag_select_kernel(choice)
+        try:
+            before = B.pipe_launch_count()
+            B.pipe_ensemble_forward(layer.desc, layer.blob, xq, sx, [y], None, True)
+            launches = B.pipe_launch_count() - before
+        finally:
+            B.pipe_diag_select_kernel(B.KERNEL_AUTO)
+        torch.cuda.synchronize()
+        ys.append(y.view(torch.int32))
+    assert torch.equal(ys[0], ys[1]) and B.pipe_poll_status() == B.PIPE_OK
+    assert launches == 2
