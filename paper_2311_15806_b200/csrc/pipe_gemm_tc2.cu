@@ -555,7 +555,12 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
     // The accumulators hold 2^(8-b) times the sums; float(2^(8-b) a) = 2^(8-b) float(a) exactly, so the shift is
     // taken as a multiplication by 2^-(8-b) after the conversion (exact for every int32, and on the pipe with the
     // most issue slots); only the verification output needs the shifted integers themselves.
-    const float unshift = __int_as_float((127 - p.shift) << 23);
+    // (ZP: a zero point outside the code range could carry its product with the row sums beyond 32 bits under that factor,
+    // which is then shifted out of both first -- not always: the shifts are 1 % of an asymmetric layer's time)
+    const int zp = ZP ? x.zp_s[t.m] : 0;
+    const bool zfar = ZP && (zp < -128 || zp > 127);
+    const int shift = zfar ? 0 : p.shift;
+    const float unshift = __int_as_float((127 - shift) << 23);
     // Token of row r (0..31) of this warp: tok_base + r for a matrix of tokens; for the implicit
     // convolution the warp holds half of an 8 x 8 pixel patch (4 image rows of 8 pixels).
     const int ttile = 2 * t.tt + x.rank;
@@ -630,7 +635,6 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
       // rewritten two tiles later, when every warp has released the accumulators of this one.)
       int* zr = x.zrow + buf * kMaxN;
       if (q == 3) {
-        const int zp = x.zp_s[t.m];
 #pragma unroll 1
         for (int c = x.part * 8; c < kMaxN; c += 8 * x.nparts) {
           int v[8];
@@ -638,7 +642,7 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           if (lane == 31) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = zp * (v[e] >> p.shift);
+            for (int e = 0; e < 8; ++e) v[e] = zp * (zfar ? v[e] >> p.shift : v[e]);
             *reinterpret_cast<int4*>(zr + c) = make_int4(v[0], v[1], v[2], v[3]);
             *reinterpret_cast<int4*>(zr + c + 4) = make_int4(v[4], v[5], v[6], v[7]);
           }
@@ -741,16 +745,17 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
               const int* zr = x.zrow + buf * kMaxN + (cols[u][ko] >= 0 ? cols[u][ko] : 0);
               const int4 z0 = *reinterpret_cast<const int4*>(zr), z1 = *reinterpret_cast<const int4*>(zr + 4);
               const int zz[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
-              // (both without the factor 2^shift: a zero point outside the code range would carry the difference beyond 32 bits)
+              if (zfar) {
 #pragma unroll
-              for (int e = 0; e < 8; ++e) {
-                acc[u][ko][e] = (acc[u][ko][e] >> p.shift) - zz[e];
-                y[e] = __fmaf_rn(__int2float_rn(acc[u][ko][e]), cs[e], y[e]);
+                for (int e = 0; e < 8; ++e) acc[u][ko][e] >>= p.shift;
               }
-            } else if constexpr (PARTIALS) {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) acc[u][ko][e] -= zz[e];
+            }
+            if constexpr (PARTIALS) {
 #pragma unroll
               for (int e = 0; e < 8; ++e) {
-                const int a = acc[u][ko][e] >> p.shift;  // exact: the accumulator holds 2^shift times the sum
+                const int a = acc[u][ko][e] >> shift;  // exact: the accumulator holds 2^shift times the sum
                 acc[u][ko][e] = a;
                 y[e] = __fmaf_rn(__int2float_rn(a), cs[e], y[e]);
               }
