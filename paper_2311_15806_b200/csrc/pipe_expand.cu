@@ -1343,11 +1343,15 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
     ch.O = L.O; ch.I = L.I; ch.I_pad = round_up(L.I, kKernelKAlign); ch.g = L.g; ch.G = L.G; ch.K = L.K; ch.qmax = L.qmax;
     ch.canon_row_bytes = L.lay.canon_row_bytes;
     ch.status = status;
-    // Two chunks per thread at 64 registers.  Between 8192 and 12288 elements three, at 80: one or two blocks of up to
-    // 384 threads are too few to hide each other's barriers there (4096 x 11008: 151 -> 143 us for the whole expansion;
-    // 11008 x 4096: 128 against 137; one chunk per thread 145 and 198, four 130 and 147).
-    const bool long_rows = ch.I_pad > 8192 && ch.I_pad <= 12288;
-    const int threads = round_up(ceil_div(ch.I_pad / 16, long_rows ? 3 : 2), 32);
+    // Two chunks per thread at 64 registers, or three at 80 where rows beyond 8192 elements leave an SM two or three blocks
+    // and three chunks make it one more, to hide the blocks' barriers behind each other.  Whole expansions of 4096 rows,
+    // int4 K = 4 / ternary K = 8 / int8 K = 2, two against three chunks: 8448 120 / 176 / 90 against 116 / 163 / 85 us,
+    // 9216 126 / 178 / 92 against 120 / 165 / 87, 11008 157 / 210 / 114 against 144 / 196 / 102, 12288 161 / 220 / 121
+    // against 149 / 200 / 108; as many blocks either way: 10240 131 / 181 / 98 against 134 / 189 / 98; shorter rows: 7168
+    // 100 / 143 against 104 / 151, 8192 113 / 154 against 116 / 162.
+    const int threads2 = round_up(ceil_div(ch.I_pad / 16, 2), 32), threads3 = round_up(ceil_div(ch.I_pad / 16, 3), 32);
+    const bool long_rows = ch.I_pad > 8192 && ch.I_pad <= 12288 && 65536 / (threads3 * 80) > 65536 / (threads2 * 64);
+    const int threads = long_rows ? threads3 : threads2;
 #define PIPE_CHAIN(B)                                                                       \
   if (long_rows) expand_chain_kernel<B, 3, 256, 3><<<L.O, threads, 0, s>>>(ch);             \
   else expand_chain_kernel<B, 2, 512, 2><<<L.O, threads, 0, s>>>(ch);
