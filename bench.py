@@ -1,7 +1,7 @@
 #!/usr/bin/env python
 """Benchmark of the residual-expanded quantized layer (one pass of the whole hot path per step).
 
-    python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME] [--impl ours|reference]
+    python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME] [--impl ours|reference] [--details FILE]
 
 A step runs the whole hot path on one seeded synthetic batch -- expand the fp32 weights, quantize the
 activations of every ensemble branch, run the (grouped) expanded GEMM -- with every phase timed on its own.
@@ -10,7 +10,8 @@ expansion is reported beside it as its own phase.  The headline workload is the 
 (cfg5); with one GPU the line also carries a `workloads` table with the GEMM of every configuration, timed
 alone, against the integer tensor peak measured in the same run (large token counts) or the measured copy
 bandwidth (T <= 16).  With N > 1 (torchrun) every rank runs an independent replica of the headline workload on
-its own GPU (the path has no exchange step).  Prints ONE JSON line on rank 0.
+its own GPU (the path has no exchange step).  Prints ONE JSON line on rank 0, short enough to be read from the end of a
+log: the headline, and of every configuration's GEMM its microseconds; `--details FILE` writes the rows behind it.
 """
 from __future__ import annotations
 
@@ -184,9 +185,8 @@ class OracleTimer:
         t_big = self.run(n_big) if n_big > n else t_small
         est_step = t_big / n_big * spec.T
         return {"value": spec.T / est_step, "unit": "tokens/s", "cores": self.cores, "kind": "oracle",
-                "sample": (f"weights expanded once beforehand ({self.t_expand:.2f} s, not in the value); quantize and forward "
-                           f"of all {spec.M} branch(es) on the first {n_big} of {spec.T} token rows ({t_big:.2f} s), "
-                           f"extrapolated to the whole step"),
+                "sample": (f"quantize and forward of all {spec.M} branch(es) on the first {n_big} of {spec.T} token rows "
+                           f"({t_big:.2f} s), extrapolated to the step; expansion ({self.t_expand:.2f} s) not in it"),
                 "seconds_per_step_estimate": est_step, "expand_seconds": self.t_expand}
 
 
@@ -347,16 +347,13 @@ def forward_row(run, spec, fwd_ms, fwd_best_ms, how, clocks, peaks, int8, sms: i
 
 def roofline_of(row, peaks, int8):
     """The `roofline` object for the GEMM of one workload (always the expanded GEMM, never another phase)."""
-    kernel = "expanded GEMM (pipe_expanded_linear / pipe_ensemble_forward / pipe_expanded_conv2d)"
-    if row["bound"] == "tensor":
-        return {"kernel": kernel, "bound": "tensor", "achieved": row["effective_tops"], "peak": int8["probe_burst"],
-                "unit": "TOP/s", "frac": row["frac_int8_probe_burst"],
-                "peak_note": "issue-bound tcgen05.mma kind::i8 probe of this run, burst (the kernel is timed alone); "
-                             f"torch._int_mm 8192^3 gave {int8.get('int_mm_8192')} and 2 x bf16 burst of {peaks['source']} "
-                             f"is {2.0 * peaks['bf16_tflops']}",
-                "traffic": row["traffic"]}
-    return {"kernel": kernel, "bound": "hbm", "achieved": row["gbs"], "peak": peaks["hbm_gbs"], "unit": "GB/s",
-            "frac": row["frac_hbm_copy"], "peak_note": f"copy bandwidth of {peaks['source']}", "traffic": row["traffic"]}
+    out = {"kernel": "expanded GEMM", "bound": row["bound"]}
+    if row["bound"] == "tensor":   # against the issue-bound probe's burst: the kernel is timed alone
+        out.update(achieved=row["effective_tops"], peak=int8["probe_burst"], unit="TOP/s", frac=row["frac_int8_probe_burst"],
+                   frac_2x_bf16_burst=row["frac_int8_2x_bf16_burst"])
+    else:
+        out.update(achieved=row["gbs"], peak=peaks["hbm_gbs"], unit="GB/s", frac=row["frac_hbm_copy"])
+    return dict(out, peaks=peaks["source"], traffic=row["traffic"])
 
 
 def host_time_per_forward_call(run, B, torch, calls: int = 300):
@@ -597,37 +594,44 @@ def run_ours(args):
     if world == 1 and not args.no_cpu_baseline:
         cpu = OracleTimer(spec).sample(12.0)
 
+    details = {"effective_tops_online_step": 2.0 * macs * world / (ms_per_step * 1e-3) / 1e12,
+               "whole_path_ms_per_step": whole_ms / args.steps,
+               "step": "online path: pipe_quantize_act of every branch input + the grouped expanded GEMM; the one-off weight "
+                       "expansion (Sec. 4.1) runs every step too but is timed as its own phase",
+               "expand": {"ms": phases["expand"], "gbs": expand_gbs, "frac_hbm_copy": expand_gbs / peaks["hbm_gbs"],
+                          "bytes": "weights read once, both code layouts and the scales written once"},
+               "quantize": {"ms": phases["quantize"], "gbs": quant_gbs,
+                            "frac_hbm_copy": (quant_gbs / peaks["hbm_gbs"]) if quant_gbs else None,
+                            "bytes": "inputs read once, codes written once"},
+               "forward": head_row, "int8_peak": int8,
+               "hbm_peak": {"copy_gbs": peaks["hbm_gbs"], "source": peaks["source"], "nominal_gbs": 8000.0},
+               "workloads": table, "wall_s_timed_region": wall, "host_us_per_forward_call_cfg4a_t1": host_us, "sha256": sha}
     line = {"metric": "expanded_layer_tokens_per_s", "value": tokens_per_s, "unit": "tokens/s", "n_gpus": world,
             "steps": args.steps, "warmup": warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "int8", "data": "synthetic",
             "config": dict(config_of(spec), l2="flush_between_steps" if flush is not None else "inputs_exceed_l2",
-                           distinct_branch_inputs=True if spec.M > 1 else False, multi_gpu="independent replicas",
-                           step="online path: pipe_quantize_act of every branch input + the grouped expanded GEMM; the "
-                                "one-off weight expansion (Sec. 4.1) runs every step too but is timed as its own phase"),
-            "effective_tops_online_step": 2.0 * macs * world / (ms_per_step * 1e-3) / 1e12,
-            "whole_path_ms_per_step": whole_ms / args.steps,
-            "phases_ms": phases,
-            "expand": {"ms": phases["expand"], "gbs": expand_gbs, "frac_hbm_copy": expand_gbs / peaks["hbm_gbs"],
-                       "bytes": run_expand_bytes_note()},
-            "quantize": {"ms": phases["quantize"], "gbs": quant_gbs,
-                         "frac_hbm_copy": (quant_gbs / peaks["hbm_gbs"]) if quant_gbs else None},
-            "forward": head_row, "roofline": roofline_of(head_row, peaks, int8), "int8_peak": int8,
-            "hbm_peak": {"copy_gbs": peaks["hbm_gbs"], "source": peaks["source"], "nominal_gbs": 8000.0},
-            "workloads": table, "clocks": dict(fclocks, during="the GEMM timing loop of the headline workload",
-                                               steps=step_clocks),
+                           parallelism=f"replicas{world}"),
+            "phases_ms": phases, "roofline": roofline_of(head_row, peaks, int8),
+            "workloads_us": {r["workload"]: r["forward_ms"] * 1e3 for r in table if "forward_ms" in r},
+            "clocks": dict(fclocks, steps_sm_mhz=step_clocks["sm_mhz"], reasons=sorted(set(fclocks["reasons"]) | set(step_clocks["reasons"]))),
             "e2e": {"value": world * T / (e2e_ms * 1e-3), "unit": "tokens/s", "h2d_bytes_per_step": h2d,
-                    "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms, "steps": e2e_steps,
-                    "pipeline": "double-buffered device inputs and outputs, upload and download on their own streams"},
-            "gpu_launches": int(launches), "wall_s_timed_region": wall, "host_us_per_forward_call_cfg4a_t1": host_us,
-            "sha256": sha, "cpu_baseline": cpu}
-    print(json.dumps(line))
+                    "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms},
+            "gpu_launches": int(launches), "cpu_baseline": cpu}
+    if args.details:
+        with open(args.details, "w") as f:
+            json.dump(dict(line, **details), f, indent=1)
+    print(json.dumps(short(line), separators=(",", ":")))
     if world > 1:
         dist.destroy_process_group()
 
 
-def run_expand_bytes_note() -> str:
-    return ("per order: fp32 rows read (+ written as residual unless last) + both code layouts written; order 1 reads "
-            "the weights once more for the row maximum")
+def short(v):
+    """The same JSON value with its floating-point numbers to six digits."""
+    if isinstance(v, dict):
+        return {k: short(x) for k, x in v.items()}
+    if isinstance(v, list):
+        return [short(x) for x in v]
+    return float(f"{v:.6g}") if isinstance(v, float) else v
 
 
 def parse_args(argv=None):
@@ -638,6 +642,7 @@ def parse_args(argv=None):
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--workload", default=DEFAULT_WORKLOAD)
     ap.add_argument("--kernel", type=int, default=None, help="force a GEMM kernel (see pipe_diag_select_kernel)")
+    ap.add_argument("--details", default=None, help="write the line and the rows behind it to this file, as JSON")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-table", action="store_true", help="skip the per-configuration GEMM table")
     return ap.parse_args(argv)

@@ -172,17 +172,14 @@ class LayerRunner:
         return codes + scales + sum(x.numel() for x in self.xq) + 4 * self.M * self.T * s.O
 
     def expand_bytes(self) -> int:
-        """Algorithmic bytes of the expansion: every processed row is read and (except at the last
-        order) written as fp32 residual, plus both code layouts written once."""
+        """Algorithmic bytes of the expansion: the weights read once, both code layouts (and the int8 copy) and the
+        scales of every kept row written once."""
         lay, s = self.layout, self.spec
-        b = 4 * s.O * s.I  # order-1 absmax pass
-        for k in range(s.K):
-            b += 4 * lay.rows[k] * s.I * (2 if k + 1 < s.K else 1)
-            b += lay.rows[k] * (lay.canon_row_bytes + lay.kernel_row_bytes)
-            if self.desc.int8_copy:
-                b += lay.rows[k] * ((s.I + 127) // 128 * 128)
-        return b
+        row = lay.canon_row_bytes + lay.kernel_row_bytes + 4
+        if self.desc.int8_copy:
+            row += (s.I + 127) // 128 * 128
+        return 4 * s.O * s.I + sum(lay.rows[k] for k in range(s.K)) * row
 
     def quantize_bytes(self) -> int:
-        """absmax pass reads fp32 once, quantize pass reads it again and writes int8."""
-        return sum(x.numel() for x in self.x) * (4 + 4 + 1)
+        """Algorithmic bytes of the quantization: fp32 read once, int8 written once (tensors beyond the L2 are read twice)."""
+        return sum(x.numel() for x in self.x) * (4 + 1)

@@ -24,3 +24,9 @@ def test_reference_arm_prints_one_contract_line():
     assert d["cpu_baseline"]["kind"] == "oracle" and d["cpu_baseline"]["cores"] >= 1 and d["cpu_baseline"]["sample"]
     assert d["e2e"]["h2d_bytes_per_step"] == 0 and d["e2e"]["d2h_bytes_per_step"] == 0
     assert d["e2e"]["value"] == d["value"]
+
+
+def test_the_line_keeps_its_numbers_to_six_digits():
+    import bench
+    got = bench.short({"a": 1.23456789, "b": [2, 3.0000001, None], "c": {"d": 6085240.885966282, "e": "x", "f": True}})
+    assert got == {"a": 1.23457, "b": [2, 3.0, None], "c": {"d": 6085240.0, "e": "x", "f": True}}
