@@ -113,18 +113,17 @@ def workload_spec(name: str):
 
 
 # ------------------------------------------------------------------------------------------------
-# DRAM read + write bytes of ONE launch of the GEMM kernel, from one ncu capture per workload of this same
-# program (summaries under profiles/, named in the comment).  A workload without a capture of the present
-# kernel has no entry and reports null.
+# DRAM read + write bytes of ONE launch of the GEMM kernel, from one ncu capture per workload
+# (profiles/ncu_pair_kernel.txt, profiles/ncu_stream_kernel.txt).  A workload without a capture has no entry and reports null.
 NCU_DRAM_BYTES_PER_LAUNCH = {
-    "cfg2": 29317632 + 51065600,           # profiles/ncu_tc2_forward_kernel_cfg2.txt
-    "cfg3a": 9438976 + 49971456,           # profiles/ncu_tc2_forward_kernel_cfg3a.txt
-    "cfg4a_t4096": 91033600 + 313256192,   # profiles/ncu_tc2_forward_kernel_cfg4a_t4096.txt
-    "cfg5": 478397440 + 1029014784,        # profiles/ncu_tc2_forward_kernel_cfg5.txt
-    "cfg4a_t1": 56559616 + 98304,          # profiles/ncu_stream_forward_kernel_cfg4a_t1.txt
-    "cfg4a_t16": 56688128 + 303872,         # profiles/ncu_stream_forward_kernel_cfg4a_t16.txt
-    "cfg4a_t4096+int8_copy": 149131520 + 316639744,   # profiles/ncu_tc2_forward_kernel_cfg4a_t4096_int8_copy.txt
-    "cfg3b+int8_copy": 31190784 + 930048,           # profiles/ncu_tc2_forward_kernel_cfg3b_int8_copy.txt
+    "cfg2": 28681984 + 50585088,
+    "cfg3a": 9456896 + 47369472,
+    "cfg4a_t4096": 91300864 + 312781824,
+    "cfg5": 445346816 + 1026677760,
+    "cfg4a_t1": 56560896 + 92160,
+    "cfg4a_t16": 56688128 + 129536,
+    "cfg4a_t4096+int8_copy": 150311936 + 315610368,
+    "cfg3b+int8_copy": 31186432 + 857088,
 }
 
 
