@@ -697,7 +697,8 @@ __global__ void block_record_kernel(const __grid_constant__ BlockRecordArgs a) {
 // K = 4, gamma = 0.5: 600 -> 280 us; 8192 x 8192 ternary, K = 8, gamma = 0.25 (8 levels computed, 2.75 used on
 // average): 464 -> 247 us.  The level storage takes the place of the residual in the workspace.
 // Layers this does not take (chain_fits) run one pass per order: the unstructured mask and the L2 score need the
-// residual itself, rows beyond 16384 do not fit a block's registers, and rows that are not whole 16-code chunks.
+// residual itself, rows beyond 16384 do not fit a block's registers, rows that are not whole 16-code chunks, and large
+// layers that use few of many levels.
 struct ChainOut {
   uint8_t* codes;
   uint8_t* kcodes;
@@ -1212,6 +1213,13 @@ static bool chain_fits(const LayerInfo& L, const float* W, int64_t ldw, ChainPla
   if (L.I % 16 != 0 || round_up(L.I, kKernelKAlign) > kChainMaxI || L.G > kSelMaxGroups) return false;
   if ((reinterpret_cast<uintptr_t>(W) & 15) || ldw % 4 != 0) return false;
   const int levels = L.n_keep == L.G ? 0 : L.K - 1;   // levels that need storage
+  // Many levels of which few are used (high orders that keep little of a large layer): a level costs 0.4 ps an element whether
+  // a row uses it or not, an order 1.5 ps an element of its kept rows (and 2000 elements' worth a row) and 10 us of
+  // selection, the first one 0.6 ps more for its maximum.  Measured, orders against chain, ternary: K = 16 16384 x 16384
+  // gamma = 0.01 897 / 1831 us, 0.1 1430 / 1874, 0.2 2025 / 1934; 28672 x 4096 0.05 721 / 736, 0.1 901 / 755; 8192 x 8192
+  // 0.01 426 / 478, 0.1 574 / 501; K = 8 16384 x 16384 0.01 692 / 817, 0.1 947 / 829, 8192 x 8192 0.01 295 / 233.
+  const double n = static_cast<double>(L.O) * L.I;
+  if (levels && 0.4 * L.K * n > 0.6 * n + 1.5 * L.lay.total_rows * (L.I + 2000.0) + 1e7 * (L.K - 1)) return false;
   c->temp_pitch = round_up(L.lay.canon_row_bytes, 16);
   uint64_t off = 0;
   c->temp = off;

@@ -88,6 +88,20 @@ def test_expand_weights_on_every_route(oracle, O, I, bits, K, g, n_keep, int8_co
     H.assert_expansion_matches(layer, e, oracle)
 
 
+@pytest.mark.parametrize("n_keep,one_pass", [(5, False), (160, True)])
+def test_large_layers_that_use_few_of_many_levels_run_by_orders(oracle, n_keep, one_pass):
+    """Sixteen orders of which the sparse ones keep 1 % (or 31 %) of a large layer: one pass per order (or all levels at
+    once, in at most five launches), the oracle's bits either way."""
+    rng = np.random.default_rng(n_keep)
+    O = I = 8192
+    W = (rng.standard_normal((O, I), dtype=np.float32) * np.float32(0.02))
+    before = B.pipe_launch_count()
+    layer = H.gpu_expand(H.desc_of(O, I, 2, 16, 16, n_keep), W)
+    assert (B.pipe_launch_count() - before <= 5) == one_pass
+    e = oracle.expand(W, 2, 16, 16, n_keep)
+    H.assert_expansion_matches(layer, e, oracle, check_kernel_layout=False)
+
+
 def _grid_weights(rng, O, I, step, top):
     """Multiples of `step` up to `top` of it, the largest in every row: an integer model's weights."""
     W = rng.integers(-top, top + 1, (O, I)).astype(np.float32)
