@@ -94,7 +94,7 @@ static pipe_status dispatch_forward(const ForwardArgs& a, const LayerInfo& L, in
   if (zp) {
     // asymmetric codes: the SM-pair kernel and, in slices of 15 tokens, the weight-streaming kernel form the row sums beside the
     // products (row of ones); the CUDA-core kernel takes every other shape.  Measured against the CUDA-core kernel from
-    // 128 x 128 to 3072 x 3072 and 1 to 2048 tokens: equal (host-bound) at 128 x 128, faster everywhere else.
+    // 128 x 128 to 3072 x 3072 and 1 to 2048 tokens: faster, with the exception below.
     if (static_cast<int64_t>(255) * L.qmax * L.I >= (static_cast<int64_t>(1) << 31)) return PIPE_ERR_ACC_OVERFLOW;
     for (int m = 0; m < M; ++m)
       if (reinterpret_cast<uintptr_t>(zp[m]) & 3) return PIPE_ERR_ALIGNMENT;
@@ -104,7 +104,13 @@ static pipe_status dispatch_forward(const ForwardArgs& a, const LayerInfo& L, in
     pipe_status st = PIPE_ERR_UNSUPPORTED;
     if (((static_cast<int64_t>(255) * L.qmax * L.I) << (8 - L.bits)) < (static_cast<int64_t>(1) << 31)) {
       st = forward_stream(a, stream, true);
-      if (st == PIPE_ERR_UNSUPPORTED) st = forward_tcgen05_pair(a, stream);
+      // A sum over predictors is one launch each on the pair kernel, one in all on the CUDA-core kernel, which is ahead on
+      // short reduction axes while its work stays small (M predictors, tokens, us, CUDA cores / pair): 4672 x 112 M = 4
+      // T = 47 46 / 73, 4016 x 64 M = 2 T = 350 25 / 38, 4160 x 240 M = 3 T = 98 49 / 58, 2448 x 176 M = 2 T = 139 35 / 37;
+      // beyond 1360 x 352 M = 3 T = 412 77 / 59, 3072 x 768 M = 2 T = 709 429 / 37.
+      const bool sum = M > 1 && a.branch[1].accumulate;
+      const bool short_sum = sum && L.I <= 256 && static_cast<int64_t>(L.lay.total_rows) * L.I * T <= static_cast<int64_t>(M) << 26;
+      if (st == PIPE_ERR_UNSUPPORTED && !short_sum) st = forward_tcgen05_pair(a, stream);
     }
     return st == PIPE_ERR_UNSUPPORTED ? forward_reference(a, stream) : st;
   }

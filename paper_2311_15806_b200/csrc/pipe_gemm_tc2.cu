@@ -468,7 +468,7 @@ struct EpiCtx {
 // outputs are summed after the layer (Sec. 3.2): every predictor's chain starts from zero, the bias closes the first
 // one, and the chains are added in ascending predictor order in this thread -- the same additions, in the same
 // order, as one launch per predictor summing into y, without the read-modify-write of y.
-// ACC: the result is added to y (a summed ensemble's later predictors); with a zero point that is found out at run time.
+// ACC: the result is added to y (a summed ensemble's later predictors).
 template <int NKMAX, bool PARTIALS, bool Q8, bool SUMMED, bool SHORT_K, bool ZP, bool ACC>
 __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) {
   constexpr int CH = (NKMAX <= 2) ? 2 : 1;   // chunks per batch of accumulator loads
@@ -542,7 +542,6 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
     locate_tile(p, x.tile_base, tile, t.m, t.cb, t.tt);
     const BranchArgs& br = p.f.branch[t.m];
     t.k0 = br.k_begin;
-    const bool accumulate = ACC || (ZP && br.accumulate);
     const int buf = tcount & 1;
     const uint32_t aph = (tcount >> 1) & 1;
     const uint32_t rec_s = x.rec0 + (tcount % kRecBufs) * kRecBytes;
@@ -595,7 +594,7 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
     // the store instructions, and rows beyond T -- for a convolution, pixels beyond the image -- are clipped by
     // the copy engine.  A sum into y keeps the path through registers, which alone adds in binary32 round-to-nearest.
     // (ZP: the last quarter holds 31 tokens; its row of sums must not be stored over the next tile's first token)
-    const bool tma_out = !Q8 && ((p.y_tma >> t.m) & 1u) && !accumulate && tile_ok && !(ZP && q == 3);
+    const bool tma_out = !Q8 && ((p.y_tma >> t.m) & 1u) && !ACC && tile_ok && !(ZP && q == 3);
     int ty1 = static_cast<int>(tok_base), ty2 = 0, ty3 = 0;   // coordinates behind the channel: token, or (x, y, image)
     if (p.f.conv_on) {
       const int patch = 2 * ttile + (q >> 1);
@@ -868,10 +867,7 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
           float4 v;
           asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(stg_r + static_cast<uint32_t>(i * 8 * 64)));
           if (add_bias) v = make_float4(__fadd_rn(v.x, bq.x), __fadd_rn(v.y, bq.y), __fadd_rn(v.z, bq.z), __fadd_rn(v.w, bq.w));
-          if (accumulate) {
-            if (!ACC) o[i] = load_row(srow[i] + 16 * grp, vec_ok);
-            v = make_float4(__fadd_rn(o[i].x, v.x), __fadd_rn(o[i].y, v.y), __fadd_rn(o[i].z, v.z), __fadd_rn(o[i].w, v.w));
-          }
+          if (ACC) v = make_float4(__fadd_rn(o[i].x, v.x), __fadd_rn(o[i].y, v.y), __fadd_rn(o[i].z, v.z), __fadd_rn(o[i].w, v.w));
           float* dst = srow[i] + 16 * grp;
           if (vec_ok) *reinterpret_cast<float4*>(dst) = v;
           else dst[0] = v.x, dst[1] = v.y, dst[2] = v.z, dst[3] = v.w;
@@ -1225,6 +1221,7 @@ static const DeviceSetup& device_setup() {
     if (cudaFuncSetAttribute(tc2_forward_kernel<false, false, true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
     if (cudaFuncSetAttribute(tc2_forward_kernel<false, false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
     if (cudaFuncSetAttribute(tc2_forward_kernel<false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
+    if (cudaFuncSetAttribute(tc2_forward_kernel<false, false, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.dyn_smem) != cudaSuccess) return;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1381,7 +1378,8 @@ static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_
   cfg.numAttrs = 2;
   // (a reduction axis of at most 8 blocks: the drain paces the layer, see STRAIGHT in the epilogue)
   const bool short_k = p.kblocks <= 8;
-  const cudaError_t e = zp          ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<false, false, false, true>, p)
+  const cudaError_t e = zp          ? (a.branch[0].accumulate ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<false, false, false, true, true>, p)
+                                                              : cudaLaunchKernelEx(&cfg, tc2_forward_kernel<false, false, false, true>, p))
                         : a.q8_out  ? (short_k ? cudaLaunchKernelEx(&cfg, tc2_forward_kernel<true, false, true>, p)
                                                : cudaLaunchKernelEx(&cfg, tc2_forward_kernel<true, false, false>, p))
                         : a.branch[0].accumulate
