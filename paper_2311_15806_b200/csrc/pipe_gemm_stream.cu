@@ -870,6 +870,10 @@ pipe_status forward_stream(const ForwardArgs& a, cudaStream_t stream, bool slice
       for (int m = 1; m < a.num_branches; ++m) split |= 1u << a.branch[m].k_begin;
       const pipe_status st = launch_stream(one, stream, slices, split, distinct);
       if (st != PIPE_ERR_UNSUPPORTED) return st;
+      // Beyond 16 tokens the pair kernel adds predictors of one input in one launch too (where the layer has the table of
+      // all orders), and slices for every predictor do not match that: 320 x 5920 ternary M = 4 T = 465 62 us in slices,
+      // 31 in one launch, 3872 x 2256 int4 M = 3 T = 49 32.5 / 21, 3776 x 48 ternary M = 4 T = 32 25 / 15.5.
+      if (shared && a.T > 16 && a.sum_blk && a.sum_rec) return PIPE_ERR_UNSUPPORTED;
     }
   }
   return launch_each_predictor(a, [&](const ForwardArgs& one, bool queue) { return launch_stream(one, stream, slices, 0, false, queue); });

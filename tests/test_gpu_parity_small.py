@@ -911,3 +911,30 @@ def test_a_declined_predictor_declines_the_ensemble(O, I, bits, g, n_keep, T):
         ys.append(y.view(torch.int32))
     assert torch.equal(ys[0], ys[1]) and B.pipe_poll_status() == B.PIPE_OK
     assert launches == 2
+
+
+@pytest.mark.parametrize("O,I,bits,K,g,n_keep,split,T", [(3872, 2256, 4, 4, 16, 30, [1, 2, 1], 49), (1272, 1456, 4, 6, 8, 159, None, 228),
+                                                         (320, 1040, 2, 5, 32, 3, [1, 2, 1, 1], 465)])
+def test_sums_on_a_shared_input_are_one_launch_beyond_the_slices(O, I, bits, K, g, n_keep, split, T):
+    """Predictors of one input, summed, in layers whose token slices take a predictor but not all of them together: the pair
+    kernel's one launch, the CUDA-core kernel's bits."""
+    M = len(split) if split else 4
+    rng = np.random.default_rng(T)
+    layer = H.gpu_expand(H.desc_of(O, I, bits, K, g, n_keep, M, split), _w(rng, O, I))
+    xq = torch.from_numpy(rng.integers(-127, 128, (T, I)).astype(np.int8)).cuda()
+    sx = torch.tensor([0.01], device="cuda")
+    bias = torch.from_numpy(rng.standard_normal(O).astype(np.float32)).cuda()
+    ys = []
+    for choice in (B.KERNEL_REFERENCE, B.KERNEL_AUTO):
+        y = torch.full((T, O), float("nan"), device="cuda")
+        B.pipe_diag_select_kernel(choice)
+        try:
+            before = B.pipe_launch_count()
+            B.pipe_ensemble_forward(layer.desc, layer.blob, [xq] * M, [sx] * M, [y], bias, True)
+            launches = B.pipe_launch_count() - before
+        finally:
+            B.pipe_diag_select_kernel(B.KERNEL_AUTO)
+        torch.cuda.synchronize()
+        ys.append(y.view(torch.int32))
+    assert torch.equal(ys[0], ys[1]) and B.pipe_poll_status() == B.PIPE_OK
+    assert launches == 1
