@@ -51,8 +51,8 @@ constexpr int kStageBOff = kSub * kABytes;
 constexpr int kTmemCols = 512;
 constexpr int kAccCols = 256;
 constexpr int kMaxRing = 3;
-constexpr int kRecBufs = 4;    // copies of block records in shared memory: a tile's, the next tile's, whose tables are made
-                               // while this tile drains, the one on its way, and one that slower warps may still be reading
+constexpr int kRecBufs = 4;    // copies of block records in shared memory: a tile's, the next tile's, whose tables may be
+                               // made while this tile drains, the one on its way, and one that slower warps may still be reading
 constexpr int kTileRing = 8;   // tiles whose stacked-row count the unpack warps keep for the MMA issuer (they are at
                                // most a ring of stages, i.e. three tiles, ahead of it)
 using namespace tcc;
@@ -358,8 +358,9 @@ __device__ __forceinline__ void unpack_role(const Params& p, const Rings& g, int
                          : "memory");
           // ... and this warp's next block into L2, a use of the ring (some 5000 cycles) ahead: where the weights come from
           // HBM -- few token tiles -- the copy then finds them there (11008 -> 4096, T = 100: 48.1 -> 44.9 us, 4096 ->
-          // 11008, T = 1024: 96.7 -> 91.3; two uses ahead 47.8, three 45.5), and it costs nothing measurable elsewhere
-          if (kbs + kUnpackWarps < p.kblocks)
+          // 11008, T = 1024: 96.7 -> 91.3; two uses ahead 47.8, three 45.5).  Not for the int8 copy, whose bytes it would
+          // ask for twice as fast (1408 x 5424, T = 121: 22.4 -> 23.6 us)
+          if (!p.direct && kbs + kUnpackWarps < p.kblocks)
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src + (static_cast<size_t>(run_stp) * kUnpackWarps << 4)), "r"(run_bytes) : "memory");
         }
         __syncwarp();
@@ -456,7 +457,7 @@ struct EpiCtx {
 // NKMAX bounds the orders of a branch (2, 4 or 8); the channel block is BN = 8 * nch_max channels.
 // Where each (order, 8-channel chunk) sits in the accumulator and the scale of every stacked row come from the
 // block's record in the blob (written by the expansion), which one lane of the CTA fetches with a bulk copy one
-// tile ahead into one of three copies; the epilogue itself does no dependent global load.
+// tile ahead into one of four copies; the epilogue itself does no dependent global load.
 // A lane computes 16 channels of its own token row at a time; the 32 x 16 block is then turned
 // through shared memory so that each store instruction writes 64 contiguous bytes of 8 rows
 // (a lane writing its own row directly would emit 32 separate 16-byte pieces per instruction,
@@ -501,15 +502,17 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
                  "l"(src), "r"(kRecBytes), "r"(bar)
                  : "memory");
   };
-  // Tables of the pair's tile number tc, by all epilogue threads of the CTA, a tile ahead of their use so that no warp
-  // waits for the slowest one between two tiles (made at the tile's start they cost 4500 cycles of the 20 000 a tile of
-  // 768 -> 3072 drains for; its fused GeLU layer 84 -> 77 us without): the products c = s_k * lambda_x of the stacked rows (once per CTA instead
-  // of once per token row) and, for the fused epilogue, the bias of the tile's channels.
-  auto make_tables = [&](uint32_t tc, int tile) -> bool {
+  // Tables of a tile, by all epilogue threads of the CTA: the products c = s_k * lambda_x of the stacked rows (once per CTA
+  // instead of once per token row) and, for the fused epilogue, the bias of the tile's channels.
+  // AHEAD: made for the pair's tile number tc a tile ahead of their use, so that no warp waits for the slowest one between
+  // two tiles (made at the tile's start they cost 4500 cycles of the 20 000 a tile of 768 -> 3072 drains for; its fused GeLU
+  // layer 84 -> 77 us without, a zero point 24.4 -> 24.0, 11008 -> 4096 summed, T = 1024 129 -> 122).  Not for plain fp32
+  // outputs, where it costs registers the chain needs (spill loads 8 -> 184 bytes: 768 -> 3072 43.7 -> 47.1 us, eight orders
+  // 73 -> 83, on a shared input 44.7 -> 46.9).
+  constexpr bool AHEAD = Q8 || ZP || ACC;
+  auto make_tables = [&](uint32_t tc, int m) -> bool {
     const uint32_t i = tc % kRecBufs, ph = (tc / kRecBufs) & 1;
     if (!mbar_wait(x.recbar0 + 8u * i, ph, x.abort_flag, p.f.status)) return false;
-    int m, cb, tt;
-    locate_tile(p, x.tile_base, tile, m, cb, tt);
     const float sx = x.sx_s[m];
     const uint32_t rec = x.rec0 + i * kRecBytes;
     const int et = (x.warp - 2 - kUnpackWarps) * 32 + lane;   // this thread among the epilogue threads
@@ -535,7 +538,11 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
       if (x.pair + x.npairs < x.num_tiles) fetch_record(1, x.pair + x.npairs);
     }
     __syncwarp();
-    tables_ok = make_tables(0, x.pair);
+    if constexpr (AHEAD) {
+      int m, cb, tt;
+      locate_tile(p, x.tile_base, x.pair, m, cb, tt);
+      tables_ok = make_tables(0, m);
+    }
   }
   for (int tile = x.pair; tables_ok && tile < x.num_tiles; tile += x.npairs, ++tcount) {
     struct { int m, cb, tt, k0; } t;
@@ -545,12 +552,26 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
     const int buf = tcount & 1;
     const uint32_t aph = (tcount >> 1) & 1;
     const uint32_t rec_s = x.rec0 + (tcount % kRecBufs) * kRecBytes;
-    if (!mbar_wait(x.prebar0 + 8u * (tcount % kRecBufs), (tcount / kRecBufs) & 1, x.abort_flag, p.f.status)) break;
+    const uint32_t rec_i = tcount % kRecBufs, rec_ph = (tcount / kRecBufs) & 1;
+    if (!mbar_wait((AHEAD ? x.prebar0 : x.recbar0) + 8u * rec_i, rec_ph, x.abort_flag, p.f.status)) break;
     int c0, c1;
     asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(c0), "=r"(c1) : "r"(rec_s));
     const int nch = (c1 - c0) >> 3;       // at most PIPE_BLOCK_CHANNELS / 8
     const uint32_t colmap_s = rec_s + kRecColmapOff;
-    const uint32_t cscale_s = smem_u32(x.cfold + (tcount % kRecBufs) * kMaxN);
+    float* cf = x.cfold + rec_i * kMaxN;
+    if constexpr (!AHEAD) {
+      const float sx = x.sx_s[t.m];
+      const int et = (x.warp - 2 - kUnpackWarps) * 32 + lane;
+      for (int r = et; r < kMaxN; r += 32 * kEpiWarps) {
+        float sc;
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(sc) : "r"(rec_s + kRecScaleOff + 4u * r));
+        cf[r] = __fmul_rn(sc, sx);
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(x.prebar0 + 8u * rec_i);
+      if (!mbar_wait(x.prebar0 + 8u * rec_i, rec_ph, x.abort_flag, p.f.status)) break;
+    }
+    const uint32_t cscale_s = smem_u32(cf);
     // The accumulators hold 2^(8-b) times the sums; float(2^(8-b) a) = 2^(8-b) float(a) exactly, so the shift is
     // taken as a multiplication by 2^-(8-b) after the conversion (exact for every int32, and on the pipe with the
     // most issue slots); only the verification output needs the shifted integers themselves.
@@ -625,9 +646,15 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
     // overwrite those of the tile before that: the accumulators just handed over were computed after every epilogue warp
     // of the pair had finished both.
     if (rec_issuer && tile + 2 * x.npairs < x.num_tiles) fetch_record(tcount + 2, tile + 2 * x.npairs);
-    __syncwarp();
-    if (tile + x.npairs < x.num_tiles) tables_ok = make_tables(tcount + 1, tile + x.npairs);
-    if (!tables_ok) break;
+    if constexpr (AHEAD) {
+      __syncwarp();
+      if (tile + x.npairs < x.num_tiles) {
+        int m, cb, tt;
+        locate_tile(p, x.tile_base, tile + x.npairs, m, cb, tt);
+        tables_ok = make_tables(tcount + 1, m);
+      }
+      if (!tables_ok) break;
+    }
     const uint32_t tbase = x.tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * kAccCols;
     if constexpr (ZP) {
       // The two warps of the last lane quarter read the row of sums, half of the columns each.  (A buffer's products are
