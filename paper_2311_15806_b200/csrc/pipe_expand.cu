@@ -694,8 +694,8 @@ __global__ void block_record_kernel(const __grid_constant__ BlockRecordArgs a) {
 // rows' packed codes from level storage to their orders (place_orders_kernel).
 // Against one pass per order this neither writes nor re-reads the fp32 residual (8 bytes an element and order) and
 // pays with codes of levels that no order uses (b / 8 bytes each, and their arithmetic): 4096 x 11008 and back, int4,
-// K = 4, gamma = 0.5: 600 -> 280 us; 8192 x 8192 ternary, K = 8, gamma = 0.25 (8 levels computed, 2.75 used on
-// average): 464 -> 247 us.  The level storage takes the place of the residual in the workspace.
+// K = 4, gamma = 0.5: 600 -> 266 us; 8192 x 8192 ternary, K = 8, gamma = 0.25 (8 levels computed, 2.75 used on
+// average): 464 -> 246 us.  The level storage takes the place of the residual in the workspace.
 // Layers this does not take (chain_fits) run one pass per order: the unstructured mask and the L2 score need the
 // residual itself, rows beyond 16384 do not fit a block's registers, rows that are not whole 16-code chunks, and large
 // layers that use few of many levels.
@@ -779,6 +779,13 @@ __device__ __forceinline__ float code_by_division(float x, float s, float fq) {
   if (s != 0.f) c = fminf(fmaxf(rintf(__fdiv_rn(x, s)), -fq), fq);
   return c;
 }
+static __device__ __noinline__ uint32_t codes4_by_division(float x0, float x1, float x2, float x3, float s, float fq) {
+  const float q[4] = {code_by_division(x0, s, fq), code_by_division(x1, s, fq), code_by_division(x2, s, fq), code_by_division(x3, s, fq)};
+  uint32_t b = 0;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) b |= (static_cast<uint32_t>(static_cast<int>(q[e])) & 0xffu) << (8 * e);
+  return b;
+}
 // Four elements through all levels up to j (out of line: a few chunks in a thousand): residual after level j and its codes
 // as the bytes of a word.  lvl_s: the scales of the levels below j.  Divides only where the estimate cannot decide, like the
 // levels themselves: weights on a coarse grid (an integer model's) put many quotients on a boundary, at several levels.
@@ -820,12 +827,18 @@ constexpr int kChainMaxI = 16384;
 // and level there are four beside the packing: r * (1 / s) + 1.5 * 2^23 (the fused addition rounds to nearest even and
 // leaves the code in the low byte), the code as a float, the residual, its maximum.  What DEFINES the code is the IEEE
 // quotient; it and the estimate can differ only next to a rounding boundary, where |residual| is within
-// s * |t| * 2^-22 of s / 2: so the maximum that the next level needs anyway tells whether a chunk has to be divided
-// (the reciprocal is off by 2^-23, the quotient's own rounding by 2^-24, relative; |t| <= qmax because |x| <= amax,
+// s * |t| * 2^-22 of s / 2: so the maximum that the next level needs anyway tells whether a chunk has to be replayed from
+// the weights, and the old residual need not be kept (the reciprocal is off by 2^-23, the quotient's own rounding by 2^-24, relative; |t| <= qmax because |x| <= amax,
 // which is also why no clamp is needed while s has a usable reciprocal).
 // (11 instructions per element and level in all, against 16 with an estimate, its distance and the update one after the
-// other and one chunk per thread; the issue slots are 77 % busy, DRAM 45 %: 11008 x 4096 in 78 us, the ternary
+// other and one chunk per thread; the issue slots are 76 % busy, DRAM 41 %: 11008 x 4096 in 76 us, the ternary
 // 8192 x 8192 with its eight levels in 190.)
+// Ordinary weights replay a few chunks in a thousand.  Weights on a coarse grid put quotients on a boundary all over, at
+// every level; a block that had to replay in an eighth of its threads therefore keeps, from the next level on, the old
+// residual of a quad until its maximum is known, and divides the quad alone.  That form alone costs ordinary weights 6 to
+// 11 % (expansion of an LLM-shaped MLP 272 -> 290 us, ternary 8192 x 8192 249 -> 281), the choice 2 %; normal weights rounded
+// to multiples of an eighth of their deviation, ternary 4096 x 4096, K = 8: 763 us with replays by division, 536 with
+// replays by estimates, 250 with the choice; by orders 234.
 template <int BITS, int PER, int MAXT, int MINB>   // PER: 16-code chunks per thread
 __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_constant__ ChainArgs p) {
   __shared__ uint32_t part[2][32];
@@ -860,12 +873,16 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
     for (int e = 0; e < 16; ++e) mk = max(mk, abs_key(r[c][e]));
   uint8_t* temp_row = p.temp + static_cast<int64_t>(o) * p.temp_pitch;   // this row in the level being written
   const int64_t temp_step = static_cast<int64_t>(p.O) * p.temp_pitch;
+  bool careful = false;
+  int replays = 0;
 #pragma unroll 1
   for (int j = 0; j < p.K; ++j) {
     // largest magnitude entering this level (one barrier per level: the partial maxima alternate between two rows)
     mk = __reduce_max_sync(0xffffffffu, mk);
     if (lane == 0) part[j & 1][warp] = mk;
-    __syncthreads();
+    // (a block that had to replay in an eighth of its threads keeps to the careful form from here on)
+    careful = __syncthreads_count(replays) * 8 > blockDim.x || careful;
+    replays = 0;
     mk = __reduce_max_sync(0xffffffffu, lane < nwarps ? part[j & 1][lane] : 0u);
     const float s = __fdiv_rn(__uint_as_float(mk), fq);
     const bool direct = j < p.direct;
@@ -880,23 +897,53 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
     mk = 0;
 #pragma unroll
     for (int c = 0; c < PER; ++c) {
+      const int chunk = tid + c * blockDim.x, e0 = chunk * 16;
       uint32_t wv[4], kern[4];
       float m = 0.f;
+      if (careful) {
 #pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        float u[4];
+        for (int w = 0; w < 4; ++w) {
+          float* x = &r[c][4 * w];
+          float u[4], x1[4];
+          float m4 = 0.f;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          float& x = r[c][4 * w + e];
-          u[e] = __fmaf_rn(x, rcp, kMagic);
-          x = __fmaf_rn(-s, __fsub_rn(u[e], kMagic), x);   // exact new residual, rounded once
-          m = fmaxf(m, fabsf(x));
+          for (int e = 0; e < 4; ++e) {
+            u[e] = __fmaf_rn(x[e], rcp, kMagic);
+            x1[e] = __fmaf_rn(-s, __fsub_rn(u[e], kMagic), x[e]);
+            m4 = fmaxf(m4, fabsf(x1[e]));
+          }
+          wv[w] = __byte_perm(__byte_perm(__float_as_uint(u[0]), __float_as_uint(u[1]), 0x0040),
+                              __byte_perm(__float_as_uint(u[2]), __float_as_uint(u[3]), 0x0040), 0x5410);
+          if (m4 >= limit) {
+            wv[w] = codes4_by_division(x[0], x[1], x[2], x[3], s, fq);
+            m4 = 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              x1[e] = __fmaf_rn(-s, static_cast<float>(static_cast<int8_t>(wv[w] >> (8 * e))), x[e]);
+              m4 = fmaxf(m4, fabsf(x1[e]));
+            }
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) x[e] = x1[e];
+          m = fmaxf(m, m4);
         }
-        wv[w] = __byte_perm(__byte_perm(__float_as_uint(u[0]), __float_as_uint(u[1]), 0x0040),
-                            __byte_perm(__float_as_uint(u[2]), __float_as_uint(u[3]), 0x0040), 0x5410);
+      } else {
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          float u[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            float& x = r[c][4 * w + e];
+            u[e] = __fmaf_rn(x, rcp, kMagic);
+            x = __fmaf_rn(-s, __fsub_rn(u[e], kMagic), x);   // exact new residual, rounded once
+            m = fmaxf(m, fabsf(x));
+          }
+          wv[w] = __byte_perm(__byte_perm(__float_as_uint(u[0]), __float_as_uint(u[1]), 0x0040),
+                              __byte_perm(__float_as_uint(u[2]), __float_as_uint(u[3]), 0x0040), 0x5410);
+        }
       }
-      const int chunk = tid + c * blockDim.x, e0 = chunk * 16;
-      if (m >= limit) {
+      if (!careful && m >= limit) {
+        replays = 1;
         // (the old residual is overwritten: the chunk goes through all levels again)
         m = 0.f;
 #pragma unroll
@@ -1522,8 +1569,8 @@ extern "C" pipe_status pipe_expand_weights_static(const pipe_layer_desc* desc, c
   void* scratch = nullptr;
   st = static_scratch(&scratch);
   if (st != PIPE_OK) return st;
-  // Nothing in the workspace has to start at zero: the residual, the row maxima, the group scores
-  // and the keep flags are all written by this call before it reads them, so what an earlier
-  // call left behind is simply overwritten.
+  // Nothing in the workspace has to start at zero: levels and their maxima, or the residual, the row maxima, the group
+  // scores and the keep flags, are all written by this call before it reads them, so what an earlier call left behind is
+  // simply overwritten.
   return pipe_expand_weights(desc, d_W, ldw, d_blob, blob_bytes, scratch, PIPE_STATIC_SCRATCH_BYTES, stream);
 }

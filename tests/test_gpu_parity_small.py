@@ -112,7 +112,7 @@ def _grid_weights(rng, O, I, step, top):
 # Rows exhausted before the last order (a step of zero), quotients on a boundary at one level after the other, steps whose
 # reciprocal is no usable estimate (binary32 underflows or overflows around them) and steps that underflow to zero.
 @pytest.mark.parametrize("bits,K", [(8, 3), (4, 4), (2, 8), (3, 5), (6, 4)])
-@pytest.mark.parametrize("kind", ["exhausted", "int8_grid", "zero_rows", "tiny", "underflow", "huge"])
+@pytest.mark.parametrize("kind", ["exhausted", "int8_grid", "coarse_grid", "zero_rows", "tiny", "underflow", "huge"])
 def test_expand_weights_of_exhausted_rows(oracle, bits, K, kind):
     rng = np.random.default_rng(bits + len(kind))
     O, I, g = 64, 528, 16
@@ -120,6 +120,8 @@ def test_expand_weights_of_exhausted_rows(oracle, bits, K, kind):
         W = _grid_weights(rng, O, I, 0.03125, 2 ** (bits - 1) - 1)
     elif kind == "int8_grid":
         W = _grid_weights(rng, O, I, 0.01, 126)
+    elif kind == "coarse_grid":
+        W = (np.rint(rng.standard_normal((O, I)) * 8.0) * 0.0025).astype(np.float32)
     elif kind == "zero_rows":
         W = _w(rng, O, I)
         W[1::2] = 0.0
@@ -129,16 +131,21 @@ def test_expand_weights_of_exhausted_rows(oracle, bits, K, kind):
     H.assert_expansion_matches(H.gpu_expand(H.desc_of(O, I, bits, K, g, 2), W), e, oracle)
 
 
-def test_expansion_of_exhausted_rows_takes_no_longer():
-    """Rows whose residual is zero after the first order take no division at all, at any level: such a layer takes about
-    0.9 of the time of one that uses every level (half as much again is allowed)."""
+@pytest.mark.parametrize("kind,allowed", [("exhausted", 1.5), ("coarse_grid", 4.0)])
+def test_expansion_of_weights_on_a_grid_keeps_its_time(kind, allowed):
+    """Rows whose residual is zero after the first order take no division at all, at any level (0.9 of the time of a layer
+    of the same size that uses every level); a grid that puts quotients on a boundary in most quads of every level
+    divides those, without going through earlier levels again (2.6 times)."""
     H.ensure_built()
     O = I = 4096
     desc = H.desc_of(O, I, 2, 8, 16, 64)
     lay = B.pipe_layout(desc)
     blob, ws = B.alloc_bytes(lay.blob_bytes), B.alloc_bytes(lay.expand_ws_bytes)
-    grid = torch.randint(-1, 2, (O, I), device="cuda").float().mul_(0.03125)
-    grid[:, 0] = 0.03125
+    if kind == "exhausted":
+        grid = torch.randint(-1, 2, (O, I), device="cuda").float().mul_(0.03125)
+        grid[:, 0] = 0.03125
+    else:
+        grid = torch.randn((O, I), device="cuda").mul_(8.0).round_().mul_(0.0025)
 
     def best_ms(W):
         best = float("inf")
@@ -152,7 +159,7 @@ def test_expansion_of_exhausted_rows_takes_no_longer():
         return best
 
     normal = best_ms(torch.randn((O, I), device="cuda"))
-    assert best_ms(grid) <= 1.5 * normal
+    assert best_ms(grid) <= allowed * normal
 
 
 @pytest.mark.parametrize("bits", [8, 4, 2])
