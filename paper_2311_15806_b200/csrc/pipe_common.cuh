@@ -211,12 +211,12 @@ inline bool has_zero_point(const ForwardArgs& a) {
 }
 
 // A summed ensemble as one launch per predictor, in order, so that y = ((y_1 + y_2) + ...) is formed in a fixed order.
-// launch(args, queue) with queue = false only says whether the kernel takes a predictor: all are asked before the first is
-// queued, for a kernel that declines a later one would have its launches repeated by the next kernel.
+// launch(args, queue) with queue = false only says whether the kernel takes a predictor: the later ones are asked before the
+// first is queued (0.2 us each), for a kernel that declines one of them would have its launches repeated by the next kernel.
 template <class Launch>
 inline pipe_status launch_each_predictor(const ForwardArgs& a, Launch launch) {
   for (int queue = 0; queue < 2; ++queue)
-    for (int m = 0; m < a.num_branches; ++m) {
+    for (int m = queue ? 0 : 1; m < a.num_branches; ++m) {
       ForwardArgs one = a;
       one.num_branches = 1;
       one.branch[0] = a.branch[m];
