@@ -116,14 +116,14 @@ def workload_spec(name: str):
 # DRAM read + write bytes of ONE launch of the GEMM kernel, from one ncu capture per workload
 # (profiles/ncu_pair_kernel.txt, profiles/ncu_stream_kernel.txt).  A workload without a capture has no entry and reports null.
 NCU_DRAM_BYTES_PER_LAUNCH = {
-    "cfg2": 28681984 + 50585088,
-    "cfg3a": 9456896 + 47369472,
-    "cfg4a_t4096": 91300864 + 312781824,
-    "cfg5": 445346816 + 1026677760,
-    "cfg4a_t1": 56560896 + 92160,
-    "cfg4a_t16": 56688128 + 129536,
-    "cfg4a_t4096+int8_copy": 150311936 + 315610368,
-    "cfg3b+int8_copy": 31186432 + 857088,
+    "cfg2": 28441344 + 50646272,
+    "cfg3a": 9420800 + 46272512,
+    "cfg4a_t4096": 90903552 + 313437696,
+    "cfg5": 437495808 + 1026217472,
+    "cfg4a_t1": 56560384 + 45056,
+    "cfg4a_t16": 56688128 + 265472,
+    "cfg4a_t4096+int8_copy": 147986944 + 315521536,
+    "cfg3b+int8_copy": 31184384 + 722176,
 }
 
 
