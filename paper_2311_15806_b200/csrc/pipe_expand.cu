@@ -831,8 +831,8 @@ constexpr int kChainMaxI = 16384;
 // the weights, and the old residual need not be kept (the reciprocal is off by 2^-23, the quotient's own rounding by 2^-24, relative; |t| <= qmax because |x| <= amax,
 // which is also why no clamp is needed while s has a usable reciprocal).
 // (11 instructions per element and level in all, against 16 with an estimate, its distance and the update one after the
-// other and one chunk per thread; the issue slots are 76 % busy, DRAM 41 %: 11008 x 4096 in 76 us, the ternary
-// 8192 x 8192 with its eight levels in 190.)
+// other and one chunk per thread; the issue slots are 77 % busy, DRAM 40 %: 11008 x 4096 in 78 us, the ternary
+// 8192 x 8192 with its eight levels in 192.)
 // Ordinary weights replay a few chunks in a thousand.  Weights on a coarse grid put quotients on a boundary all over, at
 // every level; a block that had to replay in an eighth of its threads therefore keeps, from the next level on, the old
 // residual of a quad until its maximum is known, and divides the quad alone.  That form alone costs ordinary weights 6 to

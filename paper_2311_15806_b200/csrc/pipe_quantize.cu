@@ -10,10 +10,11 @@
 // start at once: a forward call that follows sets itself up (and, where it is allowed to, fetches weights) beside it and
 // waits for it before touching the codes.  (The first launch of either form is an ordinary one, so whatever stands before
 // the quantization on the stream -- an expansion, say -- is complete when such a forward call starts.)
-// Measured against zeroing + range pass + quantize pass as three plain launches (back to back, inputs beyond L2 where
-// large; asymmetric in brackets): 4096 elements 7.2 -> 2.4 us, 65 thousand 8.2 -> 3.7, a million 8.2 -> 5.9 (13.3 -> 6.7),
-// 17 million 34.8 -> 27.0 (55 -> 33), 67 million 114.6 -> 95.3 (145 -> 113).  The one-launch form ends where one cluster's
-// SMs take longer to read the tensor than a second launch costs (131 thousand elements; at 262 thousand 7.2 against 6.0).
+// Measured against zeroing + range pass + quantize pass as three plain launches (graphs of 20 calls, inputs beyond L2 where
+// large; asymmetric in brackets): 4096 elements 8.3 -> 2.5 us (8.4 -> 2.7), 65 thousand 8.3 -> 3.7 (9.2 -> 4.5), a million
+// 8.4 -> 6.3 (13.2 -> 6.5), 17 million 35.5 -> 28.5 (56.6 -> 29.3), 67 million 115 -> 96 (145 -> 98).  The one-launch form ends
+// where one cluster's SMs take longer to read the tensor than a second launch costs (131 thousand elements; at 262 thousand
+// 7.2 against 6.0 in one run).
 #include "pipe_common.cuh"
 
 namespace pipe {
