@@ -124,6 +124,37 @@ __device__ __forceinline__ uint32_t pack4_low_bytes(float a, float b, float c, f
   return __byte_perm(ab, cd, 0x5410);
 }
 
+// Two binary32 values in a register pair, for the packed arithmetic (every operation rounds each half as its scalar form).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack_f2(float lo, float hi) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ f32x2 both_f2(float v) { return pack_f2(v, v); }
+__device__ __forceinline__ void unpack_f2(f32x2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ f32x2 fma_f2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add_f2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// Largest magnitude of three; the second form hands a NaN on (as the NaN of all ones).
+__device__ __forceinline__ float max3_abs(float a, float b, float c) {
+  float d;
+  asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ float max3_abs_nan(float a, float b, float c) {
+  float d;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 // sigma of Eq. 9 for an inner layer (Sec. 3.2 names ReLU, SiLU, GeLU and sigmoid), in binary32: kind 0 identity,
 // 1 ReLU, 2 SiLU v / (1 + exp(-v)), 3 GeLU v (1 + erf(v / sqrt 2)) / 2, 4 sigmoid 1 / (1 + exp(-v)).
 __device__ __forceinline__ float apply_activation(float v, int kind) {

@@ -823,22 +823,20 @@ static __device__ __noinline__ void replay_quad(const float4* src, const float* 
 
 constexpr int kChainMaxI = 16384;
 
-// One block per row, PER chunks of 16 consecutive elements per thread.  Bound by its instructions, so per element
-// and level there are four beside the packing: r * (1 / s) + 1.5 * 2^23 (the fused addition rounds to nearest even and
-// leaves the code in the low byte), the code as a float, the residual, its maximum.  What DEFINES the code is the IEEE
+// One block per row, PER chunks of 16 consecutive elements per thread.  Bound by its instructions, so a level costs an
+// element three packed operations (two elements each) beside half a maximum and the packing: r * (1 / s) + 1.5 * 2^23 (the
+// fused addition rounds to nearest even), the code as a float, the residual.  What DEFINES the code is the IEEE
 // quotient; it and the estimate can differ only next to a rounding boundary, where |residual| is within
 // s * |t| * 2^-22 of s / 2: so the maximum that the next level needs anyway tells whether a chunk has to be replayed from
 // the weights, and the old residual need not be kept (the reciprocal is off by 2^-23, the quotient's own rounding by 2^-24, relative; |t| <= qmax because |x| <= amax,
 // which is also why no clamp is needed while s has a usable reciprocal).
-// (11 instructions per element and level in all, against 16 with an estimate, its distance and the update one after the
-// other and one chunk per thread; the issue slots are 77 % busy, DRAM 40 %: 11008 x 4096 in 78 us, the ternary
-// 8192 x 8192 with its eight levels in 192.)
+// The packing is arithmetic too: sum_e (code_e + 2^(b-1)) 2^(b e) over the codes of 16 bits of a packed word, on top of
+// 1.5 * 2^23, is exact in binary32 and stands in the low 16 bits of its pattern; the offsets are the fields' sign bits, which
+// an exclusive or takes away.  A pair holds the elements i and i + 2 of a quad, so that its halves lead to the low and to the
+// high half of the same word.
 // Ordinary weights replay a few chunks in a thousand.  Weights on a coarse grid put quotients on a boundary all over, at
 // every level; a block that had to replay in an eighth of its threads therefore keeps, from the next level on, the old
-// residual of a quad until its maximum is known, and divides the quad alone.  That form alone costs ordinary weights 6 to
-// 11 % (expansion of an LLM-shaped MLP 272 -> 290 us, ternary 8192 x 8192 249 -> 281), the choice 2 %; normal weights rounded
-// to multiples of an eighth of their deviation, ternary 4096 x 4096, K = 8: 763 us with replays by division, 536 with
-// replays by estimates, 250 with the choice; by orders 234.
+// residual of a quad until its maximum is known, and divides the quad alone.
 template <int BITS, int PER, int MAXT, int MINB>   // PER: 16-code chunks per thread
 __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_constant__ ChainArgs p) {
   __shared__ uint32_t part[2][32];
@@ -848,10 +846,11 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
   constexpr float kMagic = 12582912.f;
   constexpr int kWords = BITS / 2;            // packed words of 16 codes
   constexpr int kStepBytes = 128 * BITS / 8;
+  constexpr uint32_t kSigns = BITS == 8 ? 0x80808080u : (BITS == 4 ? 0x88888888u : 0xAAAAAAAAu);   // sign bits of a word's fields
   // |residual| / s from which a chunk is divided: 1/2 - (qmax 2^-22 + 2^-23)
   const float near_half = 0.5f - (fq * 2.384185791015625e-07f + 1.1920928955078125e-07f);
-  float r[PER][16];
-  uint32_t mk = 0;
+  f32x2 r[PER][8];   // pair 2 w + i: elements 4 w + i and 4 w + i + 2
+  float mf = 0.f;
 #pragma unroll
   for (int c = 0; c < PER; ++c) {
     const int e0 = (tid + c * blockDim.x) * 16;
@@ -860,17 +859,23 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
         const float4 v = __ldg(src + w);
-        r[c][4 * w] = v.x; r[c][4 * w + 1] = v.y; r[c][4 * w + 2] = v.z; r[c][4 * w + 3] = v.w;
+        r[c][2 * w] = pack_f2(v.x, v.z);
+        r[c][2 * w + 1] = pack_f2(v.y, v.w);
       }
     } else {
 #pragma unroll
-      for (int e = 0; e < 16; ++e) r[c][e] = 0.f;
+      for (int i = 0; i < 8; ++i) r[c][i] = 0;
     }
   }
 #pragma unroll
   for (int c = 0; c < PER; ++c)
 #pragma unroll
-    for (int e = 0; e < 16; ++e) mk = max(mk, abs_key(r[c][e]));
+    for (int i = 0; i < 8; ++i) {
+      float lo, hi;
+      unpack_f2(r[c][i], lo, hi);
+      mf = max3_abs_nan(mf, lo, hi);
+    }
+  uint32_t mk = __float_as_uint(mf);
   uint8_t* temp_row = p.temp + static_cast<int64_t>(o) * p.temp_pitch;   // this row in the level being written
   const int64_t temp_step = static_cast<int64_t>(p.O) * p.temp_pitch;
   bool careful = false;
@@ -884,7 +889,7 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
     careful = __syncthreads_count(replays) * 8 > blockDim.x || careful;
     replays = 0;
     mk = __reduce_max_sync(0xffffffffu, lane < nwarps ? part[j & 1][lane] : 0u);
-    const float s = __fdiv_rn(__uint_as_float(mk), fq);
+    const float s = BITS == 2 ? __uint_as_float(mk) : __fdiv_rn(__uint_as_float(mk), fq);   // (2 bits: qmax = 1)
     const bool direct = j < p.direct;
     if (tid == 0) {
       lvl_s[j] = s;   // (read at later levels, behind their barriers)
@@ -894,17 +899,21 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
     }
     float rcp, limit;
     level_estimate(s, near_half, rcp, limit);
+    const f32x2 rcp2 = both_f2(rcp), neg_s2 = both_f2(-s), magic2 = both_f2(kMagic), neg_magic2 = both_f2(-kMagic);
+    constexpr float kBias = kMagic + static_cast<float>(kSigns & 0xffffu);
     mk = 0;
 #pragma unroll
     for (int c = 0; c < PER; ++c) {
       const int chunk = tid + c * blockDim.x, e0 = chunk * 16;
-      uint32_t wv[4], kern[4];
+      uint32_t kern[4];
       float m = 0.f;
       if (careful) {
+        uint32_t wv[4];
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
-          float* x = &r[c][4 * w];
-          float u[4], x1[4];
+          float x[4], u[4], x1[4];
+          unpack_f2(r[c][2 * w], x[0], x[2]);
+          unpack_f2(r[c][2 * w + 1], x[1], x[3]);
           float m4 = 0.f;
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
@@ -912,8 +921,7 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
             x1[e] = __fmaf_rn(-s, __fsub_rn(u[e], kMagic), x[e]);
             m4 = fmaxf(m4, fabsf(x1[e]));
           }
-          wv[w] = __byte_perm(__byte_perm(__float_as_uint(u[0]), __float_as_uint(u[1]), 0x0040),
-                              __byte_perm(__float_as_uint(u[2]), __float_as_uint(u[3]), 0x0040), 0x5410);
+          wv[w] = pack4_low_bytes(u[0], u[1], u[2], u[3]);
           if (m4 >= limit) {
             wv[w] = codes4_by_division(x[0], x[1], x[2], x[3], s, fq);
             m4 = 0.f;
@@ -923,39 +931,51 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
               m4 = fmaxf(m4, fabsf(x1[e]));
             }
           }
-#pragma unroll
-          for (int e = 0; e < 4; ++e) x[e] = x1[e];
+          r[c][2 * w] = pack_f2(x1[0], x1[2]);
+          r[c][2 * w + 1] = pack_f2(x1[1], x1[3]);
           m = fmaxf(m, m4);
         }
+        pack_bytes<BITS>(wv, kern);
       } else {
+        constexpr int kQuads = 8 / BITS;   // quads whose codes share a packed word
+        float m1 = 0.f;
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          float u[4];
+        for (int k = 0; k < kWords; ++k) {
+          f32x2 acc = both_f2(kBias);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            float& x = r[c][4 * w + e];
-            u[e] = __fmaf_rn(x, rcp, kMagic);
-            x = __fmaf_rn(-s, __fsub_rn(u[e], kMagic), x);   // exact new residual, rounded once
-            m = fmaxf(m, fabsf(x));
-          }
-          wv[w] = __byte_perm(__byte_perm(__float_as_uint(u[0]), __float_as_uint(u[1]), 0x0040),
-                              __byte_perm(__float_as_uint(u[2]), __float_as_uint(u[3]), 0x0040), 0x5410);
+          for (int h = 0; h < kQuads; ++h)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              f32x2& x = r[c][2 * (k * kQuads + h) + i];
+              const f32x2 q = add_f2(fma_f2(x, rcp2, magic2), neg_magic2);
+              x = fma_f2(neg_s2, q, x);   // exact new residual, rounded once
+              acc = h + i == 0 ? add_f2(q, acc) : fma_f2(q, both_f2(static_cast<float>(1u << (8 * i + BITS * h))), acc);
+              float lo, hi;
+              unpack_f2(x, lo, hi);
+              (i ? m1 : m) = max3_abs(i ? m1 : m, lo, hi);
+            }
+          float lo, hi;
+          unpack_f2(acc, lo, hi);
+          kern[k] = __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x5410) ^ kSigns;
         }
+        m = fmaxf(m, m1);
       }
       if (!careful && m >= limit) {
         replays = 1;
         // (the old residual is overwritten: the chunk goes through all levels again)
         m = 0.f;
+        uint32_t wv[4];
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
           float4 v;
           replay_quad(e0 < p.I ? reinterpret_cast<const float4*>(p.W + static_cast<int64_t>(o) * p.ldw + e0) + w : nullptr, lvl_s, j, s, fq, near_half, &v, &wv[w]);
-          r[c][4 * w] = v.x; r[c][4 * w + 1] = v.y; r[c][4 * w + 2] = v.z; r[c][4 * w + 3] = v.w;
+          r[c][2 * w] = pack_f2(v.x, v.z);
+          r[c][2 * w + 1] = pack_f2(v.y, v.w);
           m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
         }
+        pack_bytes<BITS>(wv, kern);
       }
       mk = max(mk, __float_as_uint(m));
-      pack_bytes<BITS>(wv, kern);
       auto store = [](uint8_t* dst, const uint32_t (&w)[4]) {
         if constexpr (kWords == 4) *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
         else if constexpr (kWords == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
@@ -967,9 +987,13 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
         const ChainOut& out = p.out[j];
         if (e0 < p.I_pad) {
           store(out.kcodes + (static_cast<int64_t>(e0 >> 7) * p.O + o) * kStepBytes + (e0 & 127) * BITS / 8, kern);
-          if (out.wcodes)
+          if (out.wcodes) {
+            uint32_t wv[4];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) wv[w] = bytes_of_kern<BITS>(kern[w * BITS / 8], w % (8 / BITS));
             *reinterpret_cast<uint4*>(out.wcodes + (static_cast<int64_t>(e0 >> 7) * p.O + o) * 128 + ((((e0 & 127) >> 4) ^ (o & 7)) << 4)) =
                 make_uint4(wv[0], wv[1], wv[2], wv[3]);
+          }
         }
         if (e0 < p.I) {
           uint32_t canon[4];
