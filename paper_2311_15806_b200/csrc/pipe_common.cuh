@@ -41,6 +41,31 @@ inline pipe_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? PIPE_OK : 
 
 inline pipe_status launch_status() { return cuda_ok(cudaGetLastError()); }
 
+// One launch with programmatic stream serialization: its blocks may stand on the SMs before the launch before it is complete,
+// and the kernel has to wait (grid_wait) before it touches what that launch, or one before it, may still read or write.
+// cluster: CTAs per cluster (1: none).
+template <typename... P, typename... A>
+inline cudaError_t launch_overlapped(void (*k)(P...), dim3 grid, int block, int cluster, cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block, 1, 1);
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, k, args...);
+}
+// Behind grid_wait everything queued before this launch is complete and visible.  A kernel that releases its dependents only
+// after its own wait keeps the order of the stream transitive.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 template <typename T>
 __host__ __device__ inline T ceil_div(T a, T b) {
   return (a + b - 1) / b;

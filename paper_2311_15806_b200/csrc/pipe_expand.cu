@@ -606,7 +606,11 @@ __device__ __forceinline__ void cut_table(const BlockTableArgs& a, const int m) 
   }
 }
 
-__global__ void __launch_bounds__(kTableThreads) block_table_kernel(const __grid_constant__ BlockTableArgs a) { cut_table(a, blockIdx.x); }
+__global__ void __launch_bounds__(kTableThreads) block_table_kernel(const __grid_constant__ BlockTableArgs a) {
+  grid_wait();
+  grid_release();
+  cut_table(a, blockIdx.x);
+}
 
 // Block records (layout in pipe.h): one thread block per (block of a table, table).
 struct BlockRecordArgs {
@@ -621,6 +625,8 @@ struct BlockRecordArgs {
 };
 
 __global__ void block_record_kernel(const __grid_constant__ BlockRecordArgs a) {
+  grid_wait();
+  grid_release();
   const int m = blockIdx.y, cb = blockIdx.x;
   if (!a.out[m]) return;
   const int n_blocks = a.tbl[m][0];
@@ -876,6 +882,9 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
       mf = max3_abs_nan(mf, lo, hi);
     }
   uint32_t mk = __float_as_uint(mf);
+  // (the weights were complete when the launch before this one, which zeroes the level maxima, started)
+  grid_wait();
+  grid_release();
   uint8_t* temp_row = p.temp + static_cast<int64_t>(o) * p.temp_pitch;   // this row in the level being written
   const int64_t temp_step = static_cast<int64_t>(p.O) * p.temp_pitch;
   bool careful = false;
@@ -1027,6 +1036,8 @@ __global__ void __launch_bounds__(kSelThreads) select_orders_kernel(const __grid
   __shared__ uint32_t part[2][32], part_lo[32];
   __shared__ int hist[256];
   __shared__ int found_bin, found_need, found_exact;
+  grid_wait();
+  grid_release();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nch = (p.G + kSelThreads - 1) / kSelThreads;
   if (tid < 256) hist[tid] = 0;
@@ -1163,6 +1174,8 @@ struct PlaceArgs {
 
 template <int BITS, int UW>
 __global__ void __launch_bounds__(kTableThreads) place_orders_kernel(const __grid_constant__ PlaceArgs p) {
+  grid_wait();
+  grid_release();
   if (blockIdx.x < static_cast<unsigned>(p.tables)) {
     cut_table(p.tab, blockIdx.x);
     return;
@@ -1264,6 +1277,8 @@ __global__ void write_header_kernel(uint32_t* hdr, pipe_layer_desc d) {
 }
 
 __global__ void __launch_bounds__(256) chain_init_kernel(const __grid_constant__ ChainInitArgs p) {
+  grid_wait();
+  grid_release();
   const int64_t i0 = blockIdx.x * 256ll + threadIdx.x, step = gridDim.x * 256ll;
   if (i0 == 0) write_header(p.hdr, p.desc);
   for (int64_t i = i0; i < p.n_max; i += step) p.lvl_max[i] = 0u;
@@ -1411,7 +1426,7 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
     ini.n_max = dense ? 0 : static_cast<int64_t>(L.K) * L.G;
     const int64_t init_n = ini.n_max > L.G + 1 ? ini.n_max : L.G + 1;
     const int64_t init_grid = ceil_div<int64_t>(init_n, 256);
-    chain_init_kernel<<<static_cast<int>(init_grid < 64 ? init_grid : 64), 256, 0, s>>>(ini);
+    launch_overlapped(chain_init_kernel, dim3(static_cast<int>(init_grid < 64 ? init_grid : 64)), 256, 1, s, ini);
     ch.W = d_W;
     ch.ldw = ldw;
     ch.direct = dense ? L.K : 1;
@@ -1432,8 +1447,8 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
     const bool long_rows = ch.I_pad > 8192 && ch.I_pad <= 12288 && 65536 / (threads3 * 80) > 65536 / (threads2 * 64);
     const int threads = long_rows ? threads3 : threads2;
 #define PIPE_CHAIN(B)                                                                       \
-  if (long_rows) expand_chain_kernel<B, 3, 256, 3><<<L.O, threads, 0, s>>>(ch);             \
-  else expand_chain_kernel<B, 2, 512, 2><<<L.O, threads, 0, s>>>(ch);
+  if (long_rows) launch_overlapped(expand_chain_kernel<B, 3, 256, 3>, dim3(L.O), threads, 1, s, ch);   \
+  else launch_overlapped(expand_chain_kernel<B, 2, 512, 2>, dim3(L.O), threads, 1, s, ch);
     if (L.bits == 8) { PIPE_CHAIN(8) } else if (L.bits == 4) { PIPE_CHAIN(4) } else { PIPE_CHAIN(2) }
 #undef PIPE_CHAIN
     count_launch(2);
@@ -1441,7 +1456,7 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
       sel.lvl_max = ini.lvl_max;
       sel.lvl_of = reinterpret_cast<int32_t*>(ws + plan.lvl_of);
       sel.G = L.G; sel.K = L.K; sel.n_keep = L.n_keep;
-      select_orders_kernel<<<1, kSelThreads, 0, s>>>(sel);
+      launch_overlapped(select_orders_kernel, dim3(1), kSelThreads, 1, s, sel);
       pl.lvl_of = sel.lvl_of;
       pl.lvl_scale = ch.lvl_scale;
       pl.temp = ch.temp;
@@ -1453,14 +1468,14 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
       pl.tab = t;
       const int grid = tables + (L.K - 1) * L.n_keep;
       const bool whole = L.lay.canon_row_bytes % 16 == 0;
-      if (L.bits == 8) place_orders_kernel<8, 4><<<grid, kTableThreads, 0, s>>>(pl);
-      else if (L.bits == 4 && whole) place_orders_kernel<4, 4><<<grid, kTableThreads, 0, s>>>(pl);
-      else if (L.bits == 4) place_orders_kernel<4, 2><<<grid, kTableThreads, 0, s>>>(pl);
-      else if (whole) place_orders_kernel<2, 4><<<grid, kTableThreads, 0, s>>>(pl);
-      else place_orders_kernel<2, 1><<<grid, kTableThreads, 0, s>>>(pl);
+      if (L.bits == 8) launch_overlapped(place_orders_kernel<8, 4>, dim3(grid), kTableThreads, 1, s, pl);
+      else if (L.bits == 4 && whole) launch_overlapped(place_orders_kernel<4, 4>, dim3(grid), kTableThreads, 1, s, pl);
+      else if (L.bits == 4) launch_overlapped(place_orders_kernel<4, 2>, dim3(grid), kTableThreads, 1, s, pl);
+      else if (whole) launch_overlapped(place_orders_kernel<2, 4>, dim3(grid), kTableThreads, 1, s, pl);
+      else launch_overlapped(place_orders_kernel<2, 1>, dim3(grid), kTableThreads, 1, s, pl);
       count_launch(2);
     } else if (tables) {
-      block_table_kernel<<<tables, kTableThreads, 0, s>>>(t);
+      launch_overlapped(block_table_kernel, dim3(tables), kTableThreads, 1, s, t);
       count_launch(1);
     }
   } else {
@@ -1545,7 +1560,7 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
       max_cap = max_cap > r.cap[m] ? max_cap : r.cap[m];
     }
     if (max_cap > 0) {
-      block_record_kernel<<<dim3(max_cap, L.M + 1), 256, 0, s>>>(r);
+      launch_overlapped(block_record_kernel, dim3(max_cap, L.M + 1), 256, 1, s, r);
       count_launch(1);
     }
   }

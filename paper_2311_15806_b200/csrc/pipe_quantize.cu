@@ -4,12 +4,12 @@
 // Tensors of kTinyQuads to kSmallQuads quads: ONE launch of one cluster, which keeps the tensor in registers, exchanges
 // its maxima through distributed shared memory and writes the codes.  Others: (1) a range pass whose clusters each leave
 // their maxima in the workspace (no atomics, so nothing has to be zeroed first), (2) a pass that reads those, divides /
-// rounds half to even / clamps and stores.  The second pass is launched with programmatic stream serialization -- its
-// blocks stand ready when the first pass ends -- and walks the tensor from its END, where the first pass stopped: what is
-// still in the 126 MB L2 is then read from there before it is evicted.  The last launch of either form lets ITS dependents
-// start at once: a forward call that follows sets itself up (and, where it is allowed to, fetches weights) beside it and
-// waits for it before touching the codes.  (The first launch of either form is an ordinary one, so whatever stands before
-// the quantization on the stream -- an expansion, say -- is complete when such a forward call starts.)
+// rounds half to even / clamps and stores.  Every launch uses programmatic stream serialization: its blocks stand ready when
+// the launch before ends.  The second pass walks the tensor from its END, where the first pass stopped: what is still in the
+// 126 MB L2 is then read from there before it is evicted.  The last launch of either form lets ITS dependents start at once: a
+// forward call that follows sets itself up (and, where it is allowed to, fetches weights) beside it and waits for it before
+// touching the codes.  (The first launch of either form releases only behind its own wait, so whatever stands before the
+// quantization on the stream -- an expansion, say -- is complete when such a forward call starts.)
 // Measured against zeroing + range pass + quantize pass as three plain launches (graphs of 20 calls, inputs beyond L2 where
 // large; asymmetric in brackets): 4096 elements 8.3 -> 2.5 us (8.4 -> 2.7), 65 thousand 8.3 -> 3.7 (9.2 -> 4.5), a million
 // 8.4 -> 6.3 (13.2 -> 6.5), 17 million 35.5 -> 28.5 (56.6 -> 29.3), 67 million 115 -> 96 (145 -> 98).  The one-launch form ends
@@ -207,6 +207,8 @@ __device__ __forceinline__ void load16(const QuantArgs& p, int64_t c, float (&v)
 // reads 512 contiguous bytes per instruction, four of them in flight per thread.
 template <bool EX, bool FLAT>
 __global__ void __launch_bounds__(kRangeThreads) act_range_kernel(const __grid_constant__ QuantArgs p) {
+  grid_wait();
+  grid_release();
   q_cluster_sync();   // every CTA of the cluster runs before another one writes its shared memory
   Range<EX> range;
   const int64_t first = blockIdx.x * static_cast<int64_t>(kRangeThreads) + threadIdx.x;
@@ -251,8 +253,8 @@ __global__ void __launch_bounds__(kRangeThreads) act_range_kernel(const __grid_c
 // Quantize pass: lambda_x and the codes.
 template <bool EX, bool FLAT>
 __global__ void __launch_bounds__(kQThreads) act_quantize_kernel(const __grid_constant__ QuantArgs p, int clusters) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  grid_release();
+  grid_wait();
   Range<EX> range;
   {
     const int lane = threadIdx.x & 31;
@@ -299,7 +301,8 @@ __global__ void __launch_bounds__(kQThreads) act_quantize_kernel(const __grid_co
 // Both passes in one launch of one cluster (FLAT tensors of at most PER quads per thread).
 template <bool EX, int PER>
 __global__ void __launch_bounds__(1024) act_small_kernel(const __grid_constant__ QuantArgs p) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  grid_wait();
+  grid_release();
   const int first = blockIdx.x * blockDim.x + threadIdx.x, stride = kClusterCtas * blockDim.x;
   const int quads = static_cast<int>(p.quads);
   const float4* x = reinterpret_cast<const float4*>(p.x);
@@ -324,26 +327,9 @@ __global__ void act_empty_kernel(const float* static_scale, float* sx_out, int32
   }
 }
 
-// One launch with clusters of eight CTAs, or with programmatic stream serialization.
 template <typename... P, typename... A>
 static pipe_status launch_q(void (*k)(P...), int grid, int block, bool cluster, cudaStream_t s, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  if (cluster) {
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kClusterCtas;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-  } else {
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-  }
-  cfg.gridDim = dim3(grid, 1, 1);
-  cfg.blockDim = dim3(block, 1, 1);
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, k, args...) != cudaSuccess) return PIPE_ERR_CUDA;
+  if (launch_overlapped(k, dim3(grid, 1, 1), block, cluster ? kClusterCtas : 1, s, args...) != cudaSuccess) return PIPE_ERR_CUDA;
   count_launch(1);
   return PIPE_OK;
 }
