@@ -1018,9 +1018,11 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
 
 // Which order keeps which group at which level, all orders in one block: per order the n_keep groups of largest score
 // (the maximum at the group's present level; ties to the lower index, as everywhere; non-negative floats order like
-// their bits).  The n_keep-th largest score is found by cutting the interval that holds it into up to 256 bins and
-// counting, usually twice (bisecting the bits instead, one block-wide count per bit, took 9 us per order where this
-// takes under 3), then the kept groups are compacted in index order.
+// their bits).  The n_keep-th largest score is found by counting the keys at and above three probes that quarter the interval
+// which holds it, until a probe has exactly n_keep (the usual end, after about log4 of the number of groups) or one value is
+// left.  A step of that search is one barrier, and so is the compaction, for which a thread holds neighbouring groups; the
+// block has only as many warps as leaves a thread up to eight groups, because the barriers are what an order's time goes
+// into.
 constexpr int kSelThreads = 1024;
 constexpr int kSelPer = 8;
 constexpr int kSelMaxGroups = kSelThreads * kSelPer;
@@ -1033,31 +1035,28 @@ struct SelectArgs {
 };
 
 __global__ void __launch_bounds__(kSelThreads) select_orders_kernel(const __grid_constant__ SelectArgs p) {
-  __shared__ uint32_t part[2][32], part_lo[32];
-  __shared__ int hist[256];
-  __shared__ int found_bin, found_need, found_exact;
+  __shared__ uint32_t part_lo[32], part_hi[32], part_n[2][2][32], part_c[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  const int per = (p.G + blockDim.x - 1) / blockDim.x, j0 = tid * per;   // this thread's groups: j0 .. j0 + per - 1
   grid_wait();
   grid_release();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nch = (p.G + kSelThreads - 1) / kSelThreads;
-  if (tid < 256) hist[tid] = 0;
   // key: score at the group's present level, plus one (0: no group); next: at the level behind it, asked for ahead of use
   uint32_t lvl[kSelPer], key[kSelPer], next[kSelPer];
   auto score = [&](int c, uint32_t l) -> uint32_t {
-    const int j = c * kSelThreads + tid;
-    return c < nch && j < p.G && l < static_cast<uint32_t>(p.K) ? __ldg(p.lvl_max + static_cast<int64_t>(l) * p.G + j) + 1u : 0u;
+    return c < per && j0 + c < p.G && l < static_cast<uint32_t>(p.K) ? __ldg(p.lvl_max + static_cast<int64_t>(l) * p.G + j0 + c) + 1u : 0u;
   };
 #pragma unroll
   for (int c = 0; c < kSelPer; ++c) {
     lvl[c] = 1;
     key[c] = score(c, 1);
   }
+  int round = 0;
   for (int k = 1; k < p.K; ++k) {
     uint32_t lo = 0xffffffffu, hi = 0;
 #pragma unroll
     for (int c = 0; c < kSelPer; ++c) {
       next[c] = score(c, lvl[c] + 1);
-      if (c < nch && key[c] != 0) {
+      if (key[c] != 0) {
         lo = min(lo, key[c]);
         hi = max(hi, key[c]);
       }
@@ -1066,93 +1065,89 @@ __global__ void __launch_bounds__(kSelThreads) select_orders_kernel(const __grid
     hi = __reduce_max_sync(0xffffffffu, hi);
     if (lane == 0) {
       part_lo[warp] = lo;
-      part[0][warp] = hi;
+      part_hi[warp] = hi;
     }
     __syncthreads();
-    lo = __reduce_min_sync(0xffffffffu, part_lo[lane]);
-    hi = __reduce_max_sync(0xffffffffu, part[0][lane]);
-    // of the keys in [lo, hi] the `need` largest are kept, those above hi are kept already
-    int need = p.n_keep;
-    uint32_t thr = lo;
+    lo = __reduce_min_sync(0xffffffffu, lane < nwarps ? part_lo[lane] : 0xffffffffu);
+    hi = __reduce_max_sync(0xffffffffu, lane < nwarps ? part_hi[lane] : 0u);
+    // more than n_keep keys are >= lo (every group has a key: it has been taken k - 1 times at most), `above` < n_keep are > hi
+    int above = 0;
     int ties = p.G;            // how many of the keys equal to the threshold are kept, lowest index first
+    uint32_t thr = lo;
     while (true) {
       if (lo == hi) {
         thr = lo;
-        ties = need;
+        ties = p.n_keep - above;
         break;
       }
-      const int width = 32 - __clz(hi - lo);
-      const int sh = width > 8 ? width - 8 : 0;
+      const uint32_t q = (hi - lo) >> 2;
+      const uint32_t m[3] = {lo + q + 1, lo + 2 * q + 1, lo + 3 * q + 1};   // in (lo, hi]
+      uint32_t n01 = 0, n2 = 0;
 #pragma unroll
-      for (int c = 0; c < kSelPer; ++c)
-        if (c < nch && key[c] >= lo && key[c] <= hi) atomicAdd(&hist[(key[c] - lo) >> sh], 1);
-      __syncthreads();
-      if (warp == 0) {
-        // lane L holds the bins 8 L .. 8 L + 7 (and clears them for the next use); suffix sums over the lanes
-        int h[8], tot = 0;
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-          h[b] = hist[8 * lane + b];
-          hist[8 * lane + b] = 0;
-          tot += h[b];
-        }
-        int suf = tot;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const int v = __shfl_down_sync(0xffffffffu, suf, d);
-          if (lane + d < 32) suf += v;
-        }
-        int above = suf - tot;   // keys in the lanes' bins behind this one's
-        if (above < need && suf >= need) {
-#pragma unroll
-          for (int b = 7; b >= 0; --b) {
-            if (above < need && above + h[b] >= need) {
-              found_bin = 8 * lane + b;
-              found_need = need - above;
-              found_exact = above + h[b] == need;
-            }
-            above += h[b];
-          }
-        }
+      for (int c = 0; c < kSelPer; ++c) {
+        n01 += (key[c] >= m[0] ? 1u : 0u) + (key[c] >= m[1] ? 0x10000u : 0u);
+        n2 += key[c] >= m[2] ? 1u : 0u;
+      }
+      n01 = __reduce_add_sync(0xffffffffu, n01);
+      n2 = __reduce_add_sync(0xffffffffu, n2);
+      if (lane == 0) {
+        part_n[round & 1][0][warp] = n01;
+        part_n[round & 1][1][warp] = n2;
       }
       __syncthreads();
-      lo += static_cast<uint32_t>(found_bin) << sh;
-      if (found_exact) {
-        thr = lo;
+      n01 = __reduce_add_sync(0xffffffffu, lane < nwarps ? part_n[round & 1][0][lane] : 0u);
+      n2 = __reduce_add_sync(0xffffffffu, lane < nwarps ? part_n[round & 1][1][lane] : 0u);
+      ++round;
+      const int n[3] = {static_cast<int>(n01 & 0xffffu), static_cast<int>(n01 >> 16), static_cast<int>(n2)};
+      if (n[0] == p.n_keep || n[1] == p.n_keep || n[2] == p.n_keep) {
+        thr = n[2] == p.n_keep ? m[2] : (n[1] == p.n_keep ? m[1] : m[0]);
         break;
       }
-      need = found_need;
-      hi = min(hi, lo + ((1u << sh) - 1u));
+      if (n[2] > p.n_keep) {
+        lo = m[2];
+      } else if (n[1] > p.n_keep) {
+        lo = m[1];
+        hi = m[2] - 1;
+        above = n[2];
+      } else if (n[0] > p.n_keep) {
+        lo = m[0];
+        hi = m[1] - 1;
+        above = n[1];
+      } else {
+        hi = m[0] - 1;
+        above = n[0];
+      }
     }
-    int gt_run = 0, eq_run = 0;
+    uint32_t mine = 0;   // keys above the threshold << 16, keys at it
+#pragma unroll
+    for (int c = 0; c < kSelPer; ++c) mine += (key[c] > thr ? 0x10000u : 0u) + (key[c] == thr ? 1u : 0u);
+    uint32_t incl = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += v;
+    }
+    if (lane == 31) part_c[warp] = incl;
+    __syncthreads();
+    const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? part_c[lane] : 0u) + incl - mine;
+    int gt = static_cast<int>(before >> 16), eq = static_cast<int>(before & 0xffffu);
 #pragma unroll
     for (int c = 0; c < kSelPer; ++c) {
-      if (c >= nch) continue;
-      const int j = c * kSelThreads + tid;
-      const unsigned gt = __ballot_sync(0xffffffffu, key[c] > thr), eq = __ballot_sync(0xffffffffu, key[c] == thr);
-      // (the rows of `part` alternate; the row for c = 0 is the one the interval's maximum did not use)
-      if (lane == 0) part[(c + 1) & 1][warp] = (__popc(gt) << 16) | __popc(eq);
-      __syncthreads();
-      const int mine = static_cast<int>(part[(c + 1) & 1][lane]);
-      const int before = __reduce_add_sync(0xffffffffu, lane < warp ? mine : 0), all = __reduce_add_sync(0xffffffffu, mine);
-      const unsigned below = (1u << lane) - 1u;
-      const int gb = gt_run + (before >> 16) + __popc(gt & below), eb = eq_run + (before & 0xffff) + __popc(eq & below);
-      const bool keep = ((gt >> lane) & 1u) || (((eq >> lane) & 1u) && eb < ties);
-      const int pos = gb + min(eb, ties);
-      if (j < p.G) {
-        p.cum[k][j] = pos;
-        if (keep) {
-          p.kept[k][pos] = j;
-          p.lvl_of[static_cast<int64_t>(k) * p.n_keep + pos] = static_cast<int>(lvl[c]);
-          ++lvl[c];
-          key[c] = next[c];
-        }
+      const int j = j0 + c;
+      if (c >= per || j >= p.G) continue;
+      const int pos = gt + min(eq, ties);
+      const bool over = key[c] > thr, at = key[c] == thr;
+      p.cum[k][j] = pos;
+      if (over || (at && eq < ties)) {
+        p.kept[k][pos] = j;
+        p.lvl_of[static_cast<int64_t>(k) * p.n_keep + pos] = static_cast<int>(lvl[c]);
+        ++lvl[c];
+        key[c] = next[c];
       }
-      gt_run += all >> 16;
-      eq_run += all & 0xffff;
+      gt += over;
+      eq += at;
     }
     if (tid == 0) p.cum[k][p.G] = p.n_keep;
-    __syncthreads();   // `part` and the found bin are free for the next order
   }
 }
 
@@ -1456,7 +1451,7 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
       sel.lvl_max = ini.lvl_max;
       sel.lvl_of = reinterpret_cast<int32_t*>(ws + plan.lvl_of);
       sel.G = L.G; sel.K = L.K; sel.n_keep = L.n_keep;
-      launch_overlapped(select_orders_kernel, dim3(1), kSelThreads, 1, s, sel);
+      launch_overlapped(select_orders_kernel, dim3(1), L.G <= 2048 ? 256 : (L.G <= 4096 ? 512 : kSelThreads), 1, s, sel);
       pl.lvl_of = sel.lvl_of;
       pl.lvl_scale = ch.lvl_scale;
       pl.temp = ch.temp;
