@@ -43,13 +43,13 @@ inline pipe_status launch_status() { return cuda_ok(cudaGetLastError()); }
 
 // One launch with programmatic stream serialization: its blocks may stand on the SMs before the launch before it is complete,
 // and the kernel has to wait (grid_wait) before it touches what that launch, or one before it, may still read or write.
-// cluster: CTAs per cluster (1: none).
+// cluster: CTAs per cluster (1: none); overlap = false: an ordinary launch all the same.
 template <typename... P, typename... A>
-inline cudaError_t launch_overlapped(void (*k)(P...), dim3 grid, int block, int cluster, cudaStream_t s, const A&... args) {
+inline cudaError_t launch_overlapped(void (*k)(P...), dim3 grid, int block, int cluster, bool overlap, cudaStream_t s, const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = cluster;
   attr[1].val.clusterDim.y = 1;

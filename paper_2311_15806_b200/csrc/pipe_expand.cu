@@ -1421,7 +1421,7 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
     ini.n_max = dense ? 0 : static_cast<int64_t>(L.K) * L.G;
     const int64_t init_n = ini.n_max > L.G + 1 ? ini.n_max : L.G + 1;
     const int64_t init_grid = ceil_div<int64_t>(init_n, 256);
-    launch_overlapped(chain_init_kernel, dim3(static_cast<int>(init_grid < 64 ? init_grid : 64)), 256, 1, s, ini);
+    launch_overlapped(chain_init_kernel, dim3(static_cast<int>(init_grid < 64 ? init_grid : 64)), 256, 1, true, s, ini);
     ch.W = d_W;
     ch.ldw = ldw;
     ch.direct = dense ? L.K : 1;
@@ -1442,8 +1442,8 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
     const bool long_rows = ch.I_pad > 8192 && ch.I_pad <= 12288 && 65536 / (threads3 * 80) > 65536 / (threads2 * 64);
     const int threads = long_rows ? threads3 : threads2;
 #define PIPE_CHAIN(B)                                                                       \
-  if (long_rows) launch_overlapped(expand_chain_kernel<B, 3, 256, 3>, dim3(L.O), threads, 1, s, ch);   \
-  else launch_overlapped(expand_chain_kernel<B, 2, 512, 2>, dim3(L.O), threads, 1, s, ch);
+  if (long_rows) launch_overlapped(expand_chain_kernel<B, 3, 256, 3>, dim3(L.O), threads, 1, true, s, ch);   \
+  else launch_overlapped(expand_chain_kernel<B, 2, 512, 2>, dim3(L.O), threads, 1, true, s, ch);
     if (L.bits == 8) { PIPE_CHAIN(8) } else if (L.bits == 4) { PIPE_CHAIN(4) } else { PIPE_CHAIN(2) }
 #undef PIPE_CHAIN
     count_launch(2);
@@ -1451,7 +1451,7 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
       sel.lvl_max = ini.lvl_max;
       sel.lvl_of = reinterpret_cast<int32_t*>(ws + plan.lvl_of);
       sel.G = L.G; sel.K = L.K; sel.n_keep = L.n_keep;
-      launch_overlapped(select_orders_kernel, dim3(1), L.G <= 2048 ? 256 : (L.G <= 4096 ? 512 : kSelThreads), 1, s, sel);
+      launch_overlapped(select_orders_kernel, dim3(1), L.G <= 2048 ? 256 : (L.G <= 4096 ? 512 : kSelThreads), 1, true, s, sel);
       pl.lvl_of = sel.lvl_of;
       pl.lvl_scale = ch.lvl_scale;
       pl.temp = ch.temp;
@@ -1463,14 +1463,14 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
       pl.tab = t;
       const int grid = tables + (L.K - 1) * L.n_keep;
       const bool whole = L.lay.canon_row_bytes % 16 == 0;
-      if (L.bits == 8) launch_overlapped(place_orders_kernel<8, 4>, dim3(grid), kTableThreads, 1, s, pl);
-      else if (L.bits == 4 && whole) launch_overlapped(place_orders_kernel<4, 4>, dim3(grid), kTableThreads, 1, s, pl);
-      else if (L.bits == 4) launch_overlapped(place_orders_kernel<4, 2>, dim3(grid), kTableThreads, 1, s, pl);
-      else if (whole) launch_overlapped(place_orders_kernel<2, 4>, dim3(grid), kTableThreads, 1, s, pl);
-      else launch_overlapped(place_orders_kernel<2, 1>, dim3(grid), kTableThreads, 1, s, pl);
+      if (L.bits == 8) launch_overlapped(place_orders_kernel<8, 4>, dim3(grid), kTableThreads, 1, true, s, pl);
+      else if (L.bits == 4 && whole) launch_overlapped(place_orders_kernel<4, 4>, dim3(grid), kTableThreads, 1, true, s, pl);
+      else if (L.bits == 4) launch_overlapped(place_orders_kernel<4, 2>, dim3(grid), kTableThreads, 1, true, s, pl);
+      else if (whole) launch_overlapped(place_orders_kernel<2, 4>, dim3(grid), kTableThreads, 1, true, s, pl);
+      else launch_overlapped(place_orders_kernel<2, 1>, dim3(grid), kTableThreads, 1, true, s, pl);
       count_launch(2);
     } else if (tables) {
-      launch_overlapped(block_table_kernel, dim3(tables), kTableThreads, 1, s, t);
+      launch_overlapped(block_table_kernel, dim3(tables), kTableThreads, 1, true, s, t);
       count_launch(1);
     }
   } else {
@@ -1555,7 +1555,7 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
       max_cap = max_cap > r.cap[m] ? max_cap : r.cap[m];
     }
     if (max_cap > 0) {
-      launch_overlapped(block_record_kernel, dim3(max_cap, L.M + 1), 256, 1, s, r);
+      launch_overlapped(block_record_kernel, dim3(max_cap, L.M + 1), 256, 1, true, s, r);
       count_launch(1);
     }
   }

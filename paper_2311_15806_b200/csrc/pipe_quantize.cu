@@ -4,12 +4,13 @@
 // Tensors of kTinyQuads to kSmallQuads quads: ONE launch of one cluster, which keeps the tensor in registers, exchanges
 // its maxima through distributed shared memory and writes the codes.  Others: (1) a range pass whose clusters each leave
 // their maxima in the workspace (no atomics, so nothing has to be zeroed first), (2) a pass that reads those, divides /
-// rounds half to even / clamps and stores.  Every launch uses programmatic stream serialization: its blocks stand ready when
-// the launch before ends.  The second pass walks the tensor from its END, where the first pass stopped: what is still in the
-// 126 MB L2 is then read from there before it is evicted.  The last launch of either form lets ITS dependents start at once: a
-// forward call that follows sets itself up (and, where it is allowed to, fetches weights) beside it and waits for it before
-// touching the codes.  (The first launch of either form releases only behind its own wait, so whatever stands before the
-// quantization on the stream -- an expansion, say -- is complete when such a forward call starts.)
+// rounds half to even / clamps and stores.  The launches use programmatic stream serialization: their blocks stand ready when
+// the launch before ends (but for the range pass of a large tensor, see quantize_impl).  The second pass walks the tensor from
+// its END, where the first pass stopped: what is still in the 126 MB L2 is then read from there before it is evicted.  The last
+// launch of either form lets ITS dependents start at once: a forward call that follows sets itself up (and, where it is allowed
+// to, fetches weights) beside it and waits for it before touching the codes.  (The first launch of either form releases only
+// behind its own wait, so whatever stands before the quantization on the stream -- an expansion, say -- is complete when such
+// a forward call starts.)
 // Measured against zeroing + range pass + quantize pass as three plain launches (graphs of 20 calls, inputs beyond L2 where
 // large; asymmetric in brackets): 4096 elements 8.3 -> 2.5 us (8.4 -> 2.7), 65 thousand 8.3 -> 3.7 (9.2 -> 4.5), a million
 // 8.4 -> 6.3 (13.2 -> 6.5), 17 million 35.5 -> 28.5 (56.6 -> 29.3), 67 million 115 -> 96 (145 -> 98).  The one-launch form ends
@@ -112,6 +113,7 @@ struct QuantArgs {
   int32_t* zp;
   int act_bits, asym;
   int* status;
+  int overlap;          // the range pass overlaps its neighbours' ends
 };
 
 // The quantizer of a call: scale, and for the forms of Sec. 4.3 zero point and code range.
@@ -208,7 +210,7 @@ __device__ __forceinline__ void load16(const QuantArgs& p, int64_t c, float (&v)
 template <bool EX, bool FLAT>
 __global__ void __launch_bounds__(kRangeThreads) act_range_kernel(const __grid_constant__ QuantArgs p) {
   grid_wait();
-  grid_release();
+  if (p.overlap) grid_release();
   q_cluster_sync();   // every CTA of the cluster runs before another one writes its shared memory
   Range<EX> range;
   const int64_t first = blockIdx.x * static_cast<int64_t>(kRangeThreads) + threadIdx.x;
@@ -328,8 +330,8 @@ __global__ void act_empty_kernel(const float* static_scale, float* sx_out, int32
 }
 
 template <typename... P, typename... A>
-static pipe_status launch_q(void (*k)(P...), int grid, int block, bool cluster, cudaStream_t s, A... args) {
-  if (launch_overlapped(k, dim3(grid, 1, 1), block, cluster ? kClusterCtas : 1, s, args...) != cudaSuccess) return PIPE_ERR_CUDA;
+static pipe_status launch_q(void (*k)(P...), int grid, int block, bool cluster, bool overlap, cudaStream_t s, A... args) {
+  if (launch_overlapped(k, dim3(grid, 1, 1), block, cluster ? kClusterCtas : 1, overlap, s, args...) != cudaSuccess) return PIPE_ERR_CUDA;
   count_launch(1);
   return PIPE_OK;
 }
@@ -355,8 +357,8 @@ static pipe_status quantize_impl(QuantArgs p, cudaStream_t s) {
     const int per_cta = static_cast<int>(ceil_div<int64_t>(p.quads, kClusterCtas));
     const int per = per_cta <= 1024 ? 1 : kSmallPer;
     const int threads = round_up(ceil_div(per_cta, per), 32);
-    if (per == 1) st = launch_q(act_small_kernel<EX, 1>, kClusterCtas, threads, true, s, p);
-    else st = launch_q(act_small_kernel<EX, kSmallPer>, kClusterCtas, threads, true, s, p);
+    if (per == 1) st = launch_q(act_small_kernel<EX, 1>, kClusterCtas, threads, true, true, s, p);
+    else st = launch_q(act_small_kernel<EX, kSmallPer>, kClusterCtas, threads, true, true, s, p);
     return st == PIPE_OK ? launch_status() : st;
   }
   int sms = 148, dev = 0;
@@ -366,12 +368,16 @@ static pipe_status quantize_impl(QuantArgs p, cudaStream_t s) {
   const int clusters = static_cast<int>(want_c < kRangeClusters ? want_c : kRangeClusters);
   const int64_t want = ceil_div<int64_t>(items, kQThreads);
   const int grid = static_cast<int>(want < static_cast<int64_t>(sms) * 8 ? want : static_cast<int64_t>(sms) * 8);
+  // The range pass of a tensor that fills the chip starts only when the launch before has ended, and releases nobody ahead of
+  // its end: brought in while that one still holds some SMs, its clusters crowd onto the first free ones (67 million elements,
+  // back to back: 49 us on an empty chip, 91 that way, 60 with one CTA to an SM).
+  p.overlap = clusters < kRangeClusters;
   // (with a static scale the first pass still serves the non-finite check of the input)
-  st = flat ? launch_q(act_range_kernel<EX, true>, clusters * kClusterCtas, kRangeThreads, true, s, p)
-            : launch_q(act_range_kernel<EX, false>, clusters * kClusterCtas, kRangeThreads, true, s, p);
+  st = flat ? launch_q(act_range_kernel<EX, true>, clusters * kClusterCtas, kRangeThreads, true, p.overlap != 0, s, p)
+            : launch_q(act_range_kernel<EX, false>, clusters * kClusterCtas, kRangeThreads, true, p.overlap != 0, s, p);
   if (st != PIPE_OK) return st;
-  st = flat ? launch_q(act_quantize_kernel<EX, true>, grid, kQThreads, false, s, p, clusters)
-            : launch_q(act_quantize_kernel<EX, false>, grid, kQThreads, false, s, p, clusters);
+  st = flat ? launch_q(act_quantize_kernel<EX, true>, grid, kQThreads, false, true, s, p, clusters)
+            : launch_q(act_quantize_kernel<EX, false>, grid, kQThreads, false, true, s, p, clusters);
   return st == PIPE_OK ? launch_status() : st;
 }
 
