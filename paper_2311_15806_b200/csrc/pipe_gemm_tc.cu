@@ -469,7 +469,8 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
             for (int e = 0; e < 8; ++e)
               if (add_bias) y[e] = __fadd_rn(y[e], bv[e]);
             uint32_t w0, w1;
-            q8_codes8(y, p.f.relu, ostep, orcp, ofast, w0, w1);
+            const f32x2 y2[4] = {pack_f2(y[0], y[1]), pack_f2(y[2], y[3]), pack_f2(y[4], y[5]), pack_f2(y[6], y[7])};
+            q8_codes8(y2, p.f.relu, ostep, orcp, ofast, w0, w1);
             packed[2 * (sub + u)] = w0;
             packed[2 * (sub + u) + 1] = w1;
             continue;

@@ -787,7 +787,17 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
               }
             } else {
 #pragma unroll
-              for (int e = 0; e < 8; ++e) y[e] = __fmaf_rn(__fmul_rn(__int2float_rn(acc[u][ko][e]), unshift), cs[e], y[e]);
+              for (int e = 0; e < 8; e += 2) {
+                const float f0 = __int2float_rn(acc[u][ko][e]), f1 = __int2float_rn(acc[u][ko][e + 1]);
+                if constexpr (Q8) {
+                  // (two channels per instruction, the same roundings: this drain is bound by its issue slots; the fp32 one
+                  // is not)
+                  unpack_f2(fma_f2(mul_f2(pack_f2(f0, f1), both_f2(unshift)), pack_f2(cs[e], cs[e + 1]), pack_f2(y[e], y[e + 1])), y[e], y[e + 1]);
+                } else {
+                  y[e] = __fmaf_rn(__fmul_rn(f0, unshift), cs[e], y[e]);
+                  y[e + 1] = __fmaf_rn(__fmul_rn(f1, unshift), cs[e + 1], y[e + 1]);
+                }
+              }
             }
             if (PARTIALS && own_ok) {
               int rb_ko, st_ko;   // the order's first row in the stacked block and in its own compacted rows
@@ -810,11 +820,14 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
             const uint32_t ba = smem_u32(x.bias_s + (tcount % kRecBufs) * PIPE_BLOCK_CHANNELS) + static_cast<uint32_t>(chunk * 32);
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(bv[0]), "=f"(bv[1]), "=f"(bv[2]), "=f"(bv[3]) : "r"(ba));
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(bv[4]), "=f"(bv[5]), "=f"(bv[6]), "=f"(bv[7]) : "r"(ba + 16));
+            f32x2 y2[4];
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-              if (add_bias) y[e] = __fadd_rn(y[e], bv[e]);
+            for (int e = 0; e < 4; ++e) {
+              y2[e] = pack_f2(y[2 * e], y[2 * e + 1]);
+              if (add_bias) y2[e] = add_f2(y2[e], pack_f2(bv[2 * e], bv[2 * e + 1]));
+            }
             uint32_t w0, w1;
-            q8_codes8(y, p.f.relu, ostep, orcp, ofast, w0, w1);
+            q8_codes8(y2, p.f.relu, ostep, orcp, ofast, w0, w1);
             packed[2 * (sub + u)] = w0;
             packed[2 * (sub + u) + 1] = w1;
             continue;

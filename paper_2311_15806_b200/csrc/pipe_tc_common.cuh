@@ -188,24 +188,38 @@ __device__ __forceinline__ float rcp_approx(float x) {
 //     byte permutations.)
 // Over every binary32 v in +-80 the largest distance measured (r = 1) is 0.47 (SiLU), 0.26 (GeLU), 0.47 (sigmoid) of err.
 // Scaled by r inside the estimate and without the maximum: 768 -> 3072 GeLU 78 -> 76 us, SiLU 74 -> 71, ReLU 64 -> 60.
+// (err: a number whose magnitude is the bound.)  Two at a time on the packed arithmetic, whose halves round like the scalar
+// operations; what has no packed form -- the approximate functions, an absolute value inside a multiplication -- is done twice.
 template <int KIND>
-__device__ __forceinline__ float smooth_estimate(float v, float r, float& err) {
+__device__ __forceinline__ f32x2 smooth_estimate2(f32x2 v, float r, f32x2& err) {
+  float v0, v1;
+  unpack_f2(v, v0, v1);
   if constexpr (KIND == 3) {
-    const float hv = __fmul_rn(v, __fmul_rn(0.5f, r));
-    const float t = rcp_approx(__fmaf_rn(0.23164189f, fabsf(v), 1.f));      // 0.3275911 / sqrt 2
-    const float e = ex2_approx(__fmul_rn(__fmul_rn(v, v), -0.72134752f));   // exp(-v^2 / 2)
-    float h = __fmaf_rn(t, 1.061405429f, -1.453152027f);
-    h = __fmaf_rn(t, h, 1.421413741f);
-    h = __fmaf_rn(t, h, -0.284496736f);
-    h = __fmaf_rn(t, h, 0.254829592f);
-    const float erf_v = __fmaf_rn(-__fmul_rn(t, h), e, 1.f);
-    err = __fmul_rn(fabsf(hv), 2.86102294921875e-06f);                      // |v| r (2^-20 + 2^-21)
-    return __fmaf_rn(fabsf(hv), erf_v, hv);
+    const f32x2 hv = mul_f2(v, both_f2(__fmul_rn(0.5f, r)));
+    const f32x2 t = pack_f2(rcp_approx(__fmaf_rn(0.23164189f, fabsf(v0), 1.f)), rcp_approx(__fmaf_rn(0.23164189f, fabsf(v1), 1.f)));   // 0.3275911 / sqrt 2
+    float a0, a1;
+    unpack_f2(mul_f2(mul_f2(v, v), both_f2(-0.72134752f)), a0, a1);
+    const f32x2 e = pack_f2(ex2_approx(a0), ex2_approx(a1));                // exp(-v^2 / 2)
+    f32x2 h = fma_f2(t, both_f2(-1.061405429f), both_f2(1.453152027f));     // (minus the polynomial)
+    h = fma_f2(t, h, both_f2(-1.421413741f));
+    h = fma_f2(t, h, both_f2(0.284496736f));
+    h = fma_f2(t, h, both_f2(-0.254829592f));
+    const f32x2 erf_v = fma_f2(mul_f2(t, h), e, both_f2(1.f));
+    err = mul_f2(hv, both_f2(2.86102294921875e-06f));                       // |v| r (2^-20 + 2^-21)
+    float h0, h1, f0, f1;
+    unpack_f2(hv, h0, h1);
+    unpack_f2(erf_v, f0, f1);
+    return pack_f2(__fmaf_rn(fabsf(h0), f0, h0), __fmaf_rn(fabsf(h1), f1, h1));
   } else {
-    const float q = rcp_approx(__fadd_rn(1.f, ex2_approx(__fmul_rn(v, -1.44269504f))));
-    const float t = __fmul_rn(KIND == 2 ? __fmul_rn(v, q) : q, r);
-    // |v| 2^-23 + 1.5 * 2^-20, + 2^-21
-    err = __fmul_rn(fabsf(t), __fmaf_rn(fabsf(v), 1.1920928955078125e-07f, 1.9073486328125e-06f));
+    float a0, a1;
+    unpack_f2(mul_f2(v, both_f2(-1.44269504f)), a0, a1);
+    f32x2 q = add_f2(both_f2(1.f), pack_f2(ex2_approx(a0), ex2_approx(a1)));
+    unpack_f2(q, a0, a1);
+    q = pack_f2(rcp_approx(a0), rcp_approx(a1));
+    const f32x2 t = mul_f2(KIND == 2 ? mul_f2(v, q) : q, both_f2(r));
+    // |t| (|v| 2^-23 + 1.5 * 2^-20, + 2^-21)
+    err = mul_f2(t, pack_f2(__fmaf_rn(fabsf(v0), 1.1920928955078125e-07f, 1.9073486328125e-06f),
+                            __fmaf_rn(fabsf(v1), 1.1920928955078125e-07f, 1.9073486328125e-06f)));
     return t;
   }
 }
@@ -216,27 +230,39 @@ static __device__ __noinline__ uint32_t codes4_exact(float a, float b, float c, 
          (quant_lane_exact(apply_activation(c, kind), s) << 16) | (quant_lane_exact(apply_activation(d, kind), s) << 24);
 }
 
+// Two estimates clamped to [lo, 127] and rounded by an addition (see code_magic): the codes stand in the low bytes of u0, u1.
+// RELATIVE: err is a factor, the bound its product with the clamped estimate.
+template <bool RELATIVE>
+__device__ __forceinline__ void code_magic2(f32x2 t, f32x2 err, float lo, float& u0, float& u1, float& edge) {
+  float t0, t1, d0, d1, e0, e1;
+  unpack_f2(t, t0, t1);
+  t = pack_f2(fminf(fmaxf(t0, lo), 127.f), fminf(fmaxf(t1, lo), 127.f));
+  if (RELATIVE) err = mul_f2(t, err);
+  const f32x2 u = add_f2(t, both_f2(12582912.f));
+  unpack_f2(sub_f2(t, sub_f2(u, both_f2(12582912.f))), d0, d1);
+  unpack_f2(err, e0, e1);
+  edge = max3(edge, __fadd_rn(fabsf(d0), fabsf(e0)), __fadd_rn(fabsf(d1), fabsf(e1)));
+  unpack_f2(u, u0, u1);
+}
+
 template <int KIND>
-__device__ __forceinline__ void smooth_codes8(const float (&y)[8], float r, float (&uu)[8], float& edge) {
+__device__ __forceinline__ void smooth_codes8(const f32x2 (&y)[4], float r, float (&uu)[8], float& edge) {
 #pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    float err;
-    const float t = smooth_estimate<KIND>(y[e], r, err);
-    uu[e] = code_magic(fminf(fmaxf(t, -127.f), 127.f), err, edge);
+  for (int e = 0; e < 4; ++e) {
+    f32x2 err;
+    const f32x2 t = smooth_estimate2<KIND>(y[e], r, err);
+    code_magic2<false>(t, err, -127.f, uu[2 * e], uu[2 * e + 1], edge);
   }
 }
 
 // kind: the activation; s: the output step; r = rn(1 / s), usable when `fast`.
-__device__ __forceinline__ void q8_codes8(const float (&y)[8], int kind, float s, float r, bool fast, uint32_t& w0, uint32_t& w1) {
+__device__ __forceinline__ void q8_codes8(const f32x2 (&y)[4], int kind, float s, float r, bool fast, uint32_t& w0, uint32_t& w1) {
   float uu[8];
   float edge = fast ? 0.f : 1.f;
   if (kind < 2) {
     const float lo = kind == 1 ? 0.f : -127.f;   // ReLU: max(v, 0) r = max(v r, 0)
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const float t = fminf(fmaxf(__fmul_rn(y[e], r), lo), 127.f);
-      uu[e] = code_magic(t, __fmul_rn(fabsf(t), 4.76837158203125e-07f), edge);
-    }
+    for (int e = 0; e < 4; ++e) code_magic2<true>(mul_f2(y[e], both_f2(r)), both_f2(4.76837158203125e-07f), lo, uu[2 * e], uu[2 * e + 1], edge);
   } else if (kind == 2) {
     smooth_codes8<2>(y, r, uu, edge);
   } else if (kind == 3) {
@@ -247,8 +273,11 @@ __device__ __forceinline__ void q8_codes8(const float (&y)[8], int kind, float s
   w0 = pack4_low_bytes(uu[0], uu[1], uu[2], uu[3]);
   w1 = pack4_low_bytes(uu[4], uu[5], uu[6], uu[7]);
   if (edge >= 0.5f) {   // an estimate too close to a rounding boundary to decide (or the step has no usable reciprocal)
-    w0 = codes4_exact(y[0], y[1], y[2], y[3], kind, s);
-    w1 = codes4_exact(y[4], y[5], y[6], y[7], kind, s);
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) unpack_f2(y[e], v[2 * e], v[2 * e + 1]);
+    w0 = codes4_exact(v[0], v[1], v[2], v[3], kind, s);
+    w1 = codes4_exact(v[4], v[5], v[6], v[7], kind, s);
   }
 }
 
