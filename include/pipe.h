@@ -18,8 +18,8 @@
  *   - there is no CPU fallback: without a CUDA device every compute call returns
  *     PIPE_ERR_CUDA.
  *   - the forward kernels are launched with programmatic stream serialization: their prologue
- *     may overlap the tail of the preceding launch on `stream`, and the weight-streaming kernel
- *     (at most 16 tokens) starts copying the blob's packed codes during that overlap.  The
+ *     may overlap the tail of the preceding launch on `stream`, and they start copying the
+ *     blob's packed codes during that overlap.  The
  *     library orders this correctly against its own calls (a forward call that directly follows
  *     pipe_expand_weights* on the same stream waits for it in full).  A caller that writes
  *     d_blob by other means must let that work complete -- an event, a synchronize, or any other

@@ -72,6 +72,7 @@ struct Params {
   int pk;                 // packed bytes of one row of one reduction block (128*b/8)
   int shift;              // 8 - b
   int direct;             // the weights come from the layer's int8 copy in the operand layout (bits reads 8, shift 0)
+  int early;              // the expanded layer is settled: see the kernel's first lines
   uint32_t split_mask;    // summed ensemble on one shared input, run as ONE cluster of all orders: bit k is set where
                           // order k (k > 0) opens the next predictor, whose chain the epilogue starts from zero
   int conv_pw, conv_pp, conv_np, conv_chunks;   // patches per image row / per image / in total; 128-channel chunks per tap
@@ -424,9 +425,10 @@ __device__ __forceinline__ void unpack_role(const Params& p, const Rings& g, int
   }
 }
 
+// (from L2: another SM has written it while this block may already have been standing here)
 __device__ __forceinline__ float4 load_row(const float* src, bool vec) {
-  if (vec) return *reinterpret_cast<const float4*>(src);
-  return make_float4(src[0], src[1], src[2], src[3]);
+  if (vec) return __ldcg(reinterpret_cast<const float4*>(src));
+  return make_float4(__ldcg(src), __ldcg(src + 1), __ldcg(src + 2), __ldcg(src + 3));
 }
 
 struct EpiCtx {
@@ -965,24 +967,18 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
   g.ntot = ntot_s;
 
   // A launch that follows in the stream may be brought onto the SMs as they become free (its CTAs then exist when this
-  // launch's last pair ends).  This kernel waits here, before its first access to global memory, until the launch
-  // before it is complete, and lets its own dependents start only after that: a dependent that reads weights ahead
-  // of ITS wait (the weight-streaming kernel) then never runs beside an expansion queued before this launch.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (threadIdx.x >= 32 && threadIdx.x < 32 + 2 * PIPE_MAX_ORDERS) {
-    // (inputs of this launch: written before it started)
-    const int i = threadIdx.x - 32, m = i % PIPE_MAX_ORDERS;
-    float v = 0.f;
-    if (m < p.f.num_branches) {
-      if (i < PIPE_MAX_ORDERS) v = __ldg(p.f.branch[m].sx);
-      else if (Q8) v = __ldg(p.f.branch[m].out_scale);
-    }
-    sx_s[i] = v;
-    if constexpr (ZP) {
-      if (i < PIPE_MAX_ORDERS) zp_s[i] = (m < p.f.num_branches && p.f.branch[m].zp) ? __ldg(p.f.branch[m].zp) : 0;
-    }
-  }
+  // launch's last pair ends).  Until the launch before it is complete such a pair touches nothing that launch may have
+  // written.  With p.early the host knows that the expanded layer is not being written (its last call on this stream was no
+  // expansion): what belongs to the layer -- tile counts, the first ring of weights -- is then read ahead of the wait, and
+  // what waits is the activation producer before its first copy and the epilogue before the steps, the bias and its outputs.
+  // Otherwise the pair waits here.  Its own dependents start after the wait only: a dependent that reads weights ahead of ITS
+  // wait then never runs beside an expansion queued before this launch.
+  // ACC: a later predictor of a summed ensemble.  The launch before it is the predictor before, whose blocks released it behind
+  // their wait: all that this launch reads but the sum itself is complete.  So its tiles start on the pairs that the launch
+  // before leaves idle in its last round, and only the epilogue waits.
+  const bool early = ACC || p.early;
+  if (!early) grid_wait();
+  if (ACC || !early) grid_release();
   if constexpr (ZP) {
     // the row of ones behind the 127 token rows of every activation tile of the ring (sixteen equal bytes per piece,
     // whatever the swizzle does with the pieces); the copies never write it
@@ -1046,6 +1042,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
     // completion of both CTAs' copies is counted on the FIRST CTA's stage barrier, whose expected byte count
     // (both tiles) that CTA's lane 0 posts; a copy of the second CTA may land before that, which only lets the
     // transaction count run ahead of the expectation while the barrier's one arrival is still pending.
+    if (!ACC && p.early) {
+      grid_wait();
+      grid_release();
+    }
     const int per_block = p.f.conv_on ? 2 : 1;        // copies per reduction block
     const int sub = lane / per_block, half = lane % per_block;
     if (lane < kSub * per_block) {
@@ -1163,6 +1163,21 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
     else unpack_role<2>(p, g, warp - 2, lane, smem_u32(pk_bars));
   } else {
     // ------------------------------------------------------------------ epilogue warps
+    // (inputs of this launch, and outputs that the launch before may still be reading or adding to: complete behind this)
+    if (early) grid_wait();
+    if (threadIdx.x >= kThreads - 2 * PIPE_MAX_ORDERS) {
+      const int i = threadIdx.x - (kThreads - 2 * PIPE_MAX_ORDERS), m = i % PIPE_MAX_ORDERS;
+      float v = 0.f;
+      if (m < p.f.num_branches) {
+        if (i < PIPE_MAX_ORDERS) v = __ldcg(p.f.branch[m].sx);
+        else if (Q8) v = __ldcg(p.f.branch[m].out_scale);
+      }
+      sx_s[i] = v;
+      if constexpr (ZP) {
+        if (i < PIPE_MAX_ORDERS) zp_s[i] = (m < p.f.num_branches && p.f.branch[m].zp) ? __ldcg(p.f.branch[m].zp) : 0;
+      }
+    }
+    asm volatile("bar.sync 1, %0;" ::"r"(32 * kEpiWarps) : "memory");
     EpiCtx e;
     e.tmem_base = tmem_base;
     e.tfull0 = g.tfull0;
@@ -1316,6 +1331,7 @@ static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_
   p.f = a;
   p.direct = direct ? 1 : 0;
   p.split_mask = split_mask;
+  p.early = a.blob_settled;
   const int row_bytes = direct ? round_up(a.I, kKStep) : a.kernel_row_bytes;   // bytes of a row over all reduction blocks
   if (direct) p.f.bits = 8;   // the kernel then treats the layer as one of int8 codes
   p.nkmax = max_cluster;
