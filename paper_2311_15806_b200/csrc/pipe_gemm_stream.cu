@@ -1,5 +1,6 @@
-// Small-token kernel of the expanded layer (Appendix B, Eq. 9; Sec. 3.2 for the branches): up to 16 tokens, and small
-// layers on more tokens in slices of 16 (gridDim.y; see the rule in launch_stream).
+// Weight-streaming kernel of the expanded layer (Appendix B, Eq. 9; Sec. 3.2 for the branches): small layers on more than 16
+// tokens in slices of 16 (gridDim.y; see the rule in launch_stream), and the calls of up to 16 tokens that the small-token kernel
+// (pipe_gemm_direct.cu) declines.
 //
 // With a handful of tokens the layer is bound by streaming the packed weight codes from HBM once,
 // so the kernel is built around the byte stream.  A "slab" is 8 consecutive output channels of

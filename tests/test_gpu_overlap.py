@@ -1,5 +1,6 @@
 """Launches that start ahead of the one before them: chains without synchronization whose inputs and outputs are reused from
-round to round, against the same calls one at a time.  And expansions at the edges of the packing and of the selection."""
+round to round, against the same calls one at a time.  Expansions at the edges of the packing and of the selection, and the
+small-token kernel where its split changes."""
 import numpy as np
 import pytest
 import torch
@@ -75,3 +76,45 @@ def test_expansion_of_codes_at_the_ends_of_their_range(oracle, bits, K, O, I, g)
     e = oracle.expand_ex(W, bits, K, g, n_keep) if bits in (3, 6) else oracle.expand(W, bits, K, g, n_keep)
     layer = H.gpu_expand(H.desc_of(O, I, bits, K, g, n_keep, int8_copy=g == 8), W)
     H.assert_expansion_matches(layer, e, oracle)
+
+
+# The small-token kernel.  T around the token tiles of eight (seven and fifteen beside a zero point) and the epilogue's four;
+# reduction axes of one stage, of fewer stages than a CTA has warps and of more than a ring holds, odd block counts (half a stage
+# with 2-bit codes), rows that are no whole 16 bytes; from one pair of row groups per CTA to many sets of three; orders that
+# keep next to nothing
+@pytest.mark.parametrize("T", [1, 4, 7, 8, 9, 15, 16])
+@pytest.mark.parametrize("O,I,bits,K,g,n_keep,M", [(8, 16, 4, 2, 8, 1, 1), (264, 1160, 2, 8, 8, 5, 2), (1184, 128, 8, 3, 8, 77, 3), (136, 5000, 4, 4, 8, 1, 2),
+                                                   (2368, 2432, 2, 3, 16, 20, 1), (24832, 144, 4, 8, 8, 2900, 1), (4096, 712, 8, 2, 32, 100, 2), (7104, 9000, 4, 4, 8, 400, 2)])
+def test_small_token_kernel(O, I, bits, K, g, n_keep, M, T):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(O + T)
+    layer = B.expand(B.make_desc(O, I, bits, K, g, n_keep, M), torch.empty(O, I, device="cuda").normal_(generator=gen) * 0.02)
+    bias = torch.empty(O, device="cuda").normal_(generator=gen)
+    ld = (I + 15) // 16 * 16
+    xq = [torch.randint(-127, 128, (T, ld), dtype=torch.int8, device="cuda", generator=gen)[:, :I] for _ in range(M)]
+    sx = [torch.tensor([0.01 * (1 + m)], device="cuda") for m in range(M)]
+    zp = [torch.tensor([5 - 40 * m], dtype=torch.int32, device="cuda") for m in range(M)]
+    step = [torch.tensor([0.3], device="cuda")] * M
+
+    def run(choice):
+        B.pipe_diag_select_kernel(choice)
+        try:
+            ys = [[torch.full((T, O), float("nan"), device="cuda") for _ in range(M)] for _ in range(2)]
+            yq = [torch.full((T, O), 99, dtype=torch.int8, device="cuda") for _ in range(M)]
+            sums = [torch.full((T, O), float("nan"), device="cuda") for _ in range(4)]
+            parts = [torch.zeros((T, layer.layout.total_rows), dtype=torch.int32, device="cuda") for _ in range(2)]
+            B.pipe_ensemble_forward(layer.desc, layer.blob, xq, sx, ys[0], bias, False, parts[0])
+            B.pipe_ensemble_forward_zp(layer.desc, layer.blob, xq, sx, zp, ys[1], bias, False, parts[1])
+            B.pipe_ensemble_forward(layer.desc, layer.blob, xq, sx, sums[:1], bias, True)
+            B.pipe_ensemble_forward(layer.desc, layer.blob, xq[:1] * M, sx[:1] * M, sums[1:2], bias, True)
+            B.pipe_ensemble_forward_zp(layer.desc, layer.blob, xq, sx, zp, sums[2:3], bias, True)
+            B.pipe_expanded_linear(layer.desc, layer.blob, xq[0], sx[0], sums[3], None)
+            B.pipe_ensemble_forward_q8(layer.desc, layer.blob, xq, sx, step, yq, bias, B.ACT_RELU)
+        finally:
+            B.pipe_diag_select_kernel(B.KERNEL_AUTO)
+        torch.cuda.synchronize()
+        return [y.view(torch.int32) for y in ys[0] + ys[1] + sums] + yq + parts
+
+    for a, b in zip(run(B.KERNEL_REFERENCE), run(B.KERNEL_AUTO)):
+        assert torch.equal(a, b)
+    assert B.pipe_poll_status() == B.PIPE_OK
