@@ -612,14 +612,13 @@ pipe_status forward_direct(const ForwardArgs& a, cudaStream_t stream) {
   if (a.T == 0) return PIPE_OK;
   const bool sum_mode = a.num_branches > 1 && a.branch[1].accumulate;
   if (!sum_mode) return launch_direct(a, stream, false);
-  // one launch for predictors that share their input, or two predictors of at most two orders each on inputs of their own
+  // one launch for predictors that share their input, or two predictors of at most two orders each on inputs of their own; declined,
+  // it is for the weight-streaming kernel, which also takes them together
   bool shared = true;
   for (int m = 1; m < a.num_branches; ++m)
     shared = shared && a.branch[m].xq == a.branch[0].xq && a.branch[m].sx == a.branch[0].sx && a.branch[m].zp == a.branch[0].zp;
-  if (shared || (a.num_branches == 2 && a.branch[0].k_end - a.branch[0].k_begin <= 2 && a.branch[1].k_end - a.branch[1].k_begin <= 2)) {
-    const pipe_status st = launch_direct(a, stream, true);
-    if (st != PIPE_ERR_UNSUPPORTED) return st;
-  }
+  if (shared || (a.num_branches == 2 && a.branch[0].k_end - a.branch[0].k_begin <= 2 && a.branch[1].k_end - a.branch[1].k_begin <= 2))
+    return launch_direct(a, stream, true);
   return launch_each_predictor(a, [&](const ForwardArgs& one, bool queue) { return launch_direct(one, stream, false, queue); });
 }
 
