@@ -1020,9 +1020,7 @@ __global__ void __launch_bounds__(MAXT, MINB) expand_chain_kernel(const __grid_c
 // (the maximum at the group's present level; ties to the lower index, as everywhere; non-negative floats order like
 // their bits).  The n_keep-th largest score is found by counting the keys at and above three probes that quarter the interval
 // which holds it, until a probe has exactly n_keep (the usual end, after about log4 of the number of groups) or one value is
-// left.  A step of that search is one barrier, and so is the compaction, for which a thread holds neighbouring groups; the
-// block has only as many warps as leaves a thread up to eight groups, because the barriers are what an order's time goes
-// into.
+// left.  A step of that search is one barrier, and so is the compaction, for which a thread holds neighbouring groups.
 constexpr int kSelThreads = 1024;
 constexpr int kSelPer = 8;
 constexpr int kSelMaxGroups = kSelThreads * kSelPer;
@@ -1034,6 +1032,7 @@ struct SelectArgs {
   int G, K, n_keep;
 };
 
+template <int PER>   // groups per thread: few for few groups, an order's time is its instructions one after the other
 __global__ void __launch_bounds__(kSelThreads) select_orders_kernel(const __grid_constant__ SelectArgs p) {
   __shared__ uint32_t part_lo[32], part_hi[32], part_n[2][2][32], part_c[32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
@@ -1041,12 +1040,12 @@ __global__ void __launch_bounds__(kSelThreads) select_orders_kernel(const __grid
   grid_wait();
   grid_release();
   // key: score at the group's present level, plus one (0: no group); next: at the level behind it, asked for ahead of use
-  uint32_t lvl[kSelPer], key[kSelPer], next[kSelPer];
+  uint32_t lvl[PER], key[PER], next[PER];
   auto score = [&](int c, uint32_t l) -> uint32_t {
     return c < per && j0 + c < p.G && l < static_cast<uint32_t>(p.K) ? __ldg(p.lvl_max + static_cast<int64_t>(l) * p.G + j0 + c) + 1u : 0u;
   };
 #pragma unroll
-  for (int c = 0; c < kSelPer; ++c) {
+  for (int c = 0; c < PER; ++c) {
     lvl[c] = 1;
     key[c] = score(c, 1);
   }
@@ -1054,7 +1053,7 @@ __global__ void __launch_bounds__(kSelThreads) select_orders_kernel(const __grid
   for (int k = 1; k < p.K; ++k) {
     uint32_t lo = 0xffffffffu, hi = 0;
 #pragma unroll
-    for (int c = 0; c < kSelPer; ++c) {
+    for (int c = 0; c < PER; ++c) {
       next[c] = score(c, lvl[c] + 1);
       if (key[c] != 0) {
         lo = min(lo, key[c]);
@@ -1084,7 +1083,7 @@ __global__ void __launch_bounds__(kSelThreads) select_orders_kernel(const __grid
       const uint32_t m[3] = {lo + q + 1, lo + 2 * q + 1, lo + 3 * q + 1};   // in (lo, hi]
       uint32_t n01 = 0, n2 = 0;
 #pragma unroll
-      for (int c = 0; c < kSelPer; ++c) {
+      for (int c = 0; c < PER; ++c) {
         n01 += (key[c] >= m[0] ? 1u : 0u) + (key[c] >= m[1] ? 0x10000u : 0u);
         n2 += key[c] >= m[2] ? 1u : 0u;
       }
@@ -1120,7 +1119,7 @@ __global__ void __launch_bounds__(kSelThreads) select_orders_kernel(const __grid
     }
     uint32_t mine = 0;   // keys above the threshold << 16, keys at it
 #pragma unroll
-    for (int c = 0; c < kSelPer; ++c) mine += (key[c] > thr ? 0x10000u : 0u) + (key[c] == thr ? 1u : 0u);
+    for (int c = 0; c < PER; ++c) mine += (key[c] > thr ? 0x10000u : 0u) + (key[c] == thr ? 1u : 0u);
     uint32_t incl = mine;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -1132,7 +1131,7 @@ __global__ void __launch_bounds__(kSelThreads) select_orders_kernel(const __grid
     const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? part_c[lane] : 0u) + incl - mine;
     int gt = static_cast<int>(before >> 16), eq = static_cast<int>(before & 0xffffu);
 #pragma unroll
-    for (int c = 0; c < kSelPer; ++c) {
+    for (int c = 0; c < PER; ++c) {
       const int j = j0 + c;
       if (c >= per || j >= p.G) continue;
       const int pos = gt + min(eq, ties);
@@ -1451,7 +1450,13 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
       sel.lvl_max = ini.lvl_max;
       sel.lvl_of = reinterpret_cast<int32_t*>(ws + plan.lvl_of);
       sel.G = L.G; sel.K = L.K; sel.n_keep = L.n_keep;
-      launch_overlapped(select_orders_kernel, dim3(1), L.G <= 2048 ? 256 : (L.G <= 4096 ? 512 : kSelThreads), 1, true, s, sel);
+      // (two groups per thread up to 1024 of them, four up to 2048, eight beyond: seven orders of 512 groups 18 us, 24 with eight
+      // groups per thread always)
+      const int sel_per = L.G <= 1024 ? 2 : (L.G <= 2048 ? 4 : kSelPer);
+      const int sel_threads = round_up(ceil_div(L.G, sel_per), 32);
+      if (sel_per == 2) launch_overlapped(select_orders_kernel<2>, dim3(1), sel_threads, 1, true, s, sel);
+      else if (sel_per == 4) launch_overlapped(select_orders_kernel<4>, dim3(1), sel_threads, 1, true, s, sel);
+      else launch_overlapped(select_orders_kernel<kSelPer>, dim3(1), sel_threads, 1, true, s, sel);
       pl.lvl_of = sel.lvl_of;
       pl.lvl_scale = ch.lvl_scale;
       pl.temp = ch.temp;
