@@ -169,8 +169,7 @@ __device__ __forceinline__ int rows_before(const int32_t* cum, int c, int O, int
 // FULL != 0: a consumer warp has FULL slab slots per pass and (nearly) every one of them holds a slab (the host knows:
 // one pass, FULL = ceil(slabs of a CTA / warps of a group)): the loop over a warp's slabs then runs without its per-slab
 // branches -- an absent chunk takes part with zero weights -- so that the slabs' load-and-MMA chains are one block the
-// compiler may interleave (cfg4a T = 1, five slabs per warp: 17.6 -> 16.8 us; cfg4b T = 1, two: 21.2 -> 19.4 us; with the
-// slots of the general kernel, five, a launch with two slabs per warp would do 2.5 times its work that way).
+// compiler may interleave (11008 -> 4096, T = 16, two slabs per warp: 23.3 -> 20.8 us).
 // ZP: asymmetric activations, sum_i (c - z) q = sum_i c q - z sum_i q.  The last token column of the MMAs (7, or 15 with
 // two token tiles) is fed ones instead of a token, so its accumulators are the row sums of the codes; the epilogue reads
 // them from the neighbouring lane that holds that column.
@@ -666,7 +665,7 @@ struct KernelInfo {
   const void* fn = nullptr;
   int fixed = 0, dyn_set = 0;
 };
-constexpr int kMaxKernels = 128;   // instantiations of the kernel (90)
+constexpr int kMaxKernels = 128;   // instantiations of the kernel (72)
 struct DeviceCache {
   std::mutex mu;
   bool ready = false;
@@ -759,28 +758,22 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
     if (a.bits == 8) { PIPE_ST_PICK(8, 1, false) } else if (a.bits == 4) { PIPE_ST_PICK(4, 1, false) } else { PIPE_ST_PICK(2, 1, false) }
   }
 #undef PIPE_ST_PICK
-  // the same kernel without per-slab branches, by slab slots per warp (one order pair; up to 8 tokens: 2 to 5 slots,
-  // 9 to 16 tokens: 2 or 3 -- more would spill)
+  // the same kernel without per-slab branches, by slab slots per warp (one order pair, 2 or 3 slots -- more would spill; two
+  // inputs, 1 or 2).  Two token tiles: the slices; up to 8 tokens the small-token kernel leaves this one next to nothing.
   auto full_kernel = [&](int slots) -> void (*)(const Params) {
-    if (distinct) {   // one or two slots
+    if (nt == 1) return nullptr;
+    if (distinct) {
 #define PIPE_ST_DIST(B)                                                                                                   \
-  if (slots == 1) return nt == 1 ? stream_forward_kernel<B, 1, 2, 2, 1, false> : stream_forward_kernel<B, 2, 2, 2, 1, false>; \
-  if (slots == 2) return nt == 1 ? stream_forward_kernel<B, 1, 2, 2, 2, false> : stream_forward_kernel<B, 2, 2, 2, 2, false>;
+  if (slots == 1) return stream_forward_kernel<B, 2, 2, 2, 1, false>;                                                     \
+  if (slots == 2) return stream_forward_kernel<B, 2, 2, 2, 2, false>;
       if (a.bits == 8) { PIPE_ST_DIST(8) } else if (a.bits == 4) { PIPE_ST_DIST(4) } else { PIPE_ST_DIST(2) }
 #undef PIPE_ST_DIST
       return nullptr;
     }
     if (split_mask != 0 || np != 1 || zp) return nullptr;
-#define PIPE_ST_FULL(B)                                                                                       \
-  if (nt == 1) {                                                                                              \
-    if (slots == 2) return stream_forward_kernel<B, 1, 1, 0, 2, false>;                                          \
-    if (slots == 3) return stream_forward_kernel<B, 1, 1, 0, 3, false>;                                          \
-    if (slots == 4) return stream_forward_kernel<B, 1, 1, 0, 4, false>;                                          \
-    if (slots == 5) return stream_forward_kernel<B, 1, 1, 0, 5, false>;                                          \
-  } else {                                                                                                    \
-    if (slots == 2) return stream_forward_kernel<B, 2, 1, 0, 2, false>;                                          \
-    if (slots == 3) return stream_forward_kernel<B, 2, 1, 0, 3, false>;                                          \
-  }
+#define PIPE_ST_FULL(B)                                              \
+  if (slots == 2) return stream_forward_kernel<B, 2, 1, 0, 2, false>; \
+  if (slots == 3) return stream_forward_kernel<B, 2, 1, 0, 3, false>;
     if (a.bits == 8) { PIPE_ST_FULL(8) } else if (a.bits == 4) { PIPE_ST_FULL(4) } else { PIPE_ST_FULL(2) }
 #undef PIPE_ST_FULL
     return nullptr;
