@@ -31,8 +31,8 @@ constexpr int kPlanSMs = 148;   // SMs of the B200 the decode plan is laid out f
 int* device_status_word();
 void count_launch(int n = 1);
 int kernel_choice();
-// Streams whose last library call was an expansion (which writes the blob a forward call on the same stream may be about
-// to read): an expansion marks its stream, every other call on a stream takes the mark away and learns whether it was there.
+// Streams (of whichever device is current) whose last library call was an expansion (which writes the blob a forward call on the
+// same stream may be about to read): an expansion marks its stream, every other call that has queued a kernel takes the mark away.
 void mark_expansion(cudaStream_t stream);
 bool take_expansion_mark(cudaStream_t stream);
 bool expansion_marked(cudaStream_t stream);   // the same question without clearing the mark

@@ -2,10 +2,10 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
-#include <mutex>
 
 #include "pipe_common.cuh"
 #include "pipe_diag.h"
+#include "pipe_marks.h"
 
 namespace pipe {
 
@@ -17,40 +17,16 @@ static std::atomic<int> g_kernel_choice{0};
 void count_launch(int n) { g_launches.fetch_add(static_cast<uint64_t>(n), std::memory_order_relaxed); }
 int kernel_choice() { return g_kernel_choice.load(); }
 
-namespace {
-std::mutex g_mark_mutex;
-constexpr int kMaxMarked = 64;
-cudaStream_t g_marked[kMaxMarked];
-int g_num_marked = 0;
-bool g_mark_overflow = false;   // more streams than the table holds: every call is then treated as following an expansion
-}  // namespace
+static ExpansionMarks g_marks;
 
-void mark_expansion(cudaStream_t stream) {
-  std::lock_guard<std::mutex> lock(g_mark_mutex);
-  for (int i = 0; i < g_num_marked; ++i)
-    if (g_marked[i] == stream) return;
-  if (g_num_marked < kMaxMarked) g_marked[g_num_marked++] = stream;
-  else g_mark_overflow = true;
+static StreamKey key_of(cudaStream_t stream) {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+  return stream_key(dev, static_cast<uint64_t>(reinterpret_cast<uintptr_t>(stream)));
 }
-
-bool take_expansion_mark(cudaStream_t stream) {
-  std::lock_guard<std::mutex> lock(g_mark_mutex);
-  if (g_mark_overflow) return true;
-  for (int i = 0; i < g_num_marked; ++i)
-    if (g_marked[i] == stream) {
-      g_marked[i] = g_marked[--g_num_marked];
-      return true;
-    }
-  return false;
-}
-
-bool expansion_marked(cudaStream_t stream) {
-  std::lock_guard<std::mutex> lock(g_mark_mutex);
-  if (g_mark_overflow) return true;
-  for (int i = 0; i < g_num_marked; ++i)
-    if (g_marked[i] == stream) return true;
-  return false;
-}
+void mark_expansion(cudaStream_t stream) { g_marks.mark(key_of(stream)); }
+bool take_expansion_mark(cudaStream_t stream) { return !g_marks.none() && g_marks.take(key_of(stream)); }
+bool expansion_marked(cudaStream_t stream) { return !g_marks.none() && g_marks.marked(key_of(stream)); }
 
 int* device_status_word() {
   // The symbol is per device; its address is looked up once for whichever device is current and kept.

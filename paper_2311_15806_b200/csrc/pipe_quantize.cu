@@ -498,8 +498,9 @@ extern "C" pipe_status pipe_lower_conv_input(const pipe_conv_geom* geom, const i
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t want = ceil_div<int64_t>(a.total, 256);
   const int grid = static_cast<int>(want < static_cast<int64_t>(sms) * 16 ? want : static_cast<int64_t>(sms) * 16);
-  take_expansion_mark(static_cast<cudaStream_t>(stream));
   lower_conv_input_kernel<<<grid > 0 ? grid : 1, 256, 0, static_cast<cudaStream_t>(stream)>>>(a);
   count_launch(1);
-  return launch_status();
+  const pipe_status st = launch_status();
+  if (st == PIPE_OK) take_expansion_mark(static_cast<cudaStream_t>(stream));
+  return st;
 }
