@@ -62,7 +62,9 @@ inline cudaError_t launch_overlapped(void (*k)(P...), dim3 grid, int block, int 
   return cudaLaunchKernelEx(&cfg, k, args...);
 }
 // Behind grid_wait everything queued before this launch is complete and visible.  A kernel that releases its dependents only
-// after its own wait keeps the order of the stream transitive.
+// after its own wait keeps the order of the stream transitive.  What the launch before may have written while this kernel was
+// already standing on the SMs is read by ordinary or L2 loads (__ldcg), never by __ldg: that one is for data which does not change
+// during the kernel's whole life, and the compiler may move it above the wait.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -266,8 +268,9 @@ struct ForwardArgs {
   int cHo, cWo, csh, csw;   // output height / width and the strides
   // fused inner-layer epilogue (q8_out != 0): yq = clamp(rne(act(y) / out_scale)) as int8, row pitch ldyq; y is not written
   int decode_split;   // CTAs that share a decode unit's reduction axis (from the layout; 0 = no decode tables)
-  int blob_settled;   // the library's last call on this stream was no expansion: a kernel launched with programmatic stream
-                      // serialization may read the expanded layer before it waits for the launch before it
+  int blob_settled;   // the library's last call on this stream was no expansion, so the expanded layer is complete when a kernel
+                      // launched with programmatic stream serialization starts, and may be read before that kernel waits for the
+                      // launch before it; otherwise the launch has to be an ordinary one
   int q8_out, relu;   // relu: the activation kind (see apply_activation; the name is from the first version)
   // the channel-block table and block records of the cluster of ALL orders, for a summed ensemble whose predictors
   // share one input (nullptr: the layer has none, or the call is no such ensemble)

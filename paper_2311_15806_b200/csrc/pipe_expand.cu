@@ -1043,7 +1043,7 @@ __global__ void __launch_bounds__(kSelThreads) select_orders_kernel(const __grid
   // key: score at the group's present level, plus one (0: no group); next: at the level behind it, asked for ahead of use
   uint32_t lvl[PER], key[PER], next[PER];
   auto score = [&](int c, uint32_t l) -> uint32_t {
-    return c < per && j0 + c < p.G && l < static_cast<uint32_t>(p.K) ? __ldg(p.lvl_max + static_cast<int64_t>(l) * p.G + j0 + c) + 1u : 0u;
+    return c < per && j0 + c < p.G && l < static_cast<uint32_t>(p.K) ? __ldcg(p.lvl_max + static_cast<int64_t>(l) * p.G + j0 + c) + 1u : 0u;
   };
 #pragma unroll
   for (int c = 0; c < PER; ++c) {

@@ -43,7 +43,6 @@ struct Params {
   int own_max, pairs_max;           // most slabs (of 8 channels) / pairs of row groups any CTA can have
   uint32_t split_mask;              // SUMMED: bit k marks the order (k > 0) that opens the next predictor
   int8_t input[PIPE_MAX_ORDERS];    // SUMMED: the predictor whose input an order meets
-  int prefetch;                     // the expanded layer is settled: weights may be read ahead of the dependency wait
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
@@ -266,12 +265,10 @@ __global__ void __launch_bounds__(kThreads, 2) direct_forward_kernel(const __gri
   float* scale = bias_s + p.own_max * 8;                               // [own_max][nkmax][8]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-  // With p.prefetch (the host knows that the expanded layer is not being written: its last call on this stream was no
-  // expansion) everything that belongs to the layer -- row lists, scales, the first weights -- is read ahead of the wait for the
-  // launch before, and this launch's dependents start at once: the layer before was complete, or past this same point, when
-  // this CTA started, so no expansion queued earlier is still running beside them.  Without it the CTA waits before its first
-  // access to global memory and releases its dependents only then.
-  if (!p.prefetch) grid_wait();
+  // Everything that belongs to the layer -- row lists, scales, the first weights -- is read ahead of the wait for the launch before:
+  // the layer is complete when a CTA starts (a launch directly behind an expansion is an ordinary one, see launch_direct).  This
+  // launch's dependents start at once: the launch before was complete, or past this same point, when this CTA started, so no
+  // expansion queued earlier is still running beside them.
   grid_release();
   int b = 0;
   if (!SUMMED)
@@ -349,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 2) direct_forward_kernel(const __gri
   // first activation copies
   bool waited = false, made = false;
   auto wait_once = [&]() {
-    if (!waited && p.prefetch) grid_wait();
+    if (!waited) grid_wait();
     waited = true;
   };
   auto tables_once = [&]() {
@@ -501,7 +498,6 @@ static pipe_status launch_direct(const ForwardArgs& a, cudaStream_t stream, bool
   if (!ds.ok) return PIPE_ERR_CUDA;
   Params p;
   p.f = a;
-  p.prefetch = a.blob_settled ? 1 : 0;
   p.split_mask = 0;
   int units = a.num_branches, inputs = 1;
   if (summed) {
@@ -596,7 +592,7 @@ static pipe_status launch_direct(const ForwardArgs& a, cudaStream_t stream, bool
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = a.blob_settled ? 1 : 0;   // (not where the blob may be under construction)
   cfg.gridDim = dim3(p.cta0[units], 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = static_cast<size_t>(tables + depth * kWarps * p.stage_bytes);

@@ -55,7 +55,6 @@ struct Params {
   int nkmax;              // most orders any branch has
   int chunk_ints;         // words of one slab's entry in the chunk table: chunk_entry_ints
   int own_max;            // most slabs any CTA owns
-  int prefetch;           // the expanded layer is not being written by the launch before: weights may be fetched ahead of the dependency wait
   uint32_t split_mask;    // summed ensemble on one shared input, run as ONE cluster of all orders: bit k marks the order (k > 0)
                           // that opens the next predictor, whose chain the epilogue starts from zero
   int slice_tokens;       // tokens of a slice: the CTAs of slice z compute the tokens [z, z + 1) * slice_tokens
@@ -221,13 +220,12 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
   // A launch of this kernel that follows in the stream may be brought onto the SMs as they become free: its CTAs
   // then exist when this launch's last CTA ends, instead of being launched only then (a chain of small-token layers
   // otherwise pays a launch gap and a cold start per layer).  Until the launch before it is complete such a CTA
-  // touches nothing that launch may have written: with p.prefetch (the host knows that the expanded layer is not
-  // being written: its last call on this stream was no expansion) it builds its tables and fills its whole ring
-  // with WEIGHTS first, which belong to the layer alone, and waits only then, before the first access to
-  // activations, steps, bias or outputs; without it, it waits before its first access to global memory.
-  // Its own dependents start at once in the first case (the layer before was complete, or past this same point, when
-  // this CTA started, so no expansion queued earlier is still running beside them) and after the wait in the second.
-  if (p.prefetch) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // touches nothing that launch may have written: it builds its tables and fills its whole ring with WEIGHTS first, which
+  // belong to the layer alone, and waits only then, before the first access to activations, steps, bias or outputs.  (The
+  // layer is complete when a CTA starts: a launch directly behind an expansion is an ordinary one, see launch_stream.)
+  // Its own dependents start at once: the launch before was complete, or past this same point, when this CTA started, so no
+  // expansion queued earlier is still running beside them.
+  grid_release();
   if (threadIdx.x == 0) {
     abort_flag_s = 0;
     for (int s = 0; s < depth; ++s) {
@@ -241,10 +239,6 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
   // passes: pieces of at most pass_slabs slabs of the CTA's range (which lies in one branch)
   const int npass = min((cnt + p.pass_slabs - 1) / p.pass_slabs, kMaxPasses);
   for (int e = threadIdx.x; e < p.pass_slabs * NP * NT * 4 * 32; e += kThreads) sums[e] = 0;
-  if (!p.prefetch) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  }
   // ---- which orders keep each own slab, and where its 8 rows start
   for (int e = threadIdx.x; e < cnt * p.nkmax; e += kThreads) {
     const int li = e / p.nkmax, ko = e % p.nkmax;
@@ -355,10 +349,10 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
           __syncwarp();
         }
       };
-      if (p.prefetch && it0 < static_cast<uint32_t>(depth)) {
+      if (it0 < static_cast<uint32_t>(depth)) {
         // the first use of the ring: its weights go ahead of the wait for the launch before, its activation tiles after
         issue_jobs(1);
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        grid_wait();
         issue_jobs(2);
       } else {
         issue_jobs(0);
@@ -375,7 +369,7 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
     }
   } else {
     // ================================================================== consumer warps
-    if (p.prefetch) asm volatile("griddepcontrol.wait;" ::: "memory");   // (the steps and the bias are the caller's data)
+    grid_wait();   // (the steps and the bias are the caller's data)
     const int ksecond = MODE == 2 ? __ffs(p.split_mask) - 1 : 0;   // MODE 2: first order of the second predictor
     // scale products s_k * lambda_x and bias of every own slab (needed at the end of a pass only;
     // the loads overlap the first copies)
@@ -385,14 +379,14 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
       const BranchArgs& br = p.f.branch[branch];
       const int row0 = slabmeta[li * p.nkmax + ko];
       float v = 0.f;
-      if (row0 >= 0) v = __fmul_rn(__ldg(p.f.order[br.k_begin + ko].scales + row0 + r), __ldg((MODE == 2 && ko >= ksecond) ? p.f.branch[1].sx : br.sx));
+      if (row0 >= 0) v = __fmul_rn(__ldg(p.f.order[br.k_begin + ko].scales + row0 + r), __ldcg((MODE == 2 && ko >= ksecond) ? p.f.branch[1].sx : br.sx));
       cstab[e] = v;
     }
     for (int e = threadIdx.x; e < cnt * 8; e += 32 * kConsWarps) {
       const int r = e & 7, li = e >> 3;
       const int branch = (s0 + li) / p.slabs_per_branch;
       float v = 0.f;
-      if (p.f.bias && p.f.branch[branch].add_bias) v = __ldg(p.f.bias + (s0 + li - branch * p.slabs_per_branch) * 8 + r);
+      if (p.f.bias && p.f.branch[branch].add_bias) v = __ldcg(p.f.bias + (s0 + li - branch * p.slabs_per_branch) * 8 + r);
       biastab[e] = v;
     }
     asm volatile("bar.sync 1, %0;" ::"r"(32 * kConsWarps) : "memory");   // every consumer warp arrives here unconditionally
@@ -570,7 +564,7 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
         int next_order = 1;   // orders below this one have had their predictor boundaries handled
         const float bv = biastab[li * 8 + gid];
         int zp = 0;
-        if constexpr (ZP) zp = br.zp ? __ldg(br.zp) : 0;
+        if constexpr (ZP) zp = br.zp ? __ldcg(br.zp) : 0;
         auto close_chain = [&]() {
 #pragma unroll
           for (int t = 0; t < NT; ++t)
@@ -638,7 +632,7 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
             if (p.f.q8_out) {
               // inner layer of a branch: sigma, then the next layer's input quantizer (Sec. 3.2)
               v = apply_activation(v, p.f.relu);
-              const float os = __ldg(br.out_scale);
+              const float os = *br.out_scale;
               if (!(os >= 0.f && os < __uint_as_float(0x7f800000u))) raise_status(p.f.status, PIPE_ERR_INVALID_ARG);
               br.yq[static_cast<int64_t>(tok) * p.f.ldyq + c] = static_cast<int8_t>(quant_lane_exact(v, os));
               continue;
@@ -725,7 +719,6 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
   if (max_cluster > kMaxOrd) return PIPE_ERR_UNSUPPORTED;
   Params p;
   p.f = a;
-  p.prefetch = a.blob_settled ? 1 : 0;
   p.split_mask = split_mask;
   p.slice_tokens = slice_tokens;
   const int nt = a.T <= (zp ? 7 : 8) ? 1 : 2;
@@ -826,11 +819,11 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
                                static_cast<uint64_t>(a.ldxq), 128, 16, true))
       return PIPE_ERR_CUDA;
   if (!kernel_info(kern, dyn, &smem_max, &sms, &fixed)) return PIPE_ERR_CUDA;
-  // (programmatic stream serialization: see the kernel's first lines)
+  // (programmatic stream serialization, see the kernel's first lines; not where the blob may be under construction)
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = a.blob_settled ? 1 : 0;
   cfg.gridDim = dim3(grid, nslices, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = dyn;

@@ -72,7 +72,6 @@ struct Params {
   int pk;                 // packed bytes of one row of one reduction block (128*b/8)
   int shift;              // 8 - b
   int direct;             // the weights come from the layer's int8 copy in the operand layout (bits reads 8, shift 0)
-  int early;              // the expanded layer is settled: see the kernel's first lines
   uint32_t split_mask;    // summed ensemble on one shared input, run as ONE cluster of all orders: bit k is set where
                           // order k (k > 0) opens the next predictor, whose chain the epilogue starts from zero
   int conv_pw, conv_pp, conv_np, conv_chunks;   // patches per image row / per image / in total; 128-channel chunks per tap
@@ -431,6 +430,21 @@ __device__ __forceinline__ float4 load_row(const float* src, bool vec) {
   return make_float4(__ldcg(src), __ldcg(src + 1), __ldcg(src + 2), __ldcg(src + 3));
 }
 
+// Ordinary loads of the bias, which may have been written while this block was already standing here (so not __ldg) and which
+// every row of a tile reads again (so not from L2: 3 x 3 convolution 256 -> 256 on 32 x 56 x 56, with its quantization,
+// 135.6 -> 141.6 us).  Not volatile, so that the compiler may place them as freely as __ldg; their addresses hang on the tile's
+// record, which is read behind the dependency wait, and so do they.
+__device__ __forceinline__ float late_load(const float* p) {
+  float v;
+  asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 late_load4(const float* p) {
+  float4 v;
+  asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+
 struct EpiCtx {
   uint32_t tmem_base, tfull0, tempty0;
   uint32_t recbar0;   // kRecBufs barriers: the block record of the tile has landed
@@ -522,7 +536,7 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
       int c0, c1;
       asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(c0), "=r"(c1) : "r"(rec));
       const bool bias = p.f.branch[m].add_bias && p.f.bias;
-      for (int c = et; c < c1 - c0; c += 32 * kEpiWarps) x.bias_s[i * PIPE_BLOCK_CHANNELS + c] = bias ? __ldg(p.f.bias + c0 + c) : 0.f;
+      for (int c = et; c < c1 - c0; c += 32 * kEpiWarps) x.bias_s[i * PIPE_BLOCK_CHANNELS + c] = bias ? __ldcg(p.f.bias + c0 + c) : 0.f;
     }
     for (int r = et; r < kMaxN; r += 32 * kEpiWarps) {
       float sc;
@@ -686,7 +700,7 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
       float4 bq = make_float4(0.f, 0.f, 0.f, 0.f);
       if (!Q8 && add_bias && quad_ok && !(tma_out && 2 * grp + 1 < nch)) {
         const float* bp = bias_q + 16 * grp;
-        bq = make_float4(__ldg(bp), __ldg(bp + 1), __ldg(bp + 2), __ldg(bp + 3));
+        bq = make_float4(late_load(bp), late_load(bp + 1), late_load(bp + 2), late_load(bp + 3));
       }
       // (a sum into y: the rows this lane will add to are under way while the chain runs)
       float4 o[4];
@@ -743,7 +757,7 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
               if (p.f.bias) {
                 const float* bp = p.f.bias + c0 + 8 * chunk;
 #pragma unroll
-                for (int e = 0; e < 8; ++e) y[e] = __fadd_rn(y[e], __ldg(bp + e));
+                for (int e = 0; e < 8; ++e) y[e] = __fadd_rn(y[e], late_load(bp + e));
               }
 #pragma unroll
               for (int e = 0; e < 8; ++e) ysum[e] = y[e];
@@ -842,11 +856,11 @@ __device__ __forceinline__ void epilogue_role(const Params& p, const EpiCtx& x) 
             const float* bp = p.f.bias + c0 + 8 * chunk;
             float bo[8];
             if (bias_vec) {
-              const float4 b0 = __ldg(reinterpret_cast<const float4*>(bp)), b1 = __ldg(reinterpret_cast<const float4*>(bp) + 1);
+              const float4 b0 = late_load4(bp), b1 = late_load4(bp + 4);
               bo[0] = b0.x, bo[1] = b0.y, bo[2] = b0.z, bo[3] = b0.w, bo[4] = b1.x, bo[5] = b1.y, bo[6] = b1.z, bo[7] = b1.w;
             } else {
 #pragma unroll
-              for (int e = 0; e < 8; ++e) bo[e] = __ldg(bp + e);
+              for (int e = 0; e < 8; ++e) bo[e] = late_load(bp + e);
             }
 #pragma unroll
             for (int e = 0; e < 8; ++e) y[e] = __fadd_rn(y[e], bo[e]);
@@ -969,17 +983,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
 
   // A launch that follows in the stream may be brought onto the SMs as they become free (its CTAs then exist when this
   // launch's last pair ends).  Until the launch before it is complete such a pair touches nothing that launch may have
-  // written.  With p.early the host knows that the expanded layer is not being written (its last call on this stream was no
-  // expansion): what belongs to the layer -- tile counts, the first ring of weights -- is then read ahead of the wait, and
-  // what waits is the activation producer before its first copy and the epilogue before the steps, the bias and its outputs.
-  // Otherwise the pair waits here.  Its own dependents start after the wait only: a dependent that reads weights ahead of ITS
-  // wait then never runs beside an expansion queued before this launch.
-  // ACC: a later predictor of a summed ensemble.  The launch before it is the predictor before, whose blocks released it behind
-  // their wait: all that this launch reads but the sum itself is complete.  So its tiles start on the pairs that the launch
-  // before leaves idle in its last round, and only the epilogue waits.
-  const bool early = ACC || p.early;
-  if (!early) grid_wait();
-  if (ACC || !early) grid_release();
+  // written.  What belongs to the layer -- tile counts, the first ring of weights -- is read ahead of the wait: the layer is
+  // complete when a pair starts (a launch directly behind an expansion is an ordinary one, see launch_tc2).  What waits is the
+  // activation producer before its first copy and the epilogue before the steps, the bias and its outputs.  The pair's own
+  // dependents start behind the producer's wait, when everything queued before this launch is complete.
+  // ACC: a later predictor of a summed ensemble.  The launch before it is the predictor before, of this same call: either the
+  // first, which released it behind its producer's wait, or another ACC launch, which started no earlier.  In both cases
+  // everything queued before the call was complete by then, and with it all that this launch reads but the sum itself.  So its
+  // tiles start on the pairs that the launch before leaves idle in its last round, and only the epilogue waits.  Its own
+  // dependents start at once, for the same reason: all that they may read ahead of a wait of theirs was queued before the call.
+  if (ACC) grid_release();
   if constexpr (ZP) {
     // the row of ones behind the 127 token rows of every activation tile of the ring (sixteen equal bytes per piece,
     // whatever the swizzle does with the pieces); the copies never write it
@@ -1043,7 +1056,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
     // completion of both CTAs' copies is counted on the FIRST CTA's stage barrier, whose expected byte count
     // (both tiles) that CTA's lane 0 posts; a copy of the second CTA may land before that, which only lets the
     // transaction count run ahead of the expectation while the barrier's one arrival is still pending.
-    if (!ACC && p.early) {
+    if (!ACC) {
       grid_wait();
       grid_release();
     }
@@ -1165,7 +1178,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc2_forward_kernel(const __grid_c
   } else {
     // ------------------------------------------------------------------ epilogue warps
     // (inputs of this launch, and outputs that the launch before may still be reading or adding to: complete behind this)
-    if (early) grid_wait();
+    grid_wait();
     if (threadIdx.x >= kThreads - 2 * PIPE_MAX_ORDERS) {
       const int i = threadIdx.x - (kThreads - 2 * PIPE_MAX_ORDERS), m = i % PIPE_MAX_ORDERS;
       float v = 0.f;
@@ -1332,7 +1345,6 @@ static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_
   p.f = a;
   p.direct = direct ? 1 : 0;
   p.split_mask = split_mask;
-  p.early = a.blob_settled;
   const int row_bytes = direct ? round_up(a.I, kKStep) : a.kernel_row_bytes;   // bytes of a row over all reduction blocks
   if (direct) p.f.bits = 8;   // the kernel then treats the layer as one of int8 codes
   p.nkmax = max_cluster;
@@ -1425,8 +1437,9 @@ static pipe_status launch_tc2(const ForwardArgs& a, cudaStream_t stream, uint32_
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see the kernel's first lines
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  // (see the kernel's first lines; not where the blob may be under construction -- for a later predictor it no longer is)
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = a.blob_settled || a.branch[0].accumulate ? 1 : 0;
   cfg.gridDim = dim3(2 * ds.max_pairs, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = ds.dyn_smem;

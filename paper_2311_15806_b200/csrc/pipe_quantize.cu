@@ -196,7 +196,7 @@ __device__ __forceinline__ void load16(const QuantArgs& p, int64_t c, float (&v)
   if (p.vec_in && i0 + 16 <= p.I) {
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
-      const float4 f = __ldg(reinterpret_cast<const float4*>(row + i0) + w);
+      const float4 f = __ldcg(reinterpret_cast<const float4*>(row + i0) + w);
       v[4 * w] = f.x; v[4 * w + 1] = f.y; v[4 * w + 2] = f.z; v[4 * w + 3] = f.w;
     }
   } else {
@@ -229,11 +229,11 @@ __global__ void __launch_bounds__(kRangeThreads) act_range_kernel(const __grid_c
     for (; i + (kFlatUnroll - 1) * stride < p.quads; i += kFlatUnroll * stride) {
       float4 f[kFlatUnroll];
 #pragma unroll
-      for (int u = 0; u < kFlatUnroll; ++u) f[u] = __ldg(x + i + u * stride);
+      for (int u = 0; u < kFlatUnroll; ++u) f[u] = __ldcg(x + i + u * stride);
 #pragma unroll
       for (int u = 0; u < kFlatUnroll; ++u) range.add4(f[u]);
     }
-    for (; i < p.quads; i += stride) range.add4(__ldg(x + i));
+    for (; i < p.quads; i += stride) range.add4(__ldcg(x + i));
   } else {
     for (int64_t c = first; c < p.total_chunks; c += stride) {
       float v[16];
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(kQThreads) act_quantize_kernel(const __grid_co
 #pragma unroll
       for (int u = 0; u < kFlatUnroll; ++u) xq[-(i + u * stride)] = qz.quad(f[u]);
     }
-    for (; i < p.quads; i += stride) xq[-i] = qz.quad(__ldg(x - i));
+    for (; i < p.quads; i += stride) xq[-i] = qz.quad(__ldcg(x - i));
   } else {
     for (int64_t c = first; c < p.total_chunks; c += stride) {
       float v[16];
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(1024) act_small_kernel(const __grid_constant__
   const float4* x = reinterpret_cast<const float4*>(p.x);
   float4 f[PER];
 #pragma unroll
-  for (int u = 0; u < PER; ++u) f[u] = first + u * stride < quads ? __ldg(x + first + u * stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int u = 0; u < PER; ++u) f[u] = first + u * stride < quads ? __ldcg(x + first + u * stride) : make_float4(0.f, 0.f, 0.f, 0.f);
   q_cluster_sync();   // every CTA of the cluster runs before another one writes its shared memory
   Range<EX> range;
 #pragma unroll
