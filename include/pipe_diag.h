@@ -18,10 +18,9 @@ extern "C" {
 
 /* Which GEMM kernel the forward calls use from now on, for the whole process (so only for tests and
  * measurements; concurrent users of the library would all see the change):
- * 0 = automatic, 1 = CUDA-core kernel, 2 = one-SM tcgen05 kernel, 3 = small-token kernel (the weight-streaming
- * kernel, without token slices, where that one declines),
- * 4 = SM-pair tcgen05 kernel (clusters of two CTAs), 5 = small-token tcgen05 kernel.  A forced kernel that cannot run a request makes the
- * forward call return PIPE_ERR_UNSUPPORTED. */
+ * 0 = automatic, 1 = CUDA-core kernel, 2 = one-SM tcgen05 kernel, 3 = weight-streaming kernel (without token slices),
+ * 4 = SM-pair tcgen05 kernel (clusters of two CTAs), 5 = small-token tcgen05 kernel, 6 = small-token kernel.  A forced kernel
+ * that cannot run a request makes the forward call return PIPE_ERR_UNSUPPORTED. */
 pipe_status pipe_diag_select_kernel(int32_t which);
 
 /* Issue-bound rate of tcgen05.mma kind::i8 on this device: one CTA per SM issues `mma_per_cta`

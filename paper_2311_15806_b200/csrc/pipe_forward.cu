@@ -117,12 +117,10 @@ static pipe_status dispatch_forward(const ForwardArgs& a, const LayerInfo& L, in
   }
   if (choice == 1) return forward_reference(a, stream);
   if (choice == 2) return forward_tcgen05(a, stream);
-  if (choice == 3) {
-    const pipe_status st = forward_direct(a, stream);
-    return st == PIPE_ERR_UNSUPPORTED ? forward_stream(a, stream, false) : st;
-  }
+  if (choice == 3) return forward_stream(a, stream, false);
   if (choice == 4) return forward_tcgen05_pair(a, stream);
   if (choice == 5) return forward_decode_tc(a, stream);
+  if (choice == 6) return forward_direct(a, stream);
   // T <= 16: the small-token kernel; small layers in slices of 16 tokens: weight streaming; then the SM-pair kernel; the one-SM kernel for
   // layers without channel-block tables and what the pair kernel leaves it; the CUDA-core kernel for every other shape
   pipe_status st = PIPE_ERR_UNSUPPORTED;
