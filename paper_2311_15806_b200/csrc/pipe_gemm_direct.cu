@@ -610,11 +610,15 @@ pipe_status forward_direct(const ForwardArgs& a, cudaStream_t stream) {
   if (!sum_mode) return launch_direct(a, stream, false);
   // one launch for predictors that share their input, or two predictors of at most two orders each on inputs of their own; declined,
   // it is for the weight-streaming kernel, which also takes them together
-  bool shared = true;
+  bool together = true;
   for (int m = 1; m < a.num_branches; ++m)
-    shared = shared && a.branch[m].xq == a.branch[0].xq && a.branch[m].sx == a.branch[0].sx && a.branch[m].zp == a.branch[0].zp;
-  if (shared || (a.num_branches == 2 && a.branch[0].k_end - a.branch[0].k_begin <= 2 && a.branch[1].k_end - a.branch[1].k_begin <= 2))
-    return launch_direct(a, stream, true);
+    together = together && a.branch[m].xq == a.branch[0].xq && a.branch[m].sx == a.branch[0].sx && a.branch[m].zp == a.branch[0].zp;
+  together = together || (a.num_branches == 2 && a.branch[0].k_end - a.branch[0].k_begin <= 2 && a.branch[1].k_end - a.branch[1].k_begin <= 2);
+  // Predictors of more orders than one launch takes are one launch each: the streaming kernel takes no more of them together either, and
+  // its launches are the slower ones (shared input, cold weights, us, streaming / here: 4096 x 4096 int4 K = 12, M = 6, T = 1, 8, 16
+  // 55.5 / 47.6, 56.9 / 48.4, 66.8 / 51.7; 2048 x 2048 int8 K = 10, M = 3 27.3 / 12.8, 28.1 / 13.3, 26.3 / 14.7).
+  together = together && a.branch[a.num_branches - 1].k_end - a.branch[0].k_begin <= sd::kMaxOrd;
+  if (together) return launch_direct(a, stream, true);
   return launch_each_predictor(a, [&](const ForwardArgs& one, bool queue) { return launch_direct(one, stream, false, queue); });
 }
 
