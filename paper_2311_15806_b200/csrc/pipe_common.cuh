@@ -313,7 +313,8 @@ pipe_status forward_tcgen05(const ForwardArgs& a, cudaStream_t stream);
 pipe_status forward_tcgen05_pair(const ForwardArgs& a, cudaStream_t stream);   // two-SM form (clusters of two CTAs)
 // (slices: more than 16 tokens too, in slices of 16, where the launch is small enough for the rule in launch_stream)
 pipe_status forward_stream(const ForwardArgs& a, cudaStream_t stream, bool slices);
-pipe_status forward_direct(const ForwardArgs& a, cudaStream_t stream);         // T <= 16 (15 with a zero point)
+// T <= 16 (15 with a zero point); any: also the calls that it could take but the weight-streaming kernel is ahead on
+pipe_status forward_direct(const ForwardArgs& a, cudaStream_t stream, bool any);
 pipe_status forward_decode_tc(const ForwardArgs& a, cudaStream_t stream);      // T <= 16 on tcgen05 (decode-unit tables)
 
 }  // namespace pipe

@@ -103,8 +103,9 @@ static pipe_status dispatch_forward(const ForwardArgs& a, const LayerInfo& L, in
     // (the tensor-core accumulators hold 2^(8-b) times the sums)
     pipe_status st = PIPE_ERR_UNSUPPORTED;
     if (((static_cast<int64_t>(255) * L.qmax * L.I) << (8 - L.bits)) < (static_cast<int64_t>(1) << 31)) {
-      st = forward_direct(a, stream);
+      st = forward_direct(a, stream, false);
       if (st == PIPE_ERR_UNSUPPORTED) st = forward_stream(a, stream, true);
+      if (st == PIPE_ERR_UNSUPPORTED) st = forward_direct(a, stream, true);
       // A sum over predictors is one launch each on the pair kernel, one in all on the CUDA-core kernel, which is ahead on
       // short reduction axes while its work stays small (M predictors, tokens, us, CUDA cores / pair): 4672 x 112 M = 4
       // T = 47 46 / 73, 4016 x 64 M = 2 T = 350 25 / 38, 4160 x 240 M = 3 T = 98 49 / 58, 2448 x 176 M = 2 T = 139 35 / 37;
@@ -120,15 +121,17 @@ static pipe_status dispatch_forward(const ForwardArgs& a, const LayerInfo& L, in
   if (choice == 3) return forward_stream(a, stream, false);
   if (choice == 4) return forward_tcgen05_pair(a, stream);
   if (choice == 5) return forward_decode_tc(a, stream);
-  if (choice == 6) return forward_direct(a, stream);
+  if (choice == 6) return forward_direct(a, stream, true);
   // T <= 16: the small-token kernel; small layers in slices of 16 tokens: weight streaming; then the SM-pair kernel; the one-SM kernel for
   // layers without channel-block tables and what the pair kernel leaves it; the CUDA-core kernel for every other shape
   pipe_status st = PIPE_ERR_UNSUPPORTED;
   // (the small-token tcgen05 kernel, choice 5, is measured slower than the weight-streaming kernel -- widening the
   // codes through shared memory for the tensor core triples the shared-memory traffic per weight byte -- and is
   // therefore not on the automatic path)
-  st = forward_direct(a, stream);
+  st = forward_direct(a, stream, false);
   if (st == PIPE_ERR_UNSUPPORTED) st = forward_stream(a, stream, true);
+  // (256000 x 1024 int4 K = 4, whose tables the streaming kernel has no room for, T = 1: 160 us against 180 in the next one)
+  if (st == PIPE_ERR_UNSUPPORTED) st = forward_direct(a, stream, true);
   if (T <= 16 && st == PIPE_ERR_UNSUPPORTED) st = forward_decode_tc(a, stream);
   if (st == PIPE_ERR_UNSUPPORTED) st = forward_tcgen05_pair(a, stream);
   if (st == PIPE_ERR_UNSUPPORTED) st = forward_tcgen05(a, stream);

@@ -486,8 +486,8 @@ static const DeviceSetup& device_setup() {
 }  // namespace sd
 
 // summed: a.branch[0 .. num_branches) are the predictors of a summed ensemble, whose orders run as one cluster.
-// (queue = false: only say whether the kernel takes the call)
-static pipe_status launch_direct(const ForwardArgs& a, cudaStream_t stream, bool summed, bool queue = true) {
+// (queue = false: only say whether the kernel takes the call; any: also what the streaming kernel is ahead on, see the two rules below)
+static pipe_status launch_direct(const ForwardArgs& a, cudaStream_t stream, bool summed, bool any, bool queue = true) {
   using namespace sd;
   const bool zp = has_zero_point(a);   // (its row sums take the place of a token)
   if (a.T > (zp ? 15 : 16) || a.g % 8 != 0 || a.O % 8 != 0 || (zp && a.q8_out) || a.conv_on) return PIPE_ERR_UNSUPPORTED;
@@ -567,8 +567,9 @@ static pipe_status launch_direct(const ForwardArgs& a, cudaStream_t stream, bool
   p.pairs_max = (p.own_max * p.nkmax + inputs + 1) / 2;
   const int nt = a.T <= (zp ? 7 : 8) ? 1 : 2;
   // The warps' rings: as deep as half of an SM's shared memory allows, with sets of two pairs where three would leave less than
-  // two stages (8 bits from 8 tokens on, 2 bits from 13; a CTA that takes more than half of an SM makes the grid two rounds:
-  // 4096 x 4096 int8 K = 2, T = 8 10 -> 18 us).  The whole of an SM only where even that does not fit.
+  // two stages (8 bits from 8 tokens on, 2 bits from 13), then of one.  A CTA that takes more than half of an SM makes the grid two
+  // rounds (4096 x 4096 int8 K = 2, T = 8 10 -> 18 us): the whole of an SM only where even that does not fit, whose tables are those of
+  // 100 thousand channels and more.
   const int64_t tables = 128 + static_cast<int64_t>(p.pairs_max) * nt * 512 + static_cast<int64_t>(p.own_max) * (p.nkmax * 36 + 32);
   int64_t depth = 0;
   for (p.set_pairs = kPairs; p.set_pairs > 0; --p.set_pairs) {
@@ -576,17 +577,27 @@ static pipe_status launch_direct(const ForwardArgs& a, cudaStream_t stream, bool
     depth = (ds.smem_half - tables) / (kWarps * p.stage_bytes);
     if (depth >= 2 || depth >= p.nstages) break;
   }
-  if (p.set_pairs == 0) {
+  const bool two_rounds = p.set_pairs == 0;
+  if (two_rounds) {
     p.set_pairs = 1;
     depth = (ds.smem_max - tables) / (kWarps * p.stage_bytes);
   }
   if (depth > kMaxDepth) depth = kMaxDepth;
   if (depth > p.nstages) depth = p.nstages;
   if (depth < 1) return PIPE_ERR_UNSUPPORTED;
-  // (2 bits: a stage's activations, 256 codes of every token, then outweigh its weights, and the weight-streaming kernel, which
-  // brings them once per CTA, is ahead: 11008 x 2048 K = 8 M = 2, T = 13 and 16 30 and 41 us against 27; 8192 x 8192 K = 8 M = 4,
-  // T = 16 76 against 58, but T = 13, two pairs, 44 against 58)
-  if (a.bits == 2 && (p.set_pairs < 2 || (p.set_pairs < kPairs && p.nkmax > 2))) return PIPE_ERR_UNSUPPORTED;
+  // Two rounds cost by the rows, the weight-streaming kernel by the slabs and the positions of their order pairs, half empty or not.
+  // So they pay on one token tile where a branch has more than four orders (eight positions) and at most three rows per output channel
+  // (us, streaming / here: 128256 x 2048 int4 K = 8, 2.75 rows, T = 1 and 8 200 / 154 and 200 / 180; 128256 x 2048 int8 K = 5, two rows, T = 8
+  // 183 / 139; 128256 x 1024 int4 K = 6, 3.5 rows, T = 1 104 / 120; four orders and fewer: 200000 x 1024 K = 4, T = 1 90 / 129, 128256 x 2048
+  // K = 4 M = 2, T = 8 94 / 169, K = 6 M = 2 152 / 225; two token tiles: 128256 x 4096 K = 4, T = 16 217 / 338, 98304 x 2048 K = 8 169 / 223).
+  // 2 bits: 65536 x 2048 K = 8, T = 8 75 / 85, M = 2 74 / 90.
+  if (two_rounds && !any && (nt > 1 || a.bits == 2 || p.nkmax <= 4 || total > 3 * static_cast<int64_t>(a.O) * units)) return PIPE_ERR_UNSUPPORTED;
+  // 2 bits, two token tiles, sets of one pair: a stage's activations, 256 codes of every token, are more than twice its weights, and every set
+  // brings them; the streaming kernel brings them once per CTA (8192 x 8192 K = 8 M = 4, T = 16 58 / 82 us, 8192 x 4096 M = 2 28 / 44,
+  // 11008 x 2048 23 / 28; kept rows a quarter: 19.4 / 18.6).  Sets of two pairs: T = 13 58 / 45, 8192 x 4096 28.4 / 25.4, 4096 x 4096 K = 4,
+  // T = 16 11.2 / 9.9, 11008 x 4096 K = 3 20.8 / 16.0, 4096 x 11008 K = 6 M = 2 22.6 / 23.6.  One token tile, one pair: 65536 x 2048 K = 8, T = 6
+  // 75 / 52.
+  if (a.bits == 2 && nt > 1 && p.set_pairs < 2 && !any) return PIPE_ERR_UNSUPPORTED;
   p.depth = static_cast<int>(depth);
   if (!queue) return PIPE_OK;
   cudaLaunchConfig_t cfg = {};
@@ -604,10 +615,10 @@ static pipe_status launch_direct(const ForwardArgs& a, cudaStream_t stream, bool
   return launch_status();
 }
 
-pipe_status forward_direct(const ForwardArgs& a, cudaStream_t stream) {
+pipe_status forward_direct(const ForwardArgs& a, cudaStream_t stream, bool any) {
   if (a.T == 0) return PIPE_OK;
   const bool sum_mode = a.num_branches > 1 && a.branch[1].accumulate;
-  if (!sum_mode) return launch_direct(a, stream, false);
+  if (!sum_mode) return launch_direct(a, stream, false, any);
   // one launch for predictors that share their input, or two predictors of at most two orders each on inputs of their own; declined,
   // it is for the weight-streaming kernel, which also takes them together
   bool together = true;
@@ -618,8 +629,8 @@ pipe_status forward_direct(const ForwardArgs& a, cudaStream_t stream) {
   // its launches are the slower ones (shared input, cold weights, us, streaming / here: 4096 x 4096 int4 K = 12, M = 6, T = 1, 8, 16
   // 55.5 / 47.6, 56.9 / 48.4, 66.8 / 51.7; 2048 x 2048 int8 K = 10, M = 3 27.3 / 12.8, 28.1 / 13.3, 26.3 / 14.7).
   together = together && a.branch[a.num_branches - 1].k_end - a.branch[0].k_begin <= sd::kMaxOrd;
-  if (together) return launch_direct(a, stream, true);
-  return launch_each_predictor(a, [&](const ForwardArgs& one, bool queue) { return launch_direct(one, stream, false, queue); });
+  if (together) return launch_direct(a, stream, true, any);
+  return launch_each_predictor(a, [&](const ForwardArgs& one, bool queue) { return launch_direct(one, stream, false, any, queue); });
 }
 
 }  // namespace pipe

@@ -752,7 +752,8 @@ static pipe_status launch_stream(const ForwardArgs& a, cudaStream_t stream, bool
   }
 #undef PIPE_ST_PICK
   // the same kernel without per-slab branches, by slab slots per warp (one order pair, 2 or 3 slots -- more would spill; two
-  // inputs, 1 or 2).  Two token tiles: the slices; up to 8 tokens the small-token kernel leaves this one next to nothing.
+  // inputs, 1 or 2).  Two token tiles: the slices; on one, the small-token kernel leaves this one only layers of many passes, which such a
+  // form does not serve (200000 x 1024 int4 K = 4, 128256 x 2048 M = 2 and the like).
   auto full_kernel = [&](int slots) -> void (*)(const Params) {
     if (nt == 1) return nullptr;
     if (distinct) {
