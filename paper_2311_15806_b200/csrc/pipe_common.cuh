@@ -198,6 +198,33 @@ __device__ __forceinline__ float max3_abs_nan(float a, float b, float c) {
   return d;
 }
 
+// Operands of the warp-level MMA from the streaming layout: int8 lanes (times 2^(8-b)) of MMA number mm of a 16-byte packed chunk: r0 covers the chunk's reduction offsets
+// 8mm..8mm+3, r1 covers 8mm+4..8mm+7.
+template <int BITS>
+__device__ __forceinline__ void mma_frag(const uint4& w, int mm, uint32_t& r0, uint32_t& r1) {
+  const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+  if (BITS == 8) {
+    r0 = ww[2 * mm];
+    r1 = ww[2 * mm + 1];
+  } else if (BITS == 4) {
+    r0 = (ww[mm] << 4) & 0xF0F0F0F0u;
+    r1 = ww[mm] & 0xF0F0F0F0u;
+  } else {
+    const uint32_t x = ww[mm >> 1];
+    const int h = 2 * (mm & 1);
+    r0 = (x << (6 - 2 * h)) & 0xC0C0C0C0u;
+    r1 = (x << (4 - 2 * h)) & 0xC0C0C0C0u;
+  }
+}
+
+// Number of compacted rows of an order before channel c of the branch (c a multiple of 8, c <= O).
+__device__ __forceinline__ int rows_before(const int32_t* cum, int c, int O, int g) {
+  if (c >= O) return __ldg(cum + O / g) * g;
+  const int j = c / g;
+  const int lo = __ldg(cum + j), hi = __ldg(cum + j + 1);
+  return lo * g + (hi > lo ? c - j * g : 0);
+}
+
 // sigma of Eq. 9 for an inner layer (Sec. 3.2 names ReLU, SiLU, GeLU and sigmoid), in binary32: kind 0 identity,
 // 1 ReLU, 2 SiLU v / (1 + exp(-v)), 3 GeLU v (1 + erf(v / sqrt 2)) / 2, 4 sigmoid 1 / (1 + exp(-v)).
 __device__ __forceinline__ float apply_activation(float v, int kind) {

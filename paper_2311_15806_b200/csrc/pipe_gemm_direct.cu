@@ -73,33 +73,6 @@ __device__ __forceinline__ void mma_s8(int (&c)[4], uint32_t a0, uint32_t a1, ui
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// int8 lanes (times 2^(8-b)) of MMA number mm of a 16-byte packed chunk: r0 covers the chunk's reduction offsets
-// 8mm..8mm+3, r1 covers 8mm+4..8mm+7 (see the streaming layout).
-template <int BITS>
-__device__ __forceinline__ void frag(const uint4& w, int mm, uint32_t& r0, uint32_t& r1) {
-  const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-  if (BITS == 8) {
-    r0 = ww[2 * mm];
-    r1 = ww[2 * mm + 1];
-  } else if (BITS == 4) {
-    r0 = (ww[mm] << 4) & 0xF0F0F0F0u;
-    r1 = ww[mm] & 0xF0F0F0F0u;
-  } else {
-    const uint32_t x = ww[mm >> 1];
-    const int h = 2 * (mm & 1);
-    r0 = (x << (6 - 2 * h)) & 0xC0C0C0C0u;
-    r1 = (x << (4 - 2 * h)) & 0xC0C0C0C0u;
-  }
-}
-
-// Number of compacted rows of an order before channel c of the branch (c a multiple of 8, c <= O).
-__device__ __forceinline__ int rows_before(const int32_t* cum, int c, int O, int g) {
-  if (c >= O) return __ldg(cum + O / g) * g;
-  const int j = c / g;
-  const int lo = __ldg(cum + j), hi = __ldg(cum + j + 1);
-  return lo * g + (hi > lo ? c - j * g : 0);
-}
-
 // The CTA's rows: order ko has `rows` of them from compacted row `row0` on, which are the 8-row groups g0 .. of the CTA's pool.
 // Groups of one input are consecutive; the next input's start at an even number, so no pair mixes inputs.
 struct Rows {
@@ -224,8 +197,8 @@ __device__ __forceinline__ void run_pairs(const Params& p, const Rows& rows, uin
 #pragma unroll
           for (int u = 0; u < N; ++u) {
             uint32_t a0, a1, b0, b1;
-            frag<BITS>(w[2 * u], mm, a0, a1);
-            frag<BITS>(w[2 * u + 1], mm, b0, b1);
+            mma_frag<BITS>(w[2 * u], mm, a0, a1);
+            mma_frag<BITS>(w[2 * u + 1], mm, b0, b1);
 #pragma unroll
             for (int t = 0; t < NT; ++t) mma_s8(acc[u][t], a0, b0, a1, b1, m ? x[t].z : x[t].x, m ? x[t].w : x[t].y);
           }
@@ -252,6 +225,8 @@ __device__ __forceinline__ void run_pairs(const Params& p, const Rows& rows, uin
 // SUMMED: a summed ensemble in one launch (every predictor's chain starts from zero, the bias closes the first one, the chains
 // are added in ascending predictor order), whether the predictors share their input or not.
 // ZP: asymmetric activations, sum_i (c - z) q = sum_i c q - z sum_i q.
+// (Two CTAs per SM leave a thread 128 registers.  Five of the 24 forms spill some: 2 bits with two token tiles, 12 to 24 bytes stored, and the
+// plain 8-bit one with one tile, 16.)
 template <int BITS, int NT, bool SUMMED, bool ZP>
 __global__ void __launch_bounds__(kThreads, 2) direct_forward_kernel(const __grid_constant__ Params p) {
   extern __shared__ uint8_t smem_raw[];

@@ -138,33 +138,6 @@ __device__ __forceinline__ void mma_s8(int (&c)[4], uint32_t a0, uint32_t a1, ui
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// int8 lanes (times 2^(8-b)) of MMA number mm of a 16-byte packed chunk: r0 covers the chunk's
-// reduction offsets 8mm..8mm+3, r1 covers 8mm+4..8mm+7 (see the streaming layout).
-template <int BITS>
-__device__ __forceinline__ void frag(const uint4& w, int mm, uint32_t& r0, uint32_t& r1) {
-  const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-  if (BITS == 8) {
-    r0 = ww[2 * mm];
-    r1 = ww[2 * mm + 1];
-  } else if (BITS == 4) {
-    r0 = (ww[mm] << 4) & 0xF0F0F0F0u;
-    r1 = ww[mm] & 0xF0F0F0F0u;
-  } else {
-    const uint32_t x = ww[mm >> 1];
-    const int h = 2 * (mm & 1);
-    r0 = (x << (6 - 2 * h)) & 0xC0C0C0C0u;
-    r1 = (x << (4 - 2 * h)) & 0xC0C0C0C0u;
-  }
-}
-
-// Number of compacted rows of an order before channel c of the branch (c a multiple of 8, c <= O).
-__device__ __forceinline__ int rows_before(const int32_t* cum, int c, int O, int g) {
-  if (c >= O) return __ldg(cum + O / g) * g;
-  const int j = c / g;
-  const int lo = __ldg(cum + j), hi = __ldg(cum + j + 1);
-  return lo * g + (hi > lo ? c - j * g : 0);
-}
-
 // FULL != 0: a consumer warp has FULL slab slots per pass and (nearly) every one of them holds a slab (the host knows:
 // one pass, FULL = ceil(slabs of a CTA / warps of a group)): the loop over a warp's slabs then runs without its per-slab
 // branches -- an absent chunk takes part with zero weights -- so that the slabs' load-and-MMA chains are one block the
@@ -498,8 +471,8 @@ __global__ void __launch_bounds__(kThreads, 1) stream_forward_kernel(const __gri
 #pragma unroll
               for (int mm = 0; mm < 2 * XCH; ++mm) {
                 uint32_t a0, a1, b0, b1;
-                frag<BITS>(wa, mm, a0, a1);
-                frag<BITS>(wb, mm, b0, b1);
+                mma_frag<BITS>(wa, mm, a0, a1);
+                mma_frag<BITS>(wb, mm, b0, b1);
 #pragma unroll
                 for (int t = 0; t < NT; ++t) {
                   const uint4& xr = xv[MODE == 2 ? q : 0][mm >> 1][t];
