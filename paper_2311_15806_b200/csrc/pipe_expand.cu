@@ -839,7 +839,7 @@ constexpr int kChainMaxI = 16384;
 // The packing is arithmetic too: sum_e (code_e + 2^(b-1)) 2^(b e) over the codes of 16 bits of a packed word, on top of
 // 1.5 * 2^23, is exact in binary32 and stands in the low 16 bits of its pattern; the offsets are the fields' sign bits, which
 // an exclusive or takes away.  A pair holds the elements i and i + 2 of a quad, so that its halves lead to the low and to the
-// high half of the same word.  (7.3 instructions per element and level in all, issue slots 72 % busy, against 11 with scalar
+// high half of the same word.  (9.1 instructions per element and level in all for int4, 7.3 for 2 bits, issue slots 72 % busy, against 11 with scalar
 // operations and byte permutations: 11008 x 4096 int4 K = 4 73 -> 66 us, 8192 x 8192 ternary K = 8 184 -> 155.)
 // Ordinary weights replay a few chunks in a thousand.  Weights on a coarse grid put quotients on a boundary all over, at
 // every level; a block that had to replay in an eighth of its threads therefore keeps, from the next level on, the old

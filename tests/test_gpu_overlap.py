@@ -78,7 +78,7 @@ def test_expansion_of_codes_at_the_ends_of_their_range(oracle, bits, K, O, I, g)
     H.assert_expansion_matches(layer, e, oracle)
 
 
-# The small-token kernel.  T around the token tiles of eight (seven and fifteen beside a zero point) and the epilogue's four;
+# The small-token kernel.  T around the token tiles of eight (seven and fifteen beside a zero point);
 # reduction axes of one stage, of fewer stages than a CTA has warps and of more than a ring holds, odd block counts (half a stage
 # with 2-bit codes), rows that are no whole 16 bytes; from one pair of row groups per CTA to many sets of three; orders that
 # keep next to nothing

@@ -1,7 +1,7 @@
 """Stream order between the expansion and the forward kernels.
 
-The forward kernels start under programmatic stream serialization and the weight-streaming kernel copies packed codes
-ahead of its dependency wait; a forward call queued directly behind an expansion on the same stream must nevertheless
+The forward kernels start under programmatic stream serialization and copy packed codes
+ahead of their dependency wait; a forward call queued directly behind an expansion on the same stream must nevertheless
 see that expansion's blob.  The weights change between rounds and nothing synchronizes inside a round, so a forward
 that read the blob too early would return the previous round's outputs."""
 import numpy as np
@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 
 CASES = [
     # O, I, T, bits, K, g, n_keep, M
-    (1024, 1024, 1, 4, 3, 8, 32, 1),       # weight-streaming kernel
+    (1024, 1024, 1, 4, 3, 8, 32, 1),       # small-token kernel
     (1024, 1024, 16, 8, 2, 8, 64, 2),
     (768, 1024, 200, 4, 3, 8, 24, 1),      # SM-pair kernel
 ]
