@@ -21,7 +21,8 @@
  *     may overlap the tail of the preceding launch on `stream`, and they start copying the
  *     blob's packed codes during that overlap.  The
  *     library orders this correctly against its own calls (a forward call that directly follows
- *     pipe_expand_weights* on the same stream waits for it in full).  A caller that writes
+ *     pipe_expand_weights* on the same stream waits for it in full; so does one on a stream that
+ *     has joined behind it, inside a stream capture too).  A caller that writes
  *     d_blob by other means must let that work complete -- an event, a synchronize, or any other
  *     library call in between -- before queueing a forward call on the same stream.  Inputs
  *     other than d_blob (activations, scales, bias, outputs) are only touched after the

@@ -1318,6 +1318,22 @@ static bool chain_fits(const LayerInfo& L, const float* W, int64_t ldw, ChainPla
 
 using namespace pipe;
 
+// In a stream capture the mark is not enough: a launch on ANOTHER stream that has joined behind the expansion gets an edge of the same
+// kind as one behind it on its own stream, programmatic, where outside of captures an event stands for full completion.  The
+// expansion's last kernel releases its dependents early, so it is followed by an empty node, and what comes behind it has an ordinary edge.
+static pipe_status close_in_capture(cudaStream_t s) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  cudaGraph_t graph = nullptr;
+  const cudaGraphNode_t* deps = nullptr;
+  size_t n = 0;
+  cudaError_t e = cudaStreamGetCaptureInfo(s, &status, nullptr, &graph, &deps, &n);
+  if (e != cudaSuccess || status != cudaStreamCaptureStatusActive) return cuda_ok(e);
+  cudaGraphNode_t end = nullptr;
+  e = cudaGraphAddEmptyNode(&end, graph, deps, n);
+  if (e == cudaSuccess) e = cudaStreamUpdateCaptureDependencies(s, &end, 1, cudaStreamSetCaptureDependencies);
+  return cuda_ok(e);
+}
+
 extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const float* d_W, int64_t ldw, void* d_blob,
                                            size_t blob_bytes, void* d_ws, size_t ws_bytes, void* stream) {
   LayerInfo L;
@@ -1566,7 +1582,8 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
     }
   }
   mark_expansion(s);   // a forward call that follows on this stream must not read the blob ahead of its dependency wait
-  return launch_status();
+  st = launch_status();
+  return st == PIPE_OK ? close_in_capture(s) : st;
 }
 
 // ------------------------------------------------------------------------------------------------
