@@ -33,6 +33,7 @@ void count_launch(int n = 1);
 int kernel_choice();
 // Streams (of whichever device is current) whose last library call was an expansion (which writes the blob a forward call on the
 // same stream may be about to read): an expansion marks its stream, every other call that has queued a kernel takes the mark away.
+// (Calls inside a stream capture do neither, and find no mark.)
 void mark_expansion(cudaStream_t stream);
 bool take_expansion_mark(cudaStream_t stream);
 bool expansion_marked(cudaStream_t stream);   // the same question without clearing the mark

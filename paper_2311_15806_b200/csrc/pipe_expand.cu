@@ -1318,16 +1318,18 @@ static bool chain_fits(const LayerInfo& L, const float* W, int64_t ldw, ChainPla
 
 using namespace pipe;
 
-// In a stream capture the mark is not enough: a launch on ANOTHER stream that has joined behind the expansion gets an edge of the same
+// In a stream capture a mark would not do: a launch on ANOTHER stream that has joined behind the expansion gets an edge of the same
 // kind as one behind it on its own stream, programmatic, where outside of captures an event stands for full completion.  The
 // expansion's last kernel releases its dependents early, so it is followed by an empty node, and what comes behind it has an ordinary edge.
-static pipe_status close_in_capture(cudaStream_t s) {
+// captured: the stream is in a capture.
+static pipe_status close_in_capture(cudaStream_t s, bool* captured) {
   cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
   cudaGraph_t graph = nullptr;
   const cudaGraphNode_t* deps = nullptr;
   size_t n = 0;
   cudaError_t e = cudaStreamGetCaptureInfo(s, &status, nullptr, &graph, &deps, &n);
   if (e != cudaSuccess || status != cudaStreamCaptureStatusActive) return cuda_ok(e);
+  *captured = true;
   cudaGraphNode_t end = nullptr;
   e = cudaGraphAddEmptyNode(&end, graph, deps, n);
   if (e == cudaSuccess) e = cudaStreamUpdateCaptureDependencies(s, &end, 1, cudaStreamSetCaptureDependencies);
@@ -1581,9 +1583,11 @@ extern "C" pipe_status pipe_expand_weights(const pipe_layer_desc* desc, const fl
       count_launch(1);
     }
   }
-  mark_expansion(s);   // a forward call that follows on this stream must not read the blob ahead of its dependency wait
   st = launch_status();
-  return st == PIPE_OK ? close_in_capture(s) : st;
+  bool captured = false;
+  const pipe_status closed = close_in_capture(s, &captured);
+  if (!captured) mark_expansion(s);   // a forward call that follows on this stream must not read the blob ahead of its dependency wait
+  return st == PIPE_OK ? closed : st;
 }
 
 // ------------------------------------------------------------------------------------------------

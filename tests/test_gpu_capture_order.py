@@ -128,3 +128,38 @@ def test_a_forward_behind_a_replayed_expansion(T):
     torch.cuda.synchronize()
     for r, y in got:
         assert torch.equal(y.view(torch.int32), want[r].view(torch.int32))
+
+
+@pytest.mark.parametrize("T", [1, 48, 200])
+def test_a_forward_behind_an_expansion_and_a_capture(T):
+    """A forward captured on the expansion's stream has not run there: the next one on the stream still stands directly behind the
+    expansion."""
+    c = Case(T, 3)
+    want = [c.want(r) for r in range(4)]
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    got, graphs = [], []
+    with torch.cuda.stream(s):
+        for r in (1, 2, 3, 0):
+            torch.mul(c.base, 1.0 + r, out=c.W)
+            c.expand(s)
+            graph = torch.cuda.CUDAGraph()
+            graph.capture_begin()
+            c.forward(s)
+            graph.capture_end()
+            c.forward(s)
+            got.append((r, c.y.clone()))
+            graphs.append(graph)
+    torch.cuda.synchronize()
+    for r, y in got:
+        assert torch.equal(y.view(torch.int32), want[r].view(torch.int32))
+    for r in (2, 1):
+        c.W.copy_(c.base * (1.0 + r))
+        torch.cuda.synchronize()
+        with torch.cuda.stream(s):
+            c.expand(s)
+            graphs[r].replay()   # behind the expansion, as a graph
+            y = c.y.clone()
+        torch.cuda.synchronize()
+        assert torch.equal(y.view(torch.int32), want[r].view(torch.int32))

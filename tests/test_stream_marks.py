@@ -1,5 +1,6 @@
 """The table of streams whose last library call was an expansion (csrc/pipe_marks.h): host logic, compiled on its own."""
 import os
+import re
 import subprocess
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2311_15806_b200", "csrc")
@@ -79,3 +80,12 @@ def test_the_library_asks_for_the_device_of_a_stream():
     text = open(os.path.join(CSRC, "pipe_layout.cu")).read()
     body = text[text.index("key_of("):text.index("void mark_expansion(")]
     assert "cudaGetDevice(&dev)" in body and "stream_key(dev," in body
+
+
+def test_calls_inside_a_capture_leave_the_marks_alone():
+    text = open(os.path.join(CSRC, "pipe_layout.cu")).read()
+    for name in ("take_expansion_mark", "expansion_marked"):
+        body = text[text.index(f"bool {name}(cudaStream_t stream)"):]
+        assert "!capturing(stream) &&" in body[:body.index("}")]
+    text = open(os.path.join(CSRC, "pipe_expand.cu")).read()
+    assert re.findall(r"[^\n]*mark_expansion\(s\)", text) == ["  if (!captured) mark_expansion(s)"]
