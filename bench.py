@@ -116,14 +116,15 @@ def workload_spec(name: str):
 # DRAM read + write bytes of ONE launch of the GEMM kernel, from one ncu capture per workload
 # (profiles/ncu_pair_kernel.txt, profiles/ncu_stream_kernel.txt).  A workload without a capture has no entry and reports null.
 NCU_DRAM_BYTES_PER_LAUNCH = {
-    "cfg2": 28441344 + 50646272,
-    "cfg3a": 9420800 + 46272512,
-    "cfg4a_t4096": 90903552 + 313437696,
-    "cfg5": 437495808 + 1026217472,
-    "cfg4a_t1": 56560384 + 45056,
-    "cfg4a_t16": 56688128 + 265472,
-    "cfg4a_t4096+int8_copy": 147986944 + 315521536,
-    "cfg3b+int8_copy": 31184384 + 722176,
+    "cfg2": 29143552 + 50309376,
+    "cfg3a": 9416960 + 46574592,
+    "cfg4a_t4096": 91214336 + 313686016,
+    "cfg5": 458975488 + 1029482496,
+    "cfg4a_t1": 56576000 + 47616,
+    "cfg4a_t16": 56701184 + 105216,
+    "cfg4b_t1": 56507392 + 69376,
+    "cfg4a_t4096+int8_copy": 148247552 + 315334144,
+    "cfg3b+int8_copy": 31184384 + 579584,
 }
 
 
