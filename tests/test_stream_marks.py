@@ -84,8 +84,7 @@ def test_the_library_asks_for_the_device_of_a_stream():
 
 def test_calls_inside_a_capture_leave_the_marks_alone():
     text = open(os.path.join(CSRC, "pipe_layout.cu")).read()
-    for name in ("take_expansion_mark", "expansion_marked"):
-        body = text[text.index(f"bool {name}(cudaStream_t stream)"):]
-        assert "!capturing(stream) &&" in body[:body.index("}")]
+    assert "g_marks.marked(key_of(stream)) && !capturing(stream); }" in text[text.index("bool expansion_marked(cudaStream_t stream) {"):]
+    assert "bool take_expansion_mark(cudaStream_t stream) { return expansion_marked(stream) && g_marks.take(" in text
     text = open(os.path.join(CSRC, "pipe_expand.cu")).read()
     assert re.findall(r"[^\n]*mark_expansion\(s\)", text) == ["  if (!captured) mark_expansion(s)"]
